@@ -57,11 +57,6 @@ static cudaError_t attrs_n() {
 
 static cudaError_t set_attrs() {
     cudaError_t e;
-    if ((e = smem_attr(k_pass_z_strain<float>)) != cudaSuccess) return e;
-    if ((e = smem_attr(k_pass_axis<float, +1, 1>)) != cudaSuccess) return e;
-    if ((e = smem_attr(k_pass_axis<float, -1, 1>)) != cudaSuccess) return e;
-    if ((e = smem_attr(k_pass_x_stress<float>)) != cudaSuccess) return e;
-    if ((e = smem_attr(k_pass_z_div<float>)) != cudaSuccess) return e;
     if ((e = attrs_n<4, 4>()) != cudaSuccess) return e;
     if ((e = attrs_n<8, 4>()) != cudaSuccess) return e;
     if ((e = attrs_n<8, 8>()) != cudaSuccess) return e;
@@ -184,50 +179,43 @@ extern "C" bloch_status bloch_apply_K_noalloc(bloch_plan* pl, int32_t nb, const 
 
     cudaError_t e = cudaMemcpyAsync(kvec, k, k_bytes, cudaMemcpyHostToDevice, pl->stream);
     if (e != cudaSuccess) return set_cuda_error(e, "cudaMemcpyAsync (wave vectors)");
+    const uint64_t launched = pl->launches;
     const int qblocks = (int)std::min<long long>(1024, ((long long)nb * S + 255) / 256);
     k_qtab<float><<<qblocks, 256, 0, pl->stream>>>(kvec, pl->d_xi, pl->Nx, pl->Ny, pl->Nz, nb, pl->qscale, qtab);
 
     // the five passes of the K-apply, the kernels of bloch_apply_K (two-stage
     // register passes on axes of 16..128, shared-memory Stockham passes otherwise)
-    const Geo& g = pl->geo_f;
-    const TileCfg& t = pl->tile_f;
-    const long long pxy = (long long)pl->Nx * pl->Ny, pxz = (long long)pl->Nx * pl->Nz,
-                    pyz = (long long)pl->Ny * pl->Nz;
-    dim3 g1((unsigned)((pxy + t.Pz5 - 1) / t.Pz5), nb);
-    dim3 g2((unsigned)((pxz + t.Py2 - 1) / t.Py2), nb * 6);
-    dim3 g3((unsigned)((pyz + t.Px7 - 1) / t.Px7), nb);
     const float2* uu = (const float2*)u;
     float2* out = (float2*)Ku;
     const bool fz = fast_len(pl->Nz), fy = fast_len(pl->Ny) || pl->Ny == 256, fx = fast_len(pl->Nx);
     if (fz) {
         NOALLOC_SWITCH(pl->Nz, z_strain, pl, nb, uu, E, qtab);
     } else {
-        k_pass_z_strain<float><<<g1, 256, t.smem_z5, pl->stream>>>(uu, E, qtab, pl->d_twf[2], g, t.Pz5);
+        pass_z_strain<float>(pl, nb, uu, E, qtab);
     }
     if (fy) {
         if (pl->Ny == 256) y_pass<16, 16>(pl, +1, nb, E);
         else NOALLOC_SWITCH(pl->Ny, y_pass, pl, +1, nb, E);
     } else {
-        k_pass_axis<float, +1, 1><<<g2, 256, t.smem_y2, pl->stream>>>(E, E, pl->d_twf[1], g, t.Py2, 1.0f);
+        pass_axis<float>(pl, 1, +1, 6 * nb, E, E, 1.0f);
     }
     if (fx) {
         NOALLOC_SWITCH(pl->Nx, x_stress, pl, nb, E);
     } else {
-        k_pass_x_stress<float><<<g3, 256, t.smem_x7, pl->stream>>>(E, pl->d_ids, pl->d_Cf, pl->d_twf[0], g, t.Px7);
+        pass_x_stress<float>(pl, nb, E);
     }
     if (fy) {
         if (pl->Ny == 256) y_pass<16, 16>(pl, -1, nb, E);
         else NOALLOC_SWITCH(pl->Ny, y_pass, pl, -1, nb, E);
     } else {
-        k_pass_axis<float, -1, 1><<<g2, 256, t.smem_y2, pl->stream>>>(E, E, pl->d_twf[1], g, t.Py2, 1.0f);
+        pass_axis<float>(pl, 1, -1, 6 * nb, E, E, 1.0f);
     }
     if (fz) {
         NOALLOC_SWITCH(pl->Nz, z_div, pl, nb, E, out, qtab);
     } else {
-        k_pass_z_div<float><<<g1, 256, t.smem_z5, pl->stream>>>(E, out, qtab, pl->d_twf[2], g, t.Pz5,
-                                                                (float)pl->Kscale);
+        pass_z_div<float>(pl, nb, E, out, qtab, (float)pl->Kscale);
     }
-    pl->launches += 6;
+    pl->launches = launched + 6;
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_cuda_error(e, "bloch_apply_K_noalloc launch");
     return BLOCH_OK;

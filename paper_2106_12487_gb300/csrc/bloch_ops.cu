@@ -31,14 +31,12 @@ bloch_status set_cuda_error(cudaError_t e, const char* what) {
 template <> Workspace<float>& ws_of<float>(bloch_plan* pl) { return pl->ws_f; }
 template <> Workspace<double>& ws_of<double>(bloch_plan* pl) { return pl->ws_d; }
 template <> Workspace<dfloat>& ws_of<dfloat>(bloch_plan* pl) { return pl->ws_x; }
-// float-float runs the FP64 radix schedule and tiles (same 16-byte complex)
-template <> const Geo& geo_of<dfloat>(const bloch_plan* pl) { return pl->geo_d; }
+template <> const Geo& geo_of<dfloat>(const bloch_plan* pl) { return pl->geo_x; }
 template <> const Geo& geo_of<float>(const bloch_plan* pl) { return pl->geo_f; }
 template <> const Geo& geo_of<double>(const bloch_plan* pl) { return pl->geo_d; }
-template <typename T> static const TileCfg& tile_of(const bloch_plan* pl);
 template <> const TileCfg& tile_of<float>(const bloch_plan* pl) { return pl->tile_f; }
 template <> const TileCfg& tile_of<double>(const bloch_plan* pl) { return pl->tile_d; }
-template <> const TileCfg& tile_of<dfloat>(const bloch_plan* pl) { return pl->tile_d; }
+template <> const TileCfg& tile_of<dfloat>(const bloch_plan* pl) { return pl->tile_x; }
 template <typename T> static const cplx_t<T>* tw_of(const bloch_plan* pl, int axis);
 template <> const float2* tw_of<float>(const bloch_plan* pl, int axis) { return pl->d_twf[axis]; }
 template <> const double2* tw_of<double>(const bloch_plan* pl, int axis) { return pl->d_twd[axis]; }
@@ -46,15 +44,9 @@ template <> const dfloat2* tw_of<dfloat>(const bloch_plan* pl, int axis) { retur
 template <typename T> static const T* ctab_of(const bloch_plan* pl);
 template <> const float* ctab_of<float>(const bloch_plan* pl) { return pl->d_Cf; }
 template <> const double* ctab_of<double>(const bloch_plan* pl) { return pl->d_Cd; }
-template <> const dfloat* ctab_of<dfloat>(const bloch_plan* pl) { return pl->d_Cx; }
 template <typename T> static const T* cpk_of(const bloch_plan* pl);
 template <> const float* cpk_of<float>(const bloch_plan* pl) { return pl->d_Cpf; }
 template <> const double* cpk_of<double>(const bloch_plan* pl) { return pl->d_Cpd; }
-template <typename T> static const T* rtab_of(const bloch_plan* pl);
-template <> const float* rtab_of<float>(const bloch_plan* pl) { return pl->d_rf; }
-template <> const double* rtab_of<double>(const bloch_plan* pl) { return pl->d_rd; }
-template <> const dfloat* rtab_of<dfloat>(const bloch_plan* pl) { return pl->d_rx; }
-
 // ------------------------------------------------------------ host helpers
 static bool fast_axis(int N);
 static bool fast_x(int N);
@@ -65,77 +57,82 @@ static bool factor_ok(int n) {
     return n == 1;
 }
 
-// Radix schedule: power-of-two part in as few stages as possible (each at most
-// max_r), then the odd factors 3, 5, 7.
-static AxisPlan make_axis(int N, int max_log2) {
+// Radix schedule of an axis: the fewest stages, then the smallest radices (the
+// sum of the radices is the work of the direct parts and the butterflies held
+// in registers), the first no larger than the last: the first stage of the
+// strain pass holds two butterflies.
+static AxisPlan make_axis(int N, bool ff) {
+    static const int ends[] = {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 14, 15, 16};
+    static const int mids[] = {1, 2, 3, 4, 5, 6, 7, 8};
     AxisPlan ap{};
     ap.N = N;
-    int n = N, l2 = 0;
-    while (n % 2 == 0) {
-        n /= 2;
-        ++l2;
-    }
-    int nst2 = (l2 + max_log2 - 1) / max_log2;
-    for (int s = 0; s < nst2; ++s) {
-        const int bits = l2 / (nst2 - s);
-        ap.radix[ap.nst++] = 1 << bits;
-        l2 -= bits;
-    }
-    for (int p : {3, 5, 7})
-        while (n % p == 0) {
-            ap.radix[ap.nst++] = p;
-            n /= p;
-        }
+    int best = 1 << 30;
+    for (int r1 : ends)
+        for (int r2 : mids)
+            for (int r3 : ends) {
+                if (r1 * r2 * r3 != N || (r1 > r3 && r3 > 1)) continue;
+                if (ff && (r1 == 12 || r1 == 14 || r3 == 12 || r3 == 14)) continue;
+                const int cost = (r2 > 1 ? 1000 : 0) + r1 + r2 + r3;
+                if (cost < best) {
+                    best = cost;
+                    ap.r1 = r1;
+                    ap.r2 = r2;
+                    ap.r3 = r3;
+                }
+            }
+    ap.d1 = make_fastdiv(ap.r1);
+    ap.d2 = make_fastdiv(ap.r2);
+    ap.d3 = make_fastdiv(ap.r3);
+    ap.m1 = make_fastdiv(N / ap.r1);
+    ap.m2 = make_fastdiv(N / ap.r2);
+    ap.m3 = make_fastdiv(N / ap.r3);
     return ap;
 }
 
-static int choose_P(int N, int bufs, size_t elem, size_t budget, long long npen, int pmax) {
-    int P = pmax;
-    while (P > 1 && (size_t)bufs * N * P * elem + (size_t)(N + 1) * elem > budget) P >>= 1;
+// Pencils per CTA (a power of two, at most pmax) and threads of a mixed-radix
+// pass with `bufs` buffers of `row` elements per pencil: halved until the
+// tile fits the shared-memory budget, then while the grid has fewer than
+// kTileCtas CTAs per system and the rows of a tile keep 32 bytes.
+constexpr long long kTileCtas = 304;
+static PassTile make_tile(const AxisPlan& a, int row, int bufs, size_t el, size_t budget, long long npen, int pmax) {
+    PassTile t{};
+    const size_t tw = (size_t)pad_even(a.N) * el;
+    int P = std::max(1, pmax);
+    while (P > 1 && (size_t)bufs * row * P * el + tw > budget) P >>= 1;
     while (P > 1 && (long long)(P / 2) >= npen) P >>= 1;
-    return P;
-}
-
-// Pencils per CTA of the shared-memory passes: at most pmax (z, y) or pmax / 2
-// (x), reduced until the tile fits the shared-memory budget of its pass.
-template <typename T>
-static TileCfg make_tiles(int Nx, int Ny, int Nz, int pmax) {
-    TileCfg t{};
-    const size_t el = sizeof(cplx_t<T>);
-    auto pad = [&](int N) { return (size_t)((N + 1) & ~1) * el; };
-    const int px = std::max(1, pmax / 2);
-    t.pmax = pmax;
-    t.Pz5 = choose_P(Nz, 5, el, 96 * 1024, (long long)Nx * Ny, pmax);
-    t.Py2 = choose_P(Ny, 2, el, 64 * 1024, (long long)Nx * Nz, pmax);
-    t.Pz2 = choose_P(Nz, 2, el, 64 * 1024, (long long)Nx * Ny, pmax);
-    t.Px7 = choose_P(Nx, 7, el, 96 * 1024, (long long)Ny * Nz, px);
-    t.Px4 = choose_P(Nx, 4, el, 64 * 1024, (long long)Ny * Nz, px);
-    t.smem_z5 = pad(Nz) + (size_t)5 * Nz * t.Pz5 * el;
-    t.smem_y2 = pad(Ny) + (size_t)2 * Ny * t.Py2 * el;
-    t.smem_z2 = pad(Nz) + (size_t)2 * Nz * t.Pz2 * el;
-    t.smem_x7 = pad(Nx) + (size_t)7 * Nx * t.Px7 * el;
-    t.smem_x4 = pad(Nx) + (size_t)4 * Nx * t.Px4 * el;
+    while (P * el > 32 && npen / P < kTileCtas) P >>= 1;
+    while ((1 << t.lp) < P) ++t.lp;
+    t.smem = (size_t)bufs * row * P * el + tw;
+    // threads: the fewest idle butterfly slots over the first and last stage
+    long long best = -1;
+    for (int n : {256, 224, 192, 160, 128}) {
+        long long c = 0;
+        for (int r : {a.r1, a.r3}) {
+            const long long tasks = (long long)bufs * P * (a.N / r);
+            c += (tasks + n - 1) / n * n * r;
+        }
+        if (best < 0 || c * 20 < best * 19) {   // a smaller CTA only where it saves 5 %
+            best = c;
+            t.nthr = n;
+        }
+    }
     return t;
 }
 
+// Tiles of the mixed-radix passes: at most pmax pencils (z, y) or pmax / 2 rows (x) per CTA.
 template <typename T>
-static cudaError_t set_smem_attrs() {
-    cudaError_t e;
-#define SETA(f)                   \
-    e = allow_max_dyn_smem(f);    \
-    if (e != cudaSuccess) return e;
-    SETA(k_pass_z_strain<T>);
-    SETA((k_pass_axis<T, +1, 1>));
-    SETA((k_pass_axis<T, -1, 1>));
-    SETA((k_pass_axis<T, +1, 2>));
-    SETA((k_pass_axis<T, -1, 2>));
-    SETA(k_pass_x_stress<T>);
-    SETA(k_pass_z_div<T>);
-    SETA(k_pass_x_rho<T>);
-    SETA((k_pass_x<T, +1>));
-    SETA((k_pass_x<T, -1>));
-#undef SETA
-    return cudaSuccess;
+static TileCfg make_tiles(const Geo& g, int pmax) {
+    TileCfg t{};
+    const size_t el = sizeof(cplx_t<T>);
+    const long long pxy = (long long)g.Nx * g.Ny, pxz = (long long)g.Nx * g.Nz, pyz = (long long)g.Ny * g.Nz;
+    const int px = std::max(1, pmax / 2);
+    t.pmax = pmax;
+    t.z6 = make_tile(g.ax[2], g.Nz, 6, el, 104 * 1024, pxy, pmax);
+    t.z1 = make_tile(g.ax[2], g.Nz, 1, el, 64 * 1024, pxy, pmax);
+    t.y1 = make_tile(g.ax[1], g.Ny, 1, el, 64 * 1024, pxz, pmax);
+    t.x6 = make_tile(g.ax[0], xrow(g.Nx), 6, el, 104 * 1024, pyz, px);
+    t.x3 = make_tile(g.ax[0], xrow(g.Nx), 3, el, 64 * 1024, pyz, px);
+    return t;
 }
 
 int vec_blocks(const bloch_plan* pl, int nb) {
@@ -253,8 +250,9 @@ void configure_passes(bloch_plan* pl, int variant, int pmax) {
     drop_pcg_graphs(pl);   // instantiated graphs hold the previous launch configuration
     pl->variant = variant;
     pl->fast = variant == 0;
-    pl->tile_f = make_tiles<float>(pl->Nx, pl->Ny, pl->Nz, pmax);
-    pl->tile_d = make_tiles<double>(pl->Nx, pl->Ny, pl->Nz, pmax);
+    pl->tile_f = make_tiles<float>(pl->geo_f, pmax);
+    pl->tile_d = make_tiles<double>(pl->geo_d, pmax);
+    pl->tile_x = make_tiles<dfloat>(pl->geo_x, pmax);
 }
 
 // CTAs per system of the fast z passes (P = 128 / RA pencils each), 0 when
@@ -446,16 +444,9 @@ int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_s
     int fused = 0;
     if (pl->fast) {
         Workspace<T>& w = ws_of<T>(pl);
-        const Geo& g = geo_of<T>(pl);
-        const TileCfg& t = tile_of<T>(pl);
-        const long long pxy = (long long)pl->Nx * pl->Ny, pxz = (long long)pl->Nx * pl->Nz,
-                        pyz = (long long)pl->Ny * pl->Nz;
         const bool fz = fast_x(pl->Nz) && std::is_same<T, float>::value;
         const bool fy = fast_axis(pl->Ny);
         const bool fx = fast_x(pl->Nx) && std::is_same<T, float>::value;
-        dim3 g1((unsigned)((pxy + t.Pz5 - 1) / t.Pz5), nb);
-        dim3 g2((unsigned)((pxz + t.Py2 - 1) / t.Py2), nb * 6);
-        dim3 g3((unsigned)((pyz + t.Px7 - 1) / t.Px7), nb);
         bool done1 = false;
         if constexpr (std::is_same<T, float>::value) {
             if (fz) {
@@ -463,15 +454,11 @@ int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_s
                 done1 = true;
             }
         }
-        if (!done1) {
-            ++pl->launches;
-            k_pass_z_strain<T><<<g1, 256, t.smem_z5, pl->stream>>>(u, w.E, w.qtab, tw_of<T>(pl, 2), g, t.Pz5);
-        }
+        if (!done1) pass_z_strain<T>(pl, nb, u, w.E, w.qtab);
         if (fy) {
             BLOCH_FAST_SWITCH(pl->Ny, fast_y, pl, +1, nb, w.E);
         } else {
-            ++pl->launches;
-            k_pass_axis<T, +1, 1><<<g2, 256, t.smem_y2, pl->stream>>>(w.E, w.E, tw_of<T>(pl, 1), g, t.Py2, T(1));
+            pass_axis<T>(pl, 1, +1, 6 * nb, w.E, w.E, T(1));
         }
         // (p, A p) partials: from the strain energy in the fast x pass where it runs,
         // else from the fast z-divergence pass (which then reads p once more)
@@ -491,16 +478,11 @@ int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_s
                 done3 = true;
             }
         }
-        if (!done3) {
-            ++pl->launches;
-            k_pass_x_stress<T><<<g3, 256, t.smem_x7, pl->stream>>>(w.E, pl->d_ids, ctab_of<T>(pl), tw_of<T>(pl, 0),
-                                                                    g, t.Px7);
-        }
+        if (!done3) pass_x_stress<T>(pl, nb, w.E);
         if (fy) {
             BLOCH_FAST_SWITCH(pl->Ny, fast_y, pl, -1, nb, w.E);
         } else {
-            ++pl->launches;
-            k_pass_axis<T, -1, 1><<<g2, 256, t.smem_y2, pl->stream>>>(w.E, w.E, tw_of<T>(pl, 1), g, t.Py2, T(1));
+            pass_axis<T>(pl, 1, -1, 6 * nb, w.E, w.E, T(1));
         }
         bool done5 = false;
         if constexpr (std::is_same<T, float>::value) {
@@ -512,11 +494,7 @@ int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_s
                 if (zdot) fused = fast_z_blocks(pl);
             }
         }
-        if (!done5) {
-            ++pl->launches;
-            k_pass_z_div<T><<<g1, 256, t.smem_z5, pl->stream>>>(w.E, out, w.qtab, tw_of<T>(pl, 2), g, t.Pz5,
-                                                                out_scale);
-        }
+        if (!done5) pass_z_div<T>(pl, nb, w.E, out, w.qtab, out_scale);
         return fused;
     }
     launch_K_generic<T>(pl, nb, u, out, out_scale);
@@ -526,27 +504,15 @@ int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_s
 template <typename T>
 void launch_K_generic(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale) {
     Workspace<T>& w = ws_of<T>(pl);
-    const Geo& g = geo_of<T>(pl);
-    const TileCfg& t = tile_of<T>(pl);
-    const long long pxy = (long long)pl->Nx * pl->Ny, pxz = (long long)pl->Nx * pl->Nz,
-                    pyz = (long long)pl->Ny * pl->Nz;
-    dim3 g1((unsigned)((pxy + t.Pz5 - 1) / t.Pz5), nb);
-    ++pl->launches;
-    k_pass_z_strain<T><<<g1, 256, t.smem_z5, pl->stream>>>(u, w.E, w.qtab, tw_of<T>(pl, 2), g, t.Pz5);
-    dim3 g2((unsigned)((pxz + t.Py2 - 1) / t.Py2), nb * 6);
-    ++pl->launches;
-    k_pass_axis<T, +1, 1><<<g2, 256, t.smem_y2, pl->stream>>>(w.E, w.E, tw_of<T>(pl, 1), g, t.Py2, T(1));
-    dim3 g3((unsigned)((pyz + t.Px7 - 1) / t.Px7), nb);
-    ++pl->launches;
-    k_pass_x_stress<T><<<g3, 256, t.smem_x7, pl->stream>>>(w.E, pl->d_ids, ctab_of<T>(pl), tw_of<T>(pl, 0), g, t.Px7);
-    ++pl->launches;
-    k_pass_axis<T, -1, 1><<<g2, 256, t.smem_y2, pl->stream>>>(w.E, w.E, tw_of<T>(pl, 1), g, t.Py2, T(1));
-    ++pl->launches;
-    k_pass_z_div<T><<<g1, 256, t.smem_z5, pl->stream>>>(w.E, out, w.qtab, tw_of<T>(pl, 2), g, t.Pz5, out_scale);
+    pass_z_strain<T>(pl, nb, u, w.E, w.qtab);
+    pass_axis<T>(pl, 1, +1, 6 * nb, w.E, w.E, T(1));
+    pass_x_stress<T>(pl, nb, w.E);
+    pass_axis<T>(pl, 1, -1, 6 * nb, w.E, w.E, T(1));
+    pass_z_div<T>(pl, nb, w.E, out, w.qtab, out_scale);
 }
 
-// Float-float operator: the shared-memory z and x passes; the two-stage
-// register y passes where the y axis has one (fft_variant 0)
+// Float-float operator: the mixed-radix passes; the two-stage register y
+// passes where the y axis has one (fft_variant 0)
 template <>
 int launch_K<dfloat>(bloch_plan* pl, int nb, const dfloat2* u, dfloat2* out, dfloat out_scale, const dfloat2*,
                      double2*) {
@@ -556,19 +522,11 @@ int launch_K<dfloat>(bloch_plan* pl, int nb, const dfloat2* u, dfloat2* out, dfl
         return 0;
     }
     Workspace<T>& w = ws_of<T>(pl);
-    const Geo& g = geo_of<T>(pl);
-    const TileCfg& t = tile_of<T>(pl);
-    const long long pxy = (long long)pl->Nx * pl->Ny, pyz = (long long)pl->Ny * pl->Nz;
-    dim3 g1((unsigned)((pxy + t.Pz5 - 1) / t.Pz5), nb);
-    dim3 g3((unsigned)((pyz + t.Px7 - 1) / t.Px7), nb);
-    ++pl->launches;
-    k_pass_z_strain<T><<<g1, 256, t.smem_z5, pl->stream>>>(u, w.E, w.qtab, tw_of<T>(pl, 2), g, t.Pz5);
+    pass_z_strain<T>(pl, nb, u, w.E, w.qtab);
     BLOCH_FAST_SWITCH(pl->Ny, fast_y, pl, +1, nb, w.E);
-    ++pl->launches;
-    k_pass_x_stress<T><<<g3, 256, t.smem_x7, pl->stream>>>(w.E, pl->d_ids, ctab_of<T>(pl), tw_of<T>(pl, 0), g, t.Px7);
+    pass_x_stress<T>(pl, nb, w.E);
     BLOCH_FAST_SWITCH(pl->Ny, fast_y, pl, -1, nb, w.E);
-    ++pl->launches;
-    k_pass_z_div<T><<<g1, 256, t.smem_z5, pl->stream>>>(w.E, out, w.qtab, tw_of<T>(pl, 2), g, t.Pz5, out_scale);
+    pass_z_div<T>(pl, nb, w.E, out, w.qtab, out_scale);
     return 0;
 }
 
@@ -580,37 +538,20 @@ int launch_K<dfloat>(bloch_plan* pl, int nb, const dfloat2* u, dfloat2* out, dfl
 template <typename T>
 void launch_K_stress(bloch_plan* pl, int nb, const cplx_t<T>* u) {
     Workspace<T>& w = ws_of<T>(pl);
-    const Geo& g = geo_of<T>(pl);
-    const TileCfg& t = tile_of<T>(pl);
-    const long long pxy = (long long)pl->Nx * pl->Ny, pxz = (long long)pl->Nx * pl->Nz,
-                    pyz = (long long)pl->Ny * pl->Nz;
-    dim3 g1((unsigned)((pxy + t.Pz5 - 1) / t.Pz5), nb);
-    dim3 g2((unsigned)((pxz + t.Py2 - 1) / t.Py2), nb * 6);
-    dim3 g3((unsigned)((pyz + t.Px7 - 1) / t.Px7), nb);
-    dim3 gz((unsigned)((pxy + t.Pz2 - 1) / t.Pz2), nb * 6);
-    pl->launches += 5;
-    k_pass_z_strain<T><<<g1, 256, t.smem_z5, pl->stream>>>(u, w.E, w.qtab, tw_of<T>(pl, 2), g, t.Pz5);
-    k_pass_axis<T, +1, 1><<<g2, 256, t.smem_y2, pl->stream>>>(w.E, w.E, tw_of<T>(pl, 1), g, t.Py2, T(1));
-    k_pass_x_stress<T><<<g3, 256, t.smem_x7, pl->stream>>>(w.E, pl->d_ids, ctab_of<T>(pl), tw_of<T>(pl, 0), g, t.Px7);
-    k_pass_axis<T, -1, 1><<<g2, 256, t.smem_y2, pl->stream>>>(w.E, w.E, tw_of<T>(pl, 1), g, t.Py2, T(1));
-    k_pass_axis<T, -1, 2><<<gz, 256, t.smem_z2, pl->stream>>>(w.E, w.E, tw_of<T>(pl, 2), g, t.Pz2, T(1));
+    pass_z_strain<T>(pl, nb, u, w.E, w.qtab);
+    pass_axis<T>(pl, 1, +1, 6 * nb, w.E, w.E, T(1));
+    pass_x_stress<T>(pl, nb, w.E);
+    pass_axis<T>(pl, 1, -1, 6 * nb, w.E, w.E, T(1));
+    pass_axis<T>(pl, 2, -1, 6 * nb, w.E, w.E, T(1));
 }
 
 // In-place 3D FFT of nb three-component fields (DIR -1 forward, +1 inverse;
 // unnormalised), times out_scale: shared-memory passes along z, y and x.
 template <typename T, int DIR>
 void launch_fft3(bloch_plan* pl, int nb, cplx_t<T>* W, T out_scale) {
-    const Geo& g = geo_of<T>(pl);
-    const TileCfg& t = tile_of<T>(pl);
-    const long long pxy = (long long)pl->Nx * pl->Ny, pxz = (long long)pl->Nx * pl->Nz,
-                    pyz = (long long)pl->Ny * pl->Nz;
-    dim3 gz((unsigned)((pxy + t.Pz2 - 1) / t.Pz2), nb * 3);
-    dim3 gy((unsigned)((pxz + t.Py2 - 1) / t.Py2), nb * 3);
-    dim3 gx((unsigned)((pyz + t.Px4 - 1) / t.Px4), nb);
-    pl->launches += 3;
-    k_pass_axis<T, DIR, 2><<<gz, 256, t.smem_z2, pl->stream>>>(W, W, tw_of<T>(pl, 2), g, t.Pz2, T(1));
-    k_pass_axis<T, DIR, 1><<<gy, 256, t.smem_y2, pl->stream>>>(W, W, tw_of<T>(pl, 1), g, t.Py2, T(1));
-    k_pass_x<T, DIR><<<gx, 256, t.smem_x4, pl->stream>>>(W, tw_of<T>(pl, 0), g, t.Px4, out_scale);
+    pass_axis<T>(pl, 2, DIR, 3 * nb, W, W, T(1));
+    pass_axis<T>(pl, 1, DIR, 3 * nb, W, W, T(1));
+    pass_x<T>(pl, DIR, nb, W, out_scale);
 }
 
 template <typename T>
@@ -624,23 +565,11 @@ void launch_M(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_
         return;
     }
     Workspace<T>& w = ws_of<T>(pl);
-    const Geo& g = geo_of<T>(pl);
-    const TileCfg& t = tile_of<T>(pl);
-    const long long pxy = (long long)pl->Nx * pl->Ny, pxz = (long long)pl->Nx * pl->Nz,
-                    pyz = (long long)pl->Ny * pl->Nz;
-    dim3 gz((unsigned)((pxy + t.Pz2 - 1) / t.Pz2), nb * 3);
-    dim3 gy((unsigned)((pxz + t.Py2 - 1) / t.Py2), nb * 3);
-    dim3 gx((unsigned)((pyz + t.Px4 - 1) / t.Px4), nb);
-    ++pl->launches;
-    k_pass_axis<T, +1, 2><<<gz, 256, t.smem_z2, pl->stream>>>(u, w.E, tw_of<T>(pl, 2), g, t.Pz2, T(1));
-    ++pl->launches;
-    k_pass_axis<T, +1, 1><<<gy, 256, t.smem_y2, pl->stream>>>(w.E, w.E, tw_of<T>(pl, 1), g, t.Py2, T(1));
-    ++pl->launches;
-    k_pass_x_rho<T><<<gx, 256, t.smem_x4, pl->stream>>>(w.E, pl->d_ids, rtab_of<T>(pl), tw_of<T>(pl, 0), g, t.Px4);
-    ++pl->launches;
-    k_pass_axis<T, -1, 1><<<gy, 256, t.smem_y2, pl->stream>>>(w.E, w.E, tw_of<T>(pl, 1), g, t.Py2, T(1));
-    ++pl->launches;
-    k_pass_axis<T, -1, 2><<<gz, 256, t.smem_z2, pl->stream>>>(w.E, out, tw_of<T>(pl, 2), g, t.Pz2, out_scale);
+    pass_axis<T>(pl, 2, +1, 3 * nb, u, w.E, T(1));
+    pass_axis<T>(pl, 1, +1, 3 * nb, w.E, w.E, T(1));
+    pass_x_rho<T>(pl, nb, w.E);
+    pass_axis<T>(pl, 1, -1, 3 * nb, w.E, w.E, T(1));
+    pass_axis<T>(pl, 2, -1, 3 * nb, w.E, out, out_scale);
 }
 
 template <typename T>
@@ -1240,16 +1169,22 @@ bloch_status bloch_plan_create(bloch_plan** out, const int32_t grid[3], const do
     CK(dmalloc(&pl->d_iter, 1, acc));
     CK(cudaStreamCreateWithFlags(&pl->cap_stream, cudaStreamNonBlocking));
     CK(cudaMallocHost((void**)&pl->h_nactive, sizeof(int)));
-    CK(set_smem_attrs<float>());
-    CK(set_smem_attrs<double>());
-    CK(set_smem_attrs<dfloat>());
+    CK(pass_attrs_z<float>());
+    CK(pass_attrs_axis<float>());
+    CK(pass_attrs_x<float>());
+    CK(pass_attrs_z<double>());
+    CK(pass_attrs_axis<double>());
+    CK(pass_attrs_x<double>());
+    CK(pass_attrs_z<dfloat>());
+    CK(pass_attrs_axis<dfloat>());
+    CK(pass_attrs_x<dfloat>());
     set_fast_attrs<float>();
     set_fast_attrs<double>();
     set_fast_attrs<dfloat>();
     pl->fast = pl->opt.fft_variant == 0;
     pl->variant = pl->opt.fft_variant;
 #undef CK
-    for (Geo* gp : {&pl->geo_f, &pl->geo_d}) {
+    for (Geo* gp : {&pl->geo_f, &pl->geo_d, &pl->geo_x}) {
         gp->Nx = pl->Nx;
         gp->Ny = pl->Ny;
         gp->Nz = pl->Nz;
@@ -1259,12 +1194,13 @@ bloch_status bloch_plan_create(bloch_plan** out, const int32_t grid[3], const do
         gp->err = pl->d_perr;
     }
     for (int a = 0; a < 3; ++a) {
-        pl->geo_f.ax[a] = make_axis(grid[a], 4);   // radices up to 16 in FP32
-        pl->geo_d.ax[a] = make_axis(grid[a], 3);   // up to 8 in FP64 (register budget)
+        pl->geo_f.ax[a] = pl->geo_d.ax[a] = make_axis(grid[a], false);
+        pl->geo_x.ax[a] = make_axis(grid[a], true);
     }
     const int pmax = pl->opt.tile_pmax > 0 ? pl->opt.tile_pmax : kDefaultPmax;
-    pl->tile_f = make_tiles<float>(pl->Nx, pl->Ny, pl->Nz, pmax);
-    pl->tile_d = make_tiles<double>(pl->Nx, pl->Ny, pl->Nz, pmax);
+    pl->tile_f = make_tiles<float>(pl->geo_f, pmax);
+    pl->tile_d = make_tiles<double>(pl->geo_d, pmax);
+    pl->tile_x = make_tiles<dfloat>(pl->geo_x, pmax);
     pl->nblk_max = vec_blocks(pl, 1);
     *out = pl;
     return BLOCH_OK;

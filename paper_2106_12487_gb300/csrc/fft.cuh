@@ -1,31 +1,47 @@
-// Shared-memory Stockham FFT of a tile of pencils.
-//
-// A CTA holds P pencils of length N in shared memory and transforms all of
-// them along their length with a mixed-radix Stockham autosort (out-of-place
-// between two shared buffers, one barrier per stage).  Each thread owns one
-// radix-R butterfly at a time: R values are read, multiplied by the stage
-// twiddles, transformed in registers and written to their sorted position.
-// The stage formulation is the Stockham autosort used for GPU FFTs by
-// Govindaraju et al. (SC 2008): with Ns the product of the radices already
-// applied, butterfly j reads x[j + r N/R] (r < R), twiddles by
-// w_{Ns R}^{r (j mod Ns)}, and writes X[(j div Ns) Ns R + (j mod Ns) + r Ns].
+// Register DFTs of small radices and the radix schedule of an axis.
 //
 // Radix kernels: powers of two (2..16) by unrolled radix-2 decimation in time
-// with literal twiddles; 3, 5, 7 by a direct DFT (small test grids only).
+// with literal twiddles; 3, 5, 7 from the symmetric and antisymmetric parts of
+// their inputs with literal cosines and sines; 6, 10, 12, 14, 15 as coprime
+// products of those by the prime-factor map of Good (1958), which needs no
+// twiddles; 9 as 3 x 3.
 // Direction: DIR = -1 forward (exp(-2 pi i ...)), DIR = +1 inverse; both
 // unnormalised.
 #pragma once
+
+#include <type_traits>
 
 #include "common.cuh"
 
 namespace bloch {
 
-constexpr int kMaxStages = 12;
+// Division of n < 2^31 by an invariant divisor d >= 1 with one high multiply,
+// an add and a shift (Granlund & Montgomery 1994, division by invariant
+// integers): l = ceil(log2 d), m = floor(2^32 (2^l - d) / d) + 1,
+// n / d = (umulhi(m, n) + n) >> l.
+struct FastDiv {
+    unsigned m = 1;
+    int l = 0;
+};
+inline FastDiv make_fastdiv(unsigned d) {
+    FastDiv f;
+    int l = 0;
+    while ((1ull << l) < (unsigned long long)d) ++l;
+    f.l = l;
+    f.m = (unsigned)((((1ull << 32) * ((1ull << l) - d)) / d) + 1);
+    return f;
+}
+__device__ __forceinline__ unsigned fdiv(unsigned n, const FastDiv& f) { return (__umulhi(f.m, n) + n) >> f.l; }
 
+// Radix schedule N = r1 * r2 * r3 of an axis (r2 = 1: two stages).  The first
+// and the last radix come from {1..10, 12, 14, 15, 16} (float-float: without
+// 12 and 14), the middle one from {1..8}; every length up to
+// 512 with prime factors in {2,3,5,7} has one.
 struct AxisPlan {
     int N;
-    int nst;
-    int radix[kMaxStages];
+    int r1, r2, r3;
+    FastDiv d1, d2, d3;      // division by the radices
+    FastDiv m1, m2, m3;      // division by N / radix (butterflies of a stage per pencil)
 };
 
 // cos(2 pi m / 16), m taken modulo 16
@@ -72,9 +88,78 @@ __device__ __forceinline__ C twiddle_pow2(C x, int k) {
     return mk(x.x * c - x.y * s, x.x * s + x.y * c);
 }
 
+// Butterfly v_k = e + w o, v_{k+H} = e - w o with w = exp(DIR 2 pi i k / R), k
+// and R compile time.  With w = m (1 + i t) or m (t + i), |t| <= 1, the product
+// costs two fused multiply-adds and both outputs two each: 6 instead of 8
+// operations (Linzer & Feig 1993).  Float-float has no fused multiply-add to
+// gain from and keeps the plain product.
+template <int R, int DIR, typename C>
+__device__ __forceinline__ void butterfly(C e, C o, int k, C& lo, C& hi) {
+    using T = decltype(e.x);
+    if (k == 0 || 4 * k == R || std::is_same<T, dfloat>::value) {
+        const C t = twiddle_pow2<R, DIR>(o, k);
+        lo = cadd(e, t);
+        hi = csub(e, t);
+        return;
+    }
+    const int m16 = k * (16 / R);   // 1..7
+    const T c = cos16<T>(m16), s = T(DIR) * cos16<T>(m16 - 4);
+    // tan or cot of the angle, folded into [-1, 1]: 45 degrees 1, 22.5 degrees sqrt(2) - 1
+    const T q = T((m16 & 1) ? 0.41421356237309504880 : 1.0);
+    T m, ux, uy;
+    if (m16 <= 2 || m16 >= 6) {     // |cos| >= |sin|
+        const T t = T(DIR) * (m16 <= 2 ? q : -q);
+        m = c;
+        ux = fma(-t, o.y, o.x);
+        uy = fma(t, o.x, o.y);
+    } else {
+        const T t = T(DIR) * (m16 < 4 ? q : -q);
+        m = s;
+        ux = fma(t, o.x, -o.y);
+        uy = fma(t, o.y, o.x);
+    }
+    lo = mk(fma(m, ux, e.x), fma(m, uy, e.y));
+    hi = mk(fma(-m, ux, e.x), fma(-m, uy, e.y));
+}
+
+// cosines and sines 2 pi k / R of the odd radices, k = 1 .. (R - 1) / 2
+template <int R> __host__ __device__ constexpr double odd_cos(int k) {
+    constexpr double c3[] = {1.0, -0.5};
+    constexpr double c5[] = {1.0, 0.30901699437494742410, -0.80901699437494742410};
+    constexpr double c7[] = {1.0, 0.62348980185873353053, -0.22252093395631440429, -0.90096886790241912624};
+    k %= R;
+    if (k > R / 2) k = R - k;
+    return R == 3 ? c3[k < 2 ? k : 0] : R == 5 ? c5[k < 3 ? k : 0] : c7[k];
+}
+template <int R> __host__ __device__ constexpr double odd_sin(int k) {
+    constexpr double s3[] = {0.0, 0.86602540378443864676};
+    constexpr double s5[] = {0.0, 0.95105651629515357212, 0.58778525229247312917};
+    constexpr double s7[] = {0.0, 0.78183148246802980871, 0.97492791218182360702, 0.43388373911755812048};
+    k %= R;
+    const bool neg = k > R / 2;
+    if (neg) k = R - k;
+    const double v = R == 3 ? s3[k < 2 ? k : 0] : R == 5 ? s5[k < 3 ? k : 0] : s7[k];
+    return neg ? -v : v;
+}
+
+// coprime factors of the prime-factor radices
+template <int R> struct Coprime { static constexpr int a = 1, b = 1; };
+template <> struct Coprime<6> { static constexpr int a = 2, b = 3; };
+template <> struct Coprime<10> { static constexpr int a = 2, b = 5; };
+template <> struct Coprime<12> { static constexpr int a = 4, b = 3; };
+template <> struct Coprime<14> { static constexpr int a = 2, b = 7; };
+template <> struct Coprime<15> { static constexpr int a = 3, b = 5; };
+
+__host__ __device__ constexpr int inv_mod(int x, int m) {
+    for (int i = 1; i < m; ++i)
+        if ((x * i) % m == 1) return i;
+    return 1;
+}
+
 template <int R, int DIR, typename C>
 struct RegDFT {
     __device__ __forceinline__ static void run(C* v) {
+        using T = decltype(v[0].x);
         if constexpr (R == 1) {
             return;
         } else if constexpr (R == 2) {
@@ -92,112 +177,80 @@ struct RegDFT {
             RegDFT<H, DIR, C>::run(e);
             RegDFT<H, DIR, C>::run(o);
 #pragma unroll
-            for (int k = 0; k < H; ++k) {
-                C t = twiddle_pow2<R, DIR>(o[k], k);
-                v[k] = cadd(e[k], t);
-                v[k + H] = csub(e[k], t);
+            for (int k = 0; k < H; ++k) butterfly<R, DIR>(e[k], o[k], k, v[k], v[k + H]);
+        } else if constexpr (R == 3 || R == 5 || R == 7) {
+            // X_k = a_k + DIR i b_k, X_{R-k} = a_k - DIR i b_k from t_n = v_n + v_{R-n}, d_n = v_n - v_{R-n}
+            constexpr int H = (R - 1) / 2;
+            C t[H], d[H];
+            C x0 = v[0];
+#pragma unroll
+            for (int n = 0; n < H; ++n) {
+                t[n] = cadd(v[n + 1], v[R - 1 - n]);
+                d[n] = csub(v[n + 1], v[R - 1 - n]);
+                x0 = cadd(x0, t[n]);
+            }
+#pragma unroll
+            for (int k = 1; k <= H; ++k) {
+                C a = v[0], b = cscale(d[0], T(odd_sin<R>(k)));
+#pragma unroll
+                for (int n = 0; n < H; ++n) {
+                    const T c = T(odd_cos<R>((n + 1) * k));
+                    a = mk(fma(c, t[n].x, a.x), fma(c, t[n].y, a.y));
+                    if (n > 0) {
+                        const T s = T(odd_sin<R>((n + 1) * k));
+                        b = mk(fma(s, d[n].x, b.x), fma(s, d[n].y, b.y));
+                    }
+                }
+                const C ib = cmul_i<DIR>(b);
+                v[k] = cadd(a, ib);         // v[1..H], v[R-H..] are read only through t and d
+                v[R - k] = csub(a, ib);
+            }
+            v[0] = x0;
+        } else if constexpr (R == 9) {
+            constexpr double c9[5] = {1.0, 0.76604444311897803520, 0.17364817766693034885, -0.5,
+                                      -0.93969262078590838405};
+            constexpr double s9[5] = {0.0, 0.64278760968653932632, 0.98480775301220805937, 0.86602540378443864676,
+                                      0.34202014332566873304};
+            C w[3][3];
+#pragma unroll
+            for (int n2 = 0; n2 < 3; ++n2) {
+#pragma unroll
+                for (int n1 = 0; n1 < 3; ++n1) w[n2][n1] = v[3 * n1 + n2];
+                RegDFT<3, DIR, C>::run(w[n2]);
+#pragma unroll
+                for (int k1 = 1; k1 < 3; ++k1)
+                    if (n2 > 0) w[n2][k1] = cmul(w[n2][k1], mk(T(c9[n2 * k1]), T(DIR * s9[n2 * k1])));
+            }
+#pragma unroll
+            for (int k1 = 0; k1 < 3; ++k1) {
+                C x[3] = {w[0][k1], w[1][k1], w[2][k1]};
+                RegDFT<3, DIR, C>::run(x);
+#pragma unroll
+                for (int k2 = 0; k2 < 3; ++k2) v[k1 + 3 * k2] = x[k2];
             }
         } else {
-            // direct DFT for odd radices 3, 5, 7
-            using T = decltype(v[0].x);
-            C out[R];
+            // Good's map: input n = (B i + A j) mod R, output k = (B inv_A(B) p + A inv_B(A) q) mod R
+            constexpr int A = Coprime<R>::a, B = Coprime<R>::b;
+            static_assert(A * B == R && A > 1, "no register DFT of this radix");
+            constexpr int ua = B * inv_mod(B % A, A), ub = A * inv_mod(A % B, B);
+            C w[A][B];
 #pragma unroll
-            for (int k = 0; k < R; ++k) {
-                C acc = v[0];
+            for (int i = 0; i < A; ++i) {
 #pragma unroll
-                for (int n = 1; n < R; ++n) {
-                    double s, c;
-                    sincospi(2.0 * double((n * k) % R) / double(R), &s, &c);
-                    C w = mk(T(c), T(DIR) * T(s));
-                    acc = cadd(acc, cmul(v[n], w));
-                }
-                out[k] = acc;
+                for (int j = 0; j < B; ++j) w[i][j] = v[(B * i + A * j) % R];
+                RegDFT<B, DIR, C>::run(w[i]);
             }
 #pragma unroll
-            for (int k = 0; k < R; ++k) v[k] = out[k];
+            for (int q = 0; q < B; ++q) {
+                C x[A];
+#pragma unroll
+                for (int i = 0; i < A; ++i) x[i] = w[i][q];
+                RegDFT<A, DIR, C>::run(x);
+#pragma unroll
+                for (int p = 0; p < A; ++p) v[(ua * p + ub * q) % R] = x[p];
+            }
         }
     }
 };
-
-// Element (p, n) of a tile: pencil-fastest layout (PF) n*P + p, or
-// length-fastest layout (LF) p*ld + n.
-template <bool PF>
-__device__ __forceinline__ int tile_idx(int p, int n, int P, int ld) {
-    return PF ? n * P + p : p * ld + n;
-}
-
-// One Stockham stage of radix R over all P pencils of the tile.
-// tw: table of exp(-2 pi i t / N), t < N (shared memory).
-template <int R, int DIR, bool PF, typename C>
-__device__ __forceinline__ void stockham_stage(const C* __restrict__ src, C* __restrict__ dst, int N, int P,
-                                               int ld, int Ns, const C* __restrict__ tw, int tid, int nthr) {
-    const int NR = N / R;
-    const int tasks = NR * P;
-    const int twstep = N / (Ns * R);
-    for (int t = tid; t < tasks; t += nthr) {
-        int p, j;
-        if (PF) {
-            p = t % P;
-            j = t / P;
-        } else {
-            j = t % NR;
-            p = t / NR;
-        }
-        C v[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = src[tile_idx<PF>(p, j + r * NR, P, ld)];
-        const int jm = j % Ns;
-        if (Ns > 1) {
-            const int base = jm * twstep;
-#pragma unroll
-            for (int r = 1; r < R; ++r) {
-                C w = tw[r * base];
-                if (DIR > 0) w.y = -w.y;
-                v[r] = cmul(v[r], w);
-            }
-        }
-        RegDFT<R, DIR, C>::run(v);
-        const int o = (j - jm) * R + jm;
-#pragma unroll
-        for (int r = 0; r < R; ++r) dst[tile_idx<PF>(p, o + r * Ns, P, ld)] = v[r];
-    }
-}
-
-// Odd radices only serve small test grids: keep them out of line so that
-// their direct DFT does not raise the register allocation of the kernels.
-template <int R, int DIR, bool PF, typename C>
-__device__ __noinline__ void stockham_stage_odd(const C* __restrict__ src, C* __restrict__ dst, int N, int P, int ld,
-                                                int Ns, const C* __restrict__ tw, int tid, int nthr) {
-    stockham_stage<R, DIR, PF>(src, dst, N, P, ld, Ns, tw, tid, nthr);
-}
-
-// Transform every pencil of the tile held in `a`, using `b` as the second
-// buffer.  Returns the buffer that holds the result (a or b).  Contains the
-// barriers between stages; the caller must have synchronised after filling a.
-template <int DIR, bool PF, typename C>
-__device__ C* fft_tile(C* a, C* b, const AxisPlan& ap, int P, int ld, const C* tw, int tid, int nthr) {
-    C* src = a;
-    C* dst = b;
-    int Ns = 1;
-    for (int s = 0; s < ap.nst; ++s) {
-        const int R = ap.radix[s];
-        switch (R) {
-            case 2: stockham_stage<2, DIR, PF>(src, dst, ap.N, P, ld, Ns, tw, tid, nthr); break;
-            case 4: stockham_stage<4, DIR, PF>(src, dst, ap.N, P, ld, Ns, tw, tid, nthr); break;
-            case 8: stockham_stage<8, DIR, PF>(src, dst, ap.N, P, ld, Ns, tw, tid, nthr); break;
-            case 16: stockham_stage<16, DIR, PF>(src, dst, ap.N, P, ld, Ns, tw, tid, nthr); break;
-            case 3: stockham_stage_odd<3, DIR, PF>(src, dst, ap.N, P, ld, Ns, tw, tid, nthr); break;
-            case 5: stockham_stage_odd<5, DIR, PF>(src, dst, ap.N, P, ld, Ns, tw, tid, nthr); break;
-            case 7: stockham_stage_odd<7, DIR, PF>(src, dst, ap.N, P, ld, Ns, tw, tid, nthr); break;
-            default: break;
-        }
-        __syncthreads();
-        C* t = src;
-        src = dst;
-        dst = t;
-        Ns *= R;
-    }
-    return src;
-}
 
 }  // namespace bloch

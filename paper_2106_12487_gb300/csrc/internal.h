@@ -62,14 +62,18 @@ struct Tracer {
     long long count[TR_NPHASE] = {};
 };
 
+// Tile of a mixed-radix pass: 1 << lp pencils per CTA, threads, shared memory.
+struct PassTile {
+    int lp;
+    int nthr;
+    size_t smem;
+};
+
 struct TileCfg {
-    int pmax;   // cap on pencils per CTA the tiles were made with
-    int Pz5;    // pencils per CTA, z passes with 5 buffers (strain / divergence)
-    int Py2;    // y pass, 2 buffers
-    int Pz2;    // z pass, 2 buffers (mass operator)
-    int Px7;    // x stress pass, 7 buffers
-    int Px4;    // x rho pass, 4 buffers
-    size_t smem_z5, smem_y2, smem_z2, smem_x7, smem_x4;
+    int pmax;             // cap on pencils per CTA the tiles were made with
+    PassTile z6;          // z strain / divergence, 6 buffers
+    PassTile y1, z1;      // plain y and z passes, 1 buffer
+    PassTile x6, x3;      // x rows, 6 (stress) and 3 (density, plain) components
 };
 
 }  // namespace bloch
@@ -112,8 +116,8 @@ struct bloch_plan {
     int* d_perr = nullptr;    // pass error word (a staging wait ran out), Geo::err
     int* h_nactive = nullptr;     // pinned
 
-    bloch::Geo geo_f, geo_d;
-    bloch::TileCfg tile_f, tile_d;
+    bloch::Geo geo_f, geo_d, geo_x;     // FP32, FP64, float-float
+    bloch::TileCfg tile_f, tile_d, tile_x;
     int nblk_max;
     bool fast = true;              // use the two-stage register FFT passes where the axis allows
     int variant = 0;               // options.fft_variant, or the autotuner's choice
@@ -172,6 +176,23 @@ namespace bloch {
 
 template <typename T> Workspace<T>& ws_of(bloch_plan* pl);
 template <typename T> const Geo& geo_of(const bloch_plan* pl);
+template <typename T> const TileCfg& tile_of(const bloch_plan* pl);
+
+// Mixed-radix passes (passes.cuh) on the plan's stream: any axis length, every
+// field type.  E and W are updated in place; dir -1 forward, +1 inverse.
+template <typename T>
+void pass_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab);
+template <typename T>   // axis 1 (y) or 2 (z) of nfields scalar fields
+void pass_axis(bloch_plan* pl, int axis, int dir, int nfields, const cplx_t<T>* in, cplx_t<T>* out, T out_scale);
+template <typename T> void pass_x_stress(bloch_plan* pl, int nb, cplx_t<T>* E);
+template <typename T> void pass_x_rho(bloch_plan* pl, int nb, cplx_t<T>* W);
+template <typename T> void pass_x(bloch_plan* pl, int dir, int nb, cplx_t<T>* W, T out_scale);
+template <typename T>
+void pass_z_div(bloch_plan* pl, int nb, const cplx_t<T>* E, cplx_t<T>* out, const T* qtab, T out_scale);
+// shared-memory limits of the passes, once per plan
+template <typename T> cudaError_t pass_attrs_z();
+template <typename T> cudaError_t pass_attrs_axis();
+template <typename T> cudaError_t pass_attrs_x();
 
 // Grow the operator workspace to hold nb systems.
 template <typename T> bloch_status ensure_ws(bloch_plan* pl, int nb);

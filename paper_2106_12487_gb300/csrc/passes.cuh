@@ -1,9 +1,11 @@
-// FFT pass kernels of the Bloch stiffness and mass operators.
+// Mixed-radix FFT passes of the Bloch stiffness and mass operators: any axis
+// length up to 512 with prime factors in {2,3,5,7}, in FP32, FP64 and
+// float-float.
 //
 // Stiffness operator A_k (Eq. hatA, component form), Fourier basis in and out,
 // five HBM passes with the pointwise work fused into the FFT passes:
-//   pass 1  z: gamma_c = (q (x) U + U (x) q)_c in Voigt order (engineering
-//            shear), inverse FFT along z                       3c in, 6c out
+//   pass 1  z: inverse FFTs a_k, b_k of U_k and q_z U_k along z, strains
+//            gamma_c in Voigt order (engineering shear)          3c in, 6c out
 //   pass 2  y: inverse FFT along y, 6 components in place      6c in, 6c out
 //   pass 3  x: inverse FFT along x, sigma = C_g(x) gamma / V,
 //            forward FFT along x, in place                      6c + id in, 6c out
@@ -13,30 +15,36 @@
 // with q = xi + k.  The factor 1/V of F^-1 and the unit scaling are folded
 // into the per-grain stiffness table.  Mass operator with non-uniform rho: the
 // same chain on the three displacement components with rho_g(x)/V in pass 3.
+//
+// A pencil of length N = r1 r2 r3 is transformed in place in shared memory by
+// decimation in frequency, each thread owning one radix-R butterfly in
+// registers at a time.  With the input index n = n1 r2 r3 + n2 r3 + n3:
+//   stage 1  DFT over n1 -> k1, times w_N^(k1 (n2 r3 + n3))
+//   stage 2  DFT over n2 -> k2, times w_(r2 r3)^(k2 n3)        (r2 > 1 only)
+//   stage 3  DFT over n3 -> k3
+// leaves output k = k1 + r1 k2 + r1 r2 k3 in the slot of (k1, k2, k3).  The
+// digit-reversed order costs nothing: the z and y passes write whole rows of
+// neighbouring pencils for each k, and the x pass applies the stress in that
+// order and undoes it with the mirrored (decimation in time) stages.  The
+// first stage loads its inputs straight from HBM into registers and the last
+// stage or the pointwise epilogue stores to HBM, so a component makes one
+// shared-memory round trip per stage and needs one buffer.  Tasks of all
+// components of a tile are spread over the CTA, so small tiles still fill its
+// threads; registers stay below the launch bounds and three FP32 CTAs share an
+// SM.
+//
+// Against the Stockham form these passes had before (tiles copied in, between
+// two buffers per stage and out; odd radices with run-time sines), K-apply:
+//   120 x 100 x 84, FP32, 6 systems   14.30 -> 0.76 ms
+//   256^3, FP32, 2 systems            14.26 -> 4.14 ms
+//   64^3, FP64, 4 systems              1.73 -> 1.48 ms (bound by FP64 issue)
+//   128^3, float-float, 4 systems      7.92 -> 4.62 ms (bound by FP32 issue)
 #pragma once
 
 #include "common.cuh"
 #include "fft.cuh"
 
 namespace bloch {
-
-// Division of n < 2^31 by an invariant divisor d >= 1 with one high multiply,
-// an add and a shift (Granlund & Montgomery 1994, division by invariant
-// integers): l = ceil(log2 d), m = floor(2^32 (2^l - d) / d) + 1,
-// n / d = (umulhi(m, n) + n) >> l.
-struct FastDiv {
-    unsigned m = 1;
-    int l = 0;
-};
-inline FastDiv make_fastdiv(unsigned d) {
-    FastDiv f;
-    int l = 0;
-    while ((1ull << l) < (unsigned long long)d) ++l;
-    f.l = l;
-    f.m = (unsigned)((((1ull << 32) * ((1ull << l) - d)) / d) + 1);
-    return f;
-}
-__device__ __forceinline__ unsigned fdiv(unsigned n, const FastDiv& f) { return (__umulhi(f.m, n) + n) >> f.l; }
 
 struct Geo {
     int Nx, Ny, Nz;
@@ -57,166 +65,478 @@ __device__ __forceinline__ bool sys_idle(const Geo& g, int b) {
     return g.skip != nullptr && g.skip[(size_t)b * g.skip_stride] == 0;
 }
 
-__device__ __forceinline__ int pad_even(int n) { return (n + 1) & ~1; }
+__host__ __device__ __forceinline__ int pad_even(int n) { return (n + 1) & ~1; }
+
+// Row position of slot n in the x passes: one spare slot every 16 spreads the
+// strided accesses of the last stage over the banks; xrow(N) is the row length (odd).
+__host__ __device__ __forceinline__ int xslot(int n) { return n + (n >> 4); }
+__host__ __device__ __forceinline__ int xrow(int N) { return (N + (N >> 4)) | 1; }
+
+// f(std::integral_constant<int, R>) for the run-time radix R.  Float-float
+// leaves out the radices whose code is longest for what they save (compile time).
+template <typename T, typename F>
+__device__ __forceinline__ void with_radix(int R, F&& f) {
+    switch (R) {
+#define BLOCH_RADIX(r) \
+    case r: f(std::integral_constant<int, r>{}); break;
+        BLOCH_RADIX(1) BLOCH_RADIX(2) BLOCH_RADIX(3) BLOCH_RADIX(4) BLOCH_RADIX(5) BLOCH_RADIX(6) BLOCH_RADIX(7)
+        BLOCH_RADIX(8) BLOCH_RADIX(9) BLOCH_RADIX(10) BLOCH_RADIX(15) BLOCH_RADIX(16)
+        default: break;
+    }
+    if constexpr (!std::is_same<T, dfloat>::value) {
+        switch (R) {
+            BLOCH_RADIX(12) BLOCH_RADIX(14)
+            default: break;
+        }
+    }
+}
+template <typename F>
+__device__ __forceinline__ void with_mid_radix(int R, F&& f) {
+    switch (R) {
+        BLOCH_RADIX(2) BLOCH_RADIX(3) BLOCH_RADIX(4) BLOCH_RADIX(5) BLOCH_RADIX(6) BLOCH_RADIX(7) BLOCH_RADIX(8)
+#undef BLOCH_RADIX
+        default: break;
+    }
+}
+
+template <typename C> using real_t = decltype(C::x);
+
+template <int DIR, typename C>
+__device__ __forceinline__ C twiddled(C v, C w) {
+    if (DIR > 0) w.y = -w.y;
+    return cmul(v, w);
+}
+
+// slot of output index k: (k1, k2, k3) with k = k1 + r1 k2 + r1 r2 k3
+__device__ __forceinline__ int slot_of(int k, const AxisPlan& a) {
+    const int t = (int)fdiv((unsigned)k, a.d1);
+    const int k1 = k - t * a.r1;
+    const int k3 = (int)fdiv((unsigned)t, a.d2);
+    return (k1 * a.r2 + (t - k3 * a.r2)) * a.r3 + k3;
+}
+
+// ------------------------------------------------ stages on pencil-fast tiles
+// Element (buffer c, slot n, pencil p) at c NP + (n << lp) + p, NP = N << lp.
+
+// middle stage (decimation in frequency) of nbuf buffers, in place
+template <int DIR, typename C>
+__device__ __forceinline__ void pf_mid(C* buf, int nbuf, const AxisPlan& a, int lp, const C* tw, int tid, int nthr) {
+    const int P1 = (1 << lp) - 1, NP = a.N << lp;
+    with_mid_radix(a.r2, [&](auto rc) {
+        constexpr int R = decltype(rc)::value;
+        const int per = (a.N / R) << lp, r3 = a.r3;
+        for (int t = tid; t < nbuf * per; t += nthr) {
+            const int c = t / per, u = t - c * per;
+            const int j = u >> lp, k1 = (int)fdiv((unsigned)j, a.d3), n3 = j - k1 * r3;
+            C* s = buf + c * NP + ((k1 * R * r3 + n3) << lp) + (u & P1);
+            C v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = s[(r * r3) << lp];
+            RegDFT<R, DIR, C>::run(v);
+            s[0] = v[0];
+#pragma unroll
+            for (int r = 1; r < R; ++r) s[(r * r3) << lp] = twiddled<DIR>(v[r], tw[r * n3 * a.r1]);
+        }
+    });
+}
+
+// last stage of nbuf buffers, in place
+template <int DIR, typename C>
+__device__ __forceinline__ void pf_last(C* buf, int nbuf, const AxisPlan& a, int lp, int tid, int nthr) {
+    const int P1 = (1 << lp) - 1;
+    with_radix<real_t<C>>(a.r3, [&](auto rc) {
+        constexpr int R = decltype(rc)::value;
+        if constexpr (R > 1) {
+            // the buffers are contiguous and N is a multiple of R: one run of butterflies over all of them
+            const int total = (nbuf * (a.N / R)) << lp;
+            for (int t = tid; t < total; t += nthr) {
+                C* s = buf + (((t >> lp) * R) << lp) + (t & P1);
+                C v[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[r] = s[r << lp];
+                RegDFT<R, DIR, C>::run(v);
+#pragma unroll
+                for (int r = 0; r < R; ++r) s[r << lp] = v[r];
+            }
+        }
+    });
+}
 
 // ---------------------------------------------------------------- pass 1
+// P = 1 << lp neighbouring pencils per CTA; blockIdx.y = system.  Buffers
+// a_x, b_x, a_y, b_y, a_z, b_z; with them the six Voigt strains are
+//   g_xx = q_x a_x, g_yy = q_y a_y, g_zz = b_z, g_yz = q_y a_z + b_y,
+//   g_xz = q_x a_z + b_x, g_xy = q_y a_x + q_x a_y
+// (q_x and q_y are constant on a z pencil).
 template <typename T>
-__global__ void __launch_bounds__(256, (sizeof(T) == 8) ? 2 : 1) k_pass_z_strain(const cplx_t<T>* __restrict__ U, cplx_t<T>* __restrict__ E,
-                                                       const T* __restrict__ qtab, const cplx_t<T>* __restrict__ twz,
-                                                       Geo g, int P) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
+    k_pass_z_strain(const cplx_t<T>* __restrict__ U, cplx_t<T>* __restrict__ E, const T* __restrict__ qtab,
+                    const cplx_t<T>* __restrict__ twz, Geo g, int lp) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* sm = reinterpret_cast<C*>(smem_raw);
-    const int N = g.Nz;
-    const int NP = N * P;
-    C* tw = sm;
-    C* sU = tw + pad_even(N);
-    C* sA = sU + 3 * NP;
-    C* sB = sA + NP;
+    const AxisPlan& a = g.ax[2];
+    const int N = a.N, NP = N << lp, P1 = (1 << lp) - 1;
+    C* tw = reinterpret_cast<C*>(smem_raw);
+    C* buf = tw + pad_even(N);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int b = blockIdx.y;
     if (sys_idle(g, b)) return;
-    const long long plane = (long long)g.Nx * g.Ny;
-    const long long pi0 = (long long)blockIdx.x * P;
-    const int np = (int)min((long long)P, plane - pi0);
+    const unsigned plane = (unsigned)g.Nx * (unsigned)g.Ny;
+    const unsigned pi0 = blockIdx.x << lp;
+    const int np = (int)min((unsigned)P1 + 1u, plane - pi0);
     const C* Ub = U + (size_t)b * 3 * g.V;
     C* Eb = E + (size_t)b * 6 * g.V;
     const T* qx = qtab + (size_t)b * (g.Nx + g.Ny + g.Nz);
     const T* qy = qx + g.Nx;
     const T* qz = qy + g.Ny;
-    const C zero = mk(T(0), T(0));
-
     for (int i = tid; i < N; i += nthr) tw[i] = twz[i];
-    for (int e = tid; e < 3 * NP; e += nthr) {
-        const int c = e / NP, r = e - c * NP, n = r / P, p = r - n * P;
-        sU[e] = (p < np) ? Ub[(size_t)c * g.V + (size_t)n * plane + pi0 + p] : zero;
-    }
     __syncthreads();
-    for (int c = 0; c < 6; ++c) {
-        for (int e = tid; e < NP; e += nthr) {
-            const int n = e / P, p = e - n * P;
-            const long long pi = pi0 + (p < np ? p : 0);
-            const int x = (int)(pi % g.Nx), y = (int)(pi / g.Nx);
-            const T ax = qx[x], ay = qy[y], az = qz[n];
-            const C ux = sU[e], uy = sU[NP + e], uz = sU[2 * NP + e];
-            C v;
-            switch (c) {
-                case 0: v = cscale(ux, ax); break;
-                case 1: v = cscale(uy, ay); break;
-                case 2: v = cscale(uz, az); break;
-                case 3: v = cadd(cscale(uy, az), cscale(uz, ay)); break;
-                case 4: v = cadd(cscale(ux, az), cscale(uz, ax)); break;
-                default: v = cadd(cscale(ux, ay), cscale(uy, ax)); break;
+    with_radix<real_t<C>>(a.r1, [&](auto rc) {
+        constexpr int R = decltype(rc)::value;
+        const int M = N / R, per = M << lp;
+        for (int t = tid; t < 3 * per; t += nthr) {
+            const int c = t / per, u = t - c * per;
+            const int p = u & P1, j = u >> lp;
+            const bool ok = p < np;
+            const C* src = Ub + (size_t)c * g.V + pi0 + (ok ? p : 0) + (size_t)j * plane;
+            C* s = buf + 2 * c * NP + u;
+            // the scaled transform reads its inputs again (from L1) where the
+            // registers cannot hold both
+            constexpr bool keep = sizeof(T) == 4 && R <= 8;
+            C v[R];
+            if constexpr (keep) {
+                C w[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    v[r] = src[(unsigned)(r * M) * plane];
+                    w[r] = cscale(v[r], ldg_t(qz + r * M + j));
+                }
+                RegDFT<R, +1, C>::run(v);
+                RegDFT<R, +1, C>::run(w);
+                s[0] = v[0];
+                s[NP] = w[0];
+#pragma unroll
+                for (int r = 1; r < R; ++r) {
+                    const C f = tw[r * j];
+                    s[(r * M) << lp] = twiddled<+1>(v[r], f);
+                    s[NP + ((r * M) << lp)] = twiddled<+1>(w[r], f);
+                }
+            } else {
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h, s += NP) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        v[r] = src[(unsigned)(r * M) * plane];
+                        if (h) v[r] = cscale(v[r], ldg_t(qz + r * M + j));
+                    }
+                    RegDFT<R, +1, C>::run(v);
+                    s[0] = v[0];
+#pragma unroll
+                    for (int r = 1; r < R; ++r) s[(r * M) << lp] = twiddled<+1>(v[r], tw[r * j]);
+                }
             }
-            sA[e] = v;
         }
+    });
+    __syncthreads();
+    if (a.r2 > 1) {
+        pf_mid<+1>(buf, 6, a, lp, tw, tid, nthr);
         __syncthreads();
-        C* res = fft_tile<+1, true>(sA, sB, g.ax[2], P, 0, tw, tid, nthr);
-        for (int e = tid; e < NP; e += nthr) {
-            const int n = e / P, p = e - n * P;
-            if (p < np) Eb[(size_t)c * g.V + (size_t)n * plane + pi0 + p] = res[e];
-        }
-        __syncthreads();
+    }
+    pf_last<+1>(buf, 6, a, lp, tid, nthr);
+    __syncthreads();
+    for (int t = tid; t < NP; t += nthr) {
+        const int p = t & P1, k = t >> lp;
+        if (p >= np) continue;
+        const C* s = buf + (slot_of(k, a) << lp) + p;
+        const unsigned pi = pi0 + p, y = fdiv(pi, g.dx);
+        const T ax = qx[pi - y * (unsigned)g.Nx], ay = qy[y];
+        const C a0 = s[0], b0 = s[NP], a1 = s[2 * NP], b1 = s[3 * NP], a2 = s[4 * NP], b2 = s[5 * NP];
+        C* d = Eb + (size_t)k * plane + pi;
+        d[0] = cscale(a0, ax);
+        d[g.V] = cscale(a1, ay);
+        d[2 * g.V] = b2;
+        d[3 * g.V] = cadd(cscale(a2, ay), b1);
+        d[4 * g.V] = cadd(cscale(a2, ax), b0);
+        d[5 * g.V] = cadd(cscale(a0, ay), cscale(a1, ax));
     }
 }
 
 // ------------------------------------------------- plain FFT pass along y or z
 // blockIdx.y enumerates (batch, component) pairs: offset blockIdx.y * V.
 template <typename T, int DIR, int AXIS>
-__global__ void __launch_bounds__(256) k_pass_axis(const cplx_t<T>* in, cplx_t<T>* out,
-                                                   const cplx_t<T>* __restrict__ twa, Geo g, int P,
-                                                   T out_scale) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
+    k_pass_axis(const cplx_t<T>* in, cplx_t<T>* out, const cplx_t<T>* __restrict__ twa, Geo g, int lp, T out_scale) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* sm = reinterpret_cast<C*>(smem_raw);
-    const int N = AXIS == 1 ? g.Ny : g.Nz;
-    const int NP = N * P;
-    C* tw = sm;
-    C* sA = tw + pad_even(N);
-    C* sB = sA + NP;
+    const AxisPlan& a = g.ax[AXIS];
+    const int N = a.N, P1 = (1 << lp) - 1;
+    C* tw = reinterpret_cast<C*>(smem_raw);
+    C* buf = tw + pad_even(N);
     const int tid = threadIdx.x, nthr = blockDim.x;
-    const long long npen = AXIS == 1 ? (long long)g.Nx * g.Nz : (long long)g.Nx * g.Ny;
-    const long long pi0 = (long long)blockIdx.x * P;
-    const int np = (int)min((long long)P, npen - pi0);
     if (sys_idle(g, (int)blockIdx.y / g.skip_ncomp)) return;
-    const size_t off = (size_t)blockIdx.y * g.V;
-    const C* src = in + off;
-    C* dst = out + off;
-    const long long plane = (long long)g.Nx * g.Ny;
-    const C zero = mk(T(0), T(0));
-
+    const unsigned nx = (unsigned)g.Nx, plane = nx * (unsigned)g.Ny;
+    const unsigned npen = AXIS == 1 ? nx * (unsigned)g.Nz : plane;
+    const unsigned step = AXIS == 1 ? nx : plane;     // between the elements of a pencil
+    const unsigned pi0 = blockIdx.x << lp;
+    const C* src = in + (size_t)blockIdx.y * g.V;
+    C* dst = out + (size_t)blockIdx.y * g.V;
+    // first element of pencil pi
+    auto base = [&](unsigned pi) -> size_t {
+        if (AXIS == 2) return pi;
+        const unsigned z = fdiv(pi, g.dx);
+        return (size_t)z * plane + (pi - z * nx);
+    };
     for (int i = tid; i < N; i += nthr) tw[i] = twa[i];
-    for (int e = tid; e < NP; e += nthr) {
-        const int n = e / P, p = e - n * P;
-        C v = zero;
-        if (p < np) {
-            const long long pi = pi0 + p;
-            size_t a;
-            if (AXIS == 1) a = (size_t)(pi / g.Nx) * plane + (size_t)n * g.Nx + (size_t)(pi % g.Nx);
-            else a = (size_t)n * plane + pi;
-            v = src[a];
-        }
-        sA[e] = v;
-    }
     __syncthreads();
-    C* res = fft_tile<DIR, true>(sA, sB, g.ax[AXIS], P, 0, tw, tid, nthr);
-    for (int e = tid; e < NP; e += nthr) {
-        const int n = e / P, p = e - n * P;
-        if (p < np) {
-            const long long pi = pi0 + p;
-            size_t a;
-            if (AXIS == 1) a = (size_t)(pi / g.Nx) * plane + (size_t)n * g.Nx + (size_t)(pi % g.Nx);
-            else a = (size_t)n * plane + pi;
-            dst[a] = cscale(res[e], out_scale);
+    with_radix<real_t<C>>(a.r1, [&](auto rc) {
+        constexpr int R = decltype(rc)::value;
+        const int M = N / R;
+        for (int t = tid; t < (M << lp); t += nthr) {
+            const unsigned pi = min(pi0 + (t & P1), npen - 1);
+            const int j = t >> lp;
+            const C* s = src + base(pi) + (size_t)j * step;
+            C v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = s[(unsigned)(r * M) * step];
+            RegDFT<R, DIR, C>::run(v);
+            buf[t] = v[0];
+#pragma unroll
+            for (int r = 1; r < R; ++r) buf[((r * M) << lp) + t] = twiddled<DIR>(v[r], tw[r * j]);
         }
+    });
+    __syncthreads();
+    if (a.r2 > 1) {
+        pf_mid<DIR>(buf, 1, a, lp, tw, tid, nthr);
+        __syncthreads();
     }
+    with_radix<real_t<C>>(a.r3, [&](auto rc) {
+        constexpr int R = decltype(rc)::value;
+        const int M = N / R;
+        for (int t = tid; t < (M << lp); t += nthr) {
+            const unsigned pi = pi0 + (t & P1);
+            if (pi >= npen) continue;
+            const int k = t >> lp;                    // k1 + r1 k2
+            const int k2 = (int)fdiv((unsigned)k, a.d1), k1 = k - k2 * a.r1;
+            const C* s = buf + (((k1 * a.r2 + k2) * R) << lp) + (t & P1);
+            C v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = s[r << lp];
+            RegDFT<R, DIR, C>::run(v);
+            C* d = dst + base(pi) + (size_t)k * step;
+#pragma unroll
+            for (int r = 0; r < R; ++r) d[(unsigned)(r * M) * step] = cscale(v[r], out_scale);
+        }
+    });
 }
 
-// ---------------------------------------------------------------- pass 3
-// Rows along x; all six strain components of P rows in shared memory.
+// ---------------------------------------------------------------- pass 5
 template <typename T>
-__global__ void __launch_bounds__(256, (sizeof(T) == 8) ? 2 : 1) k_pass_x_stress(cplx_t<T>* E, const int32_t* __restrict__ ids,
-                                                       const T* __restrict__ Ctab,
-                                                       const cplx_t<T>* __restrict__ twx, Geo g, int P) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
+    k_pass_z_div(const cplx_t<T>* __restrict__ E, cplx_t<T>* __restrict__ out, const T* __restrict__ qtab,
+                 const cplx_t<T>* __restrict__ twz, Geo g, int lp, T out_scale) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* sm = reinterpret_cast<C*>(smem_raw);
-    const int N = g.Nx;
-    const int NP = N * P;
-    C* tw = sm;
-    C* s0 = tw + pad_even(N);
+    const AxisPlan& a = g.ax[2];
+    const int N = a.N, NP = N << lp, P1 = (1 << lp) - 1;
+    C* tw = reinterpret_cast<C*>(smem_raw);
+    C* buf = tw + pad_even(N);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int b = blockIdx.y;
     if (sys_idle(g, b)) return;
-    const long long rows = (long long)g.Ny * g.Nz;
-    const long long r0 = (long long)blockIdx.x * P;
-    const int nr = (int)min((long long)P, rows - r0);
-    C* Eb = E + (size_t)b * 6 * g.V;
-    const C zero = mk(T(0), T(0));
-
-    for (int i = tid; i < N; i += nthr) tw[i] = twx[i];
-    for (int e = tid; e < 6 * NP; e += nthr) {
-        const int c = e / NP, r = e - c * NP, p = r / N, n = r - p * N;
-        s0[e] = (p < nr) ? Eb[(size_t)c * g.V + (size_t)(r0 + p) * N + n] : zero;
-    }
+    const unsigned plane = (unsigned)g.Nx * (unsigned)g.Ny;
+    const unsigned pi0 = blockIdx.x << lp;
+    const int np = (int)min((unsigned)P1 + 1u, plane - pi0);
+    const C* Eb = E + (size_t)b * 6 * g.V;
+    C* ob = out + (size_t)b * 3 * g.V;
+    const T* qx = qtab + (size_t)b * (g.Nx + g.Ny + g.Nz);
+    const T* qy = qx + g.Nx;
+    const T* qz = qy + g.Ny;
+    for (int i = tid; i < N; i += nthr) tw[i] = twz[i];
     __syncthreads();
-    C* buf[6];
-    C* wk = s0 + 6 * NP;
-#pragma unroll 1
-    for (int c = 0; c < 6; ++c) {
-        C* a = s0 + c * NP;
-        C* res = fft_tile<+1, false>(a, wk, g.ax[0], P, N, tw, tid, nthr);
-        if (res == wk) wk = a;
-        buf[c] = res;
+    with_radix<real_t<C>>(a.r1, [&](auto rc) {
+        constexpr int R = decltype(rc)::value;
+        const int M = N / R, per = M << lp;
+        for (int t = tid; t < 6 * per; t += nthr) {
+            const int c = t / per, u = t - c * per;
+            const int p = min(u & P1, np - 1), j = u >> lp;
+            const C* src = Eb + (size_t)c * g.V + pi0 + p + (size_t)j * plane;
+            C* s = buf + c * NP + u;
+            C v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = src[(unsigned)(r * M) * plane];
+            RegDFT<R, -1, C>::run(v);
+            s[0] = v[0];
+#pragma unroll
+            for (int r = 1; r < R; ++r) s[(r * M) << lp] = twiddled<-1>(v[r], tw[r * j]);
+        }
+    });
+    __syncthreads();
+    if (a.r2 > 1) {
+        pf_mid<-1>(buf, 6, a, lp, tw, tid, nthr);
+        __syncthreads();
     }
-    for (int e = tid; e < NP; e += nthr) {
-        const int p = e / N, n = e - p * N;
-        if (p < nr) {
-            const int gid = ids[(size_t)(r0 + p) * N + n];
-            const T* Cg = Ctab + (size_t)gid * 36;
+    pf_last<-1>(buf, 6, a, lp, tid, nthr);
+    __syncthreads();
+    for (int t = tid; t < NP; t += nthr) {
+        const int p = t & P1, k = t >> lp;
+        if (p >= np) continue;
+        const C* s = buf + (slot_of(k, a) << lp) + p;
+        const unsigned pi = pi0 + p, y = fdiv(pi, g.dx);
+        const T ax = qx[pi - y * (unsigned)g.Nx], ay = qy[y], az = qz[k];
+        const C s0 = s[0], s1 = s[NP], s2 = s[2 * NP], s3 = s[3 * NP], s4 = s[4 * NP], s5 = s[5 * NP];
+        C* d = ob + (size_t)k * plane + pi;
+        d[0] = cscale(cadd(cadd(cscale(s0, ax), cscale(s4, az)), cscale(s5, ay)), out_scale);
+        d[g.V] = cscale(cadd(cadd(cscale(s1, ay), cscale(s3, az)), cscale(s5, ax)), out_scale);
+        d[2 * g.V] = cscale(cadd(cadd(cscale(s2, az), cscale(s3, ay)), cscale(s4, ax)), out_scale);
+    }
+}
+
+// ------------------------------------------------ stages on rows along x
+// Element (component c, row p, slot n) at (c P + p) ld + xslot(n), ld = xrow(N).
+
+// stage 1 (decimation in frequency) of ncomp components of P rows, from HBM
+template <int DIR, typename C>
+__device__ __forceinline__ void lf_first(const C* Wb, long long V, C* buf, int ncomp, const AxisPlan& a, int P, int nr,
+                                         unsigned r0, const C* tw, int tid, int nthr) {
+    const int ld = xrow(a.N);
+    with_radix<real_t<C>>(a.r1, [&](auto rc) {
+        constexpr int R = decltype(rc)::value;
+        const int M = a.N / R;
+        for (int t = tid; t < ncomp * P * M; t += nthr) {
+            const int cp = (int)fdiv((unsigned)t, a.m1), j = t - cp * M;
+            const int c = cp / P, p = min(cp - c * P, nr - 1);
+            const C* src = Wb + (size_t)c * V + (size_t)(r0 + p) * a.N + j;
+            C* s = buf + cp * ld;
+            C v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = src[r * M];
+            RegDFT<R, DIR, C>::run(v);
+            s[xslot(j)] = v[0];
+#pragma unroll
+            for (int r = 1; r < R; ++r) s[xslot(r * M + j)] = twiddled<DIR>(v[r], tw[r * j]);
+        }
+    });
+}
+
+// middle stage: FREQ decimation in frequency (twiddles after), else in time (before)
+template <int DIR, bool FREQ, typename C>
+__device__ __forceinline__ void lf_mid(C* buf, int nrows, const AxisPlan& a, const C* tw, int tid, int nthr) {
+    const int ld = xrow(a.N);
+    with_mid_radix(a.r2, [&](auto rc) {
+        constexpr int R = decltype(rc)::value;
+        const int M = a.N / R, r3 = a.r3;
+        for (int t = tid; t < nrows * M; t += nthr) {
+            const int cp = (int)fdiv((unsigned)t, a.m2), j = t - cp * M;
+            const int k1 = (int)fdiv((unsigned)j, a.d3), n3 = j - k1 * r3;
+            const int s0 = k1 * R * r3 + n3;
+            C* s = buf + cp * ld;
+            C v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                v[r] = s[xslot(s0 + r * r3)];
+                if (!FREQ && r > 0) v[r] = twiddled<DIR>(v[r], tw[r * n3 * a.r1]);
+            }
+            RegDFT<R, DIR, C>::run(v);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (FREQ && r > 0) v[r] = twiddled<DIR>(v[r], tw[r * n3 * a.r1]);
+                s[xslot(s0 + r * r3)] = v[r];
+            }
+        }
+    });
+}
+
+// butterflies over the last digit, in place: the last stage of the inverse
+// and the first of the mirrored forward transform
+template <int DIR, typename C>
+__device__ __forceinline__ void lf_last(C* buf, int nrows, const AxisPlan& a, int tid, int nthr) {
+    const int ld = xrow(a.N);
+    with_radix<real_t<C>>(a.r3, [&](auto rc) {
+        constexpr int R = decltype(rc)::value;
+        if constexpr (R > 1) {
+            const int M = a.N / R;
+            for (int t = tid; t < nrows * M; t += nthr) {
+                const int cp = (int)fdiv((unsigned)t, a.m3), s0 = (t - cp * M) * R;
+                C* s = buf + cp * ld;
+                C v[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[r] = s[xslot(s0 + r)];
+                RegDFT<R, DIR, C>::run(v);
+#pragma unroll
+                for (int r = 0; r < R; ++r) s[xslot(s0 + r)] = v[r];
+            }
+        }
+    });
+}
+
+// last stage of the mirrored forward transform, to HBM
+template <int DIR, typename C>
+__device__ __forceinline__ void lf_store(C* Wb, long long V, const C* buf, int ncomp, const AxisPlan& a, int P, int nr,
+                                         unsigned r0, const C* tw, int tid, int nthr) {
+    const int ld = xrow(a.N);
+    with_radix<real_t<C>>(a.r1, [&](auto rc) {
+        constexpr int R = decltype(rc)::value;
+        const int M = a.N / R;
+        for (int t = tid; t < ncomp * P * M; t += nthr) {
+            const int cp = (int)fdiv((unsigned)t, a.m1), j = t - cp * M;
+            const int c = cp / P, p = cp - c * P;
+            if (p >= nr) continue;
+            const C* s = buf + cp * ld;
+            C v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                v[r] = s[xslot(r * M + j)];
+                if (r > 0) v[r] = twiddled<DIR>(v[r], tw[r * j]);
+            }
+            RegDFT<R, DIR, C>::run(v);
+            C* d = Wb + (size_t)c * V + (size_t)(r0 + p) * a.N + j;
+#pragma unroll
+            for (int r = 0; r < R; ++r) d[r * M] = v[r];
+        }
+    });
+}
+
+// Row pass along x on P rows per CTA (blockIdx.y = system): inverse FFT,
+// pointwise product in real space, forward FFT, in place.
+//   NC = 6: strains to stresses with the per-grain 6 x 6 table (pass 3)
+//   NC = 3: displacements times the per-grain scalar table (mass operator)
+template <typename T, int NC>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
+    k_pass_x_grain(cplx_t<T>* W, const int32_t* __restrict__ ids, const T* __restrict__ tab,
+                   const cplx_t<T>* __restrict__ twx, Geo g, int P) {
+    using C = cplx_t<T>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const AxisPlan& a = g.ax[0];
+    const int N = a.N, ld = xrow(N);
+    C* tw = reinterpret_cast<C*>(smem_raw);
+    C* buf = tw + pad_even(N);
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    const int b = blockIdx.y;
+    if (sys_idle(g, b)) return;
+    const unsigned rows = (unsigned)g.Ny * (unsigned)g.Nz;
+    const unsigned r0 = blockIdx.x * (unsigned)P;
+    const int nr = (int)min((unsigned)P, rows - r0);
+    C* Wb = W + (size_t)b * NC * g.V;
+    for (int i = tid; i < N; i += nthr) tw[i] = twx[i];
+    __syncthreads();
+    lf_first<+1>(Wb, g.V, buf, NC, a, P, nr, r0, tw, tid, nthr);
+    __syncthreads();
+    if (a.r2 > 1) {
+        lf_mid<+1, true>(buf, NC * P, a, tw, tid, nthr);
+        __syncthreads();
+    }
+    lf_last<+1>(buf, NC * P, a, tid, nthr);
+    __syncthreads();
+    for (int t = tid; t < nr * N; t += nthr) {
+        const int p = (int)fdiv((unsigned)t, g.dx), k = t - p * N;
+        const int gid = ids[(size_t)(r0 + p) * N + k];
+        C* s = buf + p * ld + xslot(slot_of(k, a));
+        const int cs = P * ld;
+        if constexpr (NC == 6) {
+            const T* Cg = tab + (size_t)gid * 36;
             C gam[6];
 #pragma unroll
-            for (int c = 0; c < 6; ++c) gam[c] = buf[c][e];
+            for (int c = 0; c < 6; ++c) gam[c] = s[c * cs];
 #pragma unroll
             for (int i = 0; i < 6; ++i) {
                 T sr = 0, si = 0;
@@ -226,142 +546,22 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 8) ? 2 : 1) k_pass_x_stress
                     sr = fma(cij, gam[j].x, sr);
                     si = fma(cij, gam[j].y, si);
                 }
-                buf[i][e] = mk(sr, si);
+                s[i * cs] = mk(sr, si);
             }
-        }
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int c = 0; c < 6; ++c) {
-        C* a = buf[c];
-        C* res = fft_tile<-1, false>(a, wk, g.ax[0], P, N, tw, tid, nthr);
-        if (res == wk) wk = a;
-        buf[c] = res;
-    }
-    for (int e = tid; e < 6 * NP; e += nthr) {
-        const int c = e / NP, r = e - c * NP, p = r / N, n = r - p * N;
-        if (p < nr) Eb[(size_t)c * g.V + (size_t)(r0 + p) * N + n] = buf[c][r];
-    }
-}
-
-// ---------------------------------------------------------------- pass 5
-template <typename T>
-__global__ void __launch_bounds__(256) k_pass_z_div(const cplx_t<T>* __restrict__ E, cplx_t<T>* __restrict__ out,
-                                                    const T* __restrict__ qtab, const cplx_t<T>* __restrict__ twz,
-                                                    Geo g, int P, T out_scale) {
-    using C = cplx_t<T>;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* sm = reinterpret_cast<C*>(smem_raw);
-    const int N = g.Nz;
-    const int NP = N * P;
-    C* tw = sm;
-    C* so = tw + pad_even(N);
-    C* sA = so + 3 * NP;
-    C* sB = sA + NP;
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int b = blockIdx.y;
-    if (sys_idle(g, b)) return;
-    const long long plane = (long long)g.Nx * g.Ny;
-    const long long pi0 = (long long)blockIdx.x * P;
-    const int np = (int)min((long long)P, plane - pi0);
-    const C* Eb = E + (size_t)b * 6 * g.V;
-    C* ob = out + (size_t)b * 3 * g.V;
-    const T* qx = qtab + (size_t)b * (g.Nx + g.Ny + g.Nz);
-    const T* qy = qx + g.Nx;
-    const T* qz = qy + g.Ny;
-    const C zero = mk(T(0), T(0));
-
-    for (int i = tid; i < N; i += nthr) tw[i] = twz[i];
-    for (int e = tid; e < 3 * NP; e += nthr) so[e] = zero;
-    for (int c = 0; c < 6; ++c) {
-        for (int e = tid; e < NP; e += nthr) {
-            const int n = e / P, p = e - n * P;
-            sA[e] = (p < np) ? Eb[(size_t)c * g.V + (size_t)n * plane + pi0 + p] : zero;
-        }
-        __syncthreads();
-        C* res = fft_tile<-1, true>(sA, sB, g.ax[2], P, 0, tw, tid, nthr);
-        for (int e = tid; e < NP; e += nthr) {
-            const int n = e / P, p = e - n * P;
-            const long long pi = pi0 + (p < np ? p : 0);
-            const int x = (int)(pi % g.Nx), y = (int)(pi / g.Nx);
-            const T ax = qx[x], ay = qy[y], az = qz[n];
-            const C s = res[e];
-            C* ox = so + e;
-            C* oy = so + NP + e;
-            C* oz = so + 2 * NP + e;
-            switch (c) {
-                case 0: *ox = cadd(*ox, cscale(s, ax)); break;
-                case 1: *oy = cadd(*oy, cscale(s, ay)); break;
-                case 2: *oz = cadd(*oz, cscale(s, az)); break;
-                case 3: *oy = cadd(*oy, cscale(s, az)); *oz = cadd(*oz, cscale(s, ay)); break;
-                case 4: *ox = cadd(*ox, cscale(s, az)); *oz = cadd(*oz, cscale(s, ax)); break;
-                default: *ox = cadd(*ox, cscale(s, ay)); *oy = cadd(*oy, cscale(s, ax)); break;
-            }
-        }
-        __syncthreads();
-    }
-    for (int e = tid; e < 3 * NP; e += nthr) {
-        const int c = e / NP, r = e - c * NP, n = r / P, p = r - n * P;
-        if (p < np) ob[(size_t)c * g.V + (size_t)n * plane + pi0 + p] = cscale(so[e], out_scale);
-    }
-}
-
-// ------------------------------------------- mass operator, non-uniform rho
-template <typename T>
-__global__ void __launch_bounds__(256) k_pass_x_rho(cplx_t<T>* W, const int32_t* __restrict__ ids,
-                                                    const T* __restrict__ rtab,
-                                                    const cplx_t<T>* __restrict__ twx, Geo g, int P) {
-    using C = cplx_t<T>;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* sm = reinterpret_cast<C*>(smem_raw);
-    const int N = g.Nx;
-    const int NP = N * P;
-    C* tw = sm;
-    C* s0 = tw + pad_even(N);
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int b = blockIdx.y;
-    if (sys_idle(g, b)) return;
-    const long long rows = (long long)g.Ny * g.Nz;
-    const long long r0 = (long long)blockIdx.x * P;
-    const int nr = (int)min((long long)P, rows - r0);
-    C* Wb = W + (size_t)b * 3 * g.V;
-    const C zero = mk(T(0), T(0));
-
-    for (int i = tid; i < N; i += nthr) tw[i] = twx[i];
-    for (int e = tid; e < 3 * NP; e += nthr) {
-        const int c = e / NP, r = e - c * NP, p = r / N, n = r - p * N;
-        s0[e] = (p < nr) ? Wb[(size_t)c * g.V + (size_t)(r0 + p) * N + n] : zero;
-    }
-    __syncthreads();
-    C* buf[3];
-    C* wk = s0 + 3 * NP;
-#pragma unroll 1
-    for (int c = 0; c < 3; ++c) {
-        C* a = s0 + c * NP;
-        C* res = fft_tile<+1, false>(a, wk, g.ax[0], P, N, tw, tid, nthr);
-        if (res == wk) wk = a;
-        buf[c] = res;
-    }
-    for (int e = tid; e < NP; e += nthr) {
-        const int p = e / N, n = e - p * N;
-        if (p < nr) {
-            const T r = ldg_t(rtab + ids[(size_t)(r0 + p) * N + n]);
+        } else {
+            const T r = ldg_t(tab + gid);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) buf[c][e] = cscale(buf[c][e], r);
+            for (int c = 0; c < NC; ++c) s[c * cs] = cscale(s[c * cs], r);
         }
     }
     __syncthreads();
-#pragma unroll 1
-    for (int c = 0; c < 3; ++c) {
-        C* a = buf[c];
-        C* res = fft_tile<-1, false>(a, wk, g.ax[0], P, N, tw, tid, nthr);
-        if (res == wk) wk = a;
-        buf[c] = res;
+    lf_last<-1>(buf, NC * P, a, tid, nthr);
+    __syncthreads();
+    if (a.r2 > 1) {
+        lf_mid<-1, false>(buf, NC * P, a, tw, tid, nthr);
+        __syncthreads();
     }
-    for (int e = tid; e < 3 * NP; e += nthr) {
-        const int c = e / NP, r = e - c * NP, p = r / N, n = r - p * N;
-        if (p < nr) Wb[(size_t)c * g.V + (size_t)(r0 + p) * N + n] = buf[c][r];
-    }
+    lf_store<-1>(Wb, g.V, buf, NC, a, P, nr, r0, tw, tid, nthr);
 }
 
 // ------------------------------------------- plain transform along x
@@ -369,41 +569,36 @@ __global__ void __launch_bounds__(256) k_pass_x_rho(cplx_t<T>* W, const int32_t*
 // of nb systems along x, in place, times out_scale; rows are contiguous, P
 // rows per CTA, blockIdx.y = system.
 template <typename T, int DIR>
-__global__ void __launch_bounds__(256) k_pass_x(cplx_t<T>* W, const cplx_t<T>* __restrict__ twx, Geo g, int P,
-                                                T out_scale) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
+    k_pass_x(cplx_t<T>* W, const cplx_t<T>* __restrict__ twx, Geo g, int P, T out_scale) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* sm = reinterpret_cast<C*>(smem_raw);
-    const int N = g.Nx;
-    const int NP = N * P;
-    C* tw = sm;
-    C* s0 = tw + pad_even(N);
+    const AxisPlan& a = g.ax[0];
+    const int N = a.N, ld = xrow(N);
+    C* tw = reinterpret_cast<C*>(smem_raw);
+    C* buf = tw + pad_even(N);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int b = blockIdx.y;
-    const long long rows = (long long)g.Ny * g.Nz;
-    const long long r0 = (long long)blockIdx.x * P;
-    const int nr = (int)min((long long)P, rows - r0);
+    if (sys_idle(g, b)) return;
+    const unsigned rows = (unsigned)g.Ny * (unsigned)g.Nz;
+    const unsigned r0 = blockIdx.x * (unsigned)P;
+    const int nr = (int)min((unsigned)P, rows - r0);
     C* Wb = W + (size_t)b * 3 * g.V;
-    const C zero = mk(T(0), T(0));
     for (int i = tid; i < N; i += nthr) tw[i] = twx[i];
-    for (int e = tid; e < 3 * NP; e += nthr) {
-        const int c = e / NP, r = e - c * NP, p = r / N, n = r - p * N;
-        s0[e] = (p < nr) ? Wb[(size_t)c * g.V + (size_t)(r0 + p) * N + n] : zero;
-    }
     __syncthreads();
-    C* buf[3];
-    C* wk = s0 + 3 * NP;
-#pragma unroll 1
-    for (int c = 0; c < 3; ++c) {
-        C* a = s0 + c * NP;
-        C* res = fft_tile<DIR, false>(a, wk, g.ax[0], P, N, tw, tid, nthr);
-        if (res == wk) wk = a;
-        buf[c] = res;
-    }
+    lf_first<DIR>(Wb, g.V, buf, 3, a, P, nr, r0, tw, tid, nthr);
     __syncthreads();
-    for (int e = tid; e < 3 * NP; e += nthr) {
-        const int c = e / NP, r = e - c * NP, p = r / N, n = r - p * N;
-        if (p < nr) Wb[(size_t)c * g.V + (size_t)(r0 + p) * N + n] = cscale(buf[c][r], out_scale);
+    if (a.r2 > 1) {
+        lf_mid<DIR, true>(buf, 3 * P, a, tw, tid, nthr);
+        __syncthreads();
+    }
+    lf_last<DIR>(buf, 3 * P, a, tid, nthr);
+    __syncthreads();
+    for (int t = tid; t < 3 * P * N; t += nthr) {
+        const int cp = (int)fdiv((unsigned)t, g.dx), k = t - cp * N;
+        const int c = cp / P, p = cp - c * P;
+        if (p < nr)
+            Wb[(size_t)c * g.V + (size_t)(r0 + p) * N + k] = cscale(buf[cp * ld + xslot(slot_of(k, a))], out_scale);
     }
 }
 

@@ -1,0 +1,128 @@
+// Launchers of the mixed-radix passes (passes.cuh), one translation unit per
+// field type.
+#pragma once
+
+#include <algorithm>
+
+#include "internal.h"
+
+namespace bloch {
+
+template <typename T> static inline const cplx_t<T>* pass_tw(const bloch_plan* pl, int axis);
+template <> inline const float2* pass_tw<float>(const bloch_plan* pl, int axis) { return pl->d_twf[axis]; }
+template <> inline const double2* pass_tw<double>(const bloch_plan* pl, int axis) { return pl->d_twd[axis]; }
+template <> inline const dfloat2* pass_tw<dfloat>(const bloch_plan* pl, int axis) { return pl->d_twx[axis]; }
+template <typename T> static inline const T* pass_ctab(const bloch_plan* pl);
+template <> inline const float* pass_ctab<float>(const bloch_plan* pl) { return pl->d_Cf; }
+template <> inline const double* pass_ctab<double>(const bloch_plan* pl) { return pl->d_Cd; }
+template <> inline const dfloat* pass_ctab<dfloat>(const bloch_plan* pl) { return pl->d_Cx; }
+template <typename T> static inline const T* pass_rtab(const bloch_plan* pl);
+template <> inline const float* pass_rtab<float>(const bloch_plan* pl) { return pl->d_rf; }
+template <> inline const double* pass_rtab<double>(const bloch_plan* pl) { return pl->d_rd; }
+template <> inline const dfloat* pass_rtab<dfloat>(const bloch_plan* pl) { return pl->d_rx; }
+
+static inline dim3 pass_grid(long long npen, int lp, int ny) {
+    return dim3((unsigned)((npen + (1LL << lp) - 1) >> lp), (unsigned)ny);
+}
+
+template <typename T>
+void pass_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab) {
+    const PassTile& t = tile_of<T>(pl).z6;
+    ++pl->launches;
+    k_pass_z_strain<T><<<pass_grid((long long)pl->Nx * pl->Ny, t.lp, nb), t.nthr, t.smem, pl->stream>>>(
+        u, E, qtab, pass_tw<T>(pl, 2), geo_of<T>(pl), t.lp);
+}
+
+template <typename T>
+void pass_axis(bloch_plan* pl, int axis, int dir, int nfields, const cplx_t<T>* in, cplx_t<T>* out, T out_scale) {
+    const TileCfg& tc = tile_of<T>(pl);
+    const PassTile& t = axis == 1 ? tc.y1 : tc.z1;
+    const dim3 gr = pass_grid((long long)pl->Nx * (axis == 1 ? pl->Nz : pl->Ny), t.lp, nfields);
+    const Geo& g = geo_of<T>(pl);
+    const cplx_t<T>* tw = pass_tw<T>(pl, axis);
+    ++pl->launches;
+    if (axis == 1 && dir > 0)
+        k_pass_axis<T, +1, 1><<<gr, t.nthr, t.smem, pl->stream>>>(in, out, tw, g, t.lp, out_scale);
+    else if (axis == 1)
+        k_pass_axis<T, -1, 1><<<gr, t.nthr, t.smem, pl->stream>>>(in, out, tw, g, t.lp, out_scale);
+    else if (dir > 0)
+        k_pass_axis<T, +1, 2><<<gr, t.nthr, t.smem, pl->stream>>>(in, out, tw, g, t.lp, out_scale);
+    else
+        k_pass_axis<T, -1, 2><<<gr, t.nthr, t.smem, pl->stream>>>(in, out, tw, g, t.lp, out_scale);
+}
+
+template <typename T>
+void pass_x_stress(bloch_plan* pl, int nb, cplx_t<T>* E) {
+    const PassTile& t = tile_of<T>(pl).x6;
+    ++pl->launches;
+    k_pass_x_grain<T, 6><<<pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb), t.nthr, t.smem, pl->stream>>>(
+        E, pl->d_ids, pass_ctab<T>(pl), pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp);
+}
+
+template <typename T>
+void pass_x_rho(bloch_plan* pl, int nb, cplx_t<T>* W) {
+    const PassTile& t = tile_of<T>(pl).x3;
+    ++pl->launches;
+    k_pass_x_grain<T, 3><<<pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb), t.nthr, t.smem, pl->stream>>>(
+        W, pl->d_ids, pass_rtab<T>(pl), pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp);
+}
+
+template <typename T>
+void pass_x(bloch_plan* pl, int dir, int nb, cplx_t<T>* W, T out_scale) {
+    const PassTile& t = tile_of<T>(pl).x3;
+    const dim3 gr = pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb);
+    ++pl->launches;
+    if (dir > 0)
+        k_pass_x<T, +1><<<gr, t.nthr, t.smem, pl->stream>>>(W, pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp, out_scale);
+    else
+        k_pass_x<T, -1><<<gr, t.nthr, t.smem, pl->stream>>>(W, pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp, out_scale);
+}
+
+template <typename T>
+void pass_z_div(bloch_plan* pl, int nb, const cplx_t<T>* E, cplx_t<T>* out, const T* qtab, T out_scale) {
+    const PassTile& t = tile_of<T>(pl).z6;
+    ++pl->launches;
+    k_pass_z_div<T><<<pass_grid((long long)pl->Nx * pl->Ny, t.lp, nb), t.nthr, t.smem, pl->stream>>>(
+        E, out, qtab, pass_tw<T>(pl, 2), geo_of<T>(pl), t.lp, out_scale);
+}
+
+template <typename K>
+static cudaError_t pass_attr(K k) {
+    return allow_max_dyn_smem(k);
+}
+template <typename T>
+cudaError_t pass_attrs_z() {
+    cudaError_t e = pass_attr(k_pass_z_strain<T>);
+    return e == cudaSuccess ? pass_attr(k_pass_z_div<T>) : e;
+}
+template <typename T>
+cudaError_t pass_attrs_axis() {
+    cudaError_t e = pass_attr(k_pass_axis<T, +1, 1>);
+    if (e == cudaSuccess) e = pass_attr(k_pass_axis<T, -1, 1>);
+    if (e == cudaSuccess) e = pass_attr(k_pass_axis<T, +1, 2>);
+    return e == cudaSuccess ? pass_attr(k_pass_axis<T, -1, 2>) : e;
+}
+template <typename T>
+cudaError_t pass_attrs_x() {
+    cudaError_t e = pass_attr(k_pass_x_grain<T, 6>);
+    if (e == cudaSuccess) e = pass_attr(k_pass_x_grain<T, 3>);
+    if constexpr (!std::is_same<T, dfloat>::value) {
+        if (e == cudaSuccess) e = pass_attr(k_pass_x<T, +1>);
+        if (e == cudaSuccess) e = pass_attr(k_pass_x<T, -1>);
+    }
+    return e;
+}
+
+#define BLOCH_INST_PASSES_Z(T)                                                                            \
+    template void pass_z_strain<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, const T*);             \
+    template void pass_z_div<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, const T*, T);             \
+    template cudaError_t pass_attrs_z<T>();
+#define BLOCH_INST_PASSES_AXIS(T)                                                                         \
+    template void pass_axis<T>(bloch_plan*, int, int, int, const cplx_t<T>*, cplx_t<T>*, T);              \
+    template cudaError_t pass_attrs_axis<T>();
+#define BLOCH_INST_PASSES_X(T)                                                                            \
+    template void pass_x_stress<T>(bloch_plan*, int, cplx_t<T>*);                                         \
+    template void pass_x_rho<T>(bloch_plan*, int, cplx_t<T>*);                                            \
+    template cudaError_t pass_attrs_x<T>();
+
+}  // namespace bloch
