@@ -231,9 +231,6 @@ bloch_status set_k(bloch_plan* pl, int nb, const double* k_host) {
 }
 
 // ------------------------------------------------------------ operators
-template <typename T>
-void launch_K_generic(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale);
-
 // ------------------------------------------------ fast two-stage passes
 static bool fast_axis(int N) { return N == 16 || N == 32 || N == 64 || N == 128 || N == 256; }
 static bool fast_x(int N) { return N == 16 || N == 32 || N == 64 || N == 128; }
@@ -285,8 +282,8 @@ static void fast_attr(K k) {
 template <typename T, int RA, int RB, bool Z>
 static void set_fast_attrs_n() {
     constexpr int PT = (RA * RB * 32 * sizeof(cplx_t<T>) <= 64 * 1024) ? 32 : 16;
-    fast_attr(k_fpass_y<T, +1, RA, RB, PT>);
-    fast_attr(k_fpass_y<T, -1, RA, RB, PT>);
+    fast_attr(k_fpass_axis<T, +1, RA, RB, PT>);
+    fast_attr(k_fpass_axis<T, -1, RA, RB, PT>);
     if constexpr (Z) {
         fast_attr(k_fpass_z_strain<T, RA, RB, kFastZThreads>);
         fast_attr(k_fpass_z_div<T, RA, RB, kFastZThreads>);
@@ -306,19 +303,24 @@ static void set_fast_attrs() {
     set_fast_attrs_n<T, 16, 16, false>();
 }
 
+// y (axis 1) or z (axis 2) pass of nfields fields
 template <typename T, int RA, int RB>
-static void fast_y(bloch_plan* pl, int DIR, int nb, cplx_t<T>* E) {
+static void fast_yz(bloch_plan* pl, int axis, int DIR, int nfields, const cplx_t<T>* in, cplx_t<T>* out, T scale) {
     const Geo& g = geo_of<T>(pl);
     constexpr int N = RA * RB;
     constexpr int PT = (N * 32 * sizeof(cplx_t<T>) <= 64 * 1024) ? 32 : 16;
-    const long long npen = (long long)pl->Nx * pl->Nz;
+    const unsigned plane = (unsigned)pl->Nx * pl->Ny;
+    const unsigned inner = axis == 1 ? (unsigned)pl->Nx : plane, outer = axis == 1 ? plane : 0;
+    const unsigned npen = axis == 1 ? (unsigned)pl->Nx * pl->Nz : plane;
     const size_t smem = (size_t)(N + N * PT) * sizeof(cplx_t<T>);
-    dim3 gr((unsigned)((npen + PT - 1) / PT), nb * 6);
+    dim3 gr((npen + PT - 1) / PT, nfields);
     ++pl->launches;
     if (DIR > 0)
-        k_fpass_y<T, +1, RA, RB, PT><<<gr, 256, smem, pl->stream>>>(E, E, tw_of<T>(pl, 1), g);
+        k_fpass_axis<T, +1, RA, RB, PT>
+            <<<gr, 256, smem, pl->stream>>>(in, out, tw_of<T>(pl, axis), g, inner, outer, npen, scale);
     else
-        k_fpass_y<T, -1, RA, RB, PT><<<gr, 256, smem, pl->stream>>>(E, E, tw_of<T>(pl, 1), g);
+        k_fpass_axis<T, -1, RA, RB, PT>
+            <<<gr, 256, smem, pl->stream>>>(in, out, tw_of<T>(pl, axis), g, inner, outer, npen, scale);
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link to the driver library)
@@ -371,48 +373,42 @@ bloch_status check_pass_err(bloch_plan* pl) {
     return BLOCH_OK;
 }
 
-template <typename T, int RA, int RB>
-static void fast_z1(bloch_plan* pl, int nb, const cplx_t<T>* u) {
-    const Geo& g = geo_of<T>(pl);
+template <int RA, int RB>
+static void fast_z1(bloch_plan* pl, int nb, const float2* u, float2* E, const float* qtab) {
     constexpr int NT = kFastZThreads;
     constexpr int P = NT / RA;
     const long long npen = (long long)pl->Nx * pl->Ny;
-    const size_t smem = fpass_z1_smem<T, RA, RB, NT>();
     dim3 gr((unsigned)((npen + P - 1) / P), nb);
     ++pl->launches;
     CUtensorMap map;
     const int tma = encode_zmap(&map, u, pl, 3LL * nb, P) ? 1 : 0;
-    k_fpass_z_strain<T, RA, RB, NT><<<gr, NT, smem, pl->stream>>>(u, ws_of<T>(pl).E, ws_of<T>(pl).qtab,
-                                                                   tw_of<T>(pl, 2), g, map, tma);
+    k_fpass_z_strain<float, RA, RB, NT><<<gr, NT, fpass_z1_smem<float, RA, RB, NT>(), pl->stream>>>(
+        u, E, qtab, pl->d_twf[2], pl->geo_f, map, tma);
 }
 
-template <typename T, int RA, int RB>
-static void fast_z5(bloch_plan* pl, int nb, cplx_t<T>* out, T out_scale, const cplx_t<T>* dotp, double2* dpart) {
-    const Geo& g = geo_of<T>(pl);
+template <int RA, int RB>
+static void fast_z5(bloch_plan* pl, int nb, const float2* E, const float* qtab, float2* out, float out_scale,
+                    const float2* dotp, double2* dpart) {
     constexpr int NT = kFastZThreads;
     constexpr int P = NT / RA;
     const long long npen = (long long)pl->Nx * pl->Ny;
-    const size_t smem = fpass_z5_smem<T, RA, RB, NT>();
     dim3 gr((unsigned)((npen + P - 1) / P), nb);
     ++pl->launches;
     CUtensorMap map;
-    const int tma = encode_zmap(&map, ws_of<T>(pl).E, pl, 6LL * nb, P) ? 1 : 0;
-    k_fpass_z_div<T, RA, RB, NT><<<gr, NT, smem, pl->stream>>>(ws_of<T>(pl).E, out, ws_of<T>(pl).qtab,
-                                                                tw_of<T>(pl, 2), g, out_scale, dotp, dpart, map,
-                                                                tma);
+    const int tma = encode_zmap(&map, E, pl, 6LL * nb, P) ? 1 : 0;
+    k_fpass_z_div<float, RA, RB, NT><<<gr, NT, fpass_z5_smem<float, RA, RB, NT>(), pl->stream>>>(
+        E, out, qtab, pl->d_twf[2], pl->geo_f, out_scale, dotp, dpart, map, tma);
 }
 
-// returns the CTAs per system (the number of (p, A p) partials written when dpart != nullptr)
-template <typename T, int RA, int RB>
-static int fast_x3(bloch_plan* pl, int nb, double2* dpart) {
-    const Geo& g = geo_of<T>(pl);
+// Returns the CTAs per system (the number of (p, A p) partials written when dpart != nullptr)
+template <int RA, int RB>
+static int fast_x3(bloch_plan* pl, int nb, float2* E, double2* dpart) {
     constexpr int P = 128 / RA;
-    const size_t smem = fpass_x_smem<T, RA, RB>();
     const long long rows = (long long)pl->Ny * pl->Nz;
     dim3 gr((unsigned)((rows + P - 1) / P), nb);
     ++pl->launches;
-    k_fpass_x_stress<T, RA, RB><<<gr, 128, smem, pl->stream>>>(ws_of<T>(pl).E, pl->d_ids, cpk_of<T>(pl),
-                                                                 tw_of<T>(pl, 0), g, dpart);
+    k_fpass_x_stress<float, RA, RB><<<gr, 128, fpass_x_smem<float, RA, RB>(), pl->stream>>>(
+        E, pl->d_ids, pl->d_Cpf, pl->d_twf[0], pl->geo_f, dpart);
     return (int)gr.x;
 }
 
@@ -424,108 +420,86 @@ static int fast_x3(bloch_plan* pl, int nb, double2* dpart) {
         case 128: FN<T, 16, 8>(__VA_ARGS__); break; \
         default: FN<T, 16, 16>(__VA_ARGS__); break; \
     }
-#define BLOCH_FAST_SWITCH_Z(N, FN, ...)             \
-    switch (N) {                                    \
-        case 16: FN<T, 4, 4>(__VA_ARGS__); break;   \
-        case 32: FN<T, 8, 4>(__VA_ARGS__); break;   \
-        case 64: FN<T, 8, 8>(__VA_ARGS__); break;   \
-        default: FN<T, 16, 8>(__VA_ARGS__); break;  \
+// FP32-only kernels on axes of 16 .. 128
+#define BLOCH_FAST_SWITCH_F(N, R, FN, ...)        \
+    switch (N) {                                  \
+        case 16: R FN<4, 4>(__VA_ARGS__); break;  \
+        case 32: R FN<8, 4>(__VA_ARGS__); break;  \
+        case 64: R FN<8, 8>(__VA_ARGS__); break;  \
+        default: R FN<16, 8>(__VA_ARGS__); break; \
     }
+
+// 1D FFTs along y (axis 1) or z (axis 2) of nfields scalar fields
+template <typename T>
+static void launch_axis(bloch_plan* pl, int axis, int DIR, int nfields, const cplx_t<T>* in, cplx_t<T>* out, T scale) {
+    const int N = axis == 1 ? pl->Ny : pl->Nz;
+    if (pl->fast && fast_axis(N)) {
+        BLOCH_FAST_SWITCH(N, fast_yz, pl, axis, DIR, nfields, in, out, scale);
+    } else {
+        pass_axis<T>(pl, axis, DIR, nfields, in, out, scale);
+    }
+}
+
+// Pass 1: strains and their inverse FFT along z
+template <typename T>
+static void launch_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab) {
+    if constexpr (std::is_same<T, float>::value) {
+        if (pl->fast && fast_x(pl->Nz)) {
+            BLOCH_FAST_SWITCH_F(pl->Nz, , fast_z1, pl, nb, u, E, qtab);
+            return;
+        }
+    }
+    pass_z_strain<T>(pl, nb, u, E, qtab);
+}
+
+// Passes 1-4: strains, their inverse FFT, stresses, forward FFT along x and y.
+// Returns the (p, A p) partials per system the x pass wrote (0: none).
+static int launch_stress_f(bloch_plan* pl, int nb, const float2* u, float2* E, const float* qtab, double2* dpart) {
+    int blk = 0;
+    launch_z_strain<float>(pl, nb, u, E, qtab);
+    launch_axis<float>(pl, 1, +1, 6 * nb, E, E, 1.0f);
+    if (pl->fast && fast_x(pl->Nx)) {
+        BLOCH_FAST_SWITCH_F(pl->Nx, blk =, fast_x3, pl, nb, E, dpart);
+    } else {
+        pass_x_stress<float>(pl, nb, E);
+    }
+    launch_axis<float>(pl, 1, -1, 6 * nb, E, E, 1.0f);
+    return dpart ? blk : 0;
+}
+
+int launch_K_on(bloch_plan* pl, int nb, const float2* u, float2* E, const float* qtab, float2* out, float out_scale,
+                const float2* dotp, double2* dpart) {
+    const bool dot = dotp && dpart;
+    int nblk = launch_stress_f(pl, nb, u, E, qtab, dot ? dpart : nullptr);
+    if (pl->fast && fast_x(pl->Nz)) {
+        // without a fast x pass the divergence forms the product and reads dotp again
+        const bool zdot = dot && nblk == 0;
+        BLOCH_FAST_SWITCH_F(pl->Nz, , fast_z5, pl, nb, E, qtab, out, out_scale, zdot ? dotp : nullptr,
+                            zdot ? dpart : nullptr);
+        if (zdot) nblk = fast_z_blocks(pl);
+    } else {
+        pass_z_div<float>(pl, nb, E, out, qtab, out_scale);
+    }
+    return nblk;
+}
 
 template <typename T>
 int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale, const cplx_t<T>* dotp,
              double2* dpart) {
-    if (pl->variant == 2) {
-        Workspace<T>& w = ws_of<T>(pl);
-        if (!cufft_launch_K<T>(pl, nb, u, out, out_scale, w.E, w.qtab, ctab_of<T>(pl), geo_of<T>(pl)))
-            pl->pending = set_error(BLOCH_ECUDA, "cuFFT plan or execution failed");
-        return 0;
-    }
-    int fused = 0;
-    if (pl->fast) {
-        Workspace<T>& w = ws_of<T>(pl);
-        const bool fz = fast_x(pl->Nz) && std::is_same<T, float>::value;
-        const bool fy = fast_axis(pl->Ny);
-        const bool fx = fast_x(pl->Nx) && std::is_same<T, float>::value;
-        bool done1 = false;
-        if constexpr (std::is_same<T, float>::value) {
-            if (fz) {
-                BLOCH_FAST_SWITCH_Z(pl->Nz, fast_z1, pl, nb, u);
-                done1 = true;
-            }
-        }
-        if (!done1) pass_z_strain<T>(pl, nb, u, w.E, w.qtab);
-        if (fy) {
-            BLOCH_FAST_SWITCH(pl->Ny, fast_y, pl, +1, nb, w.E);
-        } else {
-            pass_axis<T>(pl, 1, +1, 6 * nb, w.E, w.E, T(1));
-        }
-        // (p, A p) partials: from the strain energy in the fast x pass where it runs,
-        // else from the fast z-divergence pass (which then reads p once more)
-        bool done3 = false;
-        const bool xdot = fx && dpart && dotp;
-        if constexpr (std::is_same<T, float>::value) {
-            if (fx) {
-                double2* xd = xdot ? dpart : nullptr;
-                int xb = 0;
-                switch (pl->Nx) {
-                    case 16: xb = fast_x3<T, 4, 4>(pl, nb, xd); break;
-                    case 32: xb = fast_x3<T, 8, 4>(pl, nb, xd); break;
-                    case 64: xb = fast_x3<T, 8, 8>(pl, nb, xd); break;
-                    default: xb = fast_x3<T, 16, 8>(pl, nb, xd); break;
-                }
-                if (xdot) fused = xb;
-                done3 = true;
-            }
-        }
-        if (!done3) pass_x_stress<T>(pl, nb, w.E);
-        if (fy) {
-            BLOCH_FAST_SWITCH(pl->Ny, fast_y, pl, -1, nb, w.E);
-        } else {
-            pass_axis<T>(pl, 1, -1, 6 * nb, w.E, w.E, T(1));
-        }
-        bool done5 = false;
-        if constexpr (std::is_same<T, float>::value) {
-            if (fz) {
-                const bool zdot = !xdot && dpart && dotp;
-                BLOCH_FAST_SWITCH_Z(pl->Nz, fast_z5, pl, nb, out, out_scale, zdot ? dotp : nullptr,
-                                    zdot ? dpart : nullptr);
-                done5 = true;
-                if (zdot) fused = fast_z_blocks(pl);
-            }
-        }
-        if (!done5) pass_z_div<T>(pl, nb, w.E, out, w.qtab, out_scale);
-        return fused;
-    }
-    launch_K_generic<T>(pl, nb, u, out, out_scale);
-    return 0;
-}
-
-template <typename T>
-void launch_K_generic(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale) {
     Workspace<T>& w = ws_of<T>(pl);
-    pass_z_strain<T>(pl, nb, u, w.E, w.qtab);
-    pass_axis<T>(pl, 1, +1, 6 * nb, w.E, w.E, T(1));
-    pass_x_stress<T>(pl, nb, w.E);
-    pass_axis<T>(pl, 1, -1, 6 * nb, w.E, w.E, T(1));
-    pass_z_div<T>(pl, nb, w.E, out, w.qtab, out_scale);
-}
-
-// Float-float operator: the mixed-radix passes; the two-stage register y
-// passes where the y axis has one (fft_variant 0)
-template <>
-int launch_K<dfloat>(bloch_plan* pl, int nb, const dfloat2* u, dfloat2* out, dfloat out_scale, const dfloat2*,
-                     double2*) {
-    using T = dfloat;
-    if (!pl->fast || !fast_axis(pl->Ny)) {
-        launch_K_generic<T>(pl, nb, u, out, out_scale);
-        return 0;
+    if constexpr (!std::is_same<T, dfloat>::value) {   // cuFFT has no float-float transform
+        if (pl->variant == 2) {
+            if (!cufft_launch_K<T>(pl, nb, u, out, out_scale, w.E, w.qtab, ctab_of<T>(pl), geo_of<T>(pl)))
+                pl->pending = set_error(BLOCH_ECUDA, "cuFFT plan or execution failed");
+            return 0;
+        }
     }
-    Workspace<T>& w = ws_of<T>(pl);
+    if constexpr (std::is_same<T, float>::value)
+        return launch_K_on(pl, nb, u, w.E, w.qtab, out, out_scale, dotp, dpart);
     pass_z_strain<T>(pl, nb, u, w.E, w.qtab);
-    BLOCH_FAST_SWITCH(pl->Ny, fast_y, pl, +1, nb, w.E);
+    launch_axis<T>(pl, 1, +1, 6 * nb, w.E, w.E, T(1));
     pass_x_stress<T>(pl, nb, w.E);
-    BLOCH_FAST_SWITCH(pl->Ny, fast_y, pl, -1, nb, w.E);
+    launch_axis<T>(pl, 1, -1, 6 * nb, w.E, w.E, T(1));
     pass_z_div<T>(pl, nb, w.E, out, w.qtab, out_scale);
     return 0;
 }
@@ -534,24 +508,33 @@ int launch_K<dfloat>(bloch_plan* pl, int nb, const dfloat2* u, dfloat2* out, dfl
 // operator workspace E (6 components per system, Voigt order xx yy zz yz xz
 // xy): S = F{ C~(x) : F^-1(sym q (x) u) }, i.e. the K-apply's passes 1-4 and a
 // forward z transform of the six stress components in place of its
-// divergence.  Shared-memory passes (any grid, both precisions).
+// divergence.
 template <typename T>
 void launch_K_stress(bloch_plan* pl, int nb, const cplx_t<T>* u) {
     Workspace<T>& w = ws_of<T>(pl);
-    pass_z_strain<T>(pl, nb, u, w.E, w.qtab);
-    pass_axis<T>(pl, 1, +1, 6 * nb, w.E, w.E, T(1));
-    pass_x_stress<T>(pl, nb, w.E);
-    pass_axis<T>(pl, 1, -1, 6 * nb, w.E, w.E, T(1));
-    pass_axis<T>(pl, 2, -1, 6 * nb, w.E, w.E, T(1));
+    if constexpr (std::is_same<T, float>::value) {
+        launch_stress_f(pl, nb, u, w.E, w.qtab, nullptr);
+    } else {
+        pass_z_strain<T>(pl, nb, u, w.E, w.qtab);
+        launch_axis<T>(pl, 1, +1, 6 * nb, w.E, w.E, T(1));
+        pass_x_stress<T>(pl, nb, w.E);
+        launch_axis<T>(pl, 1, -1, 6 * nb, w.E, w.E, T(1));
+    }
+    launch_axis<T>(pl, 2, -1, 6 * nb, w.E, w.E, T(1));
 }
 
-// In-place 3D FFT of nb three-component fields (DIR -1 forward, +1 inverse;
-// unnormalised), times out_scale: shared-memory passes along z, y and x.
 template <typename T, int DIR>
-void launch_fft3(bloch_plan* pl, int nb, cplx_t<T>* W, T out_scale) {
-    pass_axis<T>(pl, 2, DIR, 3 * nb, W, W, T(1));
-    pass_axis<T>(pl, 1, DIR, 3 * nb, W, W, T(1));
-    pass_x<T>(pl, DIR, nb, W, out_scale);
+void launch_fft3(bloch_plan* pl, int nb, const cplx_t<T>* W0, cplx_t<T>* W, T out_scale, const double2* ph) {
+    launch_axis<T>(pl, 2, DIR, 3 * nb, W0, W, T(1));
+    launch_axis<T>(pl, 1, DIR, 3 * nb, W, W, T(1));
+    pass_x<T>(pl, DIR, nb, W, out_scale, ph);
+}
+
+template <typename T>
+void launch_strain_real(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* eps, T scale, const double2* ph) {
+    launch_z_strain<T>(pl, nb, u, eps, ws_of<T>(pl).qtab);
+    launch_axis<T>(pl, 1, +1, 6 * nb, eps, eps, T(1));
+    pass_x<T>(pl, +1, 2 * nb, eps, scale, ph, 2);
 }
 
 template <typename T>
@@ -565,11 +548,11 @@ void launch_M(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_
         return;
     }
     Workspace<T>& w = ws_of<T>(pl);
-    pass_axis<T>(pl, 2, +1, 3 * nb, u, w.E, T(1));
-    pass_axis<T>(pl, 1, +1, 3 * nb, w.E, w.E, T(1));
+    launch_axis<T>(pl, 2, +1, 3 * nb, u, w.E, T(1));
+    launch_axis<T>(pl, 1, +1, 3 * nb, w.E, w.E, T(1));
     pass_x_rho<T>(pl, nb, w.E);
-    pass_axis<T>(pl, 1, -1, 3 * nb, w.E, w.E, T(1));
-    pass_axis<T>(pl, 2, -1, 3 * nb, w.E, out, out_scale);
+    launch_axis<T>(pl, 1, -1, 3 * nb, w.E, w.E, T(1));
+    launch_axis<T>(pl, 2, -1, 3 * nb, w.E, out, out_scale);
 }
 
 template <typename T>
@@ -839,8 +822,9 @@ bloch_status pcg_enqueue(bloch_plan* pl, int nb, const cplx_t<T>* b, cplx_t<T>* 
     template int launch_K<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T, const cplx_t<T>*, double2*); \
     template void launch_M<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T);                        \
     template void launch_K_stress<T>(bloch_plan*, int, const cplx_t<T>*);                                 \
-    template void launch_fft3<T, -1>(bloch_plan*, int, cplx_t<T>*, T);                                   \
-    template void launch_fft3<T, +1>(bloch_plan*, int, cplx_t<T>*, T);                                   \
+    template void launch_fft3<T, -1>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T, const double2*); \
+    template void launch_fft3<T, +1>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T, const double2*); \
+    template void launch_strain_real<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T, const double2*); \
     template void launch_precond<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T);                  \
     template void launch_dot<T>(bloch_plan*, int, const cplx_t<T>*, const cplx_t<T>*, long long,         \
                                 double2*, double2*);                                                     \
@@ -852,6 +836,7 @@ INST(float)
 INST(double)
 #undef INST
 template bloch_status ensure_ws<dfloat>(bloch_plan*, int);
+template int launch_K<dfloat>(bloch_plan*, int, const dfloat2*, dfloat2*, dfloat, const dfloat2*, double2*);
 template bloch_status set_k<dfloat>(bloch_plan*, int, const double*);
 template void launch_M<dfloat>(bloch_plan*, int, const dfloat2*, dfloat2*, dfloat);
 
@@ -866,11 +851,9 @@ static bloch_status apply_K_real_impl(bloch_plan* pl, int nb, const double* k, c
     if (st != BLOCH_OK) return st;
     if ((st = set_k<T>(pl, nb, k)) != BLOCH_OK) return st;
     Workspace<T>& w = ws_of<T>(pl);
-    BLOCH_CUDA_CHECK_RET(cudaMemcpyAsync(w.Ap, u, sizeof(cplx_t<T>) * (size_t)nb * 3 * pl->V,
-                                         cudaMemcpyDeviceToDevice, pl->stream));
-    launch_fft3<T, -1>(pl, nb, w.Ap, T(1));                       // u^ = F u
+    launch_fft3<T, -1>(pl, nb, u, w.Ap, T(1));                    // u^ = F u
     launch_K<T>(pl, nb, w.Ap, Ku, T(pl->Kscale));                 // A_k u^
-    launch_fft3<T, +1>(pl, nb, Ku, T(1.0 / (double)pl->V));       // F^-1
+    launch_fft3<T, +1>(pl, nb, Ku, Ku, T(1.0 / (double)pl->V));   // F^-1
     return BLOCH_OK;
 }
 

@@ -21,61 +21,118 @@
 
 namespace bloch {
 
-constexpr int kDkVals = 9;   // d_x (re, im), d_y, d_z, a (re, im), u^H M~ u
+constexpr int kDkVals = 5;   // Re d_x, Re d_y, Re d_z, Re a, u^H M~ u
+
+// Running sum of one thread.  FP32 terms are added into an unevaluated pair
+// hi + lo with Knuth's two-sum, which keeps every rounding error of the
+// additions (48 bits); FP64 terms are added plainly.  GB300 adds FP64 at 1/64
+// of its FP32 rate: with FP64 sums of the FP32 terms this pass took ten times
+// its memory time.
+template <typename T> struct Sum;
+template <> struct Sum<float> {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float v) {
+        const dfloat s = df_two_sum(hi, v);
+        hi = s.hi;
+        lo = __fadd_rn(lo, s.lo);
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+template <> struct Sum<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double v) { s += v; }
+    __device__ __forceinline__ double value() const { return s; }
+};
+
+// Largest |component| of each FP32 vector (as bits, which order like the
+// values), so that the sums below can scale it to O(1): products of vectors of
+// any normalisation then stay inside the FP32 range.  Only ratios of the sums
+// are used, so the power of two drops out.  mx zeroed by the caller.
+static __global__ void k_absmax(const float2* __restrict__ U, long long n_per, unsigned* __restrict__ mx) {
+    const float2* u = U + (size_t)blockIdx.y * n_per;
+    float m = 0.f;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_per;
+         i += (long long)gridDim.x * blockDim.x)
+        m = fmaxf(m, fmaxf(fabsf(u[i].x), fabsf(u[i].y)));
+    unsigned b = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+    if ((threadIdx.x & 31) == 0 && b) atomicMax(mx + blockIdx.y, b);
+}
+template <typename T> __device__ __forceinline__ T unit_scale(const unsigned* mx, int b);
+template <> __device__ __forceinline__ float unit_scale<float>(const unsigned* mx, int b) {
+    const int e = min(max((int)(mx[b] >> 23), 8), 246) - 127;
+    return __uint_as_float((unsigned)(127 - e) << 23);   // 2^-e
+}
+template <> __device__ __forceinline__ double unit_scale<double>(const unsigned*, int) { return 1.0; }
+
+// enqueues the maxima of nb vectors into mx (FP32; nothing to do in FP64)
+template <typename T>
+static bloch_status launch_absmax(bloch_plan* pl, int nb, const cplx_t<T>* u, unsigned* mx) {
+    if constexpr (std::is_same<T, float>::value) {
+        const long long n3 = 3 * pl->V;
+        BLOCH_CUDA_CHECK_RET(cudaMemsetAsync(mx, 0, sizeof(unsigned) * nb, pl->stream));
+        ++pl->launches;
+        k_absmax<<<dim3((unsigned)std::max(1LL, std::min<long long>((n3 + 1023) / 1024, 512)), nb), 256, 0,
+                   pl->stream>>>(u, n3, mx);
+    }
+    return BLOCH_OK;
+}
 
 // Per system b = blockIdx.y, per block: partial sums over Fourier voxels of
-//   d_m = sum_i conj(U_i) S_im,  a = sum_ij conj(U_i) q_j S_ij,  mu = Re sum conj(U) (M~ U)
-// with M~ U = MU (non-uniform density) or rho_s U.  FP64 accumulation.
+//   Re d_m = Re sum_i conj(U_i) S_im,  Re a = sum_m q_m Re d_m (per voxel),
+//   mu = Re sum conj(U) (M~ U)
+// with M~ U = MU (non-uniform density) or rho_s U.  Terms of a voxel in the
+// field precision, sums over voxels as Sum<T> and FP64 across threads.
 template <typename T>
 __global__ void k_dk_partial(const cplx_t<T>* __restrict__ U, const cplx_t<T>* __restrict__ S,
                              const cplx_t<T>* __restrict__ MU, double rho_s, const T* __restrict__ qtab, Geo g,
-                             double* __restrict__ partial) {
+                             const unsigned* __restrict__ mx, double* __restrict__ partial) {
     using C = cplx_t<T>;
     const int b = blockIdx.y;
+    const T sc = unit_scale<T>(mx, b);
     const C* ub = U + (size_t)b * 3 * g.V;
     const C* sb = S + (size_t)b * 6 * g.V;
     const C* mb = MU ? MU + (size_t)b * 3 * g.V : nullptr;
     const T* qb = qtab + (size_t)b * (g.Nx + g.Ny + g.Nz);
     // Voigt index of S_im: rows i = x, y, z; columns m = x, y, z
     const int vo[3][3] = {{0, 5, 4}, {5, 1, 3}, {4, 3, 2}};
-    double acc[kDkVals];
-#pragma unroll
-    for (int i = 0; i < kDkVals; ++i) acc[i] = 0.0;
+    Sum<T> acc[kDkVals];
     for (unsigned v = blockIdx.x * blockDim.x + threadIdx.x; v < (unsigned)g.V; v += gridDim.x * blockDim.x) {
-        T qx, qy, qz;
-        voxel_q(qb, g, v, qx, qy, qz);
-        const double q[3] = {(double)qx, (double)qy, (double)qz};
+        T q[3];
+        voxel_q(qb, g, v, q[0], q[1], q[2]);
         C u[3], s[6];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) u[c] = ub[(size_t)c * g.V + v];
+        for (int c = 0; c < 3; ++c) u[c] = cscale(ub[(size_t)c * g.V + v], sc);
 #pragma unroll
-        for (int c = 0; c < 6; ++c) s[c] = sb[(size_t)c * g.V + v];
+        for (int c = 0; c < 6; ++c) s[c] = cscale(sb[(size_t)c * g.V + v], sc);
+        T a = T(0), mu = T(0);
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            T d = T(0);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const C sv = s[vo[i][m]];
+                d = fma(u[i].x, sv.x, fma(u[i].y, sv.y, d));
+            }
+            acc[m].add(d);
+            a = fma(q[m], d, a);
+        }
+        acc[3].add(a);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            const double ur = (double)u[i].x, ui = (double)u[i].y;
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                const C sv = s[vo[i][m]];
-                const double pr = ur * (double)sv.x + ui * (double)sv.y;   // Re conj(u) s
-                const double pim = ur * (double)sv.y - ui * (double)sv.x;  // Im conj(u) s
-                acc[2 * m] += pr;
-                acc[2 * m + 1] += pim;
-                acc[6] += q[m] * pr;
-                acc[7] += q[m] * pim;
-            }
-            if (mb) {
-                const C mv = mb[(size_t)i * g.V + v];
-                acc[8] += ur * (double)mv.x + ui * (double)mv.y;
-            } else {
-                acc[8] += rho_s * (ur * ur + ui * ui);
-            }
+            const C mv = mb ? cscale(mb[(size_t)i * g.V + v], sc) : u[i];
+            mu = fma(u[i].x, mv.x, fma(u[i].y, mv.y, mu));
         }
+        acc[4].add(mu);
     }
-    block_sum<double, kDkVals>(acc);
+    double tot[kDkVals];
+#pragma unroll
+    for (int i = 0; i < kDkVals; ++i) tot[i] = acc[i].value();
+    if (!mb) tot[4] *= rho_s;
+    block_sum<double, kDkVals>(tot);
     if (threadIdx.x == 0) {
         double* o = partial + ((size_t)b * gridDim.x + blockIdx.x) * kDkVals;
 #pragma unroll
-        for (int i = 0; i < kDkVals; ++i) o[i] = acc[i];
+        for (int i = 0; i < kDkVals; ++i) o[i] = tot[i];
     }
 }
 
@@ -97,10 +154,13 @@ static bloch_status group_velocity_impl(bloch_plan* pl, int nb, const double* k,
     const int nblk = (int)std::max(1LL, std::min<long long>((pl->V + 255) / 256, 512));
     const size_t nval = (size_t)nb * nblk * kDkVals;
     double* d_part = nullptr;
-    if ((st = plan_solver_buf(pl, 2, 0, nval * sizeof(double), (void**)&d_part)) != BLOCH_OK) return st;
+    if ((st = plan_solver_buf(pl, 2, 0, nval * sizeof(double) + nb * sizeof(unsigned), (void**)&d_part)) != BLOCH_OK)
+        return st;
+    unsigned* d_mx = (unsigned*)(d_part + nval);
+    if ((st = launch_absmax<T>(pl, nb, u, d_mx)) != BLOCH_OK) return st;
     ++pl->launches;
     k_dk_partial<T><<<dim3(nblk, nb), 256, 0, pl->stream>>>(u, w.E, MU, pl->uniform_rho ? pl->rho_uniform_scaled : 1.0,
-                                                            w.qtab, geo_of<T>(pl), d_part);
+                                                            w.qtab, geo_of<T>(pl), d_mx, d_part);
     BLOCH_CUDA_CHECK_RET(cudaGetLastError());
     std::vector<double> h(nval);
     BLOCH_CUDA_CHECK_RET(cudaMemcpyAsync(h.data(), d_part, nval * sizeof(double), cudaMemcpyDeviceToHost, pl->stream));
@@ -109,13 +169,13 @@ static bloch_status group_velocity_impl(bloch_plan* pl, int nb, const double* k,
         double s[kDkVals] = {0};
         for (int j = 0; j < nblk; ++j)
             for (int i = 0; i < kDkVals; ++i) s[i] += h[((size_t)b * nblk + j) * kDkVals + i];
-        const double uMu = pl->rho_ref * s[8];   // u^H M u (SI)
+        const double uMu = pl->rho_ref * s[4];   // u^H M u (SI)
         if (!(uMu > 0.0)) return set_error(BLOCH_EINVAL, "a vector is zero (u^H M u = 0)");
-        const double lam = pl->Kscale * s[6] / uMu;
+        const double lam = pl->Kscale * s[3] / uMu;
         const double om = lam > 0.0 ? std::sqrt(lam) : 0.0;
         if (omega_out) omega_out[b] = om;
         for (int m = 0; m < 3; ++m) {
-            const double dlam = pl->Kscale * pl->qscale * 2.0 * s[2 * m] / uMu;
+            const double dlam = pl->Kscale * pl->qscale * 2.0 * s[m] / uMu;
             c_out[(size_t)b * 3 + m] = om > 0.0 ? dlam / (2.0 * om) : 0.0;
         }
     }
@@ -129,85 +189,58 @@ static bloch_status group_velocity_impl(bloch_plan* pl, int nb, const double* k,
 // single phase, and otherwise the single phase that maximises
 // ||Re(e^{-i phi} U)|| (least squares).
 
-// partial[b][blk] = sum over the block's elements of W^2 (complex square)
+// partial[b][blk] = sum over the block's Fourier voxels m of sum_i U_i(m) U_i(-m)
+// = V sum_x sum_i (F^-1 U_i)(x)^2 (indices modulo the grid): the phase is
+// known before the inverse transforms, whose last pass then applies it.
 template <typename T>
-__global__ void k_sq_partial(const cplx_t<T>* __restrict__ W, long long n_per, double2* __restrict__ partial) {
+__global__ void k_sq_partial(const cplx_t<T>* __restrict__ U, Geo g, const unsigned* __restrict__ mx,
+                             double2* __restrict__ partial) {
     const int b = blockIdx.y;
-    const cplx_t<T>* w = W + (size_t)b * n_per;
-    double acc[2] = {0.0, 0.0};
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_per;
-         i += (long long)gridDim.x * blockDim.x) {
-        const double a = (double)w[i].x, c = (double)w[i].y;
-        acc[0] += a * a - c * c;
-        acc[1] += 2.0 * a * c;
-    }
-    block_sum<double, 2>(acc);
-    if (threadIdx.x == 0) partial[(size_t)b * gridDim.x + blockIdx.x] = make_double2(acc[0], acc[1]);
-}
-
-// W[b] *= ph[b] (complex)
-template <typename T>
-__global__ void k_phase(cplx_t<T>* W, long long n_per, const double2* __restrict__ ph) {
-    const int b = blockIdx.y;
-    const cplx_t<T> p = mk(T(ph[b].x), T(ph[b].y));
-    cplx_t<T>* w = W + (size_t)b * n_per;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_per;
-         i += (long long)gridDim.x * blockDim.x)
-        w[i] = cmul(w[i], p);
-}
-
-// Fourier-space strain of the periodic field, eps_ij = (d_j U_i + d_i U_j)/2 with
-// d_j = i xi_j (the derivative of Section 5.2's epsilon_11 = dU_1/dx_1), times
-// the phase ph[b]; Voigt-ordered tensor components (xx yy zz yz xz xy).
-// xi from the q table of a zero wave vector (scaled by qscale; s = 1/qscale).
-template <typename T>
-__global__ void k_strain_hat(const cplx_t<T>* __restrict__ U, const T* __restrict__ xitab, Geo g,
-                             const double2* __restrict__ ph, T s, cplx_t<T>* __restrict__ Eps) {
-    using C = cplx_t<T>;
-    const int b = blockIdx.y;
-    const C p = mk(T(ph[b].x), T(ph[b].y));
-    const C* ub = U + (size_t)b * 3 * g.V;
-    C* eb = Eps + (size_t)b * 6 * g.V;
+    const T sc = unit_scale<T>(mx, b);
+    const cplx_t<T>* ub = U + (size_t)b * 3 * g.V;
+    Sum<T> acc[2];
     for (unsigned v = blockIdx.x * blockDim.x + threadIdx.x; v < (unsigned)g.V; v += gridDim.x * blockDim.x) {
-        T x0, x1, x2;
-        voxel_q(xitab, g, v, x0, x1, x2);
-        const T xi[3] = {x0 * s, x1 * s, x2 * s};
-        C u[3];
+        const unsigned t = fdiv(v, g.dx);
+        const int x = (int)(v - t * (unsigned)g.Nx);
+        const int z = (int)fdiv(t, g.dy), y = (int)t - z * g.Ny;
+        const unsigned w = ((unsigned)(z ? g.Nz - z : 0) * g.Ny + (y ? g.Ny - y : 0)) * (unsigned)g.Nx +
+                           (unsigned)(x ? g.Nx - x : 0);
+        T re = T(0), im = T(0);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) u[c] = cmul(ub[(size_t)c * g.V + v], p);
-        const int pi[6] = {0, 1, 2, 1, 0, 0}, pj[6] = {0, 1, 2, 2, 2, 1};
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            const int i = pi[c], j = pj[c];
-            // (i xi_j u_i + i xi_i u_j) / 2
-            const C a = cadd(cscale(u[i], xi[j]), cscale(u[j], xi[i]));
-            eb[(size_t)c * g.V + v] = cscale(cmul_i<+1>(a), T(0.5));
+        for (int c = 0; c < 3; ++c) {
+            const cplx_t<T> a = cscale(ub[(size_t)c * g.V + v], sc), m = cscale(ub[(size_t)c * g.V + w], sc);
+            re = fma(a.x, m.x, fma(-a.y, m.y, re));
+            im = fma(a.x, m.y, fma(a.y, m.x, im));
         }
+        acc[0].add(re);
+        acc[1].add(im);
     }
+    double tot[2] = {acc[0].value(), acc[1].value()};
+    block_sum<double, 2>(tot);
+    if (threadIdx.x == 0) partial[(size_t)b * gridDim.x + blockIdx.x] = make_double2(tot[0], tot[1]);
 }
 
 template <typename T>
 static bloch_status eigvec_real_impl(bloch_plan* pl, int nb, const cplx_t<T>* uh, cplx_t<T>* ur, cplx_t<T>* eps,
                                      double* phi_out) {
-    using C = cplx_t<T>;
     bloch_status st = ensure_ws<T>(pl, nb);
     if (st != BLOCH_OK) return st;
-    const long long n3 = 3 * pl->V;
-    BLOCH_CUDA_CHECK_RET(cudaMemcpyAsync(ur, uh, sizeof(C) * (size_t)nb * n3, cudaMemcpyDeviceToDevice, pl->stream));
-    launch_fft3<T, +1>(pl, nb, ur, T(1.0 / (double)pl->V));       // F^-1 (numpy normalisation)
-    const int nblk = (int)std::max(1LL, std::min<long long>((n3 + 255) / 256, 512));
+    const int nblk = (int)std::max(1LL, std::min<long long>((pl->V + 255) / 256, 512));
     double2* d_part = nullptr;
-    if ((st = plan_solver_buf(pl, 2, 1, sizeof(double2) * ((size_t)nb * nblk + nb), (void**)&d_part)) != BLOCH_OK)
+    if ((st = plan_solver_buf(pl, 2, 1, sizeof(double2) * ((size_t)nb * nblk + 2 * nb) + nb * sizeof(unsigned),
+                              (void**)&d_part)) != BLOCH_OK)
         return st;
-    double2* d_ph = d_part + (size_t)nb * nblk;
+    double2* d_ph = d_part + (size_t)nb * nblk;   // e^{-i phi}, then i e^{-i phi}
+    unsigned* d_mx = (unsigned*)(d_ph + 2 * (size_t)nb);
+    if ((st = launch_absmax<T>(pl, nb, uh, d_mx)) != BLOCH_OK) return st;
     ++pl->launches;
-    k_sq_partial<T><<<dim3(nblk, nb), 256, 0, pl->stream>>>(ur, n3, d_part);
+    k_sq_partial<T><<<dim3(nblk, nb), 256, 0, pl->stream>>>(uh, geo_of<T>(pl), d_mx, d_part);
     BLOCH_CUDA_CHECK_RET(cudaGetLastError());
     std::vector<double2> h((size_t)nb * nblk);
     BLOCH_CUDA_CHECK_RET(
         cudaMemcpyAsync(h.data(), d_part, sizeof(double2) * h.size(), cudaMemcpyDeviceToHost, pl->stream));
     BLOCH_CUDA_CHECK_RET(cudaStreamSynchronize(pl->stream));
-    std::vector<double2> ph(nb);
+    std::vector<double2> ph(2 * (size_t)nb);
     for (int b = 0; b < nb; ++b) {
         double re = 0.0, im = 0.0;
         for (int j = 0; j < nblk; ++j) {
@@ -216,20 +249,16 @@ static bloch_status eigvec_real_impl(bloch_plan* pl, int nb, const cplx_t<T>* uh
         }
         const double phi = 0.5 * std::atan2(im, re);
         if (phi_out) phi_out[b] = phi;
-        ph[b] = make_double2(std::cos(phi), -std::sin(phi));   // e^{-i phi}
+        ph[b] = make_double2(std::cos(phi), -std::sin(phi));
+        ph[nb + b] = make_double2(std::sin(phi), std::cos(phi));
     }
-    BLOCH_CUDA_CHECK_RET(cudaMemcpyAsync(d_ph, ph.data(), sizeof(double2) * nb, cudaMemcpyHostToDevice, pl->stream));
-    const unsigned gx = (unsigned)std::min<long long>((n3 + 255) / 256, 2048);
-    ++pl->launches;
-    k_phase<T><<<dim3(gx, nb), 256, 0, pl->stream>>>(ur, n3, d_ph);
+    BLOCH_CUDA_CHECK_RET(
+        cudaMemcpyAsync(d_ph, ph.data(), sizeof(double2) * ph.size(), cudaMemcpyHostToDevice, pl->stream));
+    launch_fft3<T, +1>(pl, nb, uh, ur, T(1.0 / (double)pl->V), d_ph);       // F^-1 (numpy normalisation)
     if (eps) {
         std::vector<double> zero((size_t)nb * 3, 0.0);
         if ((st = set_k<T>(pl, nb, zero.data())) != BLOCH_OK) return st;
-        const unsigned gv = (unsigned)std::min<long long>((pl->V + 255) / 256, 2048);
-        ++pl->launches;
-        k_strain_hat<T><<<dim3(gv, nb), 256, 0, pl->stream>>>(uh, ws_of<T>(pl).qtab, geo_of<T>(pl), d_ph,
-                                                               T(1.0 / pl->qscale), eps);
-        launch_fft3<T, +1>(pl, 2 * nb, eps, T(1.0 / (double)pl->V));   // six components = two 3-component fields
+        launch_strain_real<T>(pl, nb, uh, eps, T(1.0 / (pl->qscale * (double)pl->V)), d_ph + nb);
     }
     BLOCH_CUDA_CHECK_RET(cudaGetLastError());
     BLOCH_CUDA_CHECK_RET(cudaStreamSynchronize(pl->stream));

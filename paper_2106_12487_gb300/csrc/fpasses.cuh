@@ -32,13 +32,15 @@ __device__ __forceinline__ C twmul(C v, C w, int dir) {
     return cmul(v, w);
 }
 
-// --------------------------------------------------- y pass (in place ok)
-// blockIdx.y = batch*ncomp + comp (offset blockIdx.y * V).  PT pencils (PT
-// consecutive x of the (x, z) plane) per CTA; one 32-bit division per task
-// locates the pencil, elements step by Nx along it.
+// ------------------------------------- plain pass along y or z (in place ok)
+// A pencil's elements lie `inner` apart (Nx along y, Nx Ny along z); pencil pi
+// of npen starts at (pi / inner) outer + pi mod inner.  blockIdx.y = field
+// (batch*ncomp + comp, offset blockIdx.y * V).  PT neighbouring pencils per
+// CTA; one 32-bit division per task locates the pencil.
 template <typename T, int DIR, int RA, int RB, int PT>
-__global__ void __launch_bounds__(256) k_fpass_y(const cplx_t<T>* in, cplx_t<T>* out,
-                                                 const cplx_t<T>* __restrict__ twa, Geo g) {
+__global__ void __launch_bounds__(256) k_fpass_axis(const cplx_t<T>* in, cplx_t<T>* out,
+                                                    const cplx_t<T>* __restrict__ twa, Geo g, unsigned inner,
+                                                    unsigned outer, unsigned npen, T out_scale) {
     using C = cplx_t<T>;
     constexpr int N = RA * RB;
     constexpr int NT = 256;
@@ -46,10 +48,7 @@ __global__ void __launch_bounds__(256) k_fpass_y(const cplx_t<T>* in, cplx_t<T>*
     C* tw = reinterpret_cast<C*>(smem_raw);
     C* buf = tw + N;
     const int tid = threadIdx.x;
-    const unsigned nx = (unsigned)g.Nx;
-    const unsigned npen = nx * (unsigned)g.Nz;
     const unsigned pi0 = blockIdx.x * PT;
-    const unsigned plane = nx * (unsigned)g.Ny;
     if (sys_idle(g, (int)blockIdx.y / g.skip_ncomp)) return;
     const size_t off = (size_t)blockIdx.y * g.V;
     const C* src = in + off;
@@ -61,10 +60,10 @@ __global__ void __launch_bounds__(256) k_fpass_y(const cplx_t<T>* in, cplx_t<T>*
         const unsigned pi = pi0 + p;
         C v[RA];
         if (pi < npen) {
-            const unsigned z = pi / nx;
-            const C* a = src + (z * plane + (pi - z * nx) + (unsigned)j * nx);
+            const unsigned q = pi / inner;
+            const C* a = src + (q * outer + (pi - q * inner) + (unsigned)j * inner);
 #pragma unroll
-            for (int r = 0; r < RA; ++r) v[r] = a[(unsigned)(r * RB) * nx];
+            for (int r = 0; r < RA; ++r) v[r] = a[(unsigned)(r * RB) * inner];
         } else {
 #pragma unroll
             for (int r = 0; r < RA; ++r) v[r] = mk(T(0), T(0));
@@ -85,10 +84,10 @@ __global__ void __launch_bounds__(256) k_fpass_y(const cplx_t<T>* in, cplx_t<T>*
         RegDFT<RB, DIR, C>::run(v);
         const unsigned pi = pi0 + p;
         if (pi < npen) {
-            const unsigned z = pi / nx;
-            C* a = dst + (z * plane + (pi - z * nx) + (unsigned)j * nx);
+            const unsigned q = pi / inner;
+            C* a = dst + (q * outer + (pi - q * inner) + (unsigned)j * inner);
 #pragma unroll
-            for (int r = 0; r < RB; ++r) a[(unsigned)(r * RA) * nx] = v[r];
+            for (int r = 0; r < RB; ++r) a[(unsigned)(r * RA) * inner] = cscale(v[r], out_scale);
         }
     }
 }
@@ -631,7 +630,7 @@ __device__ __forceinline__ void x_stress_single(cplx_t<T>* E, const int32_t* __r
         if (dpart) warp_sum_to(energy, red);
     }
     __syncthreads();   // the staging buffers become the forward exchange buffers; red[] complete
-    if (dpart && tid == 0) red_to<4>(red, dpart + (size_t)b * gridDim.x + blockIdx.x);
+    if (dpart && tid == 0) red_to<4>(red, dpart);
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
         C* buf = stg + (c & 1) * P * LD;
@@ -788,7 +787,7 @@ __device__ __forceinline__ void x_stress_paired(cplx_t<T>* E, const int32_t* __r
             for (int r = 0; r < RB; ++r) bufs[h * P * LD + p2 * LD + xpad(j2 * RB + r)] = v[r];
         }
         __syncthreads();   // a thread writing this buffer set again (pair m + 2) has passed the next barrier
-        if (m == 0 && dpart && tid == 0) red_to<4>(red, dpart + (size_t)blockIdx.y * gridDim.x + blockIdx.x);
+        if (m == 0 && dpart && tid == 0) red_to<4>(red, dpart);
         // forward stage 2 (radix RA): component 2m + half
         {
             C v[RA];
@@ -837,6 +836,7 @@ __global__ void __launch_bounds__(128, 4) k_fpass_x_stress(cplx_t<T>* E, const i
                                                            const cplx_t<T>* __restrict__ twx, Geo g,
                                                            double2* __restrict__ dpart) {
     if (sys_idle(g, blockIdx.y)) return;
+    if (dpart) dpart += (size_t)blockIdx.y * gridDim.x + blockIdx.x;
     if constexpr ((128 / RA) * RB == 64)
         x_stress_paired<T, RA, RB>(E, ids, Cpk, twx, g, dpart);
     else

@@ -186,7 +186,8 @@ template <typename T>   // axis 1 (y) or 2 (z) of nfields scalar fields
 void pass_axis(bloch_plan* pl, int axis, int dir, int nfields, const cplx_t<T>* in, cplx_t<T>* out, T out_scale);
 template <typename T> void pass_x_stress(bloch_plan* pl, int nb, cplx_t<T>* E);
 template <typename T> void pass_x_rho(bloch_plan* pl, int nb, cplx_t<T>* W);
-template <typename T> void pass_x(bloch_plan* pl, int dir, int nb, cplx_t<T>* W, T out_scale);
+template <typename T>   // ph, per: complex factors of the systems (k_pass_x)
+void pass_x(bloch_plan* pl, int dir, int nb, cplx_t<T>* W, T out_scale, const double2* ph = nullptr, int per = 1);
 template <typename T>
 void pass_z_div(bloch_plan* pl, int nb, const cplx_t<T>* E, cplx_t<T>* out, const T* qtab, T out_scale);
 // shared-memory limits of the passes, once per plan
@@ -207,12 +208,20 @@ template <typename T> bloch_status set_k(bloch_plan* pl, int nb, const double* k
 template <typename T>
 int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale,
              const cplx_t<T>* dotp = nullptr, double2* dpart = nullptr);
+// The FP32 operator on scratch E and q tables of the caller (launch_K's chain).
+int launch_K_on(bloch_plan* pl, int nb, const float2* u, float2* E, const float* qtab, float2* out, float out_scale,
+                const float2* dotp, double2* dpart);
 // Fourier-space stress S = F{C~ : F^-1(sym q (x) u)} of nb systems (q tables
 // set) into the operator workspace E, 6 Voigt components per system.
 template <typename T> void launch_K_stress(bloch_plan* pl, int nb, const cplx_t<T>* u);
-// In-place 3D FFT of nb three-component fields (DIR -1 forward, +1 inverse,
-// unnormalised), times out_scale; shared-memory passes.
-template <typename T, int DIR> void launch_fft3(bloch_plan* pl, int nb, cplx_t<T>* W, T out_scale);
+// 3D FFT of nb three-component fields from W0 into W (may be equal; DIR -1
+// forward, +1 inverse, unnormalised), times out_scale and, with ph, times ph[b].
+template <typename T, int DIR>
+void launch_fft3(bloch_plan* pl, int nb, const cplx_t<T>* W0, cplx_t<T>* W, T out_scale, const double2* ph = nullptr);
+// Strain of the real-space field F^-1(u): F^-1(sym d_j u_i) in tensor
+// components, from the q tables of a zero wave vector, times scale ph[b].
+template <typename T>
+void launch_strain_real(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* eps, T scale, const double2* ph);
 // Scaled mass operator: out = out_scale * M~ u (M~ = M / rho_ref).  out may alias u.
 template <typename T> void launch_M(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale);
 // Scaled preconditioner on nb systems: z = out_scale * P~^-1 r.

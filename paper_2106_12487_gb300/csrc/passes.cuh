@@ -275,8 +275,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
     const int tid = threadIdx.x, nthr = blockDim.x;
     if (sys_idle(g, (int)blockIdx.y / g.skip_ncomp)) return;
     const unsigned nx = (unsigned)g.Nx, plane = nx * (unsigned)g.Ny;
-    const unsigned npen = AXIS == 1 ? nx * (unsigned)g.Nz : plane;
     const unsigned step = AXIS == 1 ? nx : plane;     // between the elements of a pencil
+    const unsigned npen = AXIS == 1 ? nx * (unsigned)g.Nz : plane;
     const unsigned pi0 = blockIdx.x << lp;
     const C* src = in + (size_t)blockIdx.y * g.V;
     C* dst = out + (size_t)blockIdx.y * g.V;
@@ -566,11 +566,14 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
 
 // ------------------------------------------- plain transform along x
 // 1D FFT (DIR -1 forward, +1 inverse, unnormalised) of the three components
-// of nb systems along x, in place, times out_scale; rows are contiguous, P
-// rows per CTA, blockIdx.y = system.
+// of nb fields along x, in place, times out_scale; rows are contiguous, P
+// rows per CTA, blockIdx.y = field.  With ph the fields of system b (`per`
+// fields each) are also multiplied by the complex factor ph[b], and the second
+// of two fields by 1/2 (the shears of a strain field: engineering to tensor).
 template <typename T, int DIR>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
-    k_pass_x(cplx_t<T>* W, const cplx_t<T>* __restrict__ twx, Geo g, int P, T out_scale) {
+    k_pass_x(cplx_t<T>* W, const cplx_t<T>* __restrict__ twx, Geo g, int P, T out_scale,
+             const double2* __restrict__ ph, int per) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const AxisPlan& a = g.ax[0];
@@ -594,11 +597,14 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
     }
     lf_last<DIR>(buf, 3 * P, a, tid, nthr);
     __syncthreads();
+    if (per == 2 && (b & 1)) out_scale = out_scale * T(0.5);
+    const C f = ph ? mk(T(ph[b / per].x) * out_scale, T(ph[b / per].y) * out_scale) : mk(out_scale, T(0));
     for (int t = tid; t < 3 * P * N; t += nthr) {
         const int cp = (int)fdiv((unsigned)t, g.dx), k = t - cp * N;
         const int c = cp / P, p = cp - c * P;
-        if (p < nr)
-            Wb[(size_t)c * g.V + (size_t)(r0 + p) * N + k] = cscale(buf[cp * ld + xslot(slot_of(k, a))], out_scale);
+        if (p >= nr) continue;
+        const C v = buf[cp * ld + xslot(slot_of(k, a))];
+        Wb[(size_t)c * g.V + (size_t)(r0 + p) * N + k] = ph ? cmul(v, f) : cscale(v, out_scale);
     }
 }
 

@@ -68,14 +68,16 @@ void pass_x_rho(bloch_plan* pl, int nb, cplx_t<T>* W) {
 }
 
 template <typename T>
-void pass_x(bloch_plan* pl, int dir, int nb, cplx_t<T>* W, T out_scale) {
+void pass_x(bloch_plan* pl, int dir, int nb, cplx_t<T>* W, T out_scale, const double2* ph, int per) {
     const PassTile& t = tile_of<T>(pl).x3;
     const dim3 gr = pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb);
     ++pl->launches;
     if (dir > 0)
-        k_pass_x<T, +1><<<gr, t.nthr, t.smem, pl->stream>>>(W, pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp, out_scale);
+        k_pass_x<T, +1><<<gr, t.nthr, t.smem, pl->stream>>>(W, pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp, out_scale,
+                                                            ph, per);
     else
-        k_pass_x<T, -1><<<gr, t.nthr, t.smem, pl->stream>>>(W, pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp, out_scale);
+        k_pass_x<T, -1><<<gr, t.nthr, t.smem, pl->stream>>>(W, pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp, out_scale,
+                                                            ph, per);
 }
 
 template <typename T>
