@@ -83,7 +83,7 @@ bloch_status tune(bloch_plan* pl, int systems, bloch_tune_report* rep) {
         k_tune_fill<C><<<1024, 256, 0, pl->stream>>>(u, n);
         if (cudaGetLastError() != cudaSuccess) st = set_error(BLOCH_ECUDA, "autotune: fill launch failed");
     }
-    const int old_variant = pl->variant, old_pmax = pl->tile_f.pmax;
+    const int old_variant = pl->variant, old_pmax = pl->pmax;
     double best = -1.0;
     int best_v = old_variant, best_p = old_pmax, cand = 0;
     double per_var[3] = {-1.0, -1.0, -1.0};

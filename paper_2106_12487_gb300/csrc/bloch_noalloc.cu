@@ -91,7 +91,7 @@ extern "C" bloch_status bloch_apply_K_noalloc(bloch_plan* pl, int32_t nb, const 
     k_qtab<float><<<qblocks, 256, 0, pl->stream>>>(kvec, pl->d_xi, pl->Nx, pl->Ny, pl->Nz, nb, pl->qscale, qtab);
 
     ++pl->launches;
-    launch_K_on(pl, nb, (const float2*)u, E, qtab, (float2*)Ku, (float)pl->Kscale, nullptr, nullptr);
+    launch_K_on(pl, nb, (const float2*)u, E, qtab, (float2*)Ku, (float)pl->Kscale);
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_cuda_error(e, "bloch_apply_K_noalloc launch");
     return BLOCH_OK;

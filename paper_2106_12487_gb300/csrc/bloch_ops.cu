@@ -34,9 +34,6 @@ template <> Workspace<dfloat>& ws_of<dfloat>(bloch_plan* pl) { return pl->ws_x; 
 template <> const Geo& geo_of<dfloat>(const bloch_plan* pl) { return pl->geo_x; }
 template <> const Geo& geo_of<float>(const bloch_plan* pl) { return pl->geo_f; }
 template <> const Geo& geo_of<double>(const bloch_plan* pl) { return pl->geo_d; }
-template <> const TileCfg& tile_of<float>(const bloch_plan* pl) { return pl->tile_f; }
-template <> const TileCfg& tile_of<double>(const bloch_plan* pl) { return pl->tile_d; }
-template <> const TileCfg& tile_of<dfloat>(const bloch_plan* pl) { return pl->tile_x; }
 template <typename T> static const cplx_t<T>* tw_of(const bloch_plan* pl, int axis);
 template <> const float2* tw_of<float>(const bloch_plan* pl, int axis) { return pl->d_twf[axis]; }
 template <> const double2* tw_of<double>(const bloch_plan* pl, int axis) { return pl->d_twd[axis]; }
@@ -89,20 +86,36 @@ static AxisPlan make_axis(int N, bool ff) {
     return ap;
 }
 
-// Pencils per CTA (a power of two, at most pmax) and threads of a mixed-radix
-// pass with `bufs` buffers of `row` elements per pencil: halved until the
-// tile fits the shared-memory budget, then while the grid has fewer than
-// kTileCtas CTAs per system and the rows of a tile keep 32 bytes.
-constexpr long long kTileCtas = 304;
-static PassTile make_tile(const AxisPlan& a, int row, int bufs, size_t el, size_t budget, long long npen, int pmax) {
-    PassTile t{};
+// Shared memory a CTA of a six-buffer tile may take: two CTAs per SM.
+constexpr size_t kTileSmem = 104 * 1024;
+// CTAs wanted in a launch before a tile is worth its width: three per SM.
+// (48 x 40 x 36, FP32, 10 systems: 185 us per K-apply with tiles made for one
+// system, 95 us with tiles made for the launch.)
+constexpr long long kTileCtas = 456;
+
+// P pencils (rows) per CTA, a power of two of at most plan->pmax (half
+// of it along x): halved until the tile fits its shared memory, then while the
+// launch has too few CTAs to fill the chip and a tile's rows keep 32 bytes.
+template <typename T>
+PassTile pass_tile(const bloch_plan* pl, PassKind kind, int nb) {
+    const Geo& g = geo_of<T>(pl);
+    const size_t el = sizeof(cplx_t<T>);
+    const int axis = kind == PASS_Y1 ? 1 : (kind == PASS_Z6 || kind == PASS_Z1) ? 2 : 0;
+    const AxisPlan& a = g.ax[axis];
+    const bool x_ = axis == 0;
+    const int bufs = kind == PASS_Y1 || kind == PASS_Z1 ? 1 : kind == PASS_X3 ? 3 : 6;
+    const long long npen = g.V / a.N;
+    const size_t row = (size_t)(x_ ? xrow(a) : a.N) * bufs * el;
     const size_t tw = (size_t)pad_even(a.N) * el;
-    int P = std::max(1, pmax);
-    while (P > 1 && (size_t)bufs * row * P * el + tw > budget) P >>= 1;
+    const size_t budget = bufs == 1 ? 64 * 1024 : kTileSmem;
+    PassTile t{};
+    int P = std::max(1, x_ ? pl->pmax / 2 : pl->pmax);
+    while (P > 1 && row * P + tw > budget) P >>= 1;
     while (P > 1 && (long long)(P / 2) >= npen) P >>= 1;
-    while (P * el > 32 && npen / P < kTileCtas) P >>= 1;
+    // lanes run along x in row tiles: no width to keep there
+    while ((x_ ? P > 1 : P * el > 32) && npen * nb / P < kTileCtas) P >>= 1;
     while ((1 << t.lp) < P) ++t.lp;
-    t.smem = (size_t)bufs * row * P * el + tw;
+    t.smem = row * P + tw;
     // threads: the fewest idle butterfly slots over the first and last stage
     long long best = -1;
     for (int n : {256, 224, 192, 160, 128}) {
@@ -118,22 +131,9 @@ static PassTile make_tile(const AxisPlan& a, int row, int bufs, size_t el, size_
     }
     return t;
 }
-
-// Tiles of the mixed-radix passes: at most pmax pencils (z, y) or pmax / 2 rows (x) per CTA.
-template <typename T>
-static TileCfg make_tiles(const Geo& g, int pmax) {
-    TileCfg t{};
-    const size_t el = sizeof(cplx_t<T>);
-    const long long pxy = (long long)g.Nx * g.Ny, pxz = (long long)g.Nx * g.Nz, pyz = (long long)g.Ny * g.Nz;
-    const int px = std::max(1, pmax / 2);
-    t.pmax = pmax;
-    t.z6 = make_tile(g.ax[2], g.Nz, 6, el, 104 * 1024, pxy, pmax);
-    t.z1 = make_tile(g.ax[2], g.Nz, 1, el, 64 * 1024, pxy, pmax);
-    t.y1 = make_tile(g.ax[1], g.Ny, 1, el, 64 * 1024, pxz, pmax);
-    t.x6 = make_tile(g.ax[0], xrow(g.Nx), 6, el, 104 * 1024, pyz, px);
-    t.x3 = make_tile(g.ax[0], xrow(g.Nx), 3, el, 64 * 1024, pyz, px);
-    return t;
-}
+template PassTile pass_tile<float>(const bloch_plan*, PassKind, int);
+template PassTile pass_tile<double>(const bloch_plan*, PassKind, int);
+template PassTile pass_tile<dfloat>(const bloch_plan*, PassKind, int);
 
 int vec_blocks(const bloch_plan* pl, int nb) {
     long long b = (pl->V + 255) / 256;
@@ -202,12 +202,9 @@ bloch_status ensure_cg(bloch_plan* pl, int nb) {
     BLOCH_CUDA_CHECK_RET(dmalloc(&w.part2, (size_t)nb * pl->nblk_max, &pl->device_bytes));
     BLOCH_CUDA_CHECK_RET(dmalloc(&w.dots, (size_t)nb, &pl->device_bytes));
     BLOCH_CUDA_CHECK_RET(dmalloc(&w.sys, (size_t)nb, &pl->device_bytes));
-    // the fused (p, Ap) partials need one slot per CTA of the fast x or z pass that forms them,
-    // for any fast variant later chosen (>= CTAs per system for every P >= 2)
-    w.zblk = std::is_same<T, float>::value && (fast_x(pl->Nz) || fast_x(pl->Nx))
-                 ? (int)((std::max((long long)pl->Nx * pl->Ny, (long long)pl->Ny * pl->Nz) + 1) / 2)
-                 : 0;
-    if (w.zblk) BLOCH_CUDA_CHECK_RET(dmalloc(&w.partz, (size_t)nb * w.zblk, &pl->device_bytes));
+    // the (p, Ap) partials of the stress pass need one slot per CTA, at most one per row
+    w.zblk = pl->Ny * pl->Nz;
+    BLOCH_CUDA_CHECK_RET(dmalloc(&w.partz, (size_t)nb * w.zblk, &pl->device_bytes));
     w.cg_cap = nb;
     return BLOCH_OK;
 }
@@ -247,19 +244,7 @@ void configure_passes(bloch_plan* pl, int variant, int pmax) {
     drop_pcg_graphs(pl);   // instantiated graphs hold the previous launch configuration
     pl->variant = variant;
     pl->fast = variant == 0;
-    pl->tile_f = make_tiles<float>(pl->geo_f, pmax);
-    pl->tile_d = make_tiles<double>(pl->geo_d, pmax);
-    pl->tile_x = make_tiles<dfloat>(pl->geo_x, pmax);
-}
-
-// CTAs per system of the fast z passes (P = 128 / RA pencils each), 0 when
-// the fast z passes do not serve this plan in FP32
-int fast_z_blocks(const bloch_plan* pl) {
-    if (!pl->fast || !fast_x(pl->Nz)) return 0;
-    const int RA = pl->Nz == 16 ? 4 : (pl->Nz == 128 ? 16 : 8);
-    const int P = kFastZThreads / RA;
-    const long long npen = (long long)pl->Nx * pl->Ny;
-    return (int)((npen + P - 1) / P);
+    pl->pmax = pmax;
 }
 
 bool has_fast_pass(const bloch_plan* pl, int precision) {
@@ -387,8 +372,7 @@ static void fast_z1(bloch_plan* pl, int nb, const float2* u, float2* E, const fl
 }
 
 template <int RA, int RB>
-static void fast_z5(bloch_plan* pl, int nb, const float2* E, const float* qtab, float2* out, float out_scale,
-                    const float2* dotp, double2* dpart) {
+static void fast_z5(bloch_plan* pl, int nb, const float2* E, const float* qtab, float2* out, float out_scale) {
     constexpr int NT = kFastZThreads;
     constexpr int P = NT / RA;
     const long long npen = (long long)pl->Nx * pl->Ny;
@@ -397,7 +381,7 @@ static void fast_z5(bloch_plan* pl, int nb, const float2* E, const float* qtab, 
     CUtensorMap map;
     const int tma = encode_zmap(&map, E, pl, 6LL * nb, P) ? 1 : 0;
     k_fpass_z_div<float, RA, RB, NT><<<gr, NT, fpass_z5_smem<float, RA, RB, NT>(), pl->stream>>>(
-        E, out, qtab, pl->d_twf[2], pl->geo_f, out_scale, dotp, dpart, map, tma);
+        E, out, qtab, pl->d_twf[2], pl->geo_f, out_scale, map, tma);
 }
 
 // Returns the CTAs per system (the number of (p, A p) partials written when dpart != nullptr)
@@ -453,39 +437,43 @@ static void launch_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T
 }
 
 // Passes 1-4: strains, their inverse FFT, stresses, forward FFT along x and y.
-// Returns the (p, A p) partials per system the x pass wrote (0: none).
-static int launch_stress_f(bloch_plan* pl, int nb, const float2* u, float2* E, const float* qtab, double2* dpart) {
+// Returns the (u, A u) partials per system the stress pass wrote (0: none).
+template <typename T>
+static int launch_stress(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab, double2* dpart) {
     int blk = 0;
-    launch_z_strain<float>(pl, nb, u, E, qtab);
-    launch_axis<float>(pl, 1, +1, 6 * nb, E, E, 1.0f);
-    if (pl->fast && fast_x(pl->Nx)) {
-        BLOCH_FAST_SWITCH_F(pl->Nx, blk =, fast_x3, pl, nb, E, dpart);
-    } else {
-        pass_x_stress<float>(pl, nb, E);
+    launch_z_strain<T>(pl, nb, u, E, qtab);
+    launch_axis<T>(pl, 1, +1, 6 * nb, E, E, T(1));
+    bool done = false;
+    if constexpr (std::is_same<T, float>::value) {
+        if (pl->fast && fast_x(pl->Nx)) {
+            BLOCH_FAST_SWITCH_F(pl->Nx, blk =, fast_x3, pl, nb, E, dpart);
+            done = true;
+        }
     }
-    launch_axis<float>(pl, 1, -1, 6 * nb, E, E, 1.0f);
+    if (!done) blk = pass_x_stress<T>(pl, nb, E, dpart);
+    launch_axis<T>(pl, 1, -1, 6 * nb, E, E, T(1));
     return dpart ? blk : 0;
 }
 
-int launch_K_on(bloch_plan* pl, int nb, const float2* u, float2* E, const float* qtab, float2* out, float out_scale,
-                const float2* dotp, double2* dpart) {
-    const bool dot = dotp && dpart;
-    int nblk = launch_stress_f(pl, nb, u, E, qtab, dot ? dpart : nullptr);
-    if (pl->fast && fast_x(pl->Nz)) {
-        // without a fast x pass the divergence forms the product and reads dotp again
-        const bool zdot = dot && nblk == 0;
-        BLOCH_FAST_SWITCH_F(pl->Nz, , fast_z5, pl, nb, E, qtab, out, out_scale, zdot ? dotp : nullptr,
-                            zdot ? dpart : nullptr);
-        if (zdot) nblk = fast_z_blocks(pl);
-    } else {
-        pass_z_div<float>(pl, nb, E, out, qtab, out_scale);
+// Pass 5: forward FFT along z and divergence
+template <typename T>
+static void launch_z_div(bloch_plan* pl, int nb, const cplx_t<T>* E, cplx_t<T>* out, const T* qtab, T out_scale) {
+    if constexpr (std::is_same<T, float>::value) {
+        if (pl->fast && fast_x(pl->Nz)) {
+            BLOCH_FAST_SWITCH_F(pl->Nz, , fast_z5, pl, nb, E, qtab, out, out_scale);
+            return;
+        }
     }
-    return nblk;
+    pass_z_div<T>(pl, nb, E, out, qtab, out_scale);
+}
+
+void launch_K_on(bloch_plan* pl, int nb, const float2* u, float2* E, const float* qtab, float2* out, float out_scale) {
+    launch_stress<float>(pl, nb, u, E, qtab, nullptr);
+    launch_z_div<float>(pl, nb, E, out, qtab, out_scale);
 }
 
 template <typename T>
-int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale, const cplx_t<T>* dotp,
-             double2* dpart) {
+int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale, double2* dpart) {
     Workspace<T>& w = ws_of<T>(pl);
     if constexpr (!std::is_same<T, dfloat>::value) {   // cuFFT has no float-float transform
         if (pl->variant == 2) {
@@ -494,14 +482,9 @@ int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_s
             return 0;
         }
     }
-    if constexpr (std::is_same<T, float>::value)
-        return launch_K_on(pl, nb, u, w.E, w.qtab, out, out_scale, dotp, dpart);
-    pass_z_strain<T>(pl, nb, u, w.E, w.qtab);
-    launch_axis<T>(pl, 1, +1, 6 * nb, w.E, w.E, T(1));
-    pass_x_stress<T>(pl, nb, w.E);
-    launch_axis<T>(pl, 1, -1, 6 * nb, w.E, w.E, T(1));
-    pass_z_div<T>(pl, nb, w.E, out, w.qtab, out_scale);
-    return 0;
+    const int blk = launch_stress<T>(pl, nb, u, w.E, w.qtab, dpart);
+    launch_z_div<T>(pl, nb, w.E, out, w.qtab, out_scale);
+    return blk;
 }
 
 // Fourier-space stress of nb systems whose q tables are set, into the
@@ -512,14 +495,7 @@ int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_s
 template <typename T>
 void launch_K_stress(bloch_plan* pl, int nb, const cplx_t<T>* u) {
     Workspace<T>& w = ws_of<T>(pl);
-    if constexpr (std::is_same<T, float>::value) {
-        launch_stress_f(pl, nb, u, w.E, w.qtab, nullptr);
-    } else {
-        pass_z_strain<T>(pl, nb, u, w.E, w.qtab);
-        launch_axis<T>(pl, 1, +1, 6 * nb, w.E, w.E, T(1));
-        pass_x_stress<T>(pl, nb, w.E);
-        launch_axis<T>(pl, 1, -1, 6 * nb, w.E, w.E, T(1));
-    }
+    launch_stress<T>(pl, nb, u, w.E, w.qtab, nullptr);
     launch_axis<T>(pl, 2, -1, 6 * nb, w.E, w.E, T(1));
 }
 
@@ -597,7 +573,7 @@ static void pcg_iteration(bloch_plan* pl, int nb, cplx_t<T>* x, double tol2, int
     gk.skip = &w.sys[0].active;
     gk.skip_stride = (int)(sizeof(CGSys) / sizeof(int));
     gk.skip_ncomp = 6;
-    const int zb = launch_K<T>(pl, nb, w.p, w.Ap, T(1), w.p, w.partz);
+    const int zb = launch_K<T>(pl, nb, w.p, w.Ap, T(1), w.partz);
     gk.skip = nullptr;
     gk.skip_stride = 1;
     gk.skip_ncomp = 1;
@@ -819,7 +795,7 @@ bloch_status pcg_enqueue(bloch_plan* pl, int nb, const cplx_t<T>* b, cplx_t<T>* 
     template bloch_status ensure_ws<T>(bloch_plan*, int);                                                \
     template bloch_status ensure_cg<T>(bloch_plan*, int);                                                \
     template bloch_status set_k<T>(bloch_plan*, int, const double*);                                     \
-    template int launch_K<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T, const cplx_t<T>*, double2*); \
+    template int launch_K<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T, double2*);               \
     template void launch_M<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T);                        \
     template void launch_K_stress<T>(bloch_plan*, int, const cplx_t<T>*);                                 \
     template void launch_fft3<T, -1>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T, const double2*); \
@@ -836,7 +812,7 @@ INST(float)
 INST(double)
 #undef INST
 template bloch_status ensure_ws<dfloat>(bloch_plan*, int);
-template int launch_K<dfloat>(bloch_plan*, int, const dfloat2*, dfloat2*, dfloat, const dfloat2*, double2*);
+template int launch_K<dfloat>(bloch_plan*, int, const dfloat2*, dfloat2*, dfloat, double2*);
 template bloch_status set_k<dfloat>(bloch_plan*, int, const double*);
 template void launch_M<dfloat>(bloch_plan*, int, const dfloat2*, dfloat2*, dfloat);
 
@@ -1180,10 +1156,7 @@ bloch_status bloch_plan_create(bloch_plan** out, const int32_t grid[3], const do
         pl->geo_f.ax[a] = pl->geo_d.ax[a] = make_axis(grid[a], false);
         pl->geo_x.ax[a] = make_axis(grid[a], true);
     }
-    const int pmax = pl->opt.tile_pmax > 0 ? pl->opt.tile_pmax : kDefaultPmax;
-    pl->tile_f = make_tiles<float>(pl->geo_f, pmax);
-    pl->tile_d = make_tiles<double>(pl->geo_d, pmax);
-    pl->tile_x = make_tiles<dfloat>(pl->geo_x, pmax);
+    pl->pmax = pl->opt.tile_pmax > 0 ? pl->opt.tile_pmax : kDefaultPmax;
     pl->nblk_max = vec_blocks(pl, 1);
     *out = pl;
     return BLOCH_OK;

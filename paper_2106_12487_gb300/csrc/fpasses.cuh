@@ -285,14 +285,10 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>
 //   out_x = q_x S11 + q_y S12 + q_z S13, out_y = q_x S12 + q_y S22 + q_z S23,
 //   out_z = q_x S13 + q_y S23 + q_z S33   (S = forward z transform of sigma).
 // Stress components stream into shared memory two ahead (cp.async).
-// With dotp != nullptr the CTA also forms sum conj(dotp) * out over its
-// pencils (the (p, A p) product of the PCG iteration, Algorithm 2) and writes
-// it to dpart[b * gridDim.x + blockIdx.x].
 template <typename T, int RA, int RB, int NT = 128>
 __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* __restrict__ E, cplx_t<T>* __restrict__ out,
                                                         const T* __restrict__ qtab, const cplx_t<T>* __restrict__ twz,
-                                                        Geo g, T out_scale, const cplx_t<T>* __restrict__ dotp,
-                                                        double2* __restrict__ dpart,
+                                                        Geo g, T out_scale,
                                                         const __grid_constant__ CUtensorMap tmap, int use_tma) {
     using C = cplx_t<T>;
     constexpr int N = RA * RB;
@@ -450,8 +446,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* _
             stage2(c, xb);
         }
     }
-    T dre = T(0), dim = T(0);
-    const C* pb = dotp ? dotp + (size_t)b * 3 * g.V : nullptr;
     if (p2 < np) {
 #pragma unroll
         for (int r = 0; r < RB; ++r) {
@@ -461,34 +455,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* _
                 const C o = cscale(acc[i][r], out_scale);
                 if constexpr (sizeof(C) == 8) st_stream(ob + (size_t)i * g.V + a, o);
                 else ob[(size_t)i * g.V + a] = o;
-                if (pb) {
-                    const C pv = pb[(size_t)i * g.V + a];
-                    dre += pv.x * o.x + pv.y * o.y;
-                    dim += pv.x * o.y - pv.y * o.x;
-                }
             }
-        }
-    }
-    if (dotp) {   // block reduction (NT / 32 warps); deterministic order
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            dre += __shfl_xor_sync(0xffffffffu, dre, o);
-            dim += __shfl_xor_sync(0xffffffffu, dim, o);
-        }
-        __shared__ T red[2][NT / 32];
-        if ((tid & 31) == 0) {
-            red[0][tid >> 5] = dre;
-            red[1][tid >> 5] = dim;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            double sr = 0.0, si = 0.0;
-#pragma unroll
-            for (int w = 0; w < NT / 32; ++w) {
-                sr += (double)red[0][w];
-                si += (double)red[1][w];
-            }
-            dpart[(size_t)b * gridDim.x + blockIdx.x] = make_double2(sr, si);
         }
     }
 }
@@ -498,11 +465,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* _
 // blockDim.x == P * RA is required.  Shared rows are padded (one slot every 16)
 // to spread the strided Stockham writes over the banks.
 __device__ __forceinline__ int xpad(int n) { return n + (n >> 4); }
-
-// Index of C_ij (any order) in the packed upper triangle of a symmetric 6x6.
-__host__ __device__ constexpr int sym6(int i, int j) {
-    return i <= j ? i * 6 - i * (i - 1) / 2 + (j - i) : j * 6 - j * (j - 1) / 2 + (i - j);
-}
 
 // sigma = C_g gamma at the element r of every component (packed symmetric
 // table, 21 per grain), one row of C_g at a time so that few coefficients

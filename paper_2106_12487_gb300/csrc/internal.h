@@ -69,11 +69,13 @@ struct PassTile {
     size_t smem;
 };
 
-struct TileCfg {
-    int pmax;             // cap on pencils per CTA the tiles were made with
-    PassTile z6;          // z strain / divergence, 6 buffers
-    PassTile y1, z1;      // plain y and z passes, 1 buffer
-    PassTile x6, x3;      // x rows, 6 (stress) and 3 (density, plain) components
+// Mixed-radix passes by the tile they need.
+enum PassKind {
+    PASS_Z6 = 0,   // z strain / divergence, 6 buffers
+    PASS_Y1,       // plain y pass
+    PASS_Z1,       // plain z pass
+    PASS_X6,       // x rows, 6 components (stress)
+    PASS_X3        // x rows, 3 components (density, plain)
 };
 
 }  // namespace bloch
@@ -117,7 +119,7 @@ struct bloch_plan {
     int* h_nactive = nullptr;     // pinned
 
     bloch::Geo geo_f, geo_d, geo_x;     // FP32, FP64, float-float
-    bloch::TileCfg tile_f, tile_d, tile_x;
+    int pmax;                           // cap on pencils per CTA of the mixed-radix passes
     int nblk_max;
     bool fast = true;              // use the two-stage register FFT passes where the axis allows
     int variant = 0;               // options.fft_variant, or the autotuner's choice
@@ -176,7 +178,8 @@ namespace bloch {
 
 template <typename T> Workspace<T>& ws_of(bloch_plan* pl);
 template <typename T> const Geo& geo_of(const bloch_plan* pl);
-template <typename T> const TileCfg& tile_of(const bloch_plan* pl);
+// Tile of a mixed-radix pass over nb systems (plain y, z passes: fields).
+template <typename T> PassTile pass_tile(const bloch_plan* pl, PassKind kind, int nb);
 
 // Mixed-radix passes (passes.cuh) on the plan's stream: any axis length, every
 // field type.  E and W are updated in place; dir -1 forward, +1 inverse.
@@ -184,7 +187,9 @@ template <typename T>
 void pass_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab);
 template <typename T>   // axis 1 (y) or 2 (z) of nfields scalar fields
 void pass_axis(bloch_plan* pl, int axis, int dir, int nfields, const cplx_t<T>* in, cplx_t<T>* out, T out_scale);
-template <typename T> void pass_x_stress(bloch_plan* pl, int nb, cplx_t<T>* E);
+// x pass: the (u, A u) partials of each system go to dpart (nullptr: none);
+// returns their number per system.
+template <typename T> int pass_x_stress(bloch_plan* pl, int nb, cplx_t<T>* E, double2* dpart);
 template <typename T> void pass_x_rho(bloch_plan* pl, int nb, cplx_t<T>* W);
 template <typename T>   // ph, per: complex factors of the systems (k_pass_x)
 void pass_x(bloch_plan* pl, int dir, int nb, cplx_t<T>* W, T out_scale, const double2* ph = nullptr, int per = 1);
@@ -202,15 +207,13 @@ template <typename T> bloch_status ensure_cg(bloch_plan* pl, int nb);
 // Upload nb wave vectors (host, rad/m) and build the scaled q tables.
 template <typename T> bloch_status set_k(bloch_plan* pl, int nb, const double* k_host);
 // Scaled stiffness operator on nb systems whose q tables are set: out = out_scale * A~ u.
-// With dotp / dpart, a pass that can also forms per-CTA partials of
-// sum conj(dotp) * out per system in dpart and the call returns the number of
-// partials per system; it returns 0 when no pass did (the caller forms the dot).
+// With dpart, the stress pass also forms per-CTA partials of (u, A~ u) per
+// system in dpart and the call returns the number of partials per system; it
+// returns 0 when no pass did (the caller forms the product).
 template <typename T>
-int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale,
-             const cplx_t<T>* dotp = nullptr, double2* dpart = nullptr);
+int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale, double2* dpart = nullptr);
 // The FP32 operator on scratch E and q tables of the caller (launch_K's chain).
-int launch_K_on(bloch_plan* pl, int nb, const float2* u, float2* E, const float* qtab, float2* out, float out_scale,
-                const float2* dotp, double2* dpart);
+void launch_K_on(bloch_plan* pl, int nb, const float2* u, float2* E, const float* qtab, float2* out, float out_scale);
 // Fourier-space stress S = F{C~ : F^-1(sym q (x) u)} of nb systems (q tables
 // set) into the operator workspace E, 6 Voigt components per system.
 template <typename T> void launch_K_stress(bloch_plan* pl, int nb, const cplx_t<T>* u);
@@ -269,8 +272,6 @@ void configure_passes(bloch_plan* pl, int variant, int pmax);
 // Whether the fast (two-stage register) passes serve at least one pass of the
 // chain in this precision, and whether a shared-memory pass remains in it.
 bool has_fast_pass(const bloch_plan* pl, int precision);
-// CTAs per system of the fast FP32 z passes (0 when they do not serve the plan).
-int fast_z_blocks(const bloch_plan* pl);
 bool has_generic_pass(const bloch_plan* pl, int precision);
 
 // plain-form baseline (bloch_cufft.cu): Eq. (hatA) with cuFFT 3D transforms

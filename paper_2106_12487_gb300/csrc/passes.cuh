@@ -65,12 +65,22 @@ __device__ __forceinline__ bool sys_idle(const Geo& g, int b) {
     return g.skip != nullptr && g.skip[(size_t)b * g.skip_stride] == 0;
 }
 
+// Index of C_ij (any order) in the packed upper triangle of a symmetric 6x6.
+__host__ __device__ constexpr int sym6(int i, int j) {
+    return i <= j ? i * 6 - i * (i - 1) / 2 + (j - i) : j * 6 - j * (j - 1) / 2 + (i - j);
+}
+
 __host__ __device__ __forceinline__ int pad_even(int n) { return (n + 1) & ~1; }
 
-// Row position of slot n in the x passes: one spare slot every 16 spreads the
-// strided accesses of the last stage over the banks; xrow(N) is the row length (odd).
-__host__ __device__ __forceinline__ int xslot(int n) { return n + (n >> 4); }
-__host__ __device__ __forceinline__ int xrow(int N) { return (N + (N >> 4)) | 1; }
+// Rows of the x passes keep one spare element after every r3 slots when r3 is
+// even: the last stage's threads then step by an odd number of elements and
+// meet no bank conflicts.  xgroup(a) is the length of such a group, xrow(a)
+// that of a row (odd, so that rows are spread too).
+__host__ __device__ __forceinline__ int xgroup(const AxisPlan& a) { return a.r3 + ((a.r3 & 1) ^ 1); }
+__host__ __device__ __forceinline__ int xrow(const AxisPlan& a) { return (a.r1 * a.r2 * xgroup(a)) | 1; }
+
+// CTAs per SM the pass kernels leave registers for
+template <typename T> constexpr int kPassCtas = sizeof(T) == 4 ? 3 : 2;
 
 // f(std::integral_constant<int, R>) for the run-time radix R.  Float-float
 // leaves out the radices whose code is longest for what they save (compile time).
@@ -169,7 +179,7 @@ __device__ __forceinline__ void pf_last(C* buf, int nbuf, const AxisPlan& a, int
 //   g_xz = q_x a_z + b_x, g_xy = q_y a_x + q_x a_y
 // (q_x and q_y are constant on a z pencil).
 template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
+__global__ void __launch_bounds__(256, kPassCtas<T>)
     k_pass_z_strain(const cplx_t<T>* __restrict__ U, cplx_t<T>* __restrict__ E, const T* __restrict__ qtab,
                     const cplx_t<T>* __restrict__ twz, Geo g, int lp) {
     using C = cplx_t<T>;
@@ -264,7 +274,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
 // ------------------------------------------------- plain FFT pass along y or z
 // blockIdx.y enumerates (batch, component) pairs: offset blockIdx.y * V.
 template <typename T, int DIR, int AXIS>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
+__global__ void __launch_bounds__(256, kPassCtas<T>)
     k_pass_axis(const cplx_t<T>* in, cplx_t<T>* out, const cplx_t<T>* __restrict__ twa, Geo g, int lp, T out_scale) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -331,7 +341,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
 
 // ---------------------------------------------------------------- pass 5
 template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
+__global__ void __launch_bounds__(256, kPassCtas<T>)
     k_pass_z_div(const cplx_t<T>* __restrict__ E, cplx_t<T>* __restrict__ out, const T* __restrict__ qtab,
                  const cplx_t<T>* __restrict__ twz, Geo g, int lp, T out_scale) {
     using C = cplx_t<T>;
@@ -392,28 +402,28 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
 }
 
 // ------------------------------------------------ stages on rows along x
-// Element (component c, row p, slot n) at (c P + p) ld + xslot(n), ld = xrow(N).
+// Element (component c, row p, slot n) at (c P + p) xrow + (n / r3) xgroup + n mod r3.
 
 // stage 1 (decimation in frequency) of ncomp components of P rows, from HBM
 template <int DIR, typename C>
 __device__ __forceinline__ void lf_first(const C* Wb, long long V, C* buf, int ncomp, const AxisPlan& a, int P, int nr,
                                          unsigned r0, const C* tw, int tid, int nthr) {
-    const int ld = xrow(a.N);
+    const int ld = xrow(a), gr = xgroup(a);
     with_radix<real_t<C>>(a.r1, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
-        const int M = a.N / R;
+        const int M = a.N / R, Mg = a.r2 * gr;
         for (int t = tid; t < ncomp * P * M; t += nthr) {
             const int cp = (int)fdiv((unsigned)t, a.m1), j = t - cp * M;
             const int c = cp / P, p = min(cp - c * P, nr - 1);
             const C* src = Wb + (size_t)c * V + (size_t)(r0 + p) * a.N + j;
-            C* s = buf + cp * ld;
+            C* s = buf + cp * ld + j + (int)fdiv((unsigned)j, a.d3) * (gr - a.r3);
             C v[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) v[r] = src[r * M];
             RegDFT<R, DIR, C>::run(v);
-            s[xslot(j)] = v[0];
+            s[0] = v[0];
 #pragma unroll
-            for (int r = 1; r < R; ++r) s[xslot(r * M + j)] = twiddled<DIR>(v[r], tw[r * j]);
+            for (int r = 1; r < R; ++r) s[r * Mg] = twiddled<DIR>(v[r], tw[r * j]);
         }
     });
 }
@@ -421,26 +431,25 @@ __device__ __forceinline__ void lf_first(const C* Wb, long long V, C* buf, int n
 // middle stage: FREQ decimation in frequency (twiddles after), else in time (before)
 template <int DIR, bool FREQ, typename C>
 __device__ __forceinline__ void lf_mid(C* buf, int nrows, const AxisPlan& a, const C* tw, int tid, int nthr) {
-    const int ld = xrow(a.N);
+    const int ld = xrow(a), gr = xgroup(a);
     with_mid_radix(a.r2, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
-        const int M = a.N / R, r3 = a.r3;
+        const int M = a.N / R;
         for (int t = tid; t < nrows * M; t += nthr) {
             const int cp = (int)fdiv((unsigned)t, a.m2), j = t - cp * M;
-            const int k1 = (int)fdiv((unsigned)j, a.d3), n3 = j - k1 * r3;
-            const int s0 = k1 * R * r3 + n3;
-            C* s = buf + cp * ld;
+            const int k1 = (int)fdiv((unsigned)j, a.d3), n3 = j - k1 * a.r3;
+            C* s = buf + cp * ld + k1 * R * gr + n3;
             C v[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                v[r] = s[xslot(s0 + r * r3)];
+                v[r] = s[r * gr];
                 if (!FREQ && r > 0) v[r] = twiddled<DIR>(v[r], tw[r * n3 * a.r1]);
             }
             RegDFT<R, DIR, C>::run(v);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 if (FREQ && r > 0) v[r] = twiddled<DIR>(v[r], tw[r * n3 * a.r1]);
-                s[xslot(s0 + r * r3)] = v[r];
+                s[r * gr] = v[r];
             }
         }
     });
@@ -450,20 +459,20 @@ __device__ __forceinline__ void lf_mid(C* buf, int nrows, const AxisPlan& a, con
 // and the first of the mirrored forward transform
 template <int DIR, typename C>
 __device__ __forceinline__ void lf_last(C* buf, int nrows, const AxisPlan& a, int tid, int nthr) {
-    const int ld = xrow(a.N);
+    const int ld = xrow(a), gr = xgroup(a);
     with_radix<real_t<C>>(a.r3, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         if constexpr (R > 1) {
             const int M = a.N / R;
             for (int t = tid; t < nrows * M; t += nthr) {
-                const int cp = (int)fdiv((unsigned)t, a.m3), s0 = (t - cp * M) * R;
-                C* s = buf + cp * ld;
+                const int cp = (int)fdiv((unsigned)t, a.m3);
+                C* s = buf + cp * ld + (t - cp * M) * gr;
                 C v[R];
 #pragma unroll
-                for (int r = 0; r < R; ++r) v[r] = s[xslot(s0 + r)];
+                for (int r = 0; r < R; ++r) v[r] = s[r];
                 RegDFT<R, DIR, C>::run(v);
 #pragma unroll
-                for (int r = 0; r < R; ++r) s[xslot(s0 + r)] = v[r];
+                for (int r = 0; r < R; ++r) s[r] = v[r];
             }
         }
     });
@@ -473,19 +482,19 @@ __device__ __forceinline__ void lf_last(C* buf, int nrows, const AxisPlan& a, in
 template <int DIR, typename C>
 __device__ __forceinline__ void lf_store(C* Wb, long long V, const C* buf, int ncomp, const AxisPlan& a, int P, int nr,
                                          unsigned r0, const C* tw, int tid, int nthr) {
-    const int ld = xrow(a.N);
+    const int ld = xrow(a), gr = xgroup(a);
     with_radix<real_t<C>>(a.r1, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
-        const int M = a.N / R;
+        const int M = a.N / R, Mg = a.r2 * gr;
         for (int t = tid; t < ncomp * P * M; t += nthr) {
             const int cp = (int)fdiv((unsigned)t, a.m1), j = t - cp * M;
             const int c = cp / P, p = cp - c * P;
             if (p >= nr) continue;
-            const C* s = buf + cp * ld;
+            const C* s = buf + cp * ld + j + (int)fdiv((unsigned)j, a.d3) * (gr - a.r3);
             C v[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                v[r] = s[xslot(r * M + j)];
+                v[r] = s[r * Mg];
                 if (r > 0) v[r] = twiddled<DIR>(v[r], tw[r * j]);
             }
             RegDFT<R, DIR, C>::run(v);
@@ -496,18 +505,74 @@ __device__ __forceinline__ void lf_store(C* Wb, long long V, const C* buf, int n
     });
 }
 
+// Stiffness C_ij of a grain: FP32 keeps the packed upper triangle (21 per
+// grain), the wider types the full 6 x 6 table.
+template <typename T> constexpr int kCtabRow = sizeof(T) == 4 ? 21 : 36;
+template <typename T>
+__device__ __forceinline__ T ctab_at(const T* Cg, int i, int j) {
+    return ldg_t(Cg + (sizeof(T) == 4 ? sym6(i, j) : i * 6 + j));
+}
+
+// natural index k1 + r1 k2 + r1 r2 k3 of slot n = q r3 + k3, q = k1 r2 + k2
+__device__ __forceinline__ int index_of(int n, int q, const AxisPlan& a) {
+    const int k1 = (int)fdiv((unsigned)q, a.d2);
+    return k1 + a.r1 * ((q - k1 * a.r2) + a.r2 * (n - q * a.r3));
+}
+
+// sigma = C_g gamma in place on the six components s[c cs]; adds conj(gamma) sigma
+template <typename T, typename C>
+__device__ __forceinline__ void stress_smem(C* s, int cs, const T* __restrict__ Cg, T& energy) {
+    C gam[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) gam[c] = s[c * cs];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        T sr = 0, si = 0;
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            const T cij = ctab_at<T>(Cg, i, j);
+            sr = fma(cij, gam[j].x, sr);
+            si = fma(cij, gam[j].y, si);
+        }
+        s[i * cs] = mk(sr, si);
+        if constexpr (!std::is_same<T, dfloat>::value) energy = fma(gam[i].x, sr, fma(gam[i].y, si, energy));
+    }
+}
+
+// CTA sum of the threads' energies (field precision within a warp, FP64 across)
+template <typename T>
+__device__ __forceinline__ void energy_out(T e, double2* dst) {
+    if constexpr (!std::is_same<T, dfloat>::value) {
+        __shared__ double red[32];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (double)e;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double t = 0.0;
+            for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) t += red[w];
+            *dst = make_double2(t, 0.0);
+        }
+    }
+}
+
 // Row pass along x on P rows per CTA (blockIdx.y = system): inverse FFT,
 // pointwise product in real space, forward FFT, in place.
-//   NC = 6: strains to stresses with the per-grain 6 x 6 table (pass 3)
+//   NC = 6: strains to stresses with the per-grain table (pass 3)
 //   NC = 3: displacements times the per-grain scalar table (mass operator)
+// The pointwise step walks the slots in order (no bank conflicts) and gathers
+// the grain ids of a row, which its first touch brings to L1.  With dpart
+// (NC = 6) the CTA writes its share of the strain energy sum conj(gamma) sigma
+// = (u, A_k u) to dpart[b gridDim.x + blockIdx.x] (as k_fpass_x_stress).
 template <typename T, int NC>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
+__global__ void __launch_bounds__(256, kPassCtas<T>)
     k_pass_x_grain(cplx_t<T>* W, const int32_t* __restrict__ ids, const T* __restrict__ tab,
-                   const cplx_t<T>* __restrict__ twx, Geo g, int P) {
+                   const cplx_t<T>* __restrict__ twx, Geo g, int P, double2* __restrict__ dpart) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const AxisPlan& a = g.ax[0];
-    const int N = a.N, ld = xrow(N);
+    const int N = a.N, ld = xrow(a), gr = xgroup(a);
+    T energy = T(0);
     C* tw = reinterpret_cast<C*>(smem_raw);
     C* buf = tw + pad_even(N);
     const int tid = threadIdx.x, nthr = blockDim.x;
@@ -528,32 +593,20 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
     lf_last<+1>(buf, NC * P, a, tid, nthr);
     __syncthreads();
     for (int t = tid; t < nr * N; t += nthr) {
-        const int p = (int)fdiv((unsigned)t, g.dx), k = t - p * N;
-        const int gid = ids[(size_t)(r0 + p) * N + k];
-        C* s = buf + p * ld + xslot(slot_of(k, a));
+        const int p = (int)fdiv((unsigned)t, g.dx), n = t - p * N;
+        const int q = (int)fdiv((unsigned)n, a.d3);
+        const int gid = ids[(size_t)(r0 + p) * N + index_of(n, q, a)];
+        C* s = buf + p * ld + n + q * (gr - a.r3);
         const int cs = P * ld;
         if constexpr (NC == 6) {
-            const T* Cg = tab + (size_t)gid * 36;
-            C gam[6];
-#pragma unroll
-            for (int c = 0; c < 6; ++c) gam[c] = s[c * cs];
-#pragma unroll
-            for (int i = 0; i < 6; ++i) {
-                T sr = 0, si = 0;
-#pragma unroll
-                for (int j = 0; j < 6; ++j) {
-                    const T cij = ldg_t(Cg + i * 6 + j);
-                    sr = fma(cij, gam[j].x, sr);
-                    si = fma(cij, gam[j].y, si);
-                }
-                s[i * cs] = mk(sr, si);
-            }
+            stress_smem<T>(s, cs, tab + (size_t)gid * kCtabRow<T>, energy);
         } else {
             const T r = ldg_t(tab + gid);
 #pragma unroll
             for (int c = 0; c < NC; ++c) s[c * cs] = cscale(s[c * cs], r);
         }
     }
+    if (NC == 6 && dpart) energy_out(energy, dpart + (size_t)b * gridDim.x + blockIdx.x);
     __syncthreads();
     lf_last<-1>(buf, NC * P, a, tid, nthr);
     __syncthreads();
@@ -571,13 +624,13 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
 // fields each) are also multiplied by the complex factor ph[b], and the second
 // of two fields by 1/2 (the shears of a strain field: engineering to tensor).
 template <typename T, int DIR>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
+__global__ void __launch_bounds__(256, kPassCtas<T>)
     k_pass_x(cplx_t<T>* W, const cplx_t<T>* __restrict__ twx, Geo g, int P, T out_scale,
              const double2* __restrict__ ph, int per) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const AxisPlan& a = g.ax[0];
-    const int N = a.N, ld = xrow(N);
+    const int N = a.N, ld = xrow(a), gr = xgroup(a);
     C* tw = reinterpret_cast<C*>(smem_raw);
     C* buf = tw + pad_even(N);
     const int tid = threadIdx.x, nthr = blockDim.x;
@@ -603,7 +656,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
         const int cp = (int)fdiv((unsigned)t, g.dx), k = t - cp * N;
         const int c = cp / P, p = cp - c * P;
         if (p >= nr) continue;
-        const C v = buf[cp * ld + xslot(slot_of(k, a))];
+        const int s = slot_of(k, a);
+        const C v = buf[cp * ld + s + (int)fdiv((unsigned)s, a.d3) * (gr - a.r3)];
         Wb[(size_t)c * g.V + (size_t)(r0 + p) * N + k] = ph ? cmul(v, f) : cscale(v, out_scale);
     }
 }

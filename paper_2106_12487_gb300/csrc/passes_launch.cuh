@@ -13,7 +13,7 @@ template <> inline const float2* pass_tw<float>(const bloch_plan* pl, int axis) 
 template <> inline const double2* pass_tw<double>(const bloch_plan* pl, int axis) { return pl->d_twd[axis]; }
 template <> inline const dfloat2* pass_tw<dfloat>(const bloch_plan* pl, int axis) { return pl->d_twx[axis]; }
 template <typename T> static inline const T* pass_ctab(const bloch_plan* pl);
-template <> inline const float* pass_ctab<float>(const bloch_plan* pl) { return pl->d_Cf; }
+template <> inline const float* pass_ctab<float>(const bloch_plan* pl) { return pl->d_Cpf; }
 template <> inline const double* pass_ctab<double>(const bloch_plan* pl) { return pl->d_Cd; }
 template <> inline const dfloat* pass_ctab<dfloat>(const bloch_plan* pl) { return pl->d_Cx; }
 template <typename T> static inline const T* pass_rtab(const bloch_plan* pl);
@@ -27,7 +27,7 @@ static inline dim3 pass_grid(long long npen, int lp, int ny) {
 
 template <typename T>
 void pass_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab) {
-    const PassTile& t = tile_of<T>(pl).z6;
+    const PassTile t = pass_tile<T>(pl, PASS_Z6, nb);
     ++pl->launches;
     k_pass_z_strain<T><<<pass_grid((long long)pl->Nx * pl->Ny, t.lp, nb), t.nthr, t.smem, pl->stream>>>(
         u, E, qtab, pass_tw<T>(pl, 2), geo_of<T>(pl), t.lp);
@@ -35,8 +35,7 @@ void pass_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, con
 
 template <typename T>
 void pass_axis(bloch_plan* pl, int axis, int dir, int nfields, const cplx_t<T>* in, cplx_t<T>* out, T out_scale) {
-    const TileCfg& tc = tile_of<T>(pl);
-    const PassTile& t = axis == 1 ? tc.y1 : tc.z1;
+    const PassTile t = pass_tile<T>(pl, axis == 1 ? PASS_Y1 : PASS_Z1, nfields);
     const dim3 gr = pass_grid((long long)pl->Nx * (axis == 1 ? pl->Nz : pl->Ny), t.lp, nfields);
     const Geo& g = geo_of<T>(pl);
     const cplx_t<T>* tw = pass_tw<T>(pl, axis);
@@ -52,24 +51,26 @@ void pass_axis(bloch_plan* pl, int axis, int dir, int nfields, const cplx_t<T>* 
 }
 
 template <typename T>
-void pass_x_stress(bloch_plan* pl, int nb, cplx_t<T>* E) {
-    const PassTile& t = tile_of<T>(pl).x6;
+int pass_x_stress(bloch_plan* pl, int nb, cplx_t<T>* E, double2* dpart) {
+    const PassTile t = pass_tile<T>(pl, PASS_X6, nb);
+    const dim3 gr = pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb);
     ++pl->launches;
-    k_pass_x_grain<T, 6><<<pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb), t.nthr, t.smem, pl->stream>>>(
-        E, pl->d_ids, pass_ctab<T>(pl), pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp);
+    k_pass_x_grain<T, 6><<<gr, t.nthr, t.smem, pl->stream>>>(E, pl->d_ids, pass_ctab<T>(pl), pass_tw<T>(pl, 0),
+                                                             geo_of<T>(pl), 1 << t.lp, dpart);
+    return (int)gr.x;
 }
 
 template <typename T>
 void pass_x_rho(bloch_plan* pl, int nb, cplx_t<T>* W) {
-    const PassTile& t = tile_of<T>(pl).x3;
+    const PassTile t = pass_tile<T>(pl, PASS_X3, nb);
     ++pl->launches;
     k_pass_x_grain<T, 3><<<pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb), t.nthr, t.smem, pl->stream>>>(
-        W, pl->d_ids, pass_rtab<T>(pl), pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp);
+        W, pl->d_ids, pass_rtab<T>(pl), pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp, nullptr);
 }
 
 template <typename T>
 void pass_x(bloch_plan* pl, int dir, int nb, cplx_t<T>* W, T out_scale, const double2* ph, int per) {
-    const PassTile& t = tile_of<T>(pl).x3;
+    const PassTile t = pass_tile<T>(pl, PASS_X3, nb);
     const dim3 gr = pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb);
     ++pl->launches;
     if (dir > 0)
@@ -82,7 +83,7 @@ void pass_x(bloch_plan* pl, int dir, int nb, cplx_t<T>* W, T out_scale, const do
 
 template <typename T>
 void pass_z_div(bloch_plan* pl, int nb, const cplx_t<T>* E, cplx_t<T>* out, const T* qtab, T out_scale) {
-    const PassTile& t = tile_of<T>(pl).z6;
+    const PassTile t = pass_tile<T>(pl, PASS_Z6, nb);
     ++pl->launches;
     k_pass_z_div<T><<<pass_grid((long long)pl->Nx * pl->Ny, t.lp, nb), t.nthr, t.smem, pl->stream>>>(
         E, out, qtab, pass_tw<T>(pl, 2), geo_of<T>(pl), t.lp, out_scale);
@@ -123,7 +124,7 @@ cudaError_t pass_attrs_x() {
     template void pass_axis<T>(bloch_plan*, int, int, int, const cplx_t<T>*, cplx_t<T>*, T);              \
     template cudaError_t pass_attrs_axis<T>();
 #define BLOCH_INST_PASSES_X(T)                                                                            \
-    template void pass_x_stress<T>(bloch_plan*, int, cplx_t<T>*);                                         \
+    template int pass_x_stress<T>(bloch_plan*, int, cplx_t<T>*, double2*);                                \
     template void pass_x_rho<T>(bloch_plan*, int, cplx_t<T>*);                                            \
     template cudaError_t pass_attrs_x<T>();
 
