@@ -43,7 +43,6 @@ template <> const float* ctab_of<float>(const bloch_plan* pl) { return pl->d_Cf;
 template <> const double* ctab_of<double>(const bloch_plan* pl) { return pl->d_Cd; }
 template <typename T> static const T* cpk_of(const bloch_plan* pl);
 template <> const float* cpk_of<float>(const bloch_plan* pl) { return pl->d_Cpf; }
-template <> const double* cpk_of<double>(const bloch_plan* pl) { return pl->d_Cpd; }
 // ------------------------------------------------------------ host helpers
 static bool fast_axis(int N);
 static bool fast_x(int N);
@@ -86,8 +85,9 @@ static AxisPlan make_axis(int N, bool ff) {
     return ap;
 }
 
-// Shared memory a CTA of a six-buffer tile may take: two CTAs per SM.
-constexpr size_t kTileSmem = 104 * 1024;
+// Shared memory a CTA may take: two CTAs per SM for the z passes, whose rows
+// gain from width; four for the rows along x, whose do not.
+constexpr size_t kTileSmemZ = 104 * 1024, kTileSmemX = 55 * 1024;
 // CTAs wanted in a launch before a tile is worth its width: three per SM.
 // (48 x 40 x 36, FP32, 10 systems: 185 us per K-apply with tiles made for one
 // system, 95 us with tiles made for the launch.)
@@ -106,8 +106,8 @@ PassTile pass_tile(const bloch_plan* pl, PassKind kind, int nb) {
     const int bufs = kind == PASS_Y1 || kind == PASS_Z1 ? 1 : kind == PASS_X3 ? 3 : 6;
     const long long npen = g.V / a.N;
     const size_t row = (size_t)(x_ ? xrow(a) : a.N) * bufs * el;
-    const size_t tw = (size_t)pad_even(a.N) * el;
-    const size_t budget = bufs == 1 ? 64 * 1024 : kTileSmem;
+    const size_t tw = (size_t)pad_even(twtab_len(a)) * el;
+    const size_t budget = bufs == 1 ? 64 * 1024 : x_ ? kTileSmemX : kTileSmemZ;
     PassTile t{};
     int P = std::max(1, x_ ? pl->pmax / 2 : pl->pmax);
     while (P > 1 && row * P + tw > budget) P >>= 1;
@@ -297,7 +297,7 @@ static void fast_yz(bloch_plan* pl, int axis, int DIR, int nfields, const cplx_t
     const unsigned plane = (unsigned)pl->Nx * pl->Ny;
     const unsigned inner = axis == 1 ? (unsigned)pl->Nx : plane, outer = axis == 1 ? plane : 0;
     const unsigned npen = axis == 1 ? (unsigned)pl->Nx * pl->Nz : plane;
-    const size_t smem = (size_t)(N + N * PT) * sizeof(cplx_t<T>);
+    const size_t smem = (size_t)(kTwLen<RA, RB> + N * PT) * sizeof(cplx_t<T>);
     dim3 gr((npen + PT - 1) / PT, nfields);
     ++pl->launches;
     if (DIR > 0)
@@ -890,13 +890,15 @@ void bloch_plan_destroy(bloch_plan* pl) {
     cudaFree(pl->d_Cf);
     cudaFree(pl->d_Cd);
     cudaFree(pl->d_Cpf);
-    cudaFree(pl->d_Cpd);
     cudaFree(pl->d_rf);
     cudaFree(pl->d_rd);
     for (int a = 0; a < 3; ++a) {
         cudaFree(pl->d_twf[a]);
         cudaFree(pl->d_twd[a]);
         cudaFree(pl->d_twx[a]);
+        cudaFree(pl->d_mtf[a]);
+        cudaFree(pl->d_mtd[a]);
+        cudaFree(pl->d_mtx[a]);
     }
     cudaFree(pl->d_Cx);
     cudaFree(pl->d_rx);
@@ -1069,19 +1071,14 @@ bloch_status bloch_plan_create(bloch_plan** out, const int32_t grid[3], const do
             rd[g] = rho[g] / (pl->rho_ref * (double)V);
             rf[g] = (float)rd[g];
         }
-        std::vector<double> pd((size_t)G * 21);
-        std::vector<float> pf((size_t)G * 21);
+        std::vector<float> pf((size_t)G * kCtabRow<float>, 0.0f);
         for (int g = 0; g < G; ++g) {
             int k = 0;
             for (int i = 0; i < 6; ++i)
-                for (int j = i; j < 6; ++j, ++k) {
-                    pd[(size_t)g * 21 + k] = cd[(size_t)g * 36 + i * 6 + j];
-                    pf[(size_t)g * 21 + k] = (float)pd[(size_t)g * 21 + k];
-                }
+                for (int j = i; j < 6; ++j, ++k)
+                    pf[(size_t)g * kCtabRow<float> + k] = (float)cd[(size_t)g * 36 + i * 6 + j];
         }
-        CK(dmalloc(&pl->d_Cpd, pd.size(), acc));
         CK(dmalloc(&pl->d_Cpf, pf.size(), acc));
-        CK(cudaMemcpy(pl->d_Cpd, pd.data(), sizeof(double) * pd.size(), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(pl->d_Cpf, pf.data(), sizeof(float) * pf.size(), cudaMemcpyHostToDevice));
         CK(dmalloc(&pl->d_Cd, cd.size(), acc));
         CK(dmalloc(&pl->d_Cf, cf.size(), acc));
@@ -1121,6 +1118,31 @@ bloch_status bloch_plan_create(bloch_plan** out, const int32_t grid[3], const do
         }
         CK(dmalloc(&pl->d_twx[a], (size_t)N, acc));
         CK(cudaMemcpy(pl->d_twx[a], tx.data(), sizeof(dfloat2) * N, cudaMemcpyHostToDevice));
+        // the same values in the order of the mixed-radix stages
+        pl->geo_f.ax[a] = pl->geo_d.ax[a] = make_axis(N, false);
+        pl->geo_x.ax[a] = make_axis(N, true);
+        auto order = [](const AxisPlan& p) {
+            std::vector<int> o;
+            for (int r = 0; r < p.r1; ++r)
+                for (int j = 0; j < p.N / p.r1; ++j) o.push_back(r * j);
+            for (int r = 0; r < p.r2 && p.r2 > 1; ++r)
+                for (int n3 = 0; n3 < p.r3; ++n3) o.push_back(r * n3 * p.r1);
+            return o;
+        };
+        std::vector<float2> mf;
+        std::vector<double2> md;
+        std::vector<dfloat2> mx;
+        for (int t : order(pl->geo_f.ax[a])) {
+            mf.push_back(tf[t]);
+            md.push_back(td[t]);
+        }
+        for (int t : order(pl->geo_x.ax[a])) mx.push_back(tx[t]);
+        CK(dmalloc(&pl->d_mtf[a], mf.size(), acc));
+        CK(dmalloc(&pl->d_mtd[a], md.size(), acc));
+        CK(dmalloc(&pl->d_mtx[a], mx.size(), acc));
+        CK(cudaMemcpy(pl->d_mtf[a], mf.data(), sizeof(float2) * mf.size(), cudaMemcpyHostToDevice));
+        CK(cudaMemcpy(pl->d_mtd[a], md.data(), sizeof(double2) * md.size(), cudaMemcpyHostToDevice));
+        CK(cudaMemcpy(pl->d_mtx[a], mx.data(), sizeof(dfloat2) * mx.size(), cudaMemcpyHostToDevice));
     }
     CK(dmalloc(&pl->d_nactive, 1, acc));
     CK(dmalloc(&pl->d_perr, 1, acc));
@@ -1151,10 +1173,6 @@ bloch_status bloch_plan_create(bloch_plan** out, const int32_t grid[3], const do
         gp->dx = make_fastdiv((unsigned)pl->Nx);
         gp->dy = make_fastdiv((unsigned)pl->Ny);
         gp->err = pl->d_perr;
-    }
-    for (int a = 0; a < 3; ++a) {
-        pl->geo_f.ax[a] = pl->geo_d.ax[a] = make_axis(grid[a], false);
-        pl->geo_x.ax[a] = make_axis(grid[a], true);
     }
     pl->pmax = pl->opt.tile_pmax > 0 ? pl->opt.tile_pmax : kDefaultPmax;
     pl->nblk_max = vec_blocks(pl, 1);

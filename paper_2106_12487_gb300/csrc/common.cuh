@@ -69,6 +69,17 @@ __device__ __forceinline__ dfloat ldg_t(const dfloat* p) {
     const float2 v = __ldg(reinterpret_cast<const float2*>(p));
     return dfloat(v.x, v.y);
 }
+// two neighbouring entries of a 16-byte aligned table of 8-byte reals
+__device__ __forceinline__ void ldg_pair(const double* p, double& a, double& b) {
+    const double2 v = __ldg(reinterpret_cast<const double2*>(p));
+    a = v.x;
+    b = v.y;
+}
+__device__ __forceinline__ void ldg_pair(const dfloat* p, dfloat& a, dfloat& b) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+    a = dfloat(v.x, v.y);
+    b = dfloat(v.z, v.w);
+}
 #endif
 
 template <typename T> struct CplxOf;

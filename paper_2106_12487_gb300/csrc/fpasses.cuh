@@ -32,6 +32,33 @@ __device__ __forceinline__ C twmul(C v, C w, int dir) {
     return cmul(v, w);
 }
 
+// Twiddles w_N^(r j) of a radix-R stage as rows j of R + 2 values in shared
+// memory: a task reads its row in 16-byte pieces (half the loads of single FP32
+// values), and the two spare values make the rows of neighbouring j start in
+// different banks.  The natural table read at r j met up to 8-way conflicts in
+// the x pass, whose time the shared-memory pipe sets.
+template <int R> constexpr int kTwRow = R + 2;
+template <int R, int J, typename C>
+__device__ __forceinline__ void tw_fill(C* rows, const C* __restrict__ tw, int tid, int nthr) {
+    for (int i = tid; i < R * J; i += nthr) rows[(i / R) * kTwRow<R> + i % R] = tw[(i / R) * (i % R)];
+}
+template <int R, int DIR, typename C>
+__device__ __forceinline__ void tw_apply(C (&v)[R], const C* row) {
+    if constexpr (sizeof(C) == 8) {
+#pragma unroll
+        for (int r = 0; r < R; r += 2) {
+            const float4 w = *reinterpret_cast<const float4*>(row + r);
+            if (r > 0) v[r] = twmul(v[r], mk(w.x, w.y), DIR);
+            v[r + 1] = twmul(v[r + 1], mk(w.z, w.w), DIR);
+        }
+    } else {
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[r] = twmul(v[r], row[r], DIR);
+    }
+}
+// table length, a multiple of 128 bytes of FP32 values
+template <int RA, int RB> constexpr int kTwLen = (RA * kTwRow<RB> + 15) / 16 * 16;
+
 // ------------------------------------- plain pass along y or z (in place ok)
 // A pencil's elements lie `inner` apart (Nx along y, Nx Ny along z); pencil pi
 // of npen starts at (pi / inner) outer + pi mod inner.  blockIdx.y = field
@@ -46,14 +73,14 @@ __global__ void __launch_bounds__(256) k_fpass_axis(const cplx_t<T>* in, cplx_t<
     constexpr int NT = 256;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* tw = reinterpret_cast<C*>(smem_raw);
-    C* buf = tw + N;
+    C* buf = tw + kTwLen<RA, RB>;
     const int tid = threadIdx.x;
     const unsigned pi0 = blockIdx.x * PT;
     if (sys_idle(g, (int)blockIdx.y / g.skip_ncomp)) return;
     const size_t off = (size_t)blockIdx.y * g.V;
     const C* src = in + off;
     C* dst = out + off;
-    for (int i = tid; i < N; i += NT) tw[i] = twa[i];
+    tw_fill<RB, RA>(tw, twa, tid, NT);
 #pragma unroll
     for (int t = tid; t < PT * RB; t += NT) {
         const int p = t % PT, j = t / PT;
@@ -79,8 +106,7 @@ __global__ void __launch_bounds__(256) k_fpass_axis(const cplx_t<T>* in, cplx_t<
         C v[RB];
 #pragma unroll
         for (int r = 0; r < RB; ++r) v[r] = buf[(j + r * RA) * PT + p];
-#pragma unroll
-        for (int r = 1; r < RB; ++r) v[r] = twmul(v[r], tw[r * j], DIR);
+        tw_apply<RB, DIR>(v, tw + j * kTwRow<RB>);
         RegDFT<RB, DIR, C>::run(v);
         const unsigned pi = pi0 + p;
         if (pi < npen) {
@@ -121,7 +147,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t zbar[2];
     C* tw = reinterpret_cast<C*>(smem_raw + smem_pad128(smem_raw));   // 128-byte aligned (TMA destinations)
-    C* stg = tw + N;          // 2 x NP staging
+    C* stg = tw + kTwLen<RA, RB>;   // 2 x NP staging
     C* bufA = stg + 2 * NP;   // NP
     C* bufB = bufA + NP;      // NP
     const int tid = threadIdx.x;
@@ -180,7 +206,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>
     };
     stage_in(2, 0);
     stage_in(0, 1);
-    for (int i = tid; i < N; i += NT) tw[i] = twz[i];
+    tw_fill<RB, RA>(tw, twz, tid, NT);
     const int p2 = tid % P, j2 = tid / P;
     const unsigned pi = pi0 + (p2 < np ? p2 : 0);
     const T qx = qxt[pi % (unsigned)g.Nx], qy = qyt[pi / (unsigned)g.Nx];
@@ -248,11 +274,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>
             a[r] = bufA[(j2 + r * RA) * P + p2];
             bb[r] = bufB[(j2 + r * RA) * P + p2];
         }
-#pragma unroll
-        for (int r = 1; r < RB; ++r) {
-            a[r] = twmul(a[r], tw[r * j2], +1);
-            bb[r] = twmul(bb[r], tw[r * j2], +1);
-        }
+        tw_apply<RB, +1>(a, tw + j2 * kTwRow<RB>);
+        tw_apply<RB, +1>(bb, tw + j2 * kTwRow<RB>);
         RegDFT<RB, +1, C>::run(a);
         RegDFT<RB, +1, C>::run(bb);
         if (k == 2) {          // z: g_zz; keep a_z
@@ -303,7 +326,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* _
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t zbar[4];
     C* tw = reinterpret_cast<C*>(smem_raw + smem_pad128(smem_raw));   // 128-byte aligned (TMA destinations)
-    C* stg = tw + N;             // NSTG x NP staging
+    C* stg = tw + kTwLen<RA, RB>;   // NSTG x NP staging
     C* xb = stg + NSTG * NP;     // (pair ? 2 : 1) x NP exchange
     const int tid = threadIdx.x;
     const int b = blockIdx.y;
@@ -361,7 +384,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* _
     };
 #pragma unroll
     for (int c = 0; c < NSTG; ++c) stage_in(c, c);
-    for (int i = tid; i < N; i += NT) tw[i] = twz[i];
+    tw_fill<RB, RA>(tw, twz, tid, NT);
     const int p2 = tid % P, j2 = tid / P;
     const unsigned pi = pi0 + (p2 < np ? p2 : 0);
     const T qv[2] = {qxt[pi % (unsigned)g.Nx], qyt[pi / (unsigned)g.Nx]};
@@ -376,8 +399,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* _
         C v[RB];
 #pragma unroll
         for (int r = 0; r < RB; ++r) v[r] = xc[(j2 + r * RA) * P + p2];
-#pragma unroll
-        for (int r = 1; r < RB; ++r) v[r] = twmul(v[r], tw[r * j2], -1);
+        tw_apply<RB, -1>(v, tw + j2 * kTwRow<RB>);
         RegDFT<RB, -1, C>::run(v);
         const int ca = c < 3 ? c : (c == 3 ? 1 : 0);
         const int cb = c < 3 ? c : (c == 5 ? 1 : 2);
@@ -466,9 +488,10 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* _
 // to spread the strided Stockham writes over the banks.
 __device__ __forceinline__ int xpad(int n) { return n + (n >> 4); }
 
-// sigma = C_g gamma at the element r of every component (packed symmetric
-// table, 21 per grain), one row of C_g at a time so that few coefficients
-// are live next to the six components held per element.
+// sigma = C_g gamma at the element r of every component, one row of C_g at a
+// time so that few coefficients are live next to the six components held per
+// element (16-byte table loads, six at a time, spill at 128 registers: 3.03
+// against 2.99 ms per K-apply of 18 systems at 128^3).
 template <typename T, typename C, int R>
 __device__ __forceinline__ void stress_at(C (&s)[6][R], int r, const T* __restrict__ Cg, T& energy) {
     C sig[6];
@@ -514,7 +537,8 @@ __device__ __forceinline__ void x_stress_single(cplx_t<T>* E, const int32_t* __r
     constexpr int P = 128 / RA;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* tw = reinterpret_cast<C*>(smem_raw);
-    C* stg = tw + N;          // 2 x P*LD staging (rows unpadded inside), reused by the forward exchange
+    C* tw1 = tw + kTwLen<RA, RB>;     // forward radix-RA stage
+    C* stg = tw1 + kTwLen<RB, RA>;    // 2 x P*LD staging (rows unpadded inside), reused by the forward exchange
     C* xb = stg + 2 * P * LD; // P*LD exchange of the inverse transform
     const int tid = threadIdx.x;
     const int b = blockIdx.y;
@@ -543,7 +567,8 @@ __device__ __forceinline__ void x_stress_single(cplx_t<T>* E, const int32_t* __r
     };
     prefetch(0, stg);
     prefetch(1, stg + P * LD);
-    for (int i = tid; i < N; i += 128) tw[i] = twx[i];
+    tw_fill<RB, RA>(tw, twx, tid, 128);
+    tw_fill<RA, RB>(tw1, twx, tid, 128);
     // stage-2 task of this thread
     const int j2 = tid % RA, p2 = tid / RA;
     const bool own = p2 < nr;
@@ -571,8 +596,7 @@ __device__ __forceinline__ void x_stress_single(cplx_t<T>* E, const int32_t* __r
         C v[RB];
 #pragma unroll
         for (int r = 0; r < RB; ++r) v[r] = xb[p2 * LD + xpad(j2 + r * RA)];
-#pragma unroll
-        for (int r = 1; r < RB; ++r) v[r] = twmul(v[r], tw[r * j2], +1);
+        tw_apply<RB, +1>(v, tw + j2 * kTwRow<RB>);
         RegDFT<RB, +1, C>::run(v);
 #pragma unroll
         for (int r = 0; r < RB; ++r) s[c][r] = v[r];
@@ -585,7 +609,7 @@ __device__ __forceinline__ void x_stress_single(cplx_t<T>* E, const int32_t* __r
 #pragma unroll
             for (int r = 0; r < RB; ++r) {
                 T e = T(0);
-                stress_at<T>(s, r, Cpk + (size_t)ids[(size_t)(r0 + p2) * N + j2 + r * RA] * 21, e);
+                stress_at<T>(s, r, Cpk + (size_t)ids[(size_t)(r0 + p2) * N + j2 + r * RA] * kCtabRow<T>, e);
                 energy += e;
             }
         }
@@ -612,8 +636,7 @@ __device__ __forceinline__ void x_stress_single(cplx_t<T>* E, const int32_t* __r
             C v[RA];
 #pragma unroll
             for (int r = 0; r < RA; ++r) v[r] = buf[p * LD + xpad(j + r * RB)];
-#pragma unroll
-            for (int r = 1; r < RA; ++r) v[r] = twmul(v[r], tw[r * j], -1);
+            tw_apply<RA, -1>(v, tw1 + j * kTwRow<RA>);
             RegDFT<RA, -1, C>::run(v);
             if (p < nr) {
 #pragma unroll
@@ -648,7 +671,8 @@ __device__ __forceinline__ void x_stress_paired(cplx_t<T>* E, const int32_t* __r
     static_assert(P * LI * sizeof(int32_t) <= P * LD * sizeof(C), "grain-id tile must fit a staging buffer");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* tw = reinterpret_cast<C*>(smem_raw);
-    C* stg = tw + N;          // 4 x P*LD: pair buffers (set 0: 0, 1; set 1: 2, 3)
+    C* tw1 = tw + kTwLen<RA, RB>;     // forward radix-RA stage
+    C* stg = tw1 + kTwLen<RB, RA>;    // 4 x P*LD: pair buffers (set 0: 0, 1; set 1: 2, 3)
     C* xb = stg + 4 * P * LD; // 2 x P*LD exchange of the inverse transform
     int32_t* sid = reinterpret_cast<int32_t*>(stg + 2 * P * LD);   // set 1, buffer 0, once free
     const int tid = threadIdx.x;
@@ -674,7 +698,8 @@ __device__ __forceinline__ void x_stress_paired(cplx_t<T>* E, const int32_t* __r
     prefetch(2, stg + 2 * P * LD);
     prefetch(3, stg + 3 * P * LD);
     cp_async_commit();
-    for (int i = tid; i < N; i += 128) tw[i] = twx[i];
+    tw_fill<RB, RA>(tw, twx, tid, 128);
+    tw_fill<RA, RB>(tw1, twx, tid, 128);
     const int half = tid >> 6;              // radix-RA stage: component 2m + half
     const int j1 = (tid & 63) % RB, p1 = (tid & 63) / RB;
     const int j2 = tid % RA, p2 = tid / RA; // radix-RB stage and the stress: one task per thread
@@ -713,8 +738,7 @@ __device__ __forceinline__ void x_stress_paired(cplx_t<T>* E, const int32_t* __r
             C v[RB];
 #pragma unroll
             for (int r = 0; r < RB; ++r) v[r] = xb[h * P * LD + p2 * LD + xpad(j2 + r * RA)];
-#pragma unroll
-            for (int r = 1; r < RB; ++r) v[r] = twmul(v[r], tw[r * j2], +1);
+            tw_apply<RB, +1>(v, tw + j2 * kTwRow<RB>);
             RegDFT<RB, +1, C>::run(v);
 #pragma unroll
             for (int r = 0; r < RB; ++r) s[2 * m + h][r] = v[r];
@@ -729,7 +753,7 @@ __device__ __forceinline__ void x_stress_paired(cplx_t<T>* E, const int32_t* __r
 #pragma unroll
             for (int r = 0; r < RB; ++r) {
                 T e = T(0);
-                stress_at<T>(s, r, Cpk + (size_t)sid[p2 * LI + j2 + r * RA] * 21, e);
+                stress_at<T>(s, r, Cpk + (size_t)sid[p2 * LI + j2 + r * RA] * kCtabRow<T>, e);
                 energy += e;
             }
         }
@@ -756,8 +780,7 @@ __device__ __forceinline__ void x_stress_paired(cplx_t<T>* E, const int32_t* __r
             const C* bh = bufs + half * P * LD + p1 * LD;
 #pragma unroll
             for (int r = 0; r < RA; ++r) v[r] = bh[xpad(j1 + r * RB)];
-#pragma unroll
-            for (int r = 1; r < RA; ++r) v[r] = twmul(v[r], tw[r * j1], -1);
+            tw_apply<RA, -1>(v, tw1 + j1 * kTwRow<RA>);
             RegDFT<RA, -1, C>::run(v);
             if (p1 < nr) {
                 C* dst = Eb + (size_t)(2 * m + half) * g.V + (size_t)(r0 + p1) * N + j1;
@@ -771,19 +794,19 @@ __device__ __forceinline__ void x_stress_paired(cplx_t<T>* E, const int32_t* __r
 // Shared memory of k_fpass_z_strain<T, RA, RB, NT> and k_fpass_z_div<T, RA, RB, NT> (bytes).
 template <typename T, int RA, int RB, int NT>
 constexpr size_t fpass_z1_smem() {
-    return (size_t)(RA * RB + 4 * RA * RB * (NT / RA)) * sizeof(cplx_t<T>) + kSmemAlignSlack;
+    return (size_t)(kTwLen<RA, RB> + 4 * RA * RB * (NT / RA)) * sizeof(cplx_t<T>) + kSmemAlignSlack;
 }
 template <typename T, int RA, int RB, int NT>
 constexpr size_t fpass_z5_smem() {
     constexpr int P = NT / RA, NP = RA * RB * P;
-    return (size_t)(RA * RB + (2 * P * RB == NT ? 6 : 3) * NP) * sizeof(cplx_t<T>) + kSmemAlignSlack;
+    return (size_t)(kTwLen<RA, RB> + (2 * P * RB == NT ? 6 : 3) * NP) * sizeof(cplx_t<T>) + kSmemAlignSlack;
 }
 
 // Shared memory of k_fpass_x_stress<T, RA, RB> (bytes).
 template <typename T, int RA, int RB>
 constexpr size_t fpass_x_smem() {
     constexpr int N = RA * RB, LD = N + N / 16, P = 128 / RA;
-    return (size_t)(N + (P * RB == 64 ? 6 : 3) * P * LD) * sizeof(cplx_t<T>);
+    return (size_t)(kTwLen<RA, RB> + kTwLen<RB, RA> + (P * RB == 64 ? 6 : 3) * P * LD) * sizeof(cplx_t<T>);
 }
 
 // With dpart != nullptr the CTA also forms the strain energy sum over its

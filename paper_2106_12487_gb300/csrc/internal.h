@@ -104,14 +104,17 @@ struct bloch_plan {
     int32_t* d_ids = nullptr;
     float* d_Cf = nullptr;
     double* d_Cd = nullptr;
-    float* d_Cpf = nullptr;        // G x 21 packed upper triangle (fast x pass)
-    double* d_Cpd = nullptr;
+    float* d_Cpf = nullptr;        // G x 24: packed upper triangles (FP32 x passes)
     float* d_rf = nullptr;
     double* d_rd = nullptr;
     float2* d_twf[3] = {nullptr, nullptr, nullptr};
     double2* d_twd[3] = {nullptr, nullptr, nullptr};
     // float-float copies (the FP64-class check of the FP32 form on the FP32 pipes)
     dfloat2* d_twx[3] = {nullptr, nullptr, nullptr};
+    // twiddles in the order of the mixed-radix stages (twtab_len)
+    float2* d_mtf[3] = {nullptr, nullptr, nullptr};
+    double2* d_mtd[3] = {nullptr, nullptr, nullptr};
+    dfloat2* d_mtx[3] = {nullptr, nullptr, nullptr};
     dfloat* d_Cx = nullptr;
     dfloat* d_rx = nullptr;
     int* d_nactive = nullptr;

@@ -65,9 +65,54 @@ __device__ __forceinline__ bool sys_idle(const Geo& g, int b) {
     return g.skip != nullptr && g.skip[(size_t)b * g.skip_stride] == 0;
 }
 
-// Index of C_ij (any order) in the packed upper triangle of a symmetric 6x6.
+// Stiffness table of a grain.  FP32: the packed upper triangle (21 values,
+// sym6), padded to 24 so that six 16-byte loads bring it; as single values its
+// loads were half of the x passes' L1 wavefronts.  Wider types: the full 6 x 6
+// table, read in 16-byte pairs.
 __host__ __device__ constexpr int sym6(int i, int j) {
     return i <= j ? i * 6 - i * (i - 1) / 2 + (j - i) : j * 6 - j * (j - 1) / 2 + (i - j);
+}
+template <typename T> constexpr int kCtabRow = sizeof(T) == 4 ? 24 : 36;
+
+// sigma = C_g gamma at one point
+template <typename T, typename C>
+__device__ __forceinline__ void stress_of(const C (&gam)[6], C (&sig)[6], const T* __restrict__ Cg) {
+    if constexpr (std::is_same<T, float>::value) {
+        float c[24];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(Cg) + k);
+            c[4 * k] = v.x;
+            c[4 * k + 1] = v.y;
+            c[4 * k + 2] = v.z;
+            c[4 * k + 3] = v.w;
+        }
+#pragma unroll
+        for (int i = 0; i < 6; ++i) sig[i] = cscale(gam[i], c[sym6(i, i)]);
+#pragma unroll
+        for (int i = 0; i < 6; ++i)
+#pragma unroll
+            for (int j = i + 1; j < 6; ++j) {
+                const float cij = c[sym6(i, j)];
+                sig[i] = mk(fma(cij, gam[j].x, sig[i].x), fma(cij, gam[j].y, sig[i].y));
+                sig[j] = mk(fma(cij, gam[i].x, sig[j].x), fma(cij, gam[i].y, sig[j].y));
+            }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            T sr = 0, si = 0;
+#pragma unroll
+            for (int j = 0; j < 6; j += 2) {
+                T c0, c1;
+                ldg_pair(Cg + i * 6 + j, c0, c1);
+                sr = fma(c0, gam[j].x, sr);
+                si = fma(c0, gam[j].y, si);
+                sr = fma(c1, gam[j + 1].x, sr);
+                si = fma(c1, gam[j + 1].y, si);
+            }
+            sig[i] = mk(sr, si);
+        }
+    }
 }
 
 __host__ __device__ __forceinline__ int pad_even(int n) { return (n + 1) & ~1; }
@@ -79,24 +124,34 @@ __host__ __device__ __forceinline__ int pad_even(int n) { return (n + 1) & ~1; }
 __host__ __device__ __forceinline__ int xgroup(const AxisPlan& a) { return a.r3 + ((a.r3 & 1) ^ 1); }
 __host__ __device__ __forceinline__ int xrow(const AxisPlan& a) { return (a.r1 * a.r2 * xgroup(a)) | 1; }
 
-// CTAs per SM the pass kernels leave registers for
-template <typename T> constexpr int kPassCtas = sizeof(T) == 4 ? 3 : 2;
+// CTAs per SM the pass kernels leave registers for.  FP32 kernels come in two
+// forms: with radices up to 12 four CTAs share an SM (64 registers), with the
+// wide ones (14 to 16, which would spill) three.  120 x 100 x 84, 6 systems:
+// 735 us with three, 680 with four; 256^3 (16 x 16): 3.79 ms with three, 4.27
+// with four.
+template <typename T, bool WIDE> constexpr int kPassCtas = sizeof(T) != 4 ? 2 : WIDE ? 3 : 4;
 
 // f(std::integral_constant<int, R>) for the run-time radix R.  Float-float
 // leaves out the radices whose code is longest for what they save (compile time).
-template <typename T, typename F>
+template <typename T, bool WIDE, typename F>
 __device__ __forceinline__ void with_radix(int R, F&& f) {
     switch (R) {
 #define BLOCH_RADIX(r) \
     case r: f(std::integral_constant<int, r>{}); break;
         BLOCH_RADIX(1) BLOCH_RADIX(2) BLOCH_RADIX(3) BLOCH_RADIX(4) BLOCH_RADIX(5) BLOCH_RADIX(6) BLOCH_RADIX(7)
-        BLOCH_RADIX(8) BLOCH_RADIX(9) BLOCH_RADIX(10) BLOCH_RADIX(15) BLOCH_RADIX(16)
+        BLOCH_RADIX(8) BLOCH_RADIX(9) BLOCH_RADIX(10)
         default: break;
     }
     if constexpr (!std::is_same<T, dfloat>::value) {
+        if (R == 12) f(std::integral_constant<int, 12>{});
+    }
+    if constexpr (WIDE) {
         switch (R) {
-            BLOCH_RADIX(12) BLOCH_RADIX(14)
+            BLOCH_RADIX(15) BLOCH_RADIX(16)
             default: break;
+        }
+        if constexpr (!std::is_same<T, dfloat>::value) {
+            if (R == 14) f(std::integral_constant<int, 14>{});
         }
     }
 }
@@ -110,6 +165,13 @@ __device__ __forceinline__ void with_mid_radix(int R, F&& f) {
 }
 
 template <typename C> using real_t = decltype(C::x);
+
+// Twiddle table of an axis, in the order the stages read it: w_N^(r j) at
+// r (N / r1) + j for the first stage's butterflies j < N / r1, then, with a
+// middle stage, w_(r2 r3)^(r n3) at N + r r3 + n3.  Neighbouring threads of the
+// x passes take neighbouring j: the natural order w_N^t, read at r j, cost up to
+// r-way bank conflicts and two thirds of the x pass's shared-memory wavefronts.
+__host__ __device__ __forceinline__ int twtab_len(const AxisPlan& a) { return a.N + (a.r2 > 1 ? a.r2 * a.r3 : 0); }
 
 template <int DIR, typename C>
 __device__ __forceinline__ C twiddled(C v, C w) {
@@ -145,16 +207,16 @@ __device__ __forceinline__ void pf_mid(C* buf, int nbuf, const AxisPlan& a, int 
             RegDFT<R, DIR, C>::run(v);
             s[0] = v[0];
 #pragma unroll
-            for (int r = 1; r < R; ++r) s[(r * r3) << lp] = twiddled<DIR>(v[r], tw[r * n3 * a.r1]);
+            for (int r = 1; r < R; ++r) s[(r * r3) << lp] = twiddled<DIR>(v[r], tw[a.N + r * a.r3 + n3]);
         }
     });
 }
 
 // last stage of nbuf buffers, in place
-template <int DIR, typename C>
+template <int DIR, bool WIDE, typename C>
 __device__ __forceinline__ void pf_last(C* buf, int nbuf, const AxisPlan& a, int lp, int tid, int nthr) {
     const int P1 = (1 << lp) - 1;
-    with_radix<real_t<C>>(a.r3, [&](auto rc) {
+    with_radix<real_t<C>, WIDE>(a.r3, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         if constexpr (R > 1) {
             // the buffers are contiguous and N is a multiple of R: one run of butterflies over all of them
@@ -178,8 +240,8 @@ __device__ __forceinline__ void pf_last(C* buf, int nbuf, const AxisPlan& a, int
 //   g_xx = q_x a_x, g_yy = q_y a_y, g_zz = b_z, g_yz = q_y a_z + b_y,
 //   g_xz = q_x a_z + b_x, g_xy = q_y a_x + q_x a_y
 // (q_x and q_y are constant on a z pencil).
-template <typename T>
-__global__ void __launch_bounds__(256, kPassCtas<T>)
+template <typename T, bool WIDE>
+__global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     k_pass_z_strain(const cplx_t<T>* __restrict__ U, cplx_t<T>* __restrict__ E, const T* __restrict__ qtab,
                     const cplx_t<T>* __restrict__ twz, Geo g, int lp) {
     using C = cplx_t<T>;
@@ -187,7 +249,8 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
     const AxisPlan& a = g.ax[2];
     const int N = a.N, NP = N << lp, P1 = (1 << lp) - 1;
     C* tw = reinterpret_cast<C*>(smem_raw);
-    C* buf = tw + pad_even(N);
+    const int ntw = twtab_len(a);
+    C* buf = tw + pad_even(ntw);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int b = blockIdx.y;
     if (sys_idle(g, b)) return;
@@ -199,9 +262,9 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
     const T* qx = qtab + (size_t)b * (g.Nx + g.Ny + g.Nz);
     const T* qy = qx + g.Nx;
     const T* qz = qy + g.Ny;
-    for (int i = tid; i < N; i += nthr) tw[i] = twz[i];
+    for (int i = tid; i < ntw; i += nthr) tw[i] = twz[i];
     __syncthreads();
-    with_radix<real_t<C>>(a.r1, [&](auto rc) {
+    with_radix<real_t<C>, WIDE>(a.r1, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         const int M = N / R, per = M << lp;
         for (int t = tid; t < 3 * per; t += nthr) {
@@ -227,7 +290,7 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
                 s[NP] = w[0];
 #pragma unroll
                 for (int r = 1; r < R; ++r) {
-                    const C f = tw[r * j];
+                    const C f = tw[r * M + j];
                     s[(r * M) << lp] = twiddled<+1>(v[r], f);
                     s[NP + ((r * M) << lp)] = twiddled<+1>(w[r], f);
                 }
@@ -242,7 +305,7 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
                     RegDFT<R, +1, C>::run(v);
                     s[0] = v[0];
 #pragma unroll
-                    for (int r = 1; r < R; ++r) s[(r * M) << lp] = twiddled<+1>(v[r], tw[r * j]);
+                    for (int r = 1; r < R; ++r) s[(r * M) << lp] = twiddled<+1>(v[r], tw[r * M + j]);
                 }
             }
         }
@@ -252,7 +315,7 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
         pf_mid<+1>(buf, 6, a, lp, tw, tid, nthr);
         __syncthreads();
     }
-    pf_last<+1>(buf, 6, a, lp, tid, nthr);
+    pf_last<+1, WIDE>(buf, 6, a, lp, tid, nthr);
     __syncthreads();
     for (int t = tid; t < NP; t += nthr) {
         const int p = t & P1, k = t >> lp;
@@ -273,15 +336,16 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
 
 // ------------------------------------------------- plain FFT pass along y or z
 // blockIdx.y enumerates (batch, component) pairs: offset blockIdx.y * V.
-template <typename T, int DIR, int AXIS>
-__global__ void __launch_bounds__(256, kPassCtas<T>)
+template <typename T, int DIR, int AXIS, bool WIDE>
+__global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     k_pass_axis(const cplx_t<T>* in, cplx_t<T>* out, const cplx_t<T>* __restrict__ twa, Geo g, int lp, T out_scale) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const AxisPlan& a = g.ax[AXIS];
     const int N = a.N, P1 = (1 << lp) - 1;
     C* tw = reinterpret_cast<C*>(smem_raw);
-    C* buf = tw + pad_even(N);
+    const int ntw = twtab_len(a);
+    C* buf = tw + pad_even(ntw);
     const int tid = threadIdx.x, nthr = blockDim.x;
     if (sys_idle(g, (int)blockIdx.y / g.skip_ncomp)) return;
     const unsigned nx = (unsigned)g.Nx, plane = nx * (unsigned)g.Ny;
@@ -296,9 +360,9 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
         const unsigned z = fdiv(pi, g.dx);
         return (size_t)z * plane + (pi - z * nx);
     };
-    for (int i = tid; i < N; i += nthr) tw[i] = twa[i];
+    for (int i = tid; i < ntw; i += nthr) tw[i] = twa[i];
     __syncthreads();
-    with_radix<real_t<C>>(a.r1, [&](auto rc) {
+    with_radix<real_t<C>, WIDE>(a.r1, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         const int M = N / R;
         for (int t = tid; t < (M << lp); t += nthr) {
@@ -311,7 +375,7 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
             RegDFT<R, DIR, C>::run(v);
             buf[t] = v[0];
 #pragma unroll
-            for (int r = 1; r < R; ++r) buf[((r * M) << lp) + t] = twiddled<DIR>(v[r], tw[r * j]);
+            for (int r = 1; r < R; ++r) buf[((r * M) << lp) + t] = twiddled<DIR>(v[r], tw[r * M + j]);
         }
     });
     __syncthreads();
@@ -319,7 +383,7 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
         pf_mid<DIR>(buf, 1, a, lp, tw, tid, nthr);
         __syncthreads();
     }
-    with_radix<real_t<C>>(a.r3, [&](auto rc) {
+    with_radix<real_t<C>, WIDE>(a.r3, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         const int M = N / R;
         for (int t = tid; t < (M << lp); t += nthr) {
@@ -340,8 +404,8 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
 }
 
 // ---------------------------------------------------------------- pass 5
-template <typename T>
-__global__ void __launch_bounds__(256, kPassCtas<T>)
+template <typename T, bool WIDE>
+__global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     k_pass_z_div(const cplx_t<T>* __restrict__ E, cplx_t<T>* __restrict__ out, const T* __restrict__ qtab,
                  const cplx_t<T>* __restrict__ twz, Geo g, int lp, T out_scale) {
     using C = cplx_t<T>;
@@ -349,7 +413,8 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
     const AxisPlan& a = g.ax[2];
     const int N = a.N, NP = N << lp, P1 = (1 << lp) - 1;
     C* tw = reinterpret_cast<C*>(smem_raw);
-    C* buf = tw + pad_even(N);
+    const int ntw = twtab_len(a);
+    C* buf = tw + pad_even(ntw);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int b = blockIdx.y;
     if (sys_idle(g, b)) return;
@@ -361,9 +426,9 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
     const T* qx = qtab + (size_t)b * (g.Nx + g.Ny + g.Nz);
     const T* qy = qx + g.Nx;
     const T* qz = qy + g.Ny;
-    for (int i = tid; i < N; i += nthr) tw[i] = twz[i];
+    for (int i = tid; i < ntw; i += nthr) tw[i] = twz[i];
     __syncthreads();
-    with_radix<real_t<C>>(a.r1, [&](auto rc) {
+    with_radix<real_t<C>, WIDE>(a.r1, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         const int M = N / R, per = M << lp;
         for (int t = tid; t < 6 * per; t += nthr) {
@@ -377,7 +442,7 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
             RegDFT<R, -1, C>::run(v);
             s[0] = v[0];
 #pragma unroll
-            for (int r = 1; r < R; ++r) s[(r * M) << lp] = twiddled<-1>(v[r], tw[r * j]);
+            for (int r = 1; r < R; ++r) s[(r * M) << lp] = twiddled<-1>(v[r], tw[r * M + j]);
         }
     });
     __syncthreads();
@@ -385,7 +450,7 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
         pf_mid<-1>(buf, 6, a, lp, tw, tid, nthr);
         __syncthreads();
     }
-    pf_last<-1>(buf, 6, a, lp, tid, nthr);
+    pf_last<-1, WIDE>(buf, 6, a, lp, tid, nthr);
     __syncthreads();
     for (int t = tid; t < NP; t += nthr) {
         const int p = t & P1, k = t >> lp;
@@ -405,11 +470,11 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
 // Element (component c, row p, slot n) at (c P + p) xrow + (n / r3) xgroup + n mod r3.
 
 // stage 1 (decimation in frequency) of ncomp components of P rows, from HBM
-template <int DIR, typename C>
+template <int DIR, bool WIDE, typename C>
 __device__ __forceinline__ void lf_first(const C* Wb, long long V, C* buf, int ncomp, const AxisPlan& a, int P, int nr,
                                          unsigned r0, const C* tw, int tid, int nthr) {
     const int ld = xrow(a), gr = xgroup(a);
-    with_radix<real_t<C>>(a.r1, [&](auto rc) {
+    with_radix<real_t<C>, WIDE>(a.r1, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         const int M = a.N / R, Mg = a.r2 * gr;
         for (int t = tid; t < ncomp * P * M; t += nthr) {
@@ -423,7 +488,7 @@ __device__ __forceinline__ void lf_first(const C* Wb, long long V, C* buf, int n
             RegDFT<R, DIR, C>::run(v);
             s[0] = v[0];
 #pragma unroll
-            for (int r = 1; r < R; ++r) s[r * Mg] = twiddled<DIR>(v[r], tw[r * j]);
+            for (int r = 1; r < R; ++r) s[r * Mg] = twiddled<DIR>(v[r], tw[r * M + j]);
         }
     });
 }
@@ -443,12 +508,12 @@ __device__ __forceinline__ void lf_mid(C* buf, int nrows, const AxisPlan& a, con
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 v[r] = s[r * gr];
-                if (!FREQ && r > 0) v[r] = twiddled<DIR>(v[r], tw[r * n3 * a.r1]);
+                if (!FREQ && r > 0) v[r] = twiddled<DIR>(v[r], tw[a.N + r * a.r3 + n3]);
             }
             RegDFT<R, DIR, C>::run(v);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                if (FREQ && r > 0) v[r] = twiddled<DIR>(v[r], tw[r * n3 * a.r1]);
+                if (FREQ && r > 0) v[r] = twiddled<DIR>(v[r], tw[a.N + r * a.r3 + n3]);
                 s[r * gr] = v[r];
             }
         }
@@ -457,10 +522,10 @@ __device__ __forceinline__ void lf_mid(C* buf, int nrows, const AxisPlan& a, con
 
 // butterflies over the last digit, in place: the last stage of the inverse
 // and the first of the mirrored forward transform
-template <int DIR, typename C>
+template <int DIR, bool WIDE, typename C>
 __device__ __forceinline__ void lf_last(C* buf, int nrows, const AxisPlan& a, int tid, int nthr) {
     const int ld = xrow(a), gr = xgroup(a);
-    with_radix<real_t<C>>(a.r3, [&](auto rc) {
+    with_radix<real_t<C>, WIDE>(a.r3, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         if constexpr (R > 1) {
             const int M = a.N / R;
@@ -479,11 +544,11 @@ __device__ __forceinline__ void lf_last(C* buf, int nrows, const AxisPlan& a, in
 }
 
 // last stage of the mirrored forward transform, to HBM
-template <int DIR, typename C>
+template <int DIR, bool WIDE, typename C>
 __device__ __forceinline__ void lf_store(C* Wb, long long V, const C* buf, int ncomp, const AxisPlan& a, int P, int nr,
                                          unsigned r0, const C* tw, int tid, int nthr) {
     const int ld = xrow(a), gr = xgroup(a);
-    with_radix<real_t<C>>(a.r1, [&](auto rc) {
+    with_radix<real_t<C>, WIDE>(a.r1, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         const int M = a.N / R, Mg = a.r2 * gr;
         for (int t = tid; t < ncomp * P * M; t += nthr) {
@@ -495,7 +560,7 @@ __device__ __forceinline__ void lf_store(C* Wb, long long V, const C* buf, int n
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 v[r] = s[r * Mg];
-                if (r > 0) v[r] = twiddled<DIR>(v[r], tw[r * j]);
+                if (r > 0) v[r] = twiddled<DIR>(v[r], tw[r * M + j]);
             }
             RegDFT<R, DIR, C>::run(v);
             C* d = Wb + (size_t)c * V + (size_t)(r0 + p) * a.N + j;
@@ -505,37 +570,18 @@ __device__ __forceinline__ void lf_store(C* Wb, long long V, const C* buf, int n
     });
 }
 
-// Stiffness C_ij of a grain: FP32 keeps the packed upper triangle (21 per
-// grain), the wider types the full 6 x 6 table.
-template <typename T> constexpr int kCtabRow = sizeof(T) == 4 ? 21 : 36;
-template <typename T>
-__device__ __forceinline__ T ctab_at(const T* Cg, int i, int j) {
-    return ldg_t(Cg + (sizeof(T) == 4 ? sym6(i, j) : i * 6 + j));
-}
-
-// natural index k1 + r1 k2 + r1 r2 k3 of slot n = q r3 + k3, q = k1 r2 + k2
-__device__ __forceinline__ int index_of(int n, int q, const AxisPlan& a) {
-    const int k1 = (int)fdiv((unsigned)q, a.d2);
-    return k1 + a.r1 * ((q - k1 * a.r2) + a.r2 * (n - q * a.r3));
-}
-
 // sigma = C_g gamma in place on the six components s[c cs]; adds conj(gamma) sigma
 template <typename T, typename C>
 __device__ __forceinline__ void stress_smem(C* s, int cs, const T* __restrict__ Cg, T& energy) {
-    C gam[6];
+    C gam[6], sig[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) gam[c] = s[c * cs];
+    stress_of<T>(gam, sig, Cg);
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-        T sr = 0, si = 0;
-#pragma unroll
-        for (int j = 0; j < 6; ++j) {
-            const T cij = ctab_at<T>(Cg, i, j);
-            sr = fma(cij, gam[j].x, sr);
-            si = fma(cij, gam[j].y, si);
-        }
-        s[i * cs] = mk(sr, si);
-        if constexpr (!std::is_same<T, dfloat>::value) energy = fma(gam[i].x, sr, fma(gam[i].y, si, energy));
+        s[i * cs] = sig[i];
+        if constexpr (!std::is_same<T, dfloat>::value)
+            energy = fma(gam[i].x, sig[i].x, fma(gam[i].y, sig[i].y, energy));
     }
 }
 
@@ -560,12 +606,13 @@ __device__ __forceinline__ void energy_out(T e, double2* dst) {
 // pointwise product in real space, forward FFT, in place.
 //   NC = 6: strains to stresses with the per-grain table (pass 3)
 //   NC = 3: displacements times the per-grain scalar table (mass operator)
-// The pointwise step walks the slots in order (no bank conflicts) and gathers
-// the grain ids of a row, which its first touch brings to L1.  With dpart
+// The pointwise step walks a row in real-space order, so a warp meets one or
+// two grains and reads their tables once; the odd length of the slot groups
+// keeps its strided slots free of bank conflicts.  With dpart
 // (NC = 6) the CTA writes its share of the strain energy sum conj(gamma) sigma
 // = (u, A_k u) to dpart[b gridDim.x + blockIdx.x] (as k_fpass_x_stress).
-template <typename T, int NC>
-__global__ void __launch_bounds__(256, kPassCtas<T>)
+template <typename T, int NC, bool WIDE>
+__global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     k_pass_x_grain(cplx_t<T>* W, const int32_t* __restrict__ ids, const T* __restrict__ tab,
                    const cplx_t<T>* __restrict__ twx, Geo g, int P, double2* __restrict__ dpart) {
     using C = cplx_t<T>;
@@ -574,7 +621,8 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
     const int N = a.N, ld = xrow(a), gr = xgroup(a);
     T energy = T(0);
     C* tw = reinterpret_cast<C*>(smem_raw);
-    C* buf = tw + pad_even(N);
+    const int ntw = twtab_len(a);
+    C* buf = tw + pad_even(ntw);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int b = blockIdx.y;
     if (sys_idle(g, b)) return;
@@ -582,21 +630,21 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
     const unsigned r0 = blockIdx.x * (unsigned)P;
     const int nr = (int)min((unsigned)P, rows - r0);
     C* Wb = W + (size_t)b * NC * g.V;
-    for (int i = tid; i < N; i += nthr) tw[i] = twx[i];
+    for (int i = tid; i < ntw; i += nthr) tw[i] = twx[i];
     __syncthreads();
-    lf_first<+1>(Wb, g.V, buf, NC, a, P, nr, r0, tw, tid, nthr);
+    lf_first<+1, WIDE>(Wb, g.V, buf, NC, a, P, nr, r0, tw, tid, nthr);
     __syncthreads();
     if (a.r2 > 1) {
         lf_mid<+1, true>(buf, NC * P, a, tw, tid, nthr);
         __syncthreads();
     }
-    lf_last<+1>(buf, NC * P, a, tid, nthr);
+    lf_last<+1, WIDE>(buf, NC * P, a, tid, nthr);
     __syncthreads();
     for (int t = tid; t < nr * N; t += nthr) {
-        const int p = (int)fdiv((unsigned)t, g.dx), n = t - p * N;
-        const int q = (int)fdiv((unsigned)n, a.d3);
-        const int gid = ids[(size_t)(r0 + p) * N + index_of(n, q, a)];
-        C* s = buf + p * ld + n + q * (gr - a.r3);
+        const int p = (int)fdiv((unsigned)t, g.dx), k = t - p * N;
+        const int gid = ids[(size_t)(r0 + p) * N + k];
+        const int q = (int)fdiv((unsigned)k, a.d1), k3 = (int)fdiv((unsigned)q, a.d2);
+        C* s = buf + p * ld + ((k - q * a.r1) * a.r2 + (q - k3 * a.r2)) * gr + k3;   // slot (k1, k2, k3)
         const int cs = P * ld;
         if constexpr (NC == 6) {
             stress_smem<T>(s, cs, tab + (size_t)gid * kCtabRow<T>, energy);
@@ -608,13 +656,13 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
     }
     if (NC == 6 && dpart) energy_out(energy, dpart + (size_t)b * gridDim.x + blockIdx.x);
     __syncthreads();
-    lf_last<-1>(buf, NC * P, a, tid, nthr);
+    lf_last<-1, WIDE>(buf, NC * P, a, tid, nthr);
     __syncthreads();
     if (a.r2 > 1) {
         lf_mid<-1, false>(buf, NC * P, a, tw, tid, nthr);
         __syncthreads();
     }
-    lf_store<-1>(Wb, g.V, buf, NC, a, P, nr, r0, tw, tid, nthr);
+    lf_store<-1, WIDE>(Wb, g.V, buf, NC, a, P, nr, r0, tw, tid, nthr);
 }
 
 // ------------------------------------------- plain transform along x
@@ -623,8 +671,8 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
 // rows per CTA, blockIdx.y = field.  With ph the fields of system b (`per`
 // fields each) are also multiplied by the complex factor ph[b], and the second
 // of two fields by 1/2 (the shears of a strain field: engineering to tensor).
-template <typename T, int DIR>
-__global__ void __launch_bounds__(256, kPassCtas<T>)
+template <typename T, int DIR, bool WIDE>
+__global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     k_pass_x(cplx_t<T>* W, const cplx_t<T>* __restrict__ twx, Geo g, int P, T out_scale,
              const double2* __restrict__ ph, int per) {
     using C = cplx_t<T>;
@@ -632,7 +680,8 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
     const AxisPlan& a = g.ax[0];
     const int N = a.N, ld = xrow(a), gr = xgroup(a);
     C* tw = reinterpret_cast<C*>(smem_raw);
-    C* buf = tw + pad_even(N);
+    const int ntw = twtab_len(a);
+    C* buf = tw + pad_even(ntw);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int b = blockIdx.y;
     if (sys_idle(g, b)) return;
@@ -640,15 +689,15 @@ __global__ void __launch_bounds__(256, kPassCtas<T>)
     const unsigned r0 = blockIdx.x * (unsigned)P;
     const int nr = (int)min((unsigned)P, rows - r0);
     C* Wb = W + (size_t)b * 3 * g.V;
-    for (int i = tid; i < N; i += nthr) tw[i] = twx[i];
+    for (int i = tid; i < ntw; i += nthr) tw[i] = twx[i];
     __syncthreads();
-    lf_first<DIR>(Wb, g.V, buf, 3, a, P, nr, r0, tw, tid, nthr);
+    lf_first<DIR, WIDE>(Wb, g.V, buf, 3, a, P, nr, r0, tw, tid, nthr);
     __syncthreads();
     if (a.r2 > 1) {
         lf_mid<DIR, true>(buf, 3 * P, a, tw, tid, nthr);
         __syncthreads();
     }
-    lf_last<DIR>(buf, 3 * P, a, tid, nthr);
+    lf_last<DIR, WIDE>(buf, 3 * P, a, tid, nthr);
     __syncthreads();
     if (per == 2 && (b & 1)) out_scale = out_scale * T(0.5);
     const C f = ph ? mk(T(ph[b / per].x) * out_scale, T(ph[b / per].y) * out_scale) : mk(out_scale, T(0));
