@@ -154,6 +154,7 @@ bloch_status ensure_ws(bloch_plan* pl, int nb) {
     Workspace<T>& w = ws_of<T>(pl);
     if (nb <= w.cap) return BLOCH_OK;
     cudaStreamSynchronize(pl->stream);
+    drop_pcg_graphs(pl);   // they hold the buffers' addresses
     const int S = pl->Nx + pl->Ny + pl->Nz;
     if (w.E) pl->device_bytes -= (size_t)w.cap * (6 * pl->V * sizeof(cplx_t<T>) + S * sizeof(T) + 3 * sizeof(double));
     cudaFree(w.E);
@@ -177,9 +178,14 @@ bloch_status ensure_cg(bloch_plan* pl, int nb) {
     Workspace<T>& w = ws_of<T>(pl);
     if (nb <= w.cg_cap) return BLOCH_OK;
     cudaStreamSynchronize(pl->stream);
+    drop_pcg_graphs(pl);   // they hold the buffers' addresses
     const size_t vec = (size_t)3 * pl->V * sizeof(cplx_t<T>);
-    if (w.r) pl->device_bytes -= (size_t)w.cg_cap * (3 * vec + pl->nblk_max * (3 * sizeof(double) + sizeof(double2)) +
-                                                     sizeof(double2) + sizeof(CGSys) + w.zblk * sizeof(double2));
+    // (r, z), (r, r) partials: one slot per block of the vector kernels or CTA of
+    // the divergence pass (at most one per z pencil)
+    const int pblk = std::max(pl->nblk_max, pl->Nx * pl->Ny);
+    if (w.r) pl->device_bytes -= (size_t)w.cg_cap * (3 * vec + pblk * 3 * sizeof(double) +
+                                                     (pl->nblk_max + 1) * sizeof(double2) + sizeof(CGSys) +
+                                                     w.zblk * sizeof(double2));
     cudaFree(w.partz);
     w.partz = nullptr;
     cudaFree(w.r);
@@ -198,7 +204,7 @@ bloch_status ensure_cg(bloch_plan* pl, int nb) {
     BLOCH_CUDA_CHECK_RET(dmalloc(&w.r, n, &pl->device_bytes));
     BLOCH_CUDA_CHECK_RET(dmalloc(&w.p, n, &pl->device_bytes));
     BLOCH_CUDA_CHECK_RET(dmalloc(&w.Ap, n, &pl->device_bytes));
-    BLOCH_CUDA_CHECK_RET(dmalloc(&w.part3, (size_t)nb * pl->nblk_max * 3, &pl->device_bytes));
+    BLOCH_CUDA_CHECK_RET(dmalloc(&w.part3, (size_t)nb * pblk * 3, &pl->device_bytes));
     BLOCH_CUDA_CHECK_RET(dmalloc(&w.part2, (size_t)nb * pl->nblk_max, &pl->device_bytes));
     BLOCH_CUDA_CHECK_RET(dmalloc(&w.dots, (size_t)nb, &pl->device_bytes));
     BLOCH_CUDA_CHECK_RET(dmalloc(&w.sys, (size_t)nb, &pl->device_bytes));
@@ -271,7 +277,8 @@ static void set_fast_attrs_n() {
     fast_attr(k_fpass_axis<T, -1, RA, RB, PT>);
     if constexpr (Z) {
         fast_attr(k_fpass_z_strain<T, RA, RB, kFastZThreads>);
-        fast_attr(k_fpass_z_div<T, RA, RB, kFastZThreads>);
+        fast_attr(k_fpass_z_div<T, RA, RB, kFastZThreads, false>);
+        fast_attr(k_fpass_z_div<T, RA, RB, kFastZThreads, true>);
         if constexpr (RB <= 8) fast_attr(k_fpass_x_stress<T, RA, RB>);
     }
 }
@@ -359,7 +366,7 @@ bloch_status check_pass_err(bloch_plan* pl) {
 }
 
 template <int RA, int RB>
-static void fast_z1(bloch_plan* pl, int nb, const float2* u, float2* E, const float* qtab) {
+static void fast_z1(bloch_plan* pl, int nb, const float2* u, float2* E, const float* qtab, const CGSys* sys) {
     constexpr int NT = kFastZThreads;
     constexpr int P = NT / RA;
     const long long npen = (long long)pl->Nx * pl->Ny;
@@ -368,20 +375,28 @@ static void fast_z1(bloch_plan* pl, int nb, const float2* u, float2* E, const fl
     CUtensorMap map;
     const int tma = encode_zmap(&map, u, pl, 3LL * nb, P) ? 1 : 0;
     k_fpass_z_strain<float, RA, RB, NT><<<gr, NT, fpass_z1_smem<float, RA, RB, NT>(), pl->stream>>>(
-        u, E, qtab, pl->d_twf[2], pl->geo_f, map, tma);
+        u, E, qtab, pl->d_twf[2], pl->geo_f, map, tma, sys);
 }
 
+// returns the CTAs per system
 template <int RA, int RB>
-static void fast_z5(bloch_plan* pl, int nb, const float2* E, const float* qtab, float2* out, float out_scale) {
+static int fast_z5(bloch_plan* pl, int nb, const float2* E, const float* qtab, float2* out, float out_scale,
+                   const CgUpdate<float>* cg) {
     constexpr int NT = kFastZThreads;
     constexpr int P = NT / RA;
+    constexpr size_t smem = fpass_z5_smem<float, RA, RB, NT>();
     const long long npen = (long long)pl->Nx * pl->Ny;
     dim3 gr((unsigned)((npen + P - 1) / P), nb);
     ++pl->launches;
     CUtensorMap map;
     const int tma = encode_zmap(&map, E, pl, 6LL * nb, P) ? 1 : 0;
-    k_fpass_z_div<float, RA, RB, NT><<<gr, NT, fpass_z5_smem<float, RA, RB, NT>(), pl->stream>>>(
-        E, out, qtab, pl->d_twf[2], pl->geo_f, out_scale, map, tma);
+    if (cg)
+        k_fpass_z_div<float, RA, RB, NT, true>
+            <<<gr, NT, smem, pl->stream>>>(E, nullptr, qtab, pl->d_twf[2], pl->geo_f, out_scale, map, tma, *cg);
+    else
+        k_fpass_z_div<float, RA, RB, NT, false>
+            <<<gr, NT, smem, pl->stream>>>(E, out, qtab, pl->d_twf[2], pl->geo_f, out_scale, map, tma, 0);
+    return (int)gr.x;
 }
 
 // Returns the CTAs per system (the number of (p, A p) partials written when dpart != nullptr)
@@ -426,22 +441,24 @@ static void launch_axis(bloch_plan* pl, int axis, int DIR, int nfields, const cp
 
 // Pass 1: strains and their inverse FFT along z
 template <typename T>
-static void launch_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab) {
+static void launch_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab,
+                            const CGSys* sys = nullptr) {
     if constexpr (std::is_same<T, float>::value) {
         if (pl->fast && fast_x(pl->Nz)) {
-            BLOCH_FAST_SWITCH_F(pl->Nz, , fast_z1, pl, nb, u, E, qtab);
+            BLOCH_FAST_SWITCH_F(pl->Nz, , fast_z1, pl, nb, u, E, qtab, sys);
             return;
         }
     }
-    pass_z_strain<T>(pl, nb, u, E, qtab);
+    pass_z_strain<T>(pl, nb, u, E, qtab, sys);
 }
 
 // Passes 1-4: strains, their inverse FFT, stresses, forward FFT along x and y.
 // Returns the (u, A u) partials per system the stress pass wrote (0: none).
 template <typename T>
-static int launch_stress(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab, double2* dpart) {
+static int launch_stress(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab, double2* dpart,
+                         const CGSys* sys = nullptr) {
     int blk = 0;
-    launch_z_strain<T>(pl, nb, u, E, qtab);
+    launch_z_strain<T>(pl, nb, u, E, qtab, sys);
     launch_axis<T>(pl, 1, +1, 6 * nb, E, E, T(1));
     bool done = false;
     if constexpr (std::is_same<T, float>::value) {
@@ -455,16 +472,19 @@ static int launch_stress(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* 
     return dpart ? blk : 0;
 }
 
-// Pass 5: forward FFT along z and divergence
+// Pass 5: forward FFT along z and divergence, into out or (cg) into the residual
+// of the conjugate gradients; returns the CTAs per system.
 template <typename T>
-static void launch_z_div(bloch_plan* pl, int nb, const cplx_t<T>* E, cplx_t<T>* out, const T* qtab, T out_scale) {
+static int launch_z_div(bloch_plan* pl, int nb, const cplx_t<T>* E, cplx_t<T>* out, const T* qtab, T out_scale,
+                        const CgUpdate<T>* cg = nullptr) {
     if constexpr (std::is_same<T, float>::value) {
         if (pl->fast && fast_x(pl->Nz)) {
-            BLOCH_FAST_SWITCH_F(pl->Nz, , fast_z5, pl, nb, E, qtab, out, out_scale);
-            return;
+            int blk = 0;
+            BLOCH_FAST_SWITCH_F(pl->Nz, blk =, fast_z5, pl, nb, E, qtab, out, out_scale, cg);
+            return blk;
         }
     }
-    pass_z_div<T>(pl, nb, E, out, qtab, out_scale);
+    return pass_z_div<T>(pl, nb, E, out, qtab, out_scale, cg);
 }
 
 void launch_K_on(bloch_plan* pl, int nb, const float2* u, float2* E, const float* qtab, float2* out, float out_scale) {
@@ -473,18 +493,17 @@ void launch_K_on(bloch_plan* pl, int nb, const float2* u, float2* E, const float
 }
 
 template <typename T>
-int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale, double2* dpart) {
+void launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale) {
     Workspace<T>& w = ws_of<T>(pl);
     if constexpr (!std::is_same<T, dfloat>::value) {   // cuFFT has no float-float transform
         if (pl->variant == 2) {
             if (!cufft_launch_K<T>(pl, nb, u, out, out_scale, w.E, w.qtab, ctab_of<T>(pl), geo_of<T>(pl)))
                 pl->pending = set_error(BLOCH_ECUDA, "cuFFT plan or execution failed");
-            return 0;
+            return;
         }
     }
-    const int blk = launch_stress<T>(pl, nb, u, w.E, w.qtab, dpart);
+    launch_stress<T>(pl, nb, u, w.E, w.qtab, nullptr);
     launch_z_div<T>(pl, nb, w.E, out, w.qtab, out_scale);
-    return blk;
 }
 
 // Fourier-space stress of nb systems whose q tables are set, into the
@@ -550,57 +569,52 @@ void launch_dot(bloch_plan* pl, int nb, const cplx_t<T>* a, const cplx_t<T>* c, 
 }
 
 // ------------------------------------------------------------ PCG (Algorithm 2)
-// Loop condition of the graph-resident PCG: continue while a system is active
-// and the iteration cap is not reached (the cap bounds every launch).
-static __global__ void k_cg_cond(cudaGraphConditionalHandle h, const int* __restrict__ n_active, int* iter,
-                                 int max_iter) {
-    const int i = ++(*iter);
-    cudaGraphSetConditional(h, (*n_active > 0 && i < max_iter) ? 1u : 0u);
-}
-
-// One PCG iteration (operator, (p, Ap), alpha, updates, beta, p-update, loop
-// condition) enqueued on the plan's stream; captured into the WHILE body.
+// One PCG iteration enqueued on the plan's stream (captured into the WHILE body
+// with h): passes 1-4 of the operator with (p, A p) from the strain energy,
+// alpha, the divergence that updates r and forms (r, z) and (r, r), beta and the
+// loop condition, p- and x-update.
 template <typename T>
-static void pcg_iteration(bloch_plan* pl, int nb, cplx_t<T>* x, double tol2, int nblk,
-                          cudaGraphConditionalHandle* h, int max_iter) {
+static void pcg_iteration(bloch_plan* pl, int nb, cplx_t<T>* x, double tol2, cudaGraphConditionalHandle* h,
+                          int max_iter) {
     Workspace<T>& w = ws_of<T>(pl);
     const Geo& g = geo_of<T>(pl);
-    dim3 gr(nblk, nb);
-    // A p for the systems still active (the passes skip converged ones), with
-    // the (p, A p) partials fused into the last pass where it can
-    static_assert(sizeof(CGSys) % sizeof(int) == 0, "CGSys must be a whole number of ints");
-    Geo& gk = std::is_same<T, float>::value ? pl->geo_f : pl->geo_d;
-    gk.skip = &w.sys[0].active;
-    gk.skip_stride = (int)(sizeof(CGSys) / sizeof(int));
-    gk.skip_ncomp = 6;
-    const int zb = launch_K<T>(pl, nb, w.p, w.Ap, T(1), w.partz);
-    gk.skip = nullptr;
-    gk.skip_stride = 1;
-    gk.skip_ncomp = 1;
-    if (zb > 0) {
-        ++pl->launches;
-        k_dot_final<<<nb, 256, 0, pl->stream>>>(w.partz, zb, w.dots);
+    const int vblk = vec_blocks(pl, nb);
+    dim3 gr(vblk, nb);
+    int nblk = vblk;   // (r, z), (r, r) partials per system
+    const int scaled = std::is_same<T, float>::value && pl->variant != 2 ? 1 : 0;
+    if (pl->variant == 2) {
+        launch_K<T>(pl, nb, w.p, w.Ap, T(1));
+        pl->launches += 3;
+        k_dot_partial<T><<<gr, 256, 0, pl->stream>>>(w.p, w.Ap, 3 * pl->V, w.part2);
+        k_cg_alpha<<<nb, 256, 0, pl->stream>>>(w.part2, vblk, w.sys, 0, pl->d_nactive);
+        k_cg_update<T><<<gr, 256, 0, pl->stream>>>(w.r, w.Ap, w.qtab, g, pl->pc, pl->psel, w.sys, w.part3);
     } else {
-        launch_dot<T>(pl, nb, w.p, w.Ap, 3 * pl->V, w.dots, w.part2);
-    }
-    ++pl->launches;
-    k_cg_scalars<<<nb, 32, 0, pl->stream>>>(w.part3, w.dots, nblk, w.sys, 1, tol2, pl->d_nactive);
-    ++pl->launches;
-    k_cg_update<T><<<gr, 256, 0, pl->stream>>>(w.r, w.Ap, w.qtab, g, pl->pc, pl->psel, w.sys, w.part3);
-    // (mode 1 above zeroed the active count that mode 2 accumulates)
-    ++pl->launches;
-    k_cg_scalars<<<nb, 256, 0, pl->stream>>>(w.part3, w.dots, nblk, w.sys, 2, tol2, pl->d_nactive);
-    ++pl->launches;
-    k_cg_pupdate<T><<<gr, 256, 0, pl->stream>>>(w.r, w.p, x, w.qtab, g, pl->pc, pl->psel, w.sys);
-    if (h) {
+        // the passes skip converged systems
+        static_assert(sizeof(CGSys) % sizeof(int) == 0, "CGSys must be a whole number of ints");
+        Geo& gk = std::is_same<T, float>::value ? pl->geo_f : pl->geo_d;
+        gk.skip = &w.sys[0].active;
+        gk.skip_stride = (int)(sizeof(CGSys) / sizeof(int));
+        gk.skip_ncomp = 6;
+        const int xblk = launch_stress<T>(pl, nb, w.p, w.E, w.qtab, w.partz, w.sys);
         ++pl->launches;
-        k_cg_cond<<<1, 1, 0, pl->stream>>>(*h, pl->d_nactive, pl->d_iter, max_iter);
+        k_cg_alpha<<<nb, 256, 0, pl->stream>>>(w.partz, xblk, w.sys, scaled, pl->d_nactive);
+        const CgUpdate<T> cg{w.r, w.sys, w.part3, pl->pc, pl->psel};
+        nblk = launch_z_div<T>(pl, nb, w.E, nullptr, w.qtab, T(1), &cg);
+        gk.skip = nullptr;
+        gk.skip_stride = 1;
+        gk.skip_ncomp = 1;
     }
+    pl->launches += 2;
+    // residuals 16 (FP32) or 32 (FP64) digits below the start: past any recursive convergence
+    const double rz_floor = std::is_same<T, float>::value ? 1e-32 : 1e-64;
+    k_cg_beta<<<nb, 256, 0, pl->stream>>>(w.part3, nblk, w.sys, tol2, rz_floor, scaled, pl->d_nactive,
+                                          pl->d_iter + 1, h ? 1 : 0, h ? *h : cudaGraphConditionalHandle{}, pl->d_iter, max_iter);
+    k_cg_pupdate<T><<<gr, 256, 0, pl->stream>>>(w.r, w.p, x, w.qtab, g, pl->pc, pl->psel, w.sys);
 }
 
 template <typename T>
-static bloch_status pcg_graph(bloch_plan* pl, int nb, const cplx_t<T>* b, cplx_t<T>* x, double tol2, int nblk,
-                              int max_iter, cudaGraphExec_t* out, int* launches_per_iter) {
+static bloch_status pcg_graph(bloch_plan* pl, int nb, const cplx_t<T>* b, cplx_t<T>* x, double tol2, int max_iter,
+                              cudaGraphExec_t* out, int* launches_per_iter) {
     Workspace<T>& w = ws_of<T>(pl);
     const int prec = std::is_same<T, float>::value ? 1 : 0;
     for (auto& e : pl->pcg_graphs)
@@ -645,7 +659,7 @@ static bloch_status pcg_graph(bloch_plan* pl, int nb, const cplx_t<T>* b, cplx_t
     const unsigned long long l0 = pl->launches;
     cudaStream_t user = pl->stream;
     pl->stream = pl->cap_stream;
-    pcg_iteration<T>(pl, nb, x, tol2, nblk, &h, max_iter);
+    pcg_iteration<T>(pl, nb, x, tol2, &h, max_iter);
     pl->stream = user;
     const int per_iter = (int)(pl->launches - l0);
     pl->launches = l0;   // counted per executed iteration, not at capture
@@ -687,7 +701,7 @@ bloch_status pcg_run(bloch_plan* pl, int nb, const cplx_t<T>* b, cplx_t<T>* x, d
                                               T(rhs_scale), use_x0 ? 0 : 1, w.part3);
     BLOCH_CUDA_CHECK_RET(cudaMemsetAsync(pl->d_nactive, 0, sizeof(int), pl->stream));
     ++pl->launches;
-    k_cg_scalars<<<nb, 256, 0, pl->stream>>>(w.part3, w.dots, nblk, w.sys, 0, tol2, pl->d_nactive);
+    k_cg_start<<<nb, 256, 0, pl->stream>>>(w.part3, nblk, w.sys, tol2, pl->d_nactive);
     BLOCH_CUDA_CHECK_RET(
         cudaMemcpyAsync(pl->h_nactive, pl->d_nactive, sizeof(int), cudaMemcpyDeviceToHost, pl->stream));
     BLOCH_CUDA_CHECK_RET(cudaStreamSynchronize(pl->stream));
@@ -700,7 +714,7 @@ bloch_status pcg_run(bloch_plan* pl, int nb, const cplx_t<T>* b, cplx_t<T>* x, d
     if (use_graph && *pl->h_nactive > 0 && max_iter > 0) {
         cudaGraphExec_t exec;
         int per_iter = 0;
-        bloch_status gs = pcg_graph<T>(pl, nb, b, x, tol2, nblk, max_iter, &exec, &per_iter);
+        bloch_status gs = pcg_graph<T>(pl, nb, b, x, tol2, max_iter, &exec, &per_iter);
         if (gs != BLOCH_OK) return gs;
         BLOCH_CUDA_CHECK_RET(cudaMemsetAsync(pl->d_iter, 0, sizeof(int), pl->stream));
         BLOCH_CUDA_CHECK_RET(cudaGraphLaunch(exec, pl->stream));
@@ -713,7 +727,7 @@ bloch_status pcg_run(bloch_plan* pl, int nb, const cplx_t<T>* b, cplx_t<T>* x, d
     }
     while (!use_graph && *pl->h_nactive > 0 && it < max_iter) {
         tot += *pl->h_nactive;
-        pcg_iteration<T>(pl, nb, x, tol2, nblk, nullptr, max_iter);
+        pcg_iteration<T>(pl, nb, x, tol2, nullptr, max_iter);
         BLOCH_CUDA_CHECK_RET(
             cudaMemcpyAsync(pl->h_nactive, pl->d_nactive, sizeof(int), cudaMemcpyDeviceToHost, pl->stream));
         ++it;
@@ -777,10 +791,10 @@ bloch_status pcg_enqueue(bloch_plan* pl, int nb, const cplx_t<T>* b, cplx_t<T>* 
                                               w.part3);
     BLOCH_CUDA_CHECK_RET(cudaMemsetAsync(pl->d_nactive, 0, sizeof(int), pl->stream));
     ++pl->launches;
-    k_cg_scalars<<<nb, 256, 0, pl->stream>>>(w.part3, w.dots, nblk, w.sys, 0, tol2, pl->d_nactive);
+    k_cg_start<<<nb, 256, 0, pl->stream>>>(w.part3, nblk, w.sys, tol2, pl->d_nactive);
     cudaGraphExec_t exec;
     int per_iter = 0;
-    if ((st = pcg_graph<T>(pl, nb, b, x, tol2, nblk, max_iter, &exec, &per_iter)) != BLOCH_OK) return st;
+    if ((st = pcg_graph<T>(pl, nb, b, x, tol2, max_iter, &exec, &per_iter)) != BLOCH_OK) return st;
     BLOCH_CUDA_CHECK_RET(cudaMemsetAsync(pl->d_iter, 0, sizeof(int), pl->stream));
     BLOCH_CUDA_CHECK_RET(cudaGraphLaunch(exec, pl->stream));
     // launches are counted per executed iteration by the caller's tally
@@ -795,7 +809,7 @@ bloch_status pcg_enqueue(bloch_plan* pl, int nb, const cplx_t<T>* b, cplx_t<T>* 
     template bloch_status ensure_ws<T>(bloch_plan*, int);                                                \
     template bloch_status ensure_cg<T>(bloch_plan*, int);                                                \
     template bloch_status set_k<T>(bloch_plan*, int, const double*);                                     \
-    template int launch_K<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T, double2*);               \
+    template void launch_K<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T);                        \
     template void launch_M<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T);                        \
     template void launch_K_stress<T>(bloch_plan*, int, const cplx_t<T>*);                                 \
     template void launch_fft3<T, -1>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, T, const double2*); \
@@ -812,7 +826,7 @@ INST(float)
 INST(double)
 #undef INST
 template bloch_status ensure_ws<dfloat>(bloch_plan*, int);
-template int launch_K<dfloat>(bloch_plan*, int, const dfloat2*, dfloat2*, dfloat, double2*);
+template void launch_K<dfloat>(bloch_plan*, int, const dfloat2*, dfloat2*, dfloat);
 template bloch_status set_k<dfloat>(bloch_plan*, int, const double*);
 template void launch_M<dfloat>(bloch_plan*, int, const dfloat2*, dfloat2*, dfloat);
 
@@ -870,6 +884,7 @@ static void free_ws_all(bloch_plan* pl) {
         cudaFree(w.part2);
         cudaFree(w.dots);
         cudaFree(w.sys);
+        cudaFree(w.partz);
     };
     fr(pl->ws_f);
     fr(pl->ws_d);
@@ -1147,7 +1162,8 @@ bloch_status bloch_plan_create(bloch_plan** out, const int32_t grid[3], const do
     CK(dmalloc(&pl->d_nactive, 1, acc));
     CK(dmalloc(&pl->d_perr, 1, acc));
     CK(cudaMemset(pl->d_perr, 0, sizeof(int)));
-    CK(dmalloc(&pl->d_iter, 1, acc));
+    CK(dmalloc(&pl->d_iter, 2, acc));
+    CK(cudaMemset(pl->d_iter, 0, 2 * sizeof(int)));
     CK(cudaStreamCreateWithFlags(&pl->cap_stream, cudaStreamNonBlocking));
     CK(cudaMallocHost((void**)&pl->h_nactive, sizeof(int)));
     CK(pass_attrs_z<float>());

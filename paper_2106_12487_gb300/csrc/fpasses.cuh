@@ -139,7 +139,8 @@ template <typename T, int RA, int RB, int NT = 128>
 __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>* __restrict__ U, cplx_t<T>* __restrict__ E,
                                                            const T* __restrict__ qtab,
                                                            const cplx_t<T>* __restrict__ twz, Geo g,
-                                                           const __grid_constant__ CUtensorMap tmap, int use_tma) {
+                                                           const __grid_constant__ CUtensorMap tmap, int use_tma,
+                                                           const CGSys* __restrict__ sys) {
     using C = cplx_t<T>;
     constexpr int N = RA * RB;
     constexpr int P = NT / RA;
@@ -209,7 +210,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>
     tw_fill<RB, RA>(tw, twz, tid, NT);
     const int p2 = tid % P, j2 = tid / P;
     const unsigned pi = pi0 + (p2 < np ? p2 : 0);
-    const T qx = qxt[pi % (unsigned)g.Nx], qy = qyt[pi / (unsigned)g.Nx];
+    const T sc = sys ? cg_scale<T>(sys, b) : T(1);   // every strain is linear in q: scaling q scales them all
+    const T qx = qxt[pi % (unsigned)g.Nx] * sc, qy = qyt[pi / (unsigned)g.Nx] * sc;
     // stage 1 has P * RB tasks per transform and two transforms per component
     // (plain and q_z-scaled): with P * RB == NT / 2 the first half of the CTA
     // runs the plain one and the second half the scaled one
@@ -243,7 +245,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>
 #pragma unroll
             for (int r = 0; r < RA; ++r) {
                 v[r] = sb[(j1 + r * RB) * P + p1];
-                if (scaled) v[r] = cscale(v[r], qzt[j1 + r * RB]);
+                if (scaled) v[r] = cscale(v[r], qzt[j1 + r * RB] * sc);
             }
             RegDFT<RA, +1, C>::run(v);
             C* dst = scaled ? bufB : bufA;
@@ -261,7 +263,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>
 #pragma unroll
             for (int r = 0; r < RA; ++r) bufA[(j1 * RA + r) * P + p1] = v[r];
 #pragma unroll
-            for (int r = 0; r < RA; ++r) u[r] = cscale(u[r], qzt[j1 + r * RB]);
+            for (int r = 0; r < RA; ++r) u[r] = cscale(u[r], qzt[j1 + r * RB] * sc);
             RegDFT<RA, +1, C>::run(u);
 #pragma unroll
             for (int r = 0; r < RA; ++r) bufB[(j1 * RA + r) * P + p1] = u[r];
@@ -308,11 +310,15 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>
 //   out_x = q_x S11 + q_y S12 + q_z S13, out_y = q_x S12 + q_y S22 + q_z S23,
 //   out_z = q_x S13 + q_y S23 + q_z S33   (S = forward z transform of sigma).
 // Stress components stream into shared memory two ahead (cp.async).
-template <typename T, int RA, int RB, int NT = 128>
+// With CG the divergence A p is not stored: the residual of the conjugate
+// gradients is updated with it (CgUpdate), which saves writing and reading A p
+// and one launch per iteration.
+template <typename T, int RA, int RB, int NT, bool CG>
 __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* __restrict__ E, cplx_t<T>* __restrict__ out,
                                                         const T* __restrict__ qtab, const cplx_t<T>* __restrict__ twz,
                                                         Geo g, T out_scale,
-                                                        const __grid_constant__ CUtensorMap tmap, int use_tma) {
+                                                        const __grid_constant__ CUtensorMap tmap, int use_tma,
+                                                        const __grid_constant__ std::conditional_t<CG, CgUpdate<T>, int> cg) {
     using C = cplx_t<T>;
     constexpr int N = RA * RB;
     constexpr int P = NT / RA;
@@ -343,7 +349,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* _
     const unsigned pi0 = blockIdx.x * P;
     const int np = (int)min((unsigned)P, plane - pi0);
     const C* Eb = E + (size_t)b * 6 * g.V;
-    C* ob = out + (size_t)b * 3 * g.V;
     const T* qxt = qtab + (size_t)b * (g.Nx + g.Ny + g.Nz);
     const T* qyt = qxt + g.Nx;
     const T* qzt = qyt + g.Ny;
@@ -468,7 +473,33 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* _
             stage2(c, xb);
         }
     }
-    if (p2 < np) {
+    if constexpr (CG) {
+        C* rb = cg.r + (size_t)b * 3 * g.V;
+        const T sc = cg_scale<T>(cg.sys, b);
+        const T alpha = T(cg.sys[b].alpha / (double)sc);
+        T sum[2] = {T(0), T(0)};
+        if (p2 < np) {
+            constexpr int U = RB < 4 ? RB : 4;   // elements whose residuals are in flight together
+#pragma unroll
+            for (int h = 0; h < RB; h += U) {
+                C ro[U][3];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int i = 0; i < 3; ++i)
+                        ro[u][i] = rb[(size_t)i * g.V + (unsigned)(j2 + (h + u) * RA) * plane + pi0 + p2];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int r = h + u;
+                    const C ap[3] = {acc[0][r], acc[1][r], acc[2][r]};
+                    cg_update_at<T>(cg, rb, b, g.V, (unsigned)(j2 + r * RA) * plane + pi0 + p2, alpha, sc, qv[0],
+                                    qv[1], qzt[j2 + r * RA], ap, ro[u], sum);
+                }
+            }
+        }
+        cg_partial_out<T>(cg, b, sum);
+    } else if (p2 < np) {
+        C* ob = out + (size_t)b * 3 * g.V;
 #pragma unroll
         for (int r = 0; r < RB; ++r) {
             const size_t a = (size_t)(j2 + r * RA) * plane + pi0 + p2;

@@ -29,7 +29,7 @@ struct Workspace {
     C* r = nullptr;         // 3 x V x cg_cap
     C* p = nullptr;
     C* Ap = nullptr;
-    double* part3 = nullptr;  // cg_cap x nblk_max x 3
+    double* part3 = nullptr;  // cg_cap x part_blocks x 3
     double2* part2 = nullptr; // cg_cap x nblk_max
     double2* dots = nullptr;  // cg_cap
     CGSys* sys = nullptr;     // cg_cap
@@ -148,7 +148,7 @@ struct bloch_plan {
         cudaGraphExec_t exec;
     };
     std::vector<PcgGraph> pcg_graphs;
-    int* d_iter = nullptr;
+    int* d_iter = nullptr;         // loop iterations, and finished blocks of k_cg_beta behind them
     int pcg_launches_per_iter = 0;     // kernels per PCG iteration of the last enqueued graph
     cudaStream_t cap_stream = nullptr;   // private stream used only to capture graphs
 
@@ -186,8 +186,9 @@ template <typename T> PassTile pass_tile(const bloch_plan* pl, PassKind kind, in
 
 // Mixed-radix passes (passes.cuh) on the plan's stream: any axis length, every
 // field type.  E and W are updated in place; dir -1 forward, +1 inverse.
-template <typename T>
-void pass_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab);
+template <typename T>   // sys: FP32 strains times the systems' cg_scale
+void pass_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab,
+                   const CGSys* sys = nullptr);
 template <typename T>   // axis 1 (y) or 2 (z) of nfields scalar fields
 void pass_axis(bloch_plan* pl, int axis, int dir, int nfields, const cplx_t<T>* in, cplx_t<T>* out, T out_scale);
 // x pass: the (u, A u) partials of each system go to dpart (nullptr: none);
@@ -196,8 +197,9 @@ template <typename T> int pass_x_stress(bloch_plan* pl, int nb, cplx_t<T>* E, do
 template <typename T> void pass_x_rho(bloch_plan* pl, int nb, cplx_t<T>* W);
 template <typename T>   // ph, per: complex factors of the systems (k_pass_x)
 void pass_x(bloch_plan* pl, int dir, int nb, cplx_t<T>* W, T out_scale, const double2* ph = nullptr, int per = 1);
-template <typename T>
-void pass_z_div(bloch_plan* pl, int nb, const cplx_t<T>* E, cplx_t<T>* out, const T* qtab, T out_scale);
+template <typename T>   // with cg the residual is updated instead of out; returns the CTAs per system
+int pass_z_div(bloch_plan* pl, int nb, const cplx_t<T>* E, cplx_t<T>* out, const T* qtab, T out_scale,
+               const CgUpdate<T>* cg = nullptr);
 // shared-memory limits of the passes, once per plan
 template <typename T> cudaError_t pass_attrs_z();
 template <typename T> cudaError_t pass_attrs_axis();
@@ -210,11 +212,7 @@ template <typename T> bloch_status ensure_cg(bloch_plan* pl, int nb);
 // Upload nb wave vectors (host, rad/m) and build the scaled q tables.
 template <typename T> bloch_status set_k(bloch_plan* pl, int nb, const double* k_host);
 // Scaled stiffness operator on nb systems whose q tables are set: out = out_scale * A~ u.
-// With dpart, the stress pass also forms per-CTA partials of (u, A~ u) per
-// system in dpart and the call returns the number of partials per system; it
-// returns 0 when no pass did (the caller forms the product).
-template <typename T>
-int launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale, double2* dpart = nullptr);
+template <typename T> void launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale);
 // The FP32 operator on scratch E and q tables of the caller (launch_K's chain).
 void launch_K_on(bloch_plan* pl, int nb, const float2* u, float2* E, const float* qtab, float2* out, float out_scale);
 // Fourier-space stress S = F{C~ : F^-1(sym q (x) u)} of nb systems (q tables

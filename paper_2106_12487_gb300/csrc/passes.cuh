@@ -41,6 +41,7 @@
 //   128^3, float-float, 4 systems      7.92 -> 4.62 ms (bound by FP32 issue)
 #pragma once
 
+#include "cg.cuh"
 #include "common.cuh"
 #include "fft.cuh"
 
@@ -243,7 +244,7 @@ __device__ __forceinline__ void pf_last(C* buf, int nbuf, const AxisPlan& a, int
 template <typename T, bool WIDE>
 __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     k_pass_z_strain(const cplx_t<T>* __restrict__ U, cplx_t<T>* __restrict__ E, const T* __restrict__ qtab,
-                    const cplx_t<T>* __restrict__ twz, Geo g, int lp) {
+                    const cplx_t<T>* __restrict__ twz, Geo g, int lp, const CGSys* __restrict__ sys) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const AxisPlan& a = g.ax[2];
@@ -262,6 +263,15 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     const T* qx = qtab + (size_t)b * (g.Nx + g.Ny + g.Nz);
     const T* qy = qx + g.Nx;
     const T* qz = qy + g.Ny;
+    // FP32 conjugate gradients: every strain is linear in q, so scaling q scales them all
+    T sc = T(1);
+    if constexpr (sizeof(T) == 4) {
+        if (sys) sc = cg_scale<T>(sys, b);
+    }
+    auto qs = [&](T q) {
+        if constexpr (sizeof(T) == 4) return q * sc;
+        else return q;
+    };
     for (int i = tid; i < ntw; i += nthr) tw[i] = twz[i];
     __syncthreads();
     with_radix<real_t<C>, WIDE>(a.r1, [&](auto rc) {
@@ -282,7 +292,7 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     v[r] = src[(unsigned)(r * M) * plane];
-                    w[r] = cscale(v[r], ldg_t(qz + r * M + j));
+                    w[r] = cscale(v[r], qs(ldg_t(qz + r * M + j)));
                 }
                 RegDFT<R, +1, C>::run(v);
                 RegDFT<R, +1, C>::run(w);
@@ -300,7 +310,7 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
                         v[r] = src[(unsigned)(r * M) * plane];
-                        if (h) v[r] = cscale(v[r], ldg_t(qz + r * M + j));
+                        if (h) v[r] = cscale(v[r], qs(ldg_t(qz + r * M + j)));
                     }
                     RegDFT<R, +1, C>::run(v);
                     s[0] = v[0];
@@ -322,7 +332,7 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
         if (p >= np) continue;
         const C* s = buf + (slot_of(k, a) << lp) + p;
         const unsigned pi = pi0 + p, y = fdiv(pi, g.dx);
-        const T ax = qx[pi - y * (unsigned)g.Nx], ay = qy[y];
+        const T ax = qs(qx[pi - y * (unsigned)g.Nx]), ay = qs(qy[y]);
         const C a0 = s[0], b0 = s[NP], a1 = s[2 * NP], b1 = s[3 * NP], a2 = s[4 * NP], b2 = s[5 * NP];
         C* d = Eb + (size_t)k * plane + pi;
         d[0] = cscale(a0, ax);
@@ -404,10 +414,13 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
 }
 
 // ---------------------------------------------------------------- pass 5
-template <typename T, bool WIDE>
+// With CG the divergence A p is not stored: the residual of the conjugate
+// gradients is updated with it in place (CgUpdate).
+template <typename T, bool WIDE, bool CG>
 __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     k_pass_z_div(const cplx_t<T>* __restrict__ E, cplx_t<T>* __restrict__ out, const T* __restrict__ qtab,
-                 const cplx_t<T>* __restrict__ twz, Geo g, int lp, T out_scale) {
+                 const cplx_t<T>* __restrict__ twz, Geo g, int lp, T out_scale,
+                 const __grid_constant__ std::conditional_t<CG, CgUpdate<T>, int> cg) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const AxisPlan& a = g.ax[2];
@@ -422,7 +435,15 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     const unsigned pi0 = blockIdx.x << lp;
     const int np = (int)min((unsigned)P1 + 1u, plane - pi0);
     const C* Eb = E + (size_t)b * 6 * g.V;
-    C* ob = out + (size_t)b * 3 * g.V;
+    C* ob;
+    T alpha = T(0), sc = T(1), acc[2] = {T(0), T(0)};
+    if constexpr (CG) {
+        ob = cg.r + (size_t)b * 3 * g.V;
+        sc = cg_scale<T>(cg.sys, b);
+        alpha = T(cg.sys[b].alpha / (double)sc);
+    } else {
+        ob = out + (size_t)b * 3 * g.V;
+    }
     const T* qx = qtab + (size_t)b * (g.Nx + g.Ny + g.Nz);
     const T* qy = qx + g.Nx;
     const T* qz = qy + g.Ny;
@@ -452,18 +473,41 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     }
     pf_last<-1, WIDE>(buf, 6, a, lp, tid, nthr);
     __syncthreads();
-    for (int t = tid; t < NP; t += nthr) {
-        const int p = t & P1, k = t >> lp;
-        if (p >= np) continue;
-        const C* s = buf + (slot_of(k, a) << lp) + p;
-        const unsigned pi = pi0 + p, y = fdiv(pi, g.dx);
-        const T ax = qx[pi - y * (unsigned)g.Nx], ay = qy[y], az = qz[k];
-        const C s0 = s[0], s1 = s[NP], s2 = s[2 * NP], s3 = s[3 * NP], s4 = s[4 * NP], s5 = s[5 * NP];
-        C* d = ob + (size_t)k * plane + pi;
-        d[0] = cscale(cadd(cadd(cscale(s0, ax), cscale(s4, az)), cscale(s5, ay)), out_scale);
-        d[g.V] = cscale(cadd(cadd(cscale(s1, ay), cscale(s3, az)), cscale(s5, ax)), out_scale);
-        d[2 * g.V] = cscale(cadd(cadd(cscale(s2, az), cscale(s3, ay)), cscale(s4, ax)), out_scale);
+    constexpr int U = CG ? 4 : 1;   // voxels whose residuals are in flight together
+    for (int t0 = tid; t0 < NP; t0 += U * nthr) {
+        C ro[U][3];
+        if constexpr (CG) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int t = t0 + u * nthr, p = t & P1, k = t >> lp;
+                if (t < NP && p < np) {
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) ro[u][i] = ob[(size_t)i * g.V + (size_t)k * plane + pi0 + p];
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int t = t0 + u * nthr, p = t & P1, k = t >> lp;
+            if (t >= NP || p >= np) continue;
+            const C* s = buf + (slot_of(k, a) << lp) + p;
+            const unsigned pi = pi0 + p, y = fdiv(pi, g.dx);
+            const T ax = qx[pi - y * (unsigned)g.Nx], ay = qy[y], az = qz[k];
+            const C s0 = s[0], s1 = s[NP], s2 = s[2 * NP], s3 = s[3 * NP], s4 = s[4 * NP], s5 = s[5 * NP];
+            const C o[3] = {cadd(cadd(cscale(s0, ax), cscale(s4, az)), cscale(s5, ay)),
+                            cadd(cadd(cscale(s1, ay), cscale(s3, az)), cscale(s5, ax)),
+                            cadd(cadd(cscale(s2, az), cscale(s3, ay)), cscale(s4, ax))};
+            if constexpr (CG) {
+                cg_update_at<T>(cg, ob, b, g.V, (unsigned)k * plane + pi, alpha, sc, ax, ay, az, o, ro[u], acc);
+            } else {
+                C* d = ob + (size_t)k * plane + pi;
+                d[0] = cscale(o[0], out_scale);
+                d[g.V] = cscale(o[1], out_scale);
+                d[2 * g.V] = cscale(o[2], out_scale);
+            }
+        }
     }
+    if constexpr (CG) cg_partial_out<T>(cg, b, acc);
 }
 
 // ------------------------------------------------ stages on rows along x
@@ -570,18 +614,20 @@ __device__ __forceinline__ void lf_store(C* Wb, long long V, const C* buf, int n
     });
 }
 
-// sigma = C_g gamma in place on the six components s[c cs]; adds conj(gamma) sigma
+// sigma = C_g gamma in place on the six components s[c cs]; with want adds conj(gamma) sigma
 template <typename T, typename C>
-__device__ __forceinline__ void stress_smem(C* s, int cs, const T* __restrict__ Cg, T& energy) {
+__device__ __forceinline__ void stress_smem(C* s, int cs, const T* __restrict__ Cg, bool want, T& energy) {
     C gam[6], sig[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) gam[c] = s[c * cs];
     stress_of<T>(gam, sig, Cg);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        s[i * cs] = sig[i];
-        if constexpr (!std::is_same<T, dfloat>::value)
-            energy = fma(gam[i].x, sig[i].x, fma(gam[i].y, sig[i].y, energy));
+    for (int i = 0; i < 6; ++i) s[i * cs] = sig[i];
+    if constexpr (!std::is_same<T, dfloat>::value) {
+        if (want) {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) energy = fma(gam[i].x, sig[i].x, fma(gam[i].y, sig[i].y, energy));
+        }
     }
 }
 
@@ -647,7 +693,7 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
         C* s = buf + p * ld + ((k - q * a.r1) * a.r2 + (q - k3 * a.r2)) * gr + k3;   // slot (k1, k2, k3)
         const int cs = P * ld;
         if constexpr (NC == 6) {
-            stress_smem<T>(s, cs, tab + (size_t)gid * kCtabRow<T>, energy);
+            stress_smem<T>(s, cs, tab + (size_t)gid * kCtabRow<T>, dpart != nullptr, energy);
         } else {
             const T r = ldg_t(tab + gid);
 #pragma unroll

@@ -44,13 +44,13 @@ static inline void with_width(const bloch_plan* pl, int axis, F&& f) {
 }
 
 template <typename T>
-void pass_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab) {
+void pass_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, const T* qtab, const CGSys* sys) {
     const PassTile t = pass_tile<T>(pl, PASS_Z6, nb);
     ++pl->launches;
     with_width<T>(pl, 2, [&](auto w) {
         k_pass_z_strain<T, decltype(w)::value>
             <<<pass_grid((long long)pl->Nx * pl->Ny, t.lp, nb), t.nthr, t.smem, pl->stream>>>(
-                u, E, qtab, pass_tw<T>(pl, 2), geo_of<T>(pl), t.lp);
+                u, E, qtab, pass_tw<T>(pl, 2), geo_of<T>(pl), t.lp, sys);
     });
 }
 
@@ -114,14 +114,24 @@ void pass_x(bloch_plan* pl, int dir, int nb, cplx_t<T>* W, T out_scale, const do
 }
 
 template <typename T>
-void pass_z_div(bloch_plan* pl, int nb, const cplx_t<T>* E, cplx_t<T>* out, const T* qtab, T out_scale) {
+int pass_z_div(bloch_plan* pl, int nb, const cplx_t<T>* E, cplx_t<T>* out, const T* qtab, T out_scale,
+               const CgUpdate<T>* cg) {
     const PassTile t = pass_tile<T>(pl, PASS_Z6, nb);
+    const dim3 gr = pass_grid((long long)pl->Nx * pl->Ny, t.lp, nb);
     ++pl->launches;
     with_width<T>(pl, 2, [&](auto w) {
-        k_pass_z_div<T, decltype(w)::value>
-            <<<pass_grid((long long)pl->Nx * pl->Ny, t.lp, nb), t.nthr, t.smem, pl->stream>>>(
-                E, out, qtab, pass_tw<T>(pl, 2), geo_of<T>(pl), t.lp, out_scale);
+        constexpr bool W = decltype(w)::value;
+        if constexpr (!std::is_same<T, dfloat>::value) {
+            if (cg) {
+                k_pass_z_div<T, W, true><<<gr, t.nthr, t.smem, pl->stream>>>(E, nullptr, qtab, pass_tw<T>(pl, 2),
+                                                                             geo_of<T>(pl), t.lp, out_scale, *cg);
+                return;
+            }
+        }
+        k_pass_z_div<T, W, false>
+            <<<gr, t.nthr, t.smem, pl->stream>>>(E, out, qtab, pass_tw<T>(pl, 2), geo_of<T>(pl), t.lp, out_scale, 0);
     });
+    return (int)gr.x;
 }
 
 // shared-memory limits of both forms
@@ -138,7 +148,11 @@ cudaError_t pass_attrs_z() {
     return each_width<T>([](auto w) {
         constexpr bool W = decltype(w)::value;
         cudaError_t e = allow_max_dyn_smem(k_pass_z_strain<T, W>);
-        return e == cudaSuccess ? allow_max_dyn_smem(k_pass_z_div<T, W>) : e;
+        if (e == cudaSuccess) e = allow_max_dyn_smem(k_pass_z_div<T, W, false>);
+        if constexpr (!std::is_same<T, dfloat>::value) {
+            if (e == cudaSuccess) e = allow_max_dyn_smem(k_pass_z_div<T, W, true>);
+        }
+        return e;
     });
 }
 template <typename T>
@@ -166,8 +180,9 @@ cudaError_t pass_attrs_x() {
 }
 
 #define BLOCH_INST_PASSES_Z(T)                                                                            \
-    template void pass_z_strain<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, const T*);             \
-    template void pass_z_div<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, const T*, T);             \
+    template void pass_z_strain<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, const T*, const CGSys*); \
+    template int pass_z_div<T>(bloch_plan*, int, const cplx_t<T>*, cplx_t<T>*, const T*, T,               \
+                               const CgUpdate<T>*);                                                      \
     template cudaError_t pass_attrs_z<T>();
 #define BLOCH_INST_PASSES_AXIS(T)                                                                         \
     template void pass_axis<T>(bloch_plan*, int, int, int, const cplx_t<T>*, cplx_t<T>*, T);              \

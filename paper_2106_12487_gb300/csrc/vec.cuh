@@ -5,35 +5,11 @@
 // final sum per system (deterministic, no atomics).
 #pragma once
 
+#include "cg.cuh"
 #include "common.cuh"
 #include "passes.cuh"
 
 namespace bloch {
-
-// P_ik = sum_m A[ik][m] mono_m(q), pairs ik in (xx, yy, zz, yz, xz, xy) and
-// monomials (qx^2, qy^2, qz^2, qy qz, qx qz, qx qy), from the scaled C0.
-struct PrecondCoef {
-    double a[6][6];
-    float af[6][6];   // the same coefficients rounded once to FP32 (FP32 kernels read these:
-                      // no FP64 -> FP32 conversion per voxel)
-};
-template <typename T> __device__ __forceinline__ T pcoef(const PrecondCoef& pc, int i, int j);
-template <> __device__ __forceinline__ float pcoef<float>(const PrecondCoef& pc, int i, int j) { return pc.af[i][j]; }
-template <> __device__ __forceinline__ double pcoef<double>(const PrecondCoef& pc, int i, int j) { return pc.a[i][j]; }
-
-// Per-system CG scalars (device resident).
-struct CGSys {
-    double rz;       // (r, z) of the current iterate
-    double rz_new;
-    double pAp;
-    double rr;       // (r, r)
-    double bb;       // (b, b) (scaled)
-    double alpha;
-    double beta;
-    int active;
-    int iters;
-    int upd;         // took a step this iteration (x += alpha p is still to be applied)
-};
 
 // qtab[b][.] = ((xi + k_b) * qscale) for the x, y and z axes.
 template <typename T>
@@ -68,61 +44,6 @@ __device__ __forceinline__ void voxel_q(const T* qb, const Geo& g, unsigned v, T
     az = qb[g.Nx + g.Ny + z];
 }
 
-// Correctly rounded reciprocal (the FP32 form uses the rounded reciprocal
-// intrinsic instead of a full division).
-__device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
-
-// z = P^-1(q) r for one voxel (three complex components); zero where q = 0.
-template <typename T>
-__device__ __forceinline__ void green_apply(const PrecondCoef& pc, T qx, T qy, T qz, const cplx_t<T> r[3],
-                                            cplx_t<T> z[3]) {
-    const T m[6] = {qx * qx, qy * qy, qz * qz, qy * qz, qx * qz, qx * qy};
-    T P[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        T s = 0;
-#pragma unroll
-        for (int j = 0; j < 6; ++j) s = fma(pcoef<T>(pc, i, j), m[j], s);
-        P[i] = s;
-    }
-    const T a = P[0], bq = P[1], c = P[2], d = P[3], e = P[4], f = P[5];
-    const T A = bq * c - d * d, B = a * c - e * e, Cc = a * bq - f * f;
-    const T D = e * f - a * d, Ee = d * f - bq * e, F = d * e - c * f;
-    const T det = a * A + f * F + e * Ee;
-    if (m[0] + m[1] + m[2] == T(0) || det == T(0)) {
-        z[0] = z[1] = z[2] = mk(T(0), T(0));
-        return;
-    }
-    const T id = recip(det);
-    z[0] = cscale(cadd(cadd(cscale(r[0], A), cscale(r[1], F)), cscale(r[2], Ee)), id);
-    z[1] = cscale(cadd(cadd(cscale(r[0], F), cscale(r[1], B)), cscale(r[2], D)), id);
-    z[2] = cscale(cadd(cadd(cscale(r[0], Ee), cscale(r[1], D)), cscale(r[2], Cc)), id);
-}
-
-// Preconditioner selection: the Green operator P^-1 computed per voxel, or a
-// precomputed symmetric 3x3 table per voxel (the learned preconditioner), one
-// table per group of `zgroup` consecutive systems.
-struct PrecondSel {
-    const float* ztab;   // nullptr: Green operator
-    int zgroup;
-};
-
-template <typename T>
-__device__ __forceinline__ void zsym_apply(const float* __restrict__ Z, const cplx_t<T> r[3], cplx_t<T> z[3]) {
-    const T a = T(Z[0]), b = T(Z[1]), c = T(Z[2]), d = T(Z[3]), e = T(Z[4]), f = T(Z[5]);
-    z[0] = cadd(cadd(cscale(r[0], a), cscale(r[1], f)), cscale(r[2], e));
-    z[1] = cadd(cadd(cscale(r[0], f), cscale(r[1], b)), cscale(r[2], d));
-    z[2] = cadd(cadd(cscale(r[0], e), cscale(r[1], d)), cscale(r[2], c));
-}
-
-template <typename T>
-__device__ __forceinline__ void pre_apply(const PrecondSel& ps, const PrecondCoef& pc, int sys, unsigned v,
-                                          long long V, T qx, T qy, T qz, const cplx_t<T> r[3], cplx_t<T> z[3]) {
-    if (ps.ztab) zsym_apply<T>(ps.ztab + ((size_t)(sys / ps.zgroup) * V + v) * 6, r, z);
-    else green_apply(pc, qx, qy, qz, r, z);
-}
-
 template <typename T>
 __global__ void k_precond(const cplx_t<T>* r, cplx_t<T>* z, const T* __restrict__ qtab, Geo g, PrecondCoef pc,
                           PrecondSel ps, T out_scale) {
@@ -143,35 +64,6 @@ __global__ void k_precond(const cplx_t<T>* r, cplx_t<T>* z, const T* __restrict_
 }
 
 // ---------------------------------------------------------------- reductions
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Block-wide sum of NV values; result valid in thread 0.
-template <typename T, int NV>
-__device__ __forceinline__ void block_sum(T (&v)[NV]) {
-    __shared__ T red[NV][32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int i = 0; i < NV; ++i) v[i] = warp_sum(v[i]);
-    __syncthreads();
-    if (lane == 0) {
-#pragma unroll
-        for (int i = 0; i < NV; ++i) red[i][w] = v[i];
-    }
-    __syncthreads();
-    if (w == 0) {
-#pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            T s = lane < nw ? red[i][lane] : T(0);
-            v[i] = warp_sum(s);
-        }
-    }
-}
-
 // partial[b][blk] = sum over the block's voxels of conj(a) b (complex)
 template <typename T>
 __global__ void k_dot_partial(const cplx_t<T>* a, const cplx_t<T>* bv, long long n_per, double2* partial) {
@@ -244,8 +136,9 @@ __global__ void k_cg_init(const cplx_t<T>* bvec, const cplx_t<T>* Ax, cplx_t<T>*
     }
 }
 
-// r -= alpha Ap; partials (r, P^-1 r), (r, r).  The matching x += alpha p is
-// applied by k_cg_pupdate, which reads p anyway (one pass less over x here).
+// r -= alpha Ap; partials (r, P^-1 r), (r, r), for the plain-form baseline's
+// operator (the passes update r in their divergence).  The matching x += alpha p
+// is applied by k_cg_pupdate, which reads p anyway.
 template <typename T>
 __global__ void k_cg_update(cplx_t<T>* __restrict__ r, const cplx_t<T>* __restrict__ Ap,
                             const T* __restrict__ qtab, Geo g, PrecondCoef pc, PrecondSel ps, const CGSys* sys,
@@ -325,50 +218,89 @@ __global__ void k_cg_pupdate(const cplx_t<T>* __restrict__ r, cplx_t<T>* __restr
     }
 }
 
-// Final sums of the 3-wide partials and the scalar recurrences of Algorithm 2.
-// mode 0 (after init): rz, rr, bb; active = rr > tol^2 bb.
-// mode 1 (after pAp dot, partial2 holds complex (p, Ap)): alpha = rz / pAp.
-// mode 2 (after update): rz_new, rr; converge test; beta = rz_new/rz; rz = rz_new.
-static __global__ void k_cg_scalars(const double* partial3, const double2* dots, int nblk, CGSys* sys, int mode,
-                             double tol2, int* n_active) {
+// Scalar recurrences of Algorithm 2, one block per system.
+// After the initial residual: rz, rr, bb from the 3-wide partials; active = rr > tol^2 bb.
+static __global__ void k_cg_start(const double* partial3, int nblk, CGSys* sys, double tol2, int* n_active) {
     const int b = blockIdx.x;
     double acc[3] = {0.0, 0.0, 0.0};
-    if (mode != 1) {
+    for (int i = threadIdx.x; i < nblk; i += blockDim.x) {
+        const double* v = partial3 + ((size_t)b * nblk + i) * 3;
+        acc[0] += v[0];
+        acc[1] += v[1];
+        acc[2] += v[2];
+    }
+    block_sum<double, 3>(acc);
+    if (threadIdx.x != 0) return;
+    CGSys& s = sys[b];
+    s.rz = s.rz0 = acc[0];
+    s.rr = acc[1];
+    s.bb = acc[2];
+    s.iters = 0;
+    s.upd = 0;
+    s.active = (s.rr > tol2 * s.bb) ? 1 : 0;
+    if (s.active) atomicAdd(n_active, 1);
+}
+
+// After the stress pass: (p, A p) from its partials, alpha = rz / (p, A p).
+// scaled: the sums carry the square of cg_scale (here and in k_cg_beta).
+static __global__ void k_cg_alpha(const double2* partial2, int nblk, CGSys* sys, int scaled, int* n_active) {
+    const int b = blockIdx.x;
+    CGSys& s = sys[b];
+    double acc[1] = {0.0};
+    if (s.active)
+        for (int i = threadIdx.x; i < nblk; i += blockDim.x) acc[0] += partial2[(size_t)b * nblk + i].x;
+    block_sum<double, 1>(acc);
+    if (threadIdx.x != 0) return;
+    if (b == 0) *n_active = 0;   // recounted by k_cg_beta (kernels of one stream are ordered)
+    const double sc = scaled ? (double)cg_scale<float>(sys, b) : 1.0;
+    s.pAp = acc[0] / (sc * sc);
+    s.alpha = (s.active && s.pAp > 0.0) ? s.rz / s.pAp : 0.0;
+    s.upd = s.active;
+}
+
+// After the residual update: rz_new, rr; convergence test; beta = rz_new / rz.
+// A system also ends when (r, z) has fallen below rz_floor of its start: what is
+// left of r then lies where P^-1 is zero (bin 0 at k = 0 under a non-uniform
+// density), no step can reduce it, and going on to the iteration cap would only
+// drive the sums into underflow.  It still counts as not converged.
+// The last block to finish sets the condition of the graph-resident loop
+// (cond != 0): continue while a system is active and the iteration cap, which
+// bounds every launch, is not reached.  *ticket counts finished blocks and is
+// left at zero.
+static __global__ void k_cg_beta(const double* partial3, int nblk, CGSys* sys, double tol2, double rz_floor, int scaled,
+                                 int* n_active, int* ticket, int cond, cudaGraphConditionalHandle h, int* iter, int max_iter) {
+    const int b = blockIdx.x;
+    CGSys& s = sys[b];
+    double acc[2] = {0.0, 0.0};
+    const int active = s.active;
+    if (active)
         for (int i = threadIdx.x; i < nblk; i += blockDim.x) {
             const double* v = partial3 + ((size_t)b * nblk + i) * 3;
             acc[0] += v[0];
             acc[1] += v[1];
-            acc[2] += v[2];
         }
-        block_sum<double, 3>(acc);
-    }
+    block_sum<double, 2>(acc);
     if (threadIdx.x != 0) return;
-    CGSys& s = sys[b];
-    if (mode == 0) {
-        s.rz = acc[0];
-        s.rr = acc[1];
-        s.bb = acc[2];
-        s.iters = 0;
-        s.upd = 0;
-        s.active = (s.rr > tol2 * s.bb) ? 1 : 0;
-        if (s.active) atomicAdd(n_active, 1);
-    } else if (mode == 1) {
-        if (b == 0) *n_active = 0;   // recount in mode 2 (kernels of one stream are ordered)
-        s.pAp = dots[b].x;
-        s.alpha = (s.active && s.pAp > 0.0) ? s.rz / s.pAp : 0.0;
-        s.upd = s.active;
-    } else {
-        if (!s.active) return;
+    if (active) {
+        const double sc = scaled ? (double)cg_scale<float>(sys, b) : 1.0;
         s.iters += 1;
-        s.rz_new = acc[0];
-        s.rr = acc[1];
-        if (!(s.rr > tol2 * s.bb) || !(s.rz_new > 0.0)) {
+        s.rz_new = acc[0] / (sc * sc);
+        s.rr = acc[1] / (sc * sc);
+        if (!(s.rr > tol2 * s.bb) || !(s.rz_new > rz_floor * s.rz0)) {
             s.active = 0;
         } else {
             s.beta = s.rz_new / s.rz;
             s.rz = s.rz_new;
             atomicAdd(n_active, 1);
         }
+    }
+    if (!cond) return;
+    __threadfence();
+    if (atomicAdd(ticket, 1) == (int)gridDim.x - 1) {
+        *ticket = 0;
+        __threadfence();
+        const int i = ++(*iter);
+        cudaGraphSetConditional(h, (*(volatile int*)n_active > 0 && i < max_iter) ? 1u : 0u);
     }
 }
 
