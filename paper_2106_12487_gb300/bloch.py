@@ -95,7 +95,7 @@ def lib():
     L.bloch_plan_create.argtypes = [P(VP), P(I32), P(D), P(I32), I32, P(D), P(D), P(Options), VP]
     L.bloch_plan_destroy.argtypes = [VP]
     L.bloch_plan_destroy.restype = None
-    L.bloch_apply_K.argtypes = [VP, I32, P(D), I32, VP, VP]
+    L.bloch_apply_K.argtypes = [VP, I32, VP, I32, VP, VP]
     L.bloch_apply_K_real.argtypes = [VP, I32, P(D), I32, VP, VP]
     L.bloch_apply_M.argtypes = [VP, I32, I32, VP, VP]
     L.bloch_apply_K_noalloc.argtypes = [VP, I32, P(D), VP, VP]
@@ -151,6 +151,23 @@ def _dptr(arr, what):
     return ctypes.cast(arr.ctypes.data, ctypes.POINTER(what))
 
 
+def _addr(arr) -> int:
+    """Address of a contiguous numpy array's data, for a void-pointer argument."""
+    return arr.__array_interface__["data"][0]
+
+
+def _torch():
+    """The torch module, looked up once (small calls cost little more than their launches)."""
+    global _TORCH
+    if _TORCH is None:
+        import torch
+        _TORCH = torch
+    return _TORCH
+
+
+_TORCH = None
+
+
 def default_options(**kw) -> Options:
     o = Options()
     lib().bloch_default_options(ctypes.byref(o))
@@ -162,7 +179,7 @@ def default_options(**kw) -> Options:
 
 
 def _tensor_ptr(t, precision: int, n_expected: int):
-    import torch
+    torch = _torch()
     want = torch.complex64 if precision == FP32 else torch.complex128   # FP64 and FF use double2
     if t.dtype != want:
         raise TypeError(f"expected {want}, got {t.dtype}")
@@ -170,7 +187,7 @@ def _tensor_ptr(t, precision: int, n_expected: int):
         raise ValueError("device tensors must be contiguous CUDA tensors")
     if t.numel() != n_expected:
         raise ValueError(f"expected {n_expected} elements, got {t.numel()}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 class Plan:
@@ -241,6 +258,8 @@ class Plan:
 
     # ---------------------------------------------------------------- ops
     def _kv(self, k, nb):
+        if type(k) is np.ndarray and k.dtype == np.float64 and k.shape == (nb, 3) and k.flags.c_contiguous:
+            return k
         kv = np.ascontiguousarray(np.broadcast_to(np.asarray(k, dtype=np.float64).reshape(-1, 3), (nb, 3)))
         return kv
 
@@ -248,8 +267,10 @@ class Plan:
         prec = self.precision if precision is None else precision
         nb = u.numel() // (3 * self.V)
         kv = self._kv(k, nb)
-        _check(lib().bloch_apply_K(self.handle, nb, _dptr(kv, ctypes.c_double), prec,
-                                   _tensor_ptr(u, prec, nb * 3 * self.V), _tensor_ptr(out, prec, nb * 3 * self.V)))
+        n = nb * 3 * self.V
+        st = lib().bloch_apply_K(self.handle, nb, _addr(kv), prec, _tensor_ptr(u, prec, n), _tensor_ptr(out, prec, n))
+        if st != BLOCH_OK:
+            _check(st)
         return out
 
     def apply_K_real(self, k, u, out, precision: int | None = None):

@@ -85,14 +85,9 @@ extern "C" bloch_status bloch_apply_K_noalloc(bloch_plan* pl, int32_t nb, const 
     float* qtab = (float*)(b + kNoAllocPassBytes);
     double* kvec = (double*)(b + kNoAllocPassBytes + q_bytes);
 
-    cudaError_t e = cudaMemcpyAsync(kvec, k, k_bytes, cudaMemcpyHostToDevice, pl->stream);
-    if (e != cudaSuccess) return set_cuda_error(e, "cudaMemcpyAsync (wave vectors)");
-    const int qblocks = (int)std::min<long long>(1024, ((long long)nb * S + 255) / 256);
-    k_qtab<float><<<qblocks, 256, 0, pl->stream>>>(kvec, pl->d_xi, pl->Nx, pl->Ny, pl->Nz, nb, pl->qscale, qtab);
-
-    ++pl->launches;
+    if ((st = launch_qtab<float>(pl, nb, k, kvec, qtab)) != BLOCH_OK) return st;
     launch_K_on(pl, nb, (const float2*)u, E, qtab, (float2*)Ku, (float)pl->Kscale);
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return set_cuda_error(e, "bloch_apply_K_noalloc launch");
     return BLOCH_OK;
 }

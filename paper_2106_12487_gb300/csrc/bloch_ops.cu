@@ -216,6 +216,25 @@ bloch_status ensure_cg(bloch_plan* pl, int nb) {
 }
 
 template <typename T>
+bloch_status launch_qtab(bloch_plan* pl, int nb, const double* k_host, double* kvec, T* qtab) {
+    WaveParams wp;
+    if (nb <= kParamWaves) {
+        std::memcpy(wp.k, k_host, sizeof(double) * 3 * nb);
+        kvec = nullptr;
+    } else {
+        BLOCH_CUDA_CHECK_RET(
+            cudaMemcpyAsync(kvec, k_host, sizeof(double) * 3 * nb, cudaMemcpyHostToDevice, pl->stream));
+    }
+    const int S = pl->Nx + pl->Ny + pl->Nz;
+    const int blocks = (int)std::min<long long>(1024, ((long long)nb * S + 255) / 256);
+    ++pl->launches;
+    k_qtab<T><<<blocks, 256, 0, pl->stream>>>(kvec, wp, pl->d_xi, pl->Nx, pl->Ny, pl->Nz, nb, pl->qscale, qtab);
+    BLOCH_CUDA_CHECK_RET(cudaGetLastError());
+    return BLOCH_OK;
+}
+template bloch_status launch_qtab<float>(bloch_plan*, int, const double*, double*, float*);
+
+template <typename T>
 bloch_status set_k(bloch_plan* pl, int nb, const double* k_host) {
     bloch_status st = ensure_ws<T>(pl, nb);
     if (st != BLOCH_OK) return st;
@@ -223,14 +242,7 @@ bloch_status set_k(bloch_plan* pl, int nb, const double* k_host) {
         if (!std::isfinite(k_host[i])) return set_error(BLOCH_ENONFINITE, "wave vector has a non-finite component");
     Workspace<T>& w = ws_of<T>(pl);
     pl->k_host.assign(k_host, k_host + 3 * (size_t)nb);
-    BLOCH_CUDA_CHECK_RET(
-        cudaMemcpyAsync(w.kvec, k_host, sizeof(double) * 3 * nb, cudaMemcpyHostToDevice, pl->stream));
-    const int S = pl->Nx + pl->Ny + pl->Nz;
-    const int blocks = (int)std::min<long long>(1024, ((long long)nb * S + 255) / 256);
-    ++pl->launches;
-    k_qtab<T><<<blocks, 256, 0, pl->stream>>>(w.kvec, pl->d_xi, pl->Nx, pl->Ny, pl->Nz, nb, pl->qscale, w.qtab);
-    BLOCH_CUDA_CHECK_RET(cudaGetLastError());
-    return BLOCH_OK;
+    return launch_qtab<T>(pl, nb, k_host, w.kvec, w.qtab);
 }
 
 // ------------------------------------------------------------ operators
@@ -308,11 +320,9 @@ static void fast_yz(bloch_plan* pl, int axis, int DIR, int nfields, const cplx_t
     dim3 gr((npen + PT - 1) / PT, nfields);
     ++pl->launches;
     if (DIR > 0)
-        k_fpass_axis<T, +1, RA, RB, PT>
-            <<<gr, 256, smem, pl->stream>>>(in, out, tw_of<T>(pl, axis), g, inner, outer, npen, scale);
+        launch_pdl(k_fpass_axis<T, +1, RA, RB, PT>, gr, 256, smem, pl->stream, in, out, tw_of<T>(pl, axis), g, inner, outer, npen, scale);
     else
-        k_fpass_axis<T, -1, RA, RB, PT>
-            <<<gr, 256, smem, pl->stream>>>(in, out, tw_of<T>(pl, axis), g, inner, outer, npen, scale);
+        launch_pdl(k_fpass_axis<T, -1, RA, RB, PT>, gr, 256, smem, pl->stream, in, out, tw_of<T>(pl, axis), g, inner, outer, npen, scale);
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link to the driver library)
@@ -374,7 +384,7 @@ static void fast_z1(bloch_plan* pl, int nb, const float2* u, float2* E, const fl
     ++pl->launches;
     CUtensorMap map;
     const int tma = encode_zmap(&map, u, pl, 3LL * nb, P) ? 1 : 0;
-    k_fpass_z_strain<float, RA, RB, NT><<<gr, NT, fpass_z1_smem<float, RA, RB, NT>(), pl->stream>>>(
+    launch_pdl(k_fpass_z_strain<float, RA, RB, NT>, gr, NT, fpass_z1_smem<float, RA, RB, NT>(), pl->stream, 
         u, E, qtab, pl->d_twf[2], pl->geo_f, map, tma, sys);
 }
 
@@ -391,11 +401,9 @@ static int fast_z5(bloch_plan* pl, int nb, const float2* E, const float* qtab, f
     CUtensorMap map;
     const int tma = encode_zmap(&map, E, pl, 6LL * nb, P) ? 1 : 0;
     if (cg)
-        k_fpass_z_div<float, RA, RB, NT, true>
-            <<<gr, NT, smem, pl->stream>>>(E, nullptr, qtab, pl->d_twf[2], pl->geo_f, out_scale, map, tma, *cg);
+        launch_pdl(k_fpass_z_div<float, RA, RB, NT, true>, gr, NT, smem, pl->stream, E, nullptr, qtab, pl->d_twf[2], pl->geo_f, out_scale, map, tma, *cg);
     else
-        k_fpass_z_div<float, RA, RB, NT, false>
-            <<<gr, NT, smem, pl->stream>>>(E, out, qtab, pl->d_twf[2], pl->geo_f, out_scale, map, tma, 0);
+        launch_pdl(k_fpass_z_div<float, RA, RB, NT, false>, gr, NT, smem, pl->stream, E, out, qtab, pl->d_twf[2], pl->geo_f, out_scale, map, tma, 0);
     return (int)gr.x;
 }
 
@@ -406,7 +414,7 @@ static int fast_x3(bloch_plan* pl, int nb, float2* E, double2* dpart) {
     const long long rows = (long long)pl->Ny * pl->Nz;
     dim3 gr((unsigned)((rows + P - 1) / P), nb);
     ++pl->launches;
-    k_fpass_x_stress<float, RA, RB><<<gr, 128, fpass_x_smem<float, RA, RB>(), pl->stream>>>(
+    launch_pdl(k_fpass_x_stress<float, RA, RB>, gr, 128, fpass_x_smem<float, RA, RB>(), pl->stream, 
         E, pl->d_ids, pl->d_Cpf, pl->d_twf[0], pl->geo_f, dpart);
     return (int)gr.x;
 }
@@ -586,7 +594,7 @@ static void pcg_iteration(bloch_plan* pl, int nb, cplx_t<T>* x, double tol2, cud
         launch_K<T>(pl, nb, w.p, w.Ap, T(1));
         pl->launches += 3;
         k_dot_partial<T><<<gr, 256, 0, pl->stream>>>(w.p, w.Ap, 3 * pl->V, w.part2);
-        k_cg_alpha<<<nb, 256, 0, pl->stream>>>(w.part2, vblk, w.sys, 0, pl->d_nactive);
+        launch_pdl(k_cg_alpha, nb, 256, 0, pl->stream, w.part2, vblk, w.sys, 0, pl->d_nactive);
         k_cg_update<T><<<gr, 256, 0, pl->stream>>>(w.r, w.Ap, w.qtab, g, pl->pc, pl->psel, w.sys, w.part3);
     } else {
         // the passes skip converged systems
@@ -597,7 +605,7 @@ static void pcg_iteration(bloch_plan* pl, int nb, cplx_t<T>* x, double tol2, cud
         gk.skip_ncomp = 6;
         const int xblk = launch_stress<T>(pl, nb, w.p, w.E, w.qtab, w.partz, w.sys);
         ++pl->launches;
-        k_cg_alpha<<<nb, 256, 0, pl->stream>>>(w.partz, xblk, w.sys, scaled, pl->d_nactive);
+        launch_pdl(k_cg_alpha, nb, 256, 0, pl->stream, w.partz, xblk, w.sys, scaled, pl->d_nactive);
         const CgUpdate<T> cg{w.r, w.sys, w.part3, pl->pc, pl->psel};
         nblk = launch_z_div<T>(pl, nb, w.E, nullptr, w.qtab, T(1), &cg);
         gk.skip = nullptr;
@@ -607,9 +615,9 @@ static void pcg_iteration(bloch_plan* pl, int nb, cplx_t<T>* x, double tol2, cud
     pl->launches += 2;
     // residuals 16 (FP32) or 32 (FP64) digits below the start: past any recursive convergence
     const double rz_floor = std::is_same<T, float>::value ? 1e-32 : 1e-64;
-    k_cg_beta<<<nb, 256, 0, pl->stream>>>(w.part3, nblk, w.sys, tol2, rz_floor, scaled, pl->d_nactive,
+    launch_pdl(k_cg_beta, nb, 256, 0, pl->stream, w.part3, nblk, w.sys, tol2, rz_floor, scaled, pl->d_nactive,
                                           pl->d_iter + 1, h ? 1 : 0, h ? *h : cudaGraphConditionalHandle{}, pl->d_iter, max_iter);
-    k_cg_pupdate<T><<<gr, 256, 0, pl->stream>>>(w.r, w.p, x, w.qtab, g, pl->pc, pl->psel, w.sys);
+    launch_pdl(k_cg_pupdate<T>, gr, 256, 0, pl->stream, w.r, w.p, x, w.qtab, g, pl->pc, pl->psel, w.sys);
 }
 
 template <typename T>

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 // Float-float ("double-float") real: the unevaluated sum hi + lo of two
 // floats with |lo| <= ulp(hi)/2, a 48-bit significand evaluated on the FP32
 // pipes.  Sum and product are formed from the error-free transformations --
@@ -130,6 +132,32 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool sr
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
+
+// Programmatic dependent launch (sm_90 and later).  A kernel of the operator's
+// chain lets its successor start when its own CTAs have all begun
+// (pdl_launch), and does its set-up (twiddle tables, barriers) before it waits
+// for its predecessor's results (pdl_wait, before anything but constant tables is
+// touched).  Small cells are bound by the launches: a K-apply of 16^3 is six
+// kernels of a few microseconds.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... KA, typename... A>
+inline void launch_pdl(void (*k)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A&&... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = stream;
+    c.attrs = at;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, k, static_cast<KA>(std::forward<A>(args))...);
+}
+#endif
 
 // Let launches of kernel k request the device's whole opt-in shared memory
 // per block, less what k declares statically.

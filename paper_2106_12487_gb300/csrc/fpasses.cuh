@@ -76,11 +76,13 @@ __global__ void __launch_bounds__(256) k_fpass_axis(const cplx_t<T>* in, cplx_t<
     C* buf = tw + kTwLen<RA, RB>;
     const int tid = threadIdx.x;
     const unsigned pi0 = blockIdx.x * PT;
+    pdl_launch();
+    tw_fill<RB, RA>(tw, twa, tid, NT);
+    pdl_wait();
     if (sys_idle(g, (int)blockIdx.y / g.skip_ncomp)) return;
     const size_t off = (size_t)blockIdx.y * g.V;
     const C* src = in + off;
     C* dst = out + off;
-    tw_fill<RB, RA>(tw, twa, tid, NT);
 #pragma unroll
     for (int t = tid; t < PT * RB; t += NT) {
         const int p = t % PT, j = t / PT;
@@ -153,15 +155,16 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>
     C* bufB = bufA + NP;      // NP
     const int tid = threadIdx.x;
     const int b = blockIdx.y;
-    if (sys_idle(g, b)) return;
-    if (use_tma) {
-        if (tid == 0) {
-            mbar_init(smem_u32(&zbar[0]), 1);
-            mbar_init(smem_u32(&zbar[1]), 1);
-            fence_mbar_init();
-        }
-        __syncthreads();
+    pdl_launch();
+    if (use_tma && tid == 0) {
+        mbar_init(smem_u32(&zbar[0]), 1);
+        mbar_init(smem_u32(&zbar[1]), 1);
+        fence_mbar_init();
     }
+    tw_fill<RB, RA>(tw, twz, tid, NT);
+    pdl_wait();
+    if (sys_idle(g, b)) return;
+    __syncthreads();
     const unsigned plane = (unsigned)g.Nx * (unsigned)g.Ny;
     const unsigned pi0 = blockIdx.x * P;
     const int np = (int)min((unsigned)P, plane - pi0);
@@ -207,7 +210,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>
     };
     stage_in(2, 0);
     stage_in(0, 1);
-    tw_fill<RB, RA>(tw, twz, tid, NT);
     const int p2 = tid % P, j2 = tid / P;
     const unsigned pi = pi0 + (p2 < np ? p2 : 0);
     const T sc = sys ? cg_scale<T>(sys, b) : T(1);   // every strain is linear in q: scaling q scales them all
@@ -336,15 +338,16 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* _
     C* xb = stg + NSTG * NP;     // (pair ? 2 : 1) x NP exchange
     const int tid = threadIdx.x;
     const int b = blockIdx.y;
-    if (sys_idle(g, b)) return;
-    if (use_tma) {
-        if (tid == 0) {
+    pdl_launch();
+    if (use_tma && tid == 0) {
 #pragma unroll
-            for (int i = 0; i < NSTG; ++i) mbar_init(smem_u32(&zbar[i]), 1);
-            fence_mbar_init();
-        }
-        __syncthreads();
+        for (int i = 0; i < NSTG; ++i) mbar_init(smem_u32(&zbar[i]), 1);
+        fence_mbar_init();
     }
+    tw_fill<RB, RA>(tw, twz, tid, NT);
+    pdl_wait();
+    if (sys_idle(g, b)) return;
+    __syncthreads();
     const unsigned plane = (unsigned)g.Nx * (unsigned)g.Ny;
     const unsigned pi0 = blockIdx.x * P;
     const int np = (int)min((unsigned)P, plane - pi0);
@@ -389,7 +392,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* _
     };
 #pragma unroll
     for (int c = 0; c < NSTG; ++c) stage_in(c, c);
-    tw_fill<RB, RA>(tw, twz, tid, NT);
     const int p2 = tid % P, j2 = tid / P;
     const unsigned pi = pi0 + (p2 < np ? p2 : 0);
     const T qv[2] = {qxt[pi % (unsigned)g.Nx], qyt[pi / (unsigned)g.Nx]};
@@ -598,8 +600,6 @@ __device__ __forceinline__ void x_stress_single(cplx_t<T>* E, const int32_t* __r
     };
     prefetch(0, stg);
     prefetch(1, stg + P * LD);
-    tw_fill<RB, RA>(tw, twx, tid, 128);
-    tw_fill<RA, RB>(tw1, twx, tid, 128);
     // stage-2 task of this thread
     const int j2 = tid % RA, p2 = tid / RA;
     const bool own = p2 < nr;
@@ -729,8 +729,6 @@ __device__ __forceinline__ void x_stress_paired(cplx_t<T>* E, const int32_t* __r
     prefetch(2, stg + 2 * P * LD);
     prefetch(3, stg + 3 * P * LD);
     cp_async_commit();
-    tw_fill<RB, RA>(tw, twx, tid, 128);
-    tw_fill<RA, RB>(tw1, twx, tid, 128);
     const int half = tid >> 6;              // radix-RA stage: component 2m + half
     const int j1 = (tid & 63) % RB, p1 = (tid & 63) / RB;
     const int j2 = tid % RA, p2 = tid / RA; // radix-RB stage and the stress: one task per thread
@@ -851,6 +849,14 @@ __global__ void __launch_bounds__(128, 4) k_fpass_x_stress(cplx_t<T>* E, const i
                                                            const T* __restrict__ Cpk,
                                                            const cplx_t<T>* __restrict__ twx, Geo g,
                                                            double2* __restrict__ dpart) {
+    pdl_launch();
+    {
+        extern __shared__ __align__(16) unsigned char smem_raw[];
+        cplx_t<T>* tw = reinterpret_cast<cplx_t<T>*>(smem_raw);
+        tw_fill<RB, RA>(tw, twx, threadIdx.x, 128);
+        tw_fill<RA, RB>(tw + kTwLen<RA, RB>, twx, threadIdx.x, 128);
+    }
+    pdl_wait();
     if (sys_idle(g, blockIdx.y)) return;
     if (dpart) dpart += (size_t)blockIdx.y * gridDim.x + blockIdx.x;
     if constexpr ((128 / RA) * RB == 64)

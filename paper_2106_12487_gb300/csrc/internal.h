@@ -211,6 +211,9 @@ template <typename T> bloch_status ensure_ws(bloch_plan* pl, int nb);
 template <typename T> bloch_status ensure_cg(bloch_plan* pl, int nb);
 // Upload nb wave vectors (host, rad/m) and build the scaled q tables.
 template <typename T> bloch_status set_k(bloch_plan* pl, int nb, const double* k_host);
+// Scaled q tables of nb wave vectors (host, rad/m); kvec: device room for them.
+template <typename T>
+bloch_status launch_qtab(bloch_plan* pl, int nb, const double* k_host, double* kvec, T* qtab);
 // Scaled stiffness operator on nb systems whose q tables are set: out = out_scale * A~ u.
 template <typename T> void launch_K(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* out, T out_scale);
 // The FP32 operator on scratch E and q tables of the caller (launch_K's chain).

@@ -254,7 +254,6 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     C* buf = tw + pad_even(ntw);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int b = blockIdx.y;
-    if (sys_idle(g, b)) return;
     const unsigned plane = (unsigned)g.Nx * (unsigned)g.Ny;
     const unsigned pi0 = blockIdx.x << lp;
     const int np = (int)min((unsigned)P1 + 1u, plane - pi0);
@@ -265,14 +264,17 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     const T* qz = qy + g.Ny;
     // FP32 conjugate gradients: every strain is linear in q, so scaling q scales them all
     T sc = T(1);
-    if constexpr (sizeof(T) == 4) {
-        if (sys) sc = cg_scale<T>(sys, b);
-    }
     auto qs = [&](T q) {
         if constexpr (sizeof(T) == 4) return q * sc;
         else return q;
     };
+    pdl_launch();
     for (int i = tid; i < ntw; i += nthr) tw[i] = twz[i];
+    pdl_wait();
+    if (sys_idle(g, b)) return;
+    if constexpr (sizeof(T) == 4) {
+        if (sys) sc = cg_scale<T>(sys, b);
+    }
     __syncthreads();
     with_radix<real_t<C>, WIDE>(a.r1, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
@@ -357,7 +359,6 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     const int ntw = twtab_len(a);
     C* buf = tw + pad_even(ntw);
     const int tid = threadIdx.x, nthr = blockDim.x;
-    if (sys_idle(g, (int)blockIdx.y / g.skip_ncomp)) return;
     const unsigned nx = (unsigned)g.Nx, plane = nx * (unsigned)g.Ny;
     const unsigned step = AXIS == 1 ? nx : plane;     // between the elements of a pencil
     const unsigned npen = AXIS == 1 ? nx * (unsigned)g.Nz : plane;
@@ -370,7 +371,10 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
         const unsigned z = fdiv(pi, g.dx);
         return (size_t)z * plane + (pi - z * nx);
     };
+    pdl_launch();
     for (int i = tid; i < ntw; i += nthr) tw[i] = twa[i];
+    pdl_wait();
+    if (sys_idle(g, (int)blockIdx.y / g.skip_ncomp)) return;
     __syncthreads();
     with_radix<real_t<C>, WIDE>(a.r1, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
@@ -430,7 +434,6 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     C* buf = tw + pad_even(ntw);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int b = blockIdx.y;
-    if (sys_idle(g, b)) return;
     const unsigned plane = (unsigned)g.Nx * (unsigned)g.Ny;
     const unsigned pi0 = blockIdx.x << lp;
     const int np = (int)min((unsigned)P1 + 1u, plane - pi0);
@@ -439,15 +442,20 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     T alpha = T(0), sc = T(1), acc[2] = {T(0), T(0)};
     if constexpr (CG) {
         ob = cg.r + (size_t)b * 3 * g.V;
-        sc = cg_scale<T>(cg.sys, b);
-        alpha = T(cg.sys[b].alpha / (double)sc);
     } else {
         ob = out + (size_t)b * 3 * g.V;
     }
     const T* qx = qtab + (size_t)b * (g.Nx + g.Ny + g.Nz);
     const T* qy = qx + g.Nx;
     const T* qz = qy + g.Ny;
+    pdl_launch();
     for (int i = tid; i < ntw; i += nthr) tw[i] = twz[i];
+    pdl_wait();
+    if (sys_idle(g, b)) return;
+    if constexpr (CG) {
+        sc = cg_scale<T>(cg.sys, b);
+        alpha = T(cg.sys[b].alpha / (double)sc);
+    }
     __syncthreads();
     with_radix<real_t<C>, WIDE>(a.r1, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
@@ -671,12 +679,14 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     C* buf = tw + pad_even(ntw);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int b = blockIdx.y;
-    if (sys_idle(g, b)) return;
     const unsigned rows = (unsigned)g.Ny * (unsigned)g.Nz;
     const unsigned r0 = blockIdx.x * (unsigned)P;
     const int nr = (int)min((unsigned)P, rows - r0);
     C* Wb = W + (size_t)b * NC * g.V;
+    pdl_launch();
     for (int i = tid; i < ntw; i += nthr) tw[i] = twx[i];
+    pdl_wait();
+    if (sys_idle(g, b)) return;
     __syncthreads();
     lf_first<+1, WIDE>(Wb, g.V, buf, NC, a, P, nr, r0, tw, tid, nthr);
     __syncthreads();
@@ -730,12 +740,14 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     C* buf = tw + pad_even(ntw);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int b = blockIdx.y;
-    if (sys_idle(g, b)) return;
     const unsigned rows = (unsigned)g.Ny * (unsigned)g.Nz;
     const unsigned r0 = blockIdx.x * (unsigned)P;
     const int nr = (int)min((unsigned)P, rows - r0);
     C* Wb = W + (size_t)b * 3 * g.V;
+    pdl_launch();
     for (int i = tid; i < ntw; i += nthr) tw[i] = twx[i];
+    pdl_wait();
+    if (sys_idle(g, b)) return;
     __syncthreads();
     lf_first<DIR, WIDE>(Wb, g.V, buf, 3, a, P, nr, r0, tw, tid, nthr);
     __syncthreads();

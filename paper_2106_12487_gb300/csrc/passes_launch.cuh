@@ -48,8 +48,7 @@ void pass_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, con
     const PassTile t = pass_tile<T>(pl, PASS_Z6, nb);
     ++pl->launches;
     with_width<T>(pl, 2, [&](auto w) {
-        k_pass_z_strain<T, decltype(w)::value>
-            <<<pass_grid((long long)pl->Nx * pl->Ny, t.lp, nb), t.nthr, t.smem, pl->stream>>>(
+        launch_pdl(k_pass_z_strain<T, decltype(w)::value>, pass_grid((long long)pl->Nx * pl->Ny, t.lp, nb), t.nthr, t.smem, pl->stream, 
                 u, E, qtab, pass_tw<T>(pl, 2), geo_of<T>(pl), t.lp, sys);
     });
 }
@@ -64,13 +63,13 @@ void pass_axis(bloch_plan* pl, int axis, int dir, int nfields, const cplx_t<T>* 
     with_width<T>(pl, axis, [&](auto w) {
         constexpr bool W = decltype(w)::value;
         if (axis == 1 && dir > 0)
-            k_pass_axis<T, +1, 1, W><<<gr, t.nthr, t.smem, pl->stream>>>(in, out, tw, g, t.lp, out_scale);
+            launch_pdl(k_pass_axis<T, +1, 1, W>, gr, t.nthr, t.smem, pl->stream, in, out, tw, g, t.lp, out_scale);
         else if (axis == 1)
-            k_pass_axis<T, -1, 1, W><<<gr, t.nthr, t.smem, pl->stream>>>(in, out, tw, g, t.lp, out_scale);
+            launch_pdl(k_pass_axis<T, -1, 1, W>, gr, t.nthr, t.smem, pl->stream, in, out, tw, g, t.lp, out_scale);
         else if (dir > 0)
-            k_pass_axis<T, +1, 2, W><<<gr, t.nthr, t.smem, pl->stream>>>(in, out, tw, g, t.lp, out_scale);
+            launch_pdl(k_pass_axis<T, +1, 2, W>, gr, t.nthr, t.smem, pl->stream, in, out, tw, g, t.lp, out_scale);
         else
-            k_pass_axis<T, -1, 2, W><<<gr, t.nthr, t.smem, pl->stream>>>(in, out, tw, g, t.lp, out_scale);
+            launch_pdl(k_pass_axis<T, -1, 2, W>, gr, t.nthr, t.smem, pl->stream, in, out, tw, g, t.lp, out_scale);
     });
 }
 
@@ -80,7 +79,7 @@ int pass_x_stress(bloch_plan* pl, int nb, cplx_t<T>* E, double2* dpart) {
     const dim3 gr = pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb);
     ++pl->launches;
     with_width<T>(pl, 0, [&](auto w) {
-        k_pass_x_grain<T, 6, decltype(w)::value><<<gr, t.nthr, t.smem, pl->stream>>>(
+        launch_pdl(k_pass_x_grain<T, 6, decltype(w)::value>, gr, t.nthr, t.smem, pl->stream, 
             E, pl->d_ids, pass_ctab<T>(pl), pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp, dpart);
     });
     return (int)gr.x;
@@ -91,8 +90,7 @@ void pass_x_rho(bloch_plan* pl, int nb, cplx_t<T>* W) {
     const PassTile t = pass_tile<T>(pl, PASS_X3, nb);
     ++pl->launches;
     with_width<T>(pl, 0, [&](auto w) {
-        k_pass_x_grain<T, 3, decltype(w)::value>
-            <<<pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb), t.nthr, t.smem, pl->stream>>>(
+        launch_pdl(k_pass_x_grain<T, 3, decltype(w)::value>, pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb), t.nthr, t.smem, pl->stream, 
                 W, pl->d_ids, pass_rtab<T>(pl), pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp, nullptr);
     });
 }
@@ -107,9 +105,9 @@ void pass_x(bloch_plan* pl, int dir, int nb, cplx_t<T>* W, T out_scale, const do
     with_width<T>(pl, 0, [&](auto w) {
         constexpr bool WD = decltype(w)::value;
         if (dir > 0)
-            k_pass_x<T, +1, WD><<<gr, t.nthr, t.smem, pl->stream>>>(W, tw, g, 1 << t.lp, out_scale, ph, per);
+            launch_pdl(k_pass_x<T, +1, WD>, gr, t.nthr, t.smem, pl->stream, W, tw, g, 1 << t.lp, out_scale, ph, per);
         else
-            k_pass_x<T, -1, WD><<<gr, t.nthr, t.smem, pl->stream>>>(W, tw, g, 1 << t.lp, out_scale, ph, per);
+            launch_pdl(k_pass_x<T, -1, WD>, gr, t.nthr, t.smem, pl->stream, W, tw, g, 1 << t.lp, out_scale, ph, per);
     });
 }
 
@@ -123,13 +121,12 @@ int pass_z_div(bloch_plan* pl, int nb, const cplx_t<T>* E, cplx_t<T>* out, const
         constexpr bool W = decltype(w)::value;
         if constexpr (!std::is_same<T, dfloat>::value) {
             if (cg) {
-                k_pass_z_div<T, W, true><<<gr, t.nthr, t.smem, pl->stream>>>(E, nullptr, qtab, pass_tw<T>(pl, 2),
+                launch_pdl(k_pass_z_div<T, W, true>, gr, t.nthr, t.smem, pl->stream, E, nullptr, qtab, pass_tw<T>(pl, 2),
                                                                              geo_of<T>(pl), t.lp, out_scale, *cg);
                 return;
             }
         }
-        k_pass_z_div<T, W, false>
-            <<<gr, t.nthr, t.smem, pl->stream>>>(E, out, qtab, pass_tw<T>(pl, 2), geo_of<T>(pl), t.lp, out_scale, 0);
+        launch_pdl(k_pass_z_div<T, W, false>, gr, t.nthr, t.smem, pl->stream, E, out, qtab, pass_tw<T>(pl, 2), geo_of<T>(pl), t.lp, out_scale, 0);
     });
     return (int)gr.x;
 }

@@ -11,17 +11,27 @@
 
 namespace bloch {
 
-// qtab[b][.] = ((xi + k_b) * qscale) for the x, y and z axes.
+// Wave vectors of a small batch, passed as kernel arguments: no copy to the
+// device precedes the operator.
+constexpr int kParamWaves = 32;
+struct WaveParams {
+    double k[3 * kParamWaves];
+};
+
+// qtab[b][.] = ((xi + k_b) * qscale) for the x, y and z axes; k_b from kvec or,
+// with kvec == nullptr, from wp.
 template <typename T>
-__global__ void k_qtab(const double* __restrict__ kvec, const double* __restrict__ xi, int Nx, int Ny, int Nz,
-                       int nb, double qscale, T* __restrict__ qtab) {
+__global__ void k_qtab(const double* __restrict__ kvec, const __grid_constant__ WaveParams wp,
+                       const double* __restrict__ xi, int Nx, int Ny, int Nz, int nb, double qscale,
+                       T* __restrict__ qtab) {
+    pdl_launch();
     const int S = Nx + Ny + Nz;
     const long long total = (long long)nb * S;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
         const int b = (int)(i / S), j = (int)(i % S);
         const int ax = j < Nx ? 0 : (j < Nx + Ny ? 1 : 2);
-        qtab[i] = T((xi[j] + kvec[3 * b + ax]) * qscale);
+        qtab[i] = T((xi[j] + (kvec ? kvec : wp.k)[3 * b + ax]) * qscale);
     }
 }
 
@@ -188,6 +198,8 @@ __global__ void k_cg_pupdate(const cplx_t<T>* __restrict__ r, cplx_t<T>* __restr
                              const T* __restrict__ qtab, Geo g, PrecondCoef pc, PrecondSel ps, const CGSys* sys) {
     using C = cplx_t<T>;
     const int b = blockIdx.y;
+    pdl_launch();
+    pdl_wait();
     if (!sys[b].upd) return;
     const bool act = sys[b].active != 0;
     const size_t off = (size_t)b * 3 * g.V;
@@ -245,6 +257,8 @@ static __global__ void k_cg_start(const double* partial3, int nblk, CGSys* sys, 
 // scaled: the sums carry the square of cg_scale (here and in k_cg_beta).
 static __global__ void k_cg_alpha(const double2* partial2, int nblk, CGSys* sys, int scaled, int* n_active) {
     const int b = blockIdx.x;
+    pdl_launch();
+    pdl_wait();
     CGSys& s = sys[b];
     double acc[1] = {0.0};
     if (s.active)
@@ -270,6 +284,8 @@ static __global__ void k_cg_alpha(const double2* partial2, int nblk, CGSys* sys,
 static __global__ void k_cg_beta(const double* partial3, int nblk, CGSys* sys, double tol2, double rz_floor, int scaled,
                                  int* n_active, int* ticket, int cond, cudaGraphConditionalHandle h, int* iter, int max_iter) {
     const int b = blockIdx.x;
+    pdl_launch();
+    pdl_wait();
     CGSys& s = sys[b];
     double acc[2] = {0.0, 0.0};
     const int active = s.active;
