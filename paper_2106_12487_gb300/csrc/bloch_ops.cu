@@ -320,9 +320,11 @@ static void fast_yz(bloch_plan* pl, int axis, int DIR, int nfields, const cplx_t
     dim3 gr((npen + PT - 1) / PT, nfields);
     ++pl->launches;
     if (DIR > 0)
-        launch_pdl(k_fpass_axis<T, +1, RA, RB, PT>, gr, 256, smem, pl->stream, in, out, tw_of<T>(pl, axis), g, inner, outer, npen, scale);
+        launch_pdl(k_fpass_axis<T, +1, RA, RB, PT>, gr, 256, smem, pl->stream, in, out, tw_of<T>(pl, axis), g,
+                   inner, outer, npen, scale);
     else
-        launch_pdl(k_fpass_axis<T, -1, RA, RB, PT>, gr, 256, smem, pl->stream, in, out, tw_of<T>(pl, axis), g, inner, outer, npen, scale);
+        launch_pdl(k_fpass_axis<T, -1, RA, RB, PT>, gr, 256, smem, pl->stream, in, out, tw_of<T>(pl, axis), g,
+                   inner, outer, npen, scale);
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link to the driver library)
@@ -384,8 +386,8 @@ static void fast_z1(bloch_plan* pl, int nb, const float2* u, float2* E, const fl
     ++pl->launches;
     CUtensorMap map;
     const int tma = encode_zmap(&map, u, pl, 3LL * nb, P) ? 1 : 0;
-    launch_pdl(k_fpass_z_strain<float, RA, RB, NT>, gr, NT, fpass_z1_smem<float, RA, RB, NT>(), pl->stream, 
-        u, E, qtab, pl->d_twf[2], pl->geo_f, map, tma, sys);
+    launch_pdl(k_fpass_z_strain<float, RA, RB, NT>, gr, NT, fpass_z1_smem<float, RA, RB, NT>(), pl->stream, u, E,
+               qtab, pl->d_twf[2], pl->geo_f, map, tma, sys);
 }
 
 // returns the CTAs per system
@@ -401,9 +403,11 @@ static int fast_z5(bloch_plan* pl, int nb, const float2* E, const float* qtab, f
     CUtensorMap map;
     const int tma = encode_zmap(&map, E, pl, 6LL * nb, P) ? 1 : 0;
     if (cg)
-        launch_pdl(k_fpass_z_div<float, RA, RB, NT, true>, gr, NT, smem, pl->stream, E, nullptr, qtab, pl->d_twf[2], pl->geo_f, out_scale, map, tma, *cg);
+        launch_pdl(k_fpass_z_div<float, RA, RB, NT, true>, gr, NT, smem, pl->stream, E, nullptr, qtab, pl->d_twf[2],
+                   pl->geo_f, out_scale, map, tma, *cg);
     else
-        launch_pdl(k_fpass_z_div<float, RA, RB, NT, false>, gr, NT, smem, pl->stream, E, out, qtab, pl->d_twf[2], pl->geo_f, out_scale, map, tma, 0);
+        launch_pdl(k_fpass_z_div<float, RA, RB, NT, false>, gr, NT, smem, pl->stream, E, out, qtab, pl->d_twf[2],
+                   pl->geo_f, out_scale, map, tma, 0);
     return (int)gr.x;
 }
 
@@ -414,8 +418,8 @@ static int fast_x3(bloch_plan* pl, int nb, float2* E, double2* dpart) {
     const long long rows = (long long)pl->Ny * pl->Nz;
     dim3 gr((unsigned)((rows + P - 1) / P), nb);
     ++pl->launches;
-    launch_pdl(k_fpass_x_stress<float, RA, RB>, gr, 128, fpass_x_smem<float, RA, RB>(), pl->stream, 
-        E, pl->d_ids, pl->d_Cpf, pl->d_twf[0], pl->geo_f, dpart);
+    launch_pdl(k_fpass_x_stress<float, RA, RB>, gr, 128, fpass_x_smem<float, RA, RB>(), pl->stream, E,
+               pl->d_ids, pl->d_Cpf, pl->d_twf[0], pl->geo_f, dpart);
     return (int)gr.x;
 }
 
@@ -616,7 +620,7 @@ static void pcg_iteration(bloch_plan* pl, int nb, cplx_t<T>* x, double tol2, cud
     // residuals 16 (FP32) or 32 (FP64) digits below the start: past any recursive convergence
     const double rz_floor = std::is_same<T, float>::value ? 1e-32 : 1e-64;
     launch_pdl(k_cg_beta, nb, 256, 0, pl->stream, w.part3, nblk, w.sys, tol2, rz_floor, scaled, pl->d_nactive,
-                                          pl->d_iter + 1, h ? 1 : 0, h ? *h : cudaGraphConditionalHandle{}, pl->d_iter, max_iter);
+               pl->d_iter + 1, h ? 1 : 0, h ? *h : cudaGraphConditionalHandle{}, pl->d_iter, max_iter);
     launch_pdl(k_cg_pupdate<T>, gr, 256, 0, pl->stream, w.r, w.p, x, w.qtab, g, pl->pc, pl->psel, w.sys);
 }
 

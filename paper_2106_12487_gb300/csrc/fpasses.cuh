@@ -76,9 +76,9 @@ __global__ void __launch_bounds__(256) k_fpass_axis(const cplx_t<T>* in, cplx_t<
     C* buf = tw + kTwLen<RA, RB>;
     const int tid = threadIdx.x;
     const unsigned pi0 = blockIdx.x * PT;
-    pdl_launch();
     tw_fill<RB, RA>(tw, twa, tid, NT);
     pdl_wait();
+    pdl_launch();
     if (sys_idle(g, (int)blockIdx.y / g.skip_ncomp)) return;
     const size_t off = (size_t)blockIdx.y * g.V;
     const C* src = in + off;
@@ -155,7 +155,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>
     C* bufB = bufA + NP;      // NP
     const int tid = threadIdx.x;
     const int b = blockIdx.y;
-    pdl_launch();
     if (use_tma && tid == 0) {
         mbar_init(smem_u32(&zbar[0]), 1);
         mbar_init(smem_u32(&zbar[1]), 1);
@@ -163,6 +162,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>
     }
     tw_fill<RB, RA>(tw, twz, tid, NT);
     pdl_wait();
+    pdl_launch();
     if (sys_idle(g, b)) return;
     __syncthreads();
     const unsigned plane = (unsigned)g.Nx * (unsigned)g.Ny;
@@ -338,7 +338,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* _
     C* xb = stg + NSTG * NP;     // (pair ? 2 : 1) x NP exchange
     const int tid = threadIdx.x;
     const int b = blockIdx.y;
-    pdl_launch();
     if (use_tma && tid == 0) {
 #pragma unroll
         for (int i = 0; i < NSTG; ++i) mbar_init(smem_u32(&zbar[i]), 1);
@@ -346,6 +345,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* _
     }
     tw_fill<RB, RA>(tw, twz, tid, NT);
     pdl_wait();
+    pdl_launch();
     if (sys_idle(g, b)) return;
     __syncthreads();
     const unsigned plane = (unsigned)g.Nx * (unsigned)g.Ny;
@@ -849,7 +849,6 @@ __global__ void __launch_bounds__(128, 4) k_fpass_x_stress(cplx_t<T>* E, const i
                                                            const T* __restrict__ Cpk,
                                                            const cplx_t<T>* __restrict__ twx, Geo g,
                                                            double2* __restrict__ dpart) {
-    pdl_launch();
     {
         extern __shared__ __align__(16) unsigned char smem_raw[];
         cplx_t<T>* tw = reinterpret_cast<cplx_t<T>*>(smem_raw);
@@ -857,6 +856,7 @@ __global__ void __launch_bounds__(128, 4) k_fpass_x_stress(cplx_t<T>* E, const i
         tw_fill<RA, RB>(tw + kTwLen<RA, RB>, twx, threadIdx.x, 128);
     }
     pdl_wait();
+    pdl_launch();
     if (sys_idle(g, blockIdx.y)) return;
     if (dpart) dpart += (size_t)blockIdx.y * gridDim.x + blockIdx.x;
     if constexpr ((128 / RA) * RB == 64)

@@ -35,9 +35,9 @@
 //
 // Against the Stockham form these passes had before (tiles copied in, between
 // two buffers per stage and out; odd radices with run-time sines), K-apply:
-//   120 x 100 x 84, FP32, 6 systems   14.30 -> 0.76 ms
-//   256^3, FP32, 2 systems            14.26 -> 4.14 ms
-//   64^3, FP64, 4 systems              1.73 -> 1.48 ms (bound by FP64 issue)
+//   120 x 100 x 84, FP32, 6 systems   14.30 -> 0.66 ms
+//   256^3, FP32, 2 systems            14.26 -> 3.76 ms
+//   64^3, FP64, 4 systems              1.73 -> 1.51 ms (bound by FP64 issue)
 //   128^3, float-float, 4 systems      7.92 -> 4.62 ms (bound by FP32 issue)
 #pragma once
 
@@ -131,6 +131,9 @@ __host__ __device__ __forceinline__ int xrow(const AxisPlan& a) { return (a.r1 *
 // 735 us with three, 680 with four; 256^3 (16 x 16): 3.79 ms with three, 4.27
 // with four.
 template <typename T, bool WIDE> constexpr int kPassCtas = sizeof(T) != 4 ? 2 : WIDE ? 3 : 4;
+// the wide z passes' six-buffer tiles admit two CTAs anyway (256^3: 3.99 ms with
+// registers for three, which spill, 3.78 with two)
+template <typename T, bool WIDE> constexpr int kPassCtasZ = sizeof(T) != 4 || WIDE ? 2 : 4;
 
 // f(std::integral_constant<int, R>) for the run-time radix R.  Float-float
 // leaves out the radices whose code is longest for what they save (compile time).
@@ -242,7 +245,7 @@ __device__ __forceinline__ void pf_last(C* buf, int nbuf, const AxisPlan& a, int
 //   g_xz = q_x a_z + b_x, g_xy = q_y a_x + q_x a_y
 // (q_x and q_y are constant on a z pencil).
 template <typename T, bool WIDE>
-__global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
+__global__ void __launch_bounds__(256, kPassCtasZ<T, WIDE>)
     k_pass_z_strain(const cplx_t<T>* __restrict__ U, cplx_t<T>* __restrict__ E, const T* __restrict__ qtab,
                     const cplx_t<T>* __restrict__ twz, Geo g, int lp, const CGSys* __restrict__ sys) {
     using C = cplx_t<T>;
@@ -268,9 +271,9 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
         if constexpr (sizeof(T) == 4) return q * sc;
         else return q;
     };
-    pdl_launch();
     for (int i = tid; i < ntw; i += nthr) tw[i] = twz[i];
     pdl_wait();
+    pdl_launch();
     if (sys_idle(g, b)) return;
     if constexpr (sizeof(T) == 4) {
         if (sys) sc = cg_scale<T>(sys, b);
@@ -371,9 +374,9 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
         const unsigned z = fdiv(pi, g.dx);
         return (size_t)z * plane + (pi - z * nx);
     };
-    pdl_launch();
     for (int i = tid; i < ntw; i += nthr) tw[i] = twa[i];
     pdl_wait();
+    pdl_launch();
     if (sys_idle(g, (int)blockIdx.y / g.skip_ncomp)) return;
     __syncthreads();
     with_radix<real_t<C>, WIDE>(a.r1, [&](auto rc) {
@@ -421,7 +424,7 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
 // With CG the divergence A p is not stored: the residual of the conjugate
 // gradients is updated with it in place (CgUpdate).
 template <typename T, bool WIDE, bool CG>
-__global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
+__global__ void __launch_bounds__(256, kPassCtasZ<T, WIDE>)
     k_pass_z_div(const cplx_t<T>* __restrict__ E, cplx_t<T>* __restrict__ out, const T* __restrict__ qtab,
                  const cplx_t<T>* __restrict__ twz, Geo g, int lp, T out_scale,
                  const __grid_constant__ std::conditional_t<CG, CgUpdate<T>, int> cg) {
@@ -448,9 +451,9 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     const T* qx = qtab + (size_t)b * (g.Nx + g.Ny + g.Nz);
     const T* qy = qx + g.Nx;
     const T* qz = qy + g.Ny;
-    pdl_launch();
     for (int i = tid; i < ntw; i += nthr) tw[i] = twz[i];
     pdl_wait();
+    pdl_launch();
     if (sys_idle(g, b)) return;
     if constexpr (CG) {
         sc = cg_scale<T>(cg.sys, b);
@@ -683,9 +686,9 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     const unsigned r0 = blockIdx.x * (unsigned)P;
     const int nr = (int)min((unsigned)P, rows - r0);
     C* Wb = W + (size_t)b * NC * g.V;
-    pdl_launch();
     for (int i = tid; i < ntw; i += nthr) tw[i] = twx[i];
     pdl_wait();
+    pdl_launch();
     if (sys_idle(g, b)) return;
     __syncthreads();
     lf_first<+1, WIDE>(Wb, g.V, buf, NC, a, P, nr, r0, tw, tid, nthr);
@@ -744,9 +747,9 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     const unsigned r0 = blockIdx.x * (unsigned)P;
     const int nr = (int)min((unsigned)P, rows - r0);
     C* Wb = W + (size_t)b * 3 * g.V;
-    pdl_launch();
     for (int i = tid; i < ntw; i += nthr) tw[i] = twx[i];
     pdl_wait();
+    pdl_launch();
     if (sys_idle(g, b)) return;
     __syncthreads();
     lf_first<DIR, WIDE>(Wb, g.V, buf, 3, a, P, nr, r0, tw, tid, nthr);

@@ -48,7 +48,8 @@ void pass_z_strain(bloch_plan* pl, int nb, const cplx_t<T>* u, cplx_t<T>* E, con
     const PassTile t = pass_tile<T>(pl, PASS_Z6, nb);
     ++pl->launches;
     with_width<T>(pl, 2, [&](auto w) {
-        launch_pdl(k_pass_z_strain<T, decltype(w)::value>, pass_grid((long long)pl->Nx * pl->Ny, t.lp, nb), t.nthr, t.smem, pl->stream, 
+        launch_pdl(k_pass_z_strain<T, decltype(w)::value>, pass_grid((long long)pl->Nx * pl->Ny, t.lp, nb), t.nthr,
+                   t.smem, pl->stream,
                 u, E, qtab, pass_tw<T>(pl, 2), geo_of<T>(pl), t.lp, sys);
     });
 }
@@ -79,7 +80,7 @@ int pass_x_stress(bloch_plan* pl, int nb, cplx_t<T>* E, double2* dpart) {
     const dim3 gr = pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb);
     ++pl->launches;
     with_width<T>(pl, 0, [&](auto w) {
-        launch_pdl(k_pass_x_grain<T, 6, decltype(w)::value>, gr, t.nthr, t.smem, pl->stream, 
+        launch_pdl(k_pass_x_grain<T, 6, decltype(w)::value>, gr, t.nthr, t.smem, pl->stream,
             E, pl->d_ids, pass_ctab<T>(pl), pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp, dpart);
     });
     return (int)gr.x;
@@ -90,7 +91,8 @@ void pass_x_rho(bloch_plan* pl, int nb, cplx_t<T>* W) {
     const PassTile t = pass_tile<T>(pl, PASS_X3, nb);
     ++pl->launches;
     with_width<T>(pl, 0, [&](auto w) {
-        launch_pdl(k_pass_x_grain<T, 3, decltype(w)::value>, pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb), t.nthr, t.smem, pl->stream, 
+        launch_pdl(k_pass_x_grain<T, 3, decltype(w)::value>, pass_grid((long long)pl->Ny * pl->Nz, t.lp, nb),
+                   t.nthr, t.smem, pl->stream,
                 W, pl->d_ids, pass_rtab<T>(pl), pass_tw<T>(pl, 0), geo_of<T>(pl), 1 << t.lp, nullptr);
     });
 }
@@ -121,12 +123,14 @@ int pass_z_div(bloch_plan* pl, int nb, const cplx_t<T>* E, cplx_t<T>* out, const
         constexpr bool W = decltype(w)::value;
         if constexpr (!std::is_same<T, dfloat>::value) {
             if (cg) {
-                launch_pdl(k_pass_z_div<T, W, true>, gr, t.nthr, t.smem, pl->stream, E, nullptr, qtab, pass_tw<T>(pl, 2),
+                launch_pdl(k_pass_z_div<T, W, true>, gr, t.nthr, t.smem, pl->stream, E, nullptr, qtab,
+                           pass_tw<T>(pl, 2),
                                                                              geo_of<T>(pl), t.lp, out_scale, *cg);
                 return;
             }
         }
-        launch_pdl(k_pass_z_div<T, W, false>, gr, t.nthr, t.smem, pl->stream, E, out, qtab, pass_tw<T>(pl, 2), geo_of<T>(pl), t.lp, out_scale, 0);
+        launch_pdl(k_pass_z_div<T, W, false>, gr, t.nthr, t.smem, pl->stream, E, out, qtab, pass_tw<T>(pl, 2),
+                   geo_of<T>(pl), t.lp, out_scale, 0);
     });
     return (int)gr.x;
 }

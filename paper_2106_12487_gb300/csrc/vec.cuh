@@ -198,8 +198,8 @@ __global__ void k_cg_pupdate(const cplx_t<T>* __restrict__ r, cplx_t<T>* __restr
                              const T* __restrict__ qtab, Geo g, PrecondCoef pc, PrecondSel ps, const CGSys* sys) {
     using C = cplx_t<T>;
     const int b = blockIdx.y;
-    pdl_launch();
     pdl_wait();
+    pdl_launch();
     if (!sys[b].upd) return;
     const bool act = sys[b].active != 0;
     const size_t off = (size_t)b * 3 * g.V;
@@ -257,8 +257,8 @@ static __global__ void k_cg_start(const double* partial3, int nblk, CGSys* sys, 
 // scaled: the sums carry the square of cg_scale (here and in k_cg_beta).
 static __global__ void k_cg_alpha(const double2* partial2, int nblk, CGSys* sys, int scaled, int* n_active) {
     const int b = blockIdx.x;
-    pdl_launch();
     pdl_wait();
+    pdl_launch();
     CGSys& s = sys[b];
     double acc[1] = {0.0};
     if (s.active)
@@ -284,8 +284,8 @@ static __global__ void k_cg_alpha(const double2* partial2, int nblk, CGSys* sys,
 static __global__ void k_cg_beta(const double* partial3, int nblk, CGSys* sys, double tol2, double rz_floor, int scaled,
                                  int* n_active, int* ticket, int cond, cudaGraphConditionalHandle h, int* iter, int max_iter) {
     const int b = blockIdx.x;
-    pdl_launch();
     pdl_wait();
+    pdl_launch();
     CGSys& s = sys[b];
     double acc[2] = {0.0, 0.0};
     const int active = s.active;
