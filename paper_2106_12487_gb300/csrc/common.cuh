@@ -112,42 +112,6 @@ template <int DIR, typename C> __host__ __device__ __forceinline__ C cmul_i(C a)
     return DIR < 0 ? mk(a.y, -a.x) : mk(-a.y, a.x);
 }
 
-#ifdef __CUDACC__
-// Sums and fused multiply-adds of both parts of an FP32 complex value in one
-// instruction (add / fma .f32x2, sm_100 and later; each part rounded as by the
-// scalar instruction): half the issue slots of the butterflies' additions.
-// K-apply, 128^3 x 18: 2.98 -> 2.95 ms; 64^3 x 10: 237 -> 232 us.
-__device__ __forceinline__ unsigned long long pack2(float2 v) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(unsigned long long r) {
-    float2 v;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(r));
-    return v;
-}
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
-    return unpack2(r);
-}
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)), "l"(pack2(c)));
-    return unpack2(r);
-}
-// a + b, a - b and c + m a of a butterfly (m real)
-template <typename C> __device__ __forceinline__ C badd(C a, C b) { return cadd(a, b); }
-template <typename C> __device__ __forceinline__ C bsub(C a, C b) { return csub(a, b); }
-template <typename C, typename T> __device__ __forceinline__ C bfma(T m, C a, C c) {
-    return mk(fma(m, a.x, c.x), fma(m, a.y, c.y));
-}
-__device__ __forceinline__ float2 badd(float2 a, float2 b) { return add2(a, b); }
-__device__ __forceinline__ float2 bsub(float2 a, float2 b) { return fma2(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ float2 bfma(float m, float2 a, float2 c) { return fma2(make_float2(m, m), a, c); }
-#endif
-
 // Asynchronous global -> shared copy of one complex value (8 or 16 bytes);
 // src_valid = false fills zeros without reading.
 template <typename C>

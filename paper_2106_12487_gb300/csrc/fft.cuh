@@ -105,8 +105,8 @@ __device__ __forceinline__ void butterfly(C e, C o, int k, C& lo, C& hi) {
     using T = decltype(e.x);
     if (k == 0 || 4 * k == R || std::is_same<T, dfloat>::value) {
         const C t = twiddle_pow2<R, DIR>(o, k);
-        lo = badd(e, t);
-        hi = bsub(e, t);
+        lo = cadd(e, t);
+        hi = csub(e, t);
         return;
     }
     const int m16 = k * (16 / R);   // 1..7
@@ -125,8 +125,8 @@ __device__ __forceinline__ void butterfly(C e, C o, int k, C& lo, C& hi) {
         ux = fma(t, o.x, -o.y);
         uy = fma(t, o.y, o.x);
     }
-    lo = bfma(m, mk(ux, uy), e);
-    hi = bfma(-m, mk(ux, uy), e);
+    lo = mk(fma(m, ux, e.x), fma(m, uy, e.y));
+    hi = mk(fma(-m, ux, e.x), fma(-m, uy, e.y));
 }
 
 // cosines and sines 2 pi k / R of the odd radices, k = 1 .. (R - 1) / 2
@@ -171,8 +171,8 @@ struct RegDFT {
             return;
         } else if constexpr (R == 2) {
             C a = v[0], b = v[1];
-            v[0] = badd(a, b);
-            v[1] = bsub(a, b);
+            v[0] = cadd(a, b);
+            v[1] = csub(a, b);
         } else if constexpr ((R & (R - 1)) == 0) {
             constexpr int H = R / 2;
             C e[H], o[H];
@@ -192,21 +192,25 @@ struct RegDFT {
             C x0 = v[0];
 #pragma unroll
             for (int n = 0; n < H; ++n) {
-                t[n] = badd(v[n + 1], v[R - 1 - n]);
-                d[n] = bsub(v[n + 1], v[R - 1 - n]);
-                x0 = badd(x0, t[n]);
+                t[n] = cadd(v[n + 1], v[R - 1 - n]);
+                d[n] = csub(v[n + 1], v[R - 1 - n]);
+                x0 = cadd(x0, t[n]);
             }
 #pragma unroll
             for (int k = 1; k <= H; ++k) {
                 C a = v[0], b = cscale(d[0], T(odd_sin<R>(k)));
 #pragma unroll
                 for (int n = 0; n < H; ++n) {
-                    a = bfma(T(odd_cos<R>((n + 1) * k)), t[n], a);
-                    if (n > 0) b = bfma(T(odd_sin<R>((n + 1) * k)), d[n], b);
+                    const T c = T(odd_cos<R>((n + 1) * k));
+                    a = mk(fma(c, t[n].x, a.x), fma(c, t[n].y, a.y));
+                    if (n > 0) {
+                        const T s = T(odd_sin<R>((n + 1) * k));
+                        b = mk(fma(s, d[n].x, b.x), fma(s, d[n].y, b.y));
+                    }
                 }
                 const C ib = cmul_i<DIR>(b);
-                v[k] = badd(a, ib);         // v[1..H], v[R-H..] are read only through t and d
-                v[R - k] = bsub(a, ib);
+                v[k] = cadd(a, ib);         // v[1..H], v[R-H..] are read only through t and d
+                v[R - k] = csub(a, ib);
             }
             v[0] = x0;
         } else if constexpr (R == 9) {
