@@ -74,7 +74,7 @@ struct PrecondSel {
 };
 
 template <typename T>
-__device__ __forceinline__ void zsym_apply(const float* __restrict__ Z, const cplx_t<T> r[3], cplx_t<T> z[3]) {
+__device__ __forceinline__ void zsym_apply(const float* Z, const cplx_t<T> r[3], cplx_t<T> z[3]) {
     const T a = T(Z[0]), b = T(Z[1]), c = T(Z[2]), d = T(Z[3]), e = T(Z[4]), f = T(Z[5]);
     z[0] = cadd(cadd(cscale(r[0], a), cscale(r[1], f)), cscale(r[2], e));
     z[1] = cadd(cadd(cscale(r[0], f), cscale(r[1], b)), cscale(r[2], d));

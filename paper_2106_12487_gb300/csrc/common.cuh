@@ -134,11 +134,20 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
 
 // Programmatic dependent launch (sm_90 and later).  A kernel of the operator's
-// chain lets its successor start when its own CTAs have all begun
-// (pdl_launch), and does its set-up (twiddle tables, barriers) before it waits
-// for its predecessor's results (pdl_wait, before anything but constant tables is
-// touched).  Small cells are bound by the launches: a K-apply of 16^3 is six
+// chain does its set-up (twiddle tables, barriers), waits for its predecessor's
+// results (pdl_wait, before anything but constant tables is touched) and then
+// lets its successor start (pdl_launch): a successor becomes resident once every
+// CTA of this kernel has passed its wait, so at most two kernels of a chain
+// overlap.  Small cells are bound by the launches: a K-apply of 16^3 is six
 // kernels of a few microseconds.
+//
+// A kernel started this way lives while its predecessor still writes.  The
+// read-only forms of a load (__ldg, and `const ... __restrict__`, which lets the
+// compiler choose the non-coherent path or move the load across pdl_wait) are
+// specified for memory that no one writes during the kernel's whole lifetime:
+// they stand for the plan's constants only (twiddles, grain ids, stiffness and
+// density tables).  Whatever is made on the stream (fields, q tables, CG scalars,
+// phases) is read by plain loads after the wait.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -138,11 +138,11 @@ __global__ void __launch_bounds__(256) k_fpass_axis(const cplx_t<T>* in, cplx_t<
 // as [system * component][z][y * Nx + x] of 8-byte values), completed on an
 // mbarrier; otherwise by cp.async.  A wait that runs out sets *g.err.
 template <typename T, int RA, int RB, int NT = 128>
-__global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>* __restrict__ U, cplx_t<T>* __restrict__ E,
-                                                           const T* __restrict__ qtab,
+__global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>* U, cplx_t<T>* __restrict__ E,
+                                                           const T* qtab,
                                                            const cplx_t<T>* __restrict__ twz, Geo g,
                                                            const __grid_constant__ CUtensorMap tmap, int use_tma,
-                                                           const CGSys* __restrict__ sys) {
+                                                           const CGSys* sys) {
     using C = cplx_t<T>;
     constexpr int N = RA * RB;
     constexpr int P = NT / RA;
@@ -316,8 +316,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_strain(const cplx_t<T>
 // gradients is updated with it (CgUpdate), which saves writing and reading A p
 // and one launch per iteration.
 template <typename T, int RA, int RB, int NT, bool CG>
-__global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* __restrict__ E, cplx_t<T>* __restrict__ out,
-                                                        const T* __restrict__ qtab, const cplx_t<T>* __restrict__ twz,
+__global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* E, cplx_t<T>* __restrict__ out,
+                                                        const T* qtab, const cplx_t<T>* __restrict__ twz,
                                                         Geo g, T out_scale,
                                                         const __grid_constant__ CUtensorMap tmap, int use_tma,
                                                         const __grid_constant__ std::conditional_t<CG, CgUpdate<T>, int> cg) {

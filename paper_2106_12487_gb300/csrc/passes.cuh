@@ -245,8 +245,8 @@ __device__ __forceinline__ void pf_last(C* buf, int nbuf, const AxisPlan& a, int
 // (q_x and q_y are constant on a z pencil).
 template <typename T, bool WIDE>
 __global__ void __launch_bounds__(256, kPassCtasZ<T, WIDE>)
-    k_pass_z_strain(const cplx_t<T>* __restrict__ U, cplx_t<T>* __restrict__ E, const T* __restrict__ qtab,
-                    const cplx_t<T>* __restrict__ twz, Geo g, int lp, const CGSys* __restrict__ sys) {
+    k_pass_z_strain(const cplx_t<T>* U, cplx_t<T>* __restrict__ E, const T* qtab, const cplx_t<T>* __restrict__ twz,
+                    Geo g, int lp, const CGSys* sys) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const AxisPlan& a = g.ax[2];
@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(256, kPassCtasZ<T, WIDE>)
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     v[r] = src[(unsigned)(r * M) * plane];
-                    w[r] = cscale(v[r], qs(ldg_t(qz + r * M + j)));
+                    w[r] = cscale(v[r], qs(qz[r * M + j]));
                 }
                 RegDFT<R, +1, C>::run(v);
                 RegDFT<R, +1, C>::run(w);
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(256, kPassCtasZ<T, WIDE>)
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
                         v[r] = src[(unsigned)(r * M) * plane];
-                        if (h) v[r] = cscale(v[r], qs(ldg_t(qz + r * M + j)));
+                        if (h) v[r] = cscale(v[r], qs(qz[r * M + j]));
                     }
                     RegDFT<R, +1, C>::run(v);
                     s[0] = v[0];
@@ -424,8 +424,8 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
 // gradients is updated with it in place (CgUpdate).
 template <typename T, bool WIDE, bool CG>
 __global__ void __launch_bounds__(256, kPassCtasZ<T, WIDE>)
-    k_pass_z_div(const cplx_t<T>* __restrict__ E, cplx_t<T>* __restrict__ out, const T* __restrict__ qtab,
-                 const cplx_t<T>* __restrict__ twz, Geo g, int lp, T out_scale,
+    k_pass_z_div(const cplx_t<T>* E, cplx_t<T>* __restrict__ out, const T* qtab, const cplx_t<T>* __restrict__ twz,
+                 Geo g, int lp, T out_scale,
                  const __grid_constant__ std::conditional_t<CG, CgUpdate<T>, int> cg) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -732,7 +732,7 @@ __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
 template <typename T, int DIR, bool WIDE>
 __global__ void __launch_bounds__(256, kPassCtas<T, WIDE>)
     k_pass_x(cplx_t<T>* W, const cplx_t<T>* __restrict__ twx, Geo g, int P, T out_scale,
-             const double2* __restrict__ ph, int per) {
+             const double2* ph, int per) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const AxisPlan& a = g.ax[0];

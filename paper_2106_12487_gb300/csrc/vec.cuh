@@ -194,8 +194,8 @@ __global__ void k_cg_update(cplx_t<T>* __restrict__ r, const cplx_t<T>* __restri
 // For systems that took a step: x += alpha p (old p); then, if still active,
 // p = P^-1 r + beta p.
 template <typename T>
-__global__ void k_cg_pupdate(const cplx_t<T>* __restrict__ r, cplx_t<T>* __restrict__ p, cplx_t<T>* __restrict__ x,
-                             const T* __restrict__ qtab, Geo g, PrecondCoef pc, PrecondSel ps, const CGSys* sys) {
+__global__ void k_cg_pupdate(const cplx_t<T>* r, cplx_t<T>* __restrict__ p, cplx_t<T>* __restrict__ x,
+                             const T* qtab, Geo g, PrecondCoef pc, PrecondSel ps, const CGSys* sys) {
     using C = cplx_t<T>;
     const int b = blockIdx.y;
     pdl_wait();
