@@ -117,17 +117,26 @@ __device__ __forceinline__ void block_sum(T (&v)[NV]) {
     }
 }
 
-// Power of two near 1 / sqrt((r, z)) of a system.  The FP32 iteration forms its
-// products from the scaled direction and residual, so that they neither
-// underflow nor overflow whatever the size of the right-hand side and however
-// small the residual gets (a power of two changes no digit); the scalars are
-// kept unscaled in FP64.  FP64 needs none.
-template <typename T> __device__ __forceinline__ T cg_scale(const CGSys* sys, int b);
-template <> __device__ __forceinline__ float cg_scale<float>(const CGSys* sys, int b) {
-    const int e = ((__double2hiint(sys[b].rz) >> 20) & 0x7ff) - 1023;
+// Powers of two near 1 / sqrt((r, z)) and 1 / sqrt((r, r)) of a system.  The FP32
+// iteration forms its products from the direction and residual times the first,
+// and (r, r) from the residual times the second, so that neither underflows nor
+// overflows however small the residual gets (a power of two changes no digit).
+// One scale does not do for both: a part of r that P^-1 does not see (bin 0 at
+// k = 0) keeps (r, r) up while (r, z) falls by 32 digits, and its scaled square
+// would leave the FP32 range.  The scalars are kept unscaled in FP64.  FP64 fields
+// need no scale.
+template <typename T> __device__ __forceinline__ T inv_sqrt_pow2(double v);
+template <> __device__ __forceinline__ float inv_sqrt_pow2<float>(double v) {
+    const int e = ((__double2hiint(v) >> 20) & 0x7ff) - 1023;
     return __int_as_float((127 + min(max(-(e >> 1), -100), 100)) << 23);
 }
-template <> __device__ __forceinline__ double cg_scale<double>(const CGSys*, int) { return 1.0; }
+template <> __device__ __forceinline__ double inv_sqrt_pow2<double>(double) { return 1.0; }
+template <typename T> __device__ __forceinline__ T cg_scale(const CGSys* sys, int b) {
+    return inv_sqrt_pow2<T>(sys[b].rz);
+}
+template <typename T> __device__ __forceinline__ T cg_scale_rr(const CGSys* sys, int b) {
+    return inv_sqrt_pow2<T>(sys[b].rr);
+}
 
 // What the divergence pass needs to update the residual in place of storing
 // A p: r -= alpha A p, partials (r, P^-1 r) and (r, r) per CTA at
@@ -142,26 +151,25 @@ struct CgUpdate {
 };
 
 // Residual update at one voxel whose old residual is ro: ap = A p there times
-// the system's scale sc, alpha likewise divided by it; acc += (r, z), (r, r),
-// times sc^2.  Callers read the residuals of several voxels before the first
+// the system's scale sc, alpha likewise divided by it; acc += (r, z) times sc^2
+// and (r, r) times sr^2 (sr = cg_scale_rr).  Callers read the residuals of several voxels before the first
 // update: a load cannot pass the stores of r before it.
 template <typename T>
 __device__ __forceinline__ void cg_update_at(const CgUpdate<T>& cg, cplx_t<T>* rb, int b, long long V, unsigned v, T alpha,
-                                             T sc, T qx, T qy, T qz, const cplx_t<T> (&ap)[3],
+                                             T sc, T sr, T qx, T qy, T qz, const cplx_t<T> (&ap)[3],
                                              const cplx_t<T> (&ro)[3], T (&acc)[2]) {
     cplx_t<T> rv[3], zv[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         rv[c] = mk(fma(-alpha, ap[c].x, ro[c].x), fma(-alpha, ap[c].y, ro[c].y));
         rb[c * V + v] = rv[c];
+        const cplx_t<T> w = sizeof(T) == 4 ? cscale(rv[c], sr) : rv[c];
+        acc[1] += w.x * w.x + w.y * w.y;
         if constexpr (sizeof(T) == 4) rv[c] = cscale(rv[c], sc);
     }
     pre_apply<T>(cg.ps, cg.pc, b, v, V, qx, qy, qz, rv, zv);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        acc[0] += rv[c].x * zv[c].x + rv[c].y * zv[c].y;
-        acc[1] += rv[c].x * rv[c].x + rv[c].y * rv[c].y;
-    }
+    for (int c = 0; c < 3; ++c) acc[0] += rv[c].x * zv[c].x + rv[c].y * zv[c].y;
 }
 template <typename T>
 __device__ __forceinline__ void cg_partial_out(const CgUpdate<T>& cg, int b, T (&acc)[2]) {

@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* E
     }
     if constexpr (CG) {
         C* rb = cg.r + (size_t)b * 3 * g.V;
-        const T sc = cg_scale<T>(cg.sys, b);
+        const T sc = cg_scale<T>(cg.sys, b), sr = cg_scale_rr<T>(cg.sys, b);
         const T alpha = T(cg.sys[b].alpha / (double)sc);
         T sum[2] = {T(0), T(0)};
         if (p2 < np) {
@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_fpass_z_div(const cplx_t<T>* E
                 for (int u = 0; u < U; ++u) {
                     const int r = h + u;
                     const C ap[3] = {acc[0][r], acc[1][r], acc[2][r]};
-                    cg_update_at<T>(cg, rb, b, g.V, (unsigned)(j2 + r * RA) * plane + pi0 + p2, alpha, sc, qv[0],
+                    cg_update_at<T>(cg, rb, b, g.V, (unsigned)(j2 + r * RA) * plane + pi0 + p2, alpha, sc, sr, qv[0],
                                     qv[1], qzt[j2 + r * RA], ap, ro[u], sum);
                 }
             }

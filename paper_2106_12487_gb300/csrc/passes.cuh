@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(256, kPassCtasZ<T, WIDE>)
     const int np = (int)min((unsigned)P1 + 1u, plane - pi0);
     const C* Eb = E + (size_t)b * 6 * g.V;
     C* ob;
-    T alpha = T(0), sc = T(1), acc[2] = {T(0), T(0)};
+    T alpha = T(0), sc = T(1), sr = T(1), acc[2] = {T(0), T(0)};
     if constexpr (CG) {
         ob = cg.r + (size_t)b * 3 * g.V;
     } else {
@@ -456,6 +456,7 @@ __global__ void __launch_bounds__(256, kPassCtasZ<T, WIDE>)
     if (sys_idle(g, b)) return;
     if constexpr (CG) {
         sc = cg_scale<T>(cg.sys, b);
+        sr = cg_scale_rr<T>(cg.sys, b);
         alpha = T(cg.sys[b].alpha / (double)sc);
     }
     __syncthreads();
@@ -508,7 +509,7 @@ __global__ void __launch_bounds__(256, kPassCtasZ<T, WIDE>)
                             cadd(cadd(cscale(s1, ay), cscale(s3, az)), cscale(s5, ax)),
                             cadd(cadd(cscale(s2, az), cscale(s3, ay)), cscale(s4, ax))};
             if constexpr (CG) {
-                cg_update_at<T>(cg, ob, b, g.V, (unsigned)k * plane + pi, alpha, sc, ax, ay, az, o, ro[u], acc);
+                cg_update_at<T>(cg, ob, b, g.V, (unsigned)k * plane + pi, alpha, sc, sr, ax, ay, az, o, ro[u], acc);
             } else {
                 C* d = ob + (size_t)k * plane + pi;
                 d[0] = cscale(o[0], out_scale);

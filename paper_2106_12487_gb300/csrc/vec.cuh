@@ -254,7 +254,8 @@ static __global__ void k_cg_start(const double* partial3, int nblk, CGSys* sys, 
 }
 
 // After the stress pass: (p, A p) from its partials, alpha = rz / (p, A p).
-// scaled: the sums carry the square of cg_scale (here and in k_cg_beta).
+// scaled: the sum carries the square of cg_scale (in k_cg_beta (r, z) likewise,
+// and (r, r) the square of cg_scale_rr).
 static __global__ void k_cg_alpha(const double2* partial2, int nblk, CGSys* sys, int scaled, int* n_active) {
     const int b = blockIdx.x;
     pdl_wait();
@@ -299,9 +300,10 @@ static __global__ void k_cg_beta(const double* partial3, int nblk, CGSys* sys, d
     if (threadIdx.x != 0) return;
     if (active) {
         const double sc = scaled ? (double)cg_scale<float>(sys, b) : 1.0;
+        const double sr = scaled ? (double)cg_scale_rr<float>(sys, b) : 1.0;   // of the old (r, r)
         s.iters += 1;
         s.rz_new = acc[0] / (sc * sc);
-        s.rr = acc[1] / (sc * sc);
+        s.rr = acc[1] / (sr * sr);
         if (!(s.rr > tol2 * s.bb) || !(s.rz_new > rz_floor * s.rz0)) {
             s.active = 0;
         } else {
