@@ -120,7 +120,9 @@ __device__ __forceinline__ void block_sum(T (&v)[NV]) {
 // Powers of two near 1 / sqrt((r, z)) and 1 / sqrt((r, r)) of a system.  The FP32
 // iteration forms its products from the direction and residual times the first,
 // and (r, r) from the residual times the second, so that neither underflows nor
-// overflows however small the residual gets (a power of two changes no digit).
+// overflows however small the residual gets (a power of two changes no digit; the
+// sums of the start residual carry their own units, k_cg_init).  The operator of
+// the plain-form baseline (fft_variant 2) forms its products unscaled.
 // One scale does not do for both: a part of r that P^-1 does not see (bin 0 at
 // k = 0) keeps (r, r) up while (r, z) falls by 32 digits, and its scaled square
 // would leave the FP32 range.  The scalars are kept unscaled in FP64.  FP64 fields

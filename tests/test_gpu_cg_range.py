@@ -1,4 +1,6 @@
 """FP32 conjugate gradients over the range of their numbers."""
+import math
+
 import numpy as np
 import pytest
 
@@ -45,3 +47,22 @@ def test_large_irreducible_part(B, grid, amp):
     assert abs(rel[0] - np.linalg.norm(b[..., 0, 0, 0]) / np.linalg.norm(b)) < 1e-5
     # same bound as for amplitude 1: a small condition number times the tolerance
     assert np.linalg.norm(x - want) < 1e-4 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("use_x0", [False, True])
+@pytest.mark.parametrize("e", [-75, -60, 40, 64])
+@pytest.mark.parametrize("grid", GRIDS)
+def test_right_hand_sides_of_any_size(B, grid, e, use_x0):
+    """A power of two on b (and x0) changes no digit of a step, so iterations
+    and solution are those of b, also where the squares of b over the operator's
+    scale (about 7e18 here) leave the FP32 range."""
+    plan = B.Plan.from_problem(synth.small_polycrystal(grid, 5, 7), precision=1)
+    k = np.array([[0.4, 0.2, -0.3], [0.9, 0.0, 0.1]]) * math.pi / 1e-3
+    b = (synth.random_field(grid, 3, batch=2) * 1e18).astype(np.complex64)
+    x0 = solve(B, plan, k, b, 1e-1)[0] if use_x0 else None
+    f = np.float32(2.0 ** e)
+    ref, it0, rel0, st0 = solve(B, plan, k, b, 1e-5, x0=x0)
+    x, it, rel, st = solve(B, plan, k, b * f, 1e-5, x0=None if x0 is None else x0 * f)
+    assert st0 == 0 and st == 0 and np.array_equal(it, it0) and it.min() > 0
+    assert np.allclose(rel, rel0, rtol=1e-5)
+    assert np.linalg.norm(x.astype(np.complex128) * 2.0 ** -e - ref) <= 1e-6 * np.linalg.norm(ref)
