@@ -244,9 +244,9 @@ bloch_status bloch_apply_precond(bloch_plan* plan, int32_t nb, const double* k, 
  *   max_iter   iteration cap
  *   iters      host, nb (may be NULL): iterations taken per system
  *   rel_res    host, nb (may be NULL): final recursive relative residual per system
- * A system whose preconditioned residual (r, z) has fallen below 1e-32 (FP32)
- * or 1e-64 (FP64) of its start stops there: what is left of r (bin 0 at k = 0)
- * cannot be reduced.
+ * A residual in the bin where xi + k = 0 (bin 0 at k = 0) cannot be reduced.  If
+ * it alone exceeds tol ||b||, the system stops, as not converged, once the rest
+ * is solved for: (r, z) below 1e-32 (FP32) or 1e-64 (FP64) of its start.
  * Synchronises the stream.  Returns BLOCH_ENOTCONV_CG if any system missed tol,
  * and BLOCH_ECUDA if a pass kernel since the previous synchronising call gave
  * up waiting for its staging copies (the plan's pass error word; then cleared).

@@ -617,7 +617,8 @@ static void pcg_iteration(bloch_plan* pl, int nb, cplx_t<T>* x, double tol2, cud
         gk.skip_ncomp = 1;
     }
     pl->launches += 2;
-    // residuals 16 (FP32) or 32 (FP64) digits below the start: past any recursive convergence
+    // a system that cannot converge: (r, z) 32 (FP32) or 64 (FP64) digits below its start, which is
+    // the square of a residual 16 or 32 digits below
     const double rz_floor = std::is_same<T, float>::value ? 1e-32 : 1e-64;
     launch_pdl(k_cg_beta, nb, 256, 0, pl->stream, w.part3, nblk, w.sys, tol2, rz_floor, scaled, pl->d_nactive,
                pl->d_iter + 1, h ? 1 : 0, h ? *h : cudaGraphConditionalHandle{}, pl->d_iter, max_iter);
@@ -713,7 +714,7 @@ bloch_status pcg_run(bloch_plan* pl, int nb, const cplx_t<T>* b, cplx_t<T>* x, d
                                               T(rhs_scale), use_x0 ? 0 : 1, w.part3);
     BLOCH_CUDA_CHECK_RET(cudaMemsetAsync(pl->d_nactive, 0, sizeof(int), pl->stream));
     ++pl->launches;
-    k_cg_start<<<nb, 256, 0, pl->stream>>>(w.part3, nblk, w.sys, tol2, pl->d_nactive);
+    k_cg_start<T><<<nb, 256, 0, pl->stream>>>(w.part3, nblk, w.sys, tol2, pl->d_nactive, w.r, w.qtab, g);
     BLOCH_CUDA_CHECK_RET(
         cudaMemcpyAsync(pl->h_nactive, pl->d_nactive, sizeof(int), cudaMemcpyDeviceToHost, pl->stream));
     BLOCH_CUDA_CHECK_RET(cudaStreamSynchronize(pl->stream));
@@ -803,7 +804,7 @@ bloch_status pcg_enqueue(bloch_plan* pl, int nb, const cplx_t<T>* b, cplx_t<T>* 
                                               w.part3);
     BLOCH_CUDA_CHECK_RET(cudaMemsetAsync(pl->d_nactive, 0, sizeof(int), pl->stream));
     ++pl->launches;
-    k_cg_start<<<nb, 256, 0, pl->stream>>>(w.part3, nblk, w.sys, tol2, pl->d_nactive);
+    k_cg_start<T><<<nb, 256, 0, pl->stream>>>(w.part3, nblk, w.sys, tol2, pl->d_nactive, w.r, w.qtab, g);
     cudaGraphExec_t exec;
     int per_iter = 0;
     if ((st = pcg_graph<T>(pl, nb, b, x, tol2, max_iter, &exec, &per_iter)) != BLOCH_OK) return st;

@@ -31,6 +31,7 @@ struct CGSys {
     int active;
     int iters;
     int upd;         // took a step this iteration (x += alpha p is still to be applied)
+    int stuck;       // cannot converge: |r|^2 in the bin where q = 0 exceeds tol^2 bb
 };
 
 // Correctly rounded reciprocal (the FP32 form uses the rounded reciprocal

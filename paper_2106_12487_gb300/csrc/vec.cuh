@@ -297,8 +297,22 @@ __global__ void k_cg_pupdate(const cplx_t<T>* r, cplx_t<T>* __restrict__ p, cplx
 
 // Scalar recurrences of Algorithm 2, one block per system.
 // After the initial residual: rz, rr, bb from the 3-wide partials; active = rr > tol^2 bb.
-static __global__ void k_cg_start(const double* partial3, int nblk, CGSys* sys, double tol2, int* n_active) {
+// A p is zero in a bin where q = xi + k is zero (k = 0, or k on the reciprocal
+// lattice), so no step changes r there: a system whose residual in that bin alone
+// exceeds the tolerance can never meet it (stuck).
+template <typename T>
+__global__ void k_cg_start(const double* partial3, int nblk, CGSys* sys, double tol2, int* n_active,
+                           const cplx_t<T>* r, const T* qtab, Geo g) {
     const int b = blockIdx.x;
+    __shared__ int zero[3];   // index of q = 0 along each axis
+    if (threadIdx.x < 3) zero[threadIdx.x] = -1;
+    __syncthreads();
+    const T* qb = qtab + (size_t)b * (g.Nx + g.Ny + g.Nz);
+    for (int i = threadIdx.x; i < g.Nx + g.Ny + g.Nz; i += blockDim.x)
+        if (qb[i] == T(0)) {
+            const int ax = i < g.Nx ? 0 : (i < g.Nx + g.Ny ? 1 : 2);
+            zero[ax] = i - (ax > 0 ? g.Nx : 0) - (ax > 1 ? g.Ny : 0);
+        }
     double acc[3] = {0.0, 0.0, 0.0};
     for (int i = threadIdx.x; i < nblk; i += blockDim.x) {
         const double* v = partial3 + ((size_t)b * nblk + i) * 3;
@@ -315,6 +329,15 @@ static __global__ void k_cg_start(const double* partial3, int nblk, CGSys* sys, 
     s.iters = 0;
     s.upd = 0;
     s.active = (s.rr > tol2 * s.bb) ? 1 : 0;
+    double rest = 0.0;
+    if (zero[0] >= 0 && zero[1] >= 0 && zero[2] >= 0) {
+        const size_t v = ((size_t)zero[2] * g.Ny + zero[1]) * g.Nx + zero[0];
+        for (int c = 0; c < 3; ++c) {
+            const cplx_t<T> w = r[((size_t)b * 3 + c) * g.V + v];
+            rest += (double)w.x * w.x + (double)w.y * w.y;
+        }
+    }
+    s.stuck = rest > tol2 * s.bb ? 1 : 0;
     if (s.active) atomicAdd(n_active, 1);
 }
 
@@ -339,10 +362,10 @@ static __global__ void k_cg_alpha(const double2* partial2, int nblk, CGSys* sys,
 }
 
 // After the residual update: rz_new, rr; convergence test; beta = rz_new / rz.
-// A system also ends when (r, z) has fallen below rz_floor of its start: what is
-// left of r then lies where P^-1 is zero (bin 0 at k = 0 under a non-uniform
-// density), no step can reduce it, and going on to the iteration cap would only
-// drive the sums into underflow.  It still counts as not converged.
+// A system that cannot converge (stuck, k_cg_start) also ends when (r, z) has
+// fallen below rz_floor of its start: the rest of r is then solved for as far as
+// its digits go, and going on to the iteration cap would change nothing.  It counts
+// as not converged.  Every other system goes on as long as the tolerance asks.
 // The last block to finish sets the condition of the graph-resident loop
 // (cond != 0): continue while a system is active and the iteration cap, which
 // bounds every launch, is not reached.  *ticket counts finished blocks and is
@@ -369,7 +392,7 @@ static __global__ void k_cg_beta(const double* partial3, int nblk, CGSys* sys, d
         s.iters += 1;
         s.rz_new = acc[0] / (sc * sc);
         s.rr = acc[1] / (sr * sr);
-        if (!(s.rr > tol2 * s.bb) || !(s.rz_new > rz_floor * s.rz0)) {
+        if (!(s.rr > tol2 * s.bb) || !(s.rz_new > (s.stuck ? rz_floor * s.rz0 : 0.0))) {
             s.active = 0;
         } else {
             s.beta = s.rz_new / s.rz;

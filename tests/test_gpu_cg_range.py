@@ -66,3 +66,17 @@ def test_right_hand_sides_of_any_size(B, grid, e, use_x0):
     assert st0 == 0 and st == 0 and np.array_equal(it, it0) and it.min() > 0
     assert np.allclose(rel, rel0, rtol=1e-5)
     assert np.linalg.norm(x.astype(np.complex128) * 2.0 ** -e - ref) <= 1e-6 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("grid", GRIDS)
+def test_tolerance_below_the_fp32_digits(B, grid):
+    """The recursive residual of a system that can converge is followed as far
+    as asked, and a tolerance that is not reached within the cap takes the
+    iterations of the cap."""
+    plan = B.Plan.from_problem(synth.small_polycrystal(grid, 5, 7), precision=1)
+    k = np.array([[0.4, 0.2, -0.3]]) * math.pi / 1e-3
+    b = synth.random_field(grid, 3, batch=1) * 1e18
+    _, iters, rel, st = solve(B, plan, k, b, 1e-20)
+    assert st == 0 and rel[0] <= 1e-20 and iters[0] < 500
+    _, n, _, st = solve(B, plan, k, b, 1e-30, max_iter=int(iters[0]) - 1)
+    assert st == 4 and n[0] == iters[0] - 1
