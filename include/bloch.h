@@ -288,8 +288,8 @@ bloch_status bloch_solve_bands(bloch_plan* plan, int32_t n_k, const double* k_li
  * speeds of Section 5.2 are |c| of the acoustic branches at small k.
  *   nb         vectors (1..10922)
  *   k          host, nb x 3 (rad/m), the wave vector of each vector
- *   precision  BLOCH_FP32 or BLOCH_FP64 (u's type; arithmetic in that type,
- *              sums in FP64)
+ *   precision  BLOCH_FP32 or BLOCH_FP64 (u's type; stresses in that type, the
+ *              sums over voxels from exact products to 48 bits or in FP64)
  *   u          device, nb x 3 x V complex, Fourier basis
  *   omega_out  host, nb (may be NULL): sqrt of the Rayleigh quotient (rad/s)
  *   c_out      host, nb x 3 (m/s); 0 where omega = 0 (rigid translations at k = 0)

@@ -23,24 +23,39 @@ namespace bloch {
 
 constexpr int kDkVals = 5;   // Re d_x, Re d_y, Re d_z, Re a, u^H M~ u
 
-// Running sum of one thread.  FP32 terms are added into an unevaluated pair
-// hi + lo with Knuth's two-sum, which keeps every rounding error of the
-// additions (48 bits); FP64 terms are added plainly.  GB300 adds FP64 at 1/64
-// of its FP32 rate: with FP64 sums of the FP32 terms this pass took ten times
-// its memory time.
+// Sum of products of one thread.  For FP32 values a pair hi + lo: the rounding
+// error of a product is one fused multiply-add, that of an addition Knuth's
+// two-sum, and both go to lo, so the products are exact and the sum carries about
+// 48 bits.  FP64 values are added plainly.  GB300 runs FP64 at 1/64 of its FP32
+// rate: with FP64 products and sums of FP32 values this pass took ten times its
+// memory time.  Exact products cost 1.4 % of the property calls over rounded ones
+// (128^3, 10 vectors: 4.21 -> 4.27 ms); the phase is then that of the FP32 values
+// to 1e-15 (3e-9 from real-space FP32 fields in FP64 sums, 1e-9 with rounded
+// products).
 template <typename T> struct Sum;
 template <> struct Sum<float> {
     float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float v) {
+    __device__ __forceinline__ void add(float v, float err) {
         const dfloat s = df_two_sum(hi, v);
         hi = s.hi;
-        lo = __fadd_rn(lo, s.lo);
+        lo = __fadd_rn(lo, __fadd_rn(s.lo, err));
     }
+    __device__ __forceinline__ void mul(float a, float b) {   // += a b
+        const float p = __fmul_rn(a, b);
+        add(p, __fmaf_rn(a, b, -p));
+    }
+    __device__ __forceinline__ void mul(float a, const Sum& b) {   // += a b
+        mul(a, b.hi);
+        lo = __fmaf_rn(a, b.lo, lo);
+    }
+    __device__ __forceinline__ void add(const Sum& b) { add(b.hi, b.lo); }
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 template <> struct Sum<double> {
     double s = 0.0;
-    __device__ __forceinline__ void add(double v) { s += v; }
+    __device__ __forceinline__ void mul(double a, double b) { s = fma(a, b, s); }
+    __device__ __forceinline__ void mul(double a, const Sum& b) { s = fma(a, b.s, s); }
+    __device__ __forceinline__ void add(const Sum& b) { s += b.s; }
     __device__ __forceinline__ double value() const { return s; }
 };
 
@@ -80,8 +95,8 @@ static bloch_status launch_absmax(bloch_plan* pl, int nb, const cplx_t<T>* u, un
 // Per system b = blockIdx.y, per block: partial sums over Fourier voxels of
 //   Re d_m = Re sum_i conj(U_i) S_im,  Re a = sum_m q_m Re d_m (per voxel),
 //   mu = Re sum conj(U) (M~ U)
-// with M~ U = MU (non-uniform density) or rho_s U.  Terms of a voxel in the
-// field precision, sums over voxels as Sum<T> and FP64 across threads.
+// with M~ U = MU (non-uniform density) or rho_s U.  Products and sums of a thread
+// as Sum<T>, FP64 across threads.
 template <typename T>
 __global__ void k_dk_partial(const cplx_t<T>* __restrict__ U, const cplx_t<T>* __restrict__ S,
                              const cplx_t<T>* __restrict__ MU, double rho_s, const T* __restrict__ qtab, Geo g,
@@ -104,25 +119,24 @@ __global__ void k_dk_partial(const cplx_t<T>* __restrict__ U, const cplx_t<T>* _
         for (int c = 0; c < 3; ++c) u[c] = cscale(ub[(size_t)c * g.V + v], sc);
 #pragma unroll
         for (int c = 0; c < 6; ++c) s[c] = cscale(sb[(size_t)c * g.V + v], sc);
-        T a = T(0), mu = T(0);
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
-            T d = T(0);
+            Sum<T> d;
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
                 const C sv = s[vo[i][m]];
-                d = fma(u[i].x, sv.x, fma(u[i].y, sv.y, d));
+                d.mul(u[i].x, sv.x);
+                d.mul(u[i].y, sv.y);
             }
             acc[m].add(d);
-            a = fma(q[m], d, a);
+            acc[3].mul(q[m], d);
         }
-        acc[3].add(a);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             const C mv = mb ? cscale(mb[(size_t)i * g.V + v], sc) : u[i];
-            mu = fma(u[i].x, mv.x, fma(u[i].y, mv.y, mu));
+            acc[4].mul(u[i].x, mv.x);
+            acc[4].mul(u[i].y, mv.y);
         }
-        acc[4].add(mu);
     }
     double tot[kDkVals];
 #pragma unroll
@@ -205,15 +219,14 @@ __global__ void k_sq_partial(const cplx_t<T>* __restrict__ U, Geo g, const unsig
         const int z = (int)fdiv(t, g.dy), y = (int)t - z * g.Ny;
         const unsigned w = ((unsigned)(z ? g.Nz - z : 0) * g.Ny + (y ? g.Ny - y : 0)) * (unsigned)g.Nx +
                            (unsigned)(x ? g.Nx - x : 0);
-        T re = T(0), im = T(0);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const cplx_t<T> a = cscale(ub[(size_t)c * g.V + v], sc), m = cscale(ub[(size_t)c * g.V + w], sc);
-            re = fma(a.x, m.x, fma(-a.y, m.y, re));
-            im = fma(a.x, m.y, fma(a.y, m.x, im));
+            acc[0].mul(a.x, m.x);
+            acc[0].mul(-a.y, m.y);
+            acc[1].mul(a.x, m.y);
+            acc[1].mul(a.y, m.x);
         }
-        acc[0].add(re);
-        acc[1].add(im);
     }
     double tot[2] = {acc[0].value(), acc[1].value()};
     block_sum<double, 2>(tot);
