@@ -195,7 +195,8 @@ void bloch_plan_destroy(bloch_plan* plan);
  * vector, held by the plan and grown on demand.  The FP32 fast z passes stage
  * their pencils with TMA tiles when u is 16-byte aligned and Nx * Ny is even
  * (cp.async otherwise); a staging wait that runs out sets the plan's pass
- * error word, reported by the next bloch_pcg or bloch_solve_bands.
+ * error word, reported by the next bloch_pcg, bloch_solve_bands,
+ * bloch_group_velocity or bloch_eigvec_real.
  */
 bloch_status bloch_apply_K(bloch_plan* plan, int32_t nb, const double* k, int32_t precision,
                            const void* u, void* Ku);
@@ -294,7 +295,8 @@ bloch_status bloch_solve_bands(bloch_plan* plan, int32_t n_k, const double* k_li
  *   omega_out  host, nb (may be NULL): sqrt of the Rayleigh quotient (rad/s)
  *   c_out      host, nb x 3 (m/s); 0 where omega = 0 (rigid translations at k = 0)
  * Synchronises the plan's stream.  Errors: BLOCH_EINVAL (arguments, a zero
- * vector), BLOCH_ENONFINITE (k), BLOCH_ENOMEM, BLOCH_ECUDA.
+ * vector), BLOCH_ENONFINITE (k), BLOCH_ENOMEM, BLOCH_ECUDA (also when the plan's
+ * pass error word is set, as bloch_pcg).
  */
 bloch_status bloch_group_velocity(bloch_plan* plan, int32_t nb, const double* k, int32_t precision, const void* u,
                                   double* omega_out, double* c_out);
@@ -314,7 +316,8 @@ bloch_status bloch_group_velocity(bloch_plan* plan, int32_t nb, const double* k,
  *   strain     device, nb x 6 x V complex, tensor components (xx yy zz yz xz
  *              xy), or NULL
  *   phi_out    host, nb (may be NULL): phi (rad)
- * Outputs may not alias u_hat.  Synchronises the plan's stream.
+ * Outputs may not alias u_hat.  Synchronises the plan's stream; returns BLOCH_ECUDA
+ * when the plan's pass error word is set (as bloch_pcg).
  */
 bloch_status bloch_eigvec_real(bloch_plan* plan, int32_t nb, int32_t precision, const void* u_hat, void* u_real,
                                void* strain, double* phi_out);

@@ -367,10 +367,10 @@ bool encode_zmap(CUtensorMap* map, const void* base, const bloch_plan* pl, long 
 }
 
 bloch_status check_pass_err(bloch_plan* pl) {
-    int e = 0;
-    BLOCH_CUDA_CHECK_RET(cudaMemcpyAsync(&e, pl->d_perr, sizeof(int), cudaMemcpyDeviceToHost, pl->stream));
+    int* e = pl->h_nactive + 1;
+    BLOCH_CUDA_CHECK_RET(cudaMemcpyAsync(e, pl->d_perr, sizeof(int), cudaMemcpyDeviceToHost, pl->stream));
     BLOCH_CUDA_CHECK_RET(cudaStreamSynchronize(pl->stream));
-    if (e) {
+    if (*e) {
         cudaMemsetAsync(pl->d_perr, 0, sizeof(int), pl->stream);
         return set_error(BLOCH_ECUDA, "a pass's staging copy did not complete within its wait bound");
     }
@@ -1178,7 +1178,7 @@ bloch_status bloch_plan_create(bloch_plan** out, const int32_t grid[3], const do
     CK(dmalloc(&pl->d_iter, 2, acc));
     CK(cudaMemset(pl->d_iter, 0, 2 * sizeof(int)));
     CK(cudaStreamCreateWithFlags(&pl->cap_stream, cudaStreamNonBlocking));
-    CK(cudaMallocHost((void**)&pl->h_nactive, sizeof(int)));
+    CK(cudaMallocHost((void**)&pl->h_nactive, 2 * sizeof(int)));
     CK(pass_attrs_z<float>());
     CK(pass_attrs_axis<float>());
     CK(pass_attrs_x<float>());

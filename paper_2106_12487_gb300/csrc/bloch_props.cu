@@ -147,6 +147,8 @@ __global__ void k_dk_partial(const cplx_t<T>* __restrict__ U, const cplx_t<T>* _
         double* o = partial + ((size_t)b * gridDim.x + blockIdx.x) * kDkVals;
 #pragma unroll
         for (int i = 0; i < kDkVals; ++i) o[i] = tot[i];
+        // the pass error word rides behind the partials: the host reads it in the same copy
+        if (b == 0 && blockIdx.x == 0) partial[(size_t)gridDim.y * gridDim.x * kDkVals] = *g.err ? 1.0 : 0.0;
     }
 }
 
@@ -168,17 +170,19 @@ static bloch_status group_velocity_impl(bloch_plan* pl, int nb, const double* k,
     const int nblk = (int)std::max(1LL, std::min<long long>((pl->V + 255) / 256, 512));
     const size_t nval = (size_t)nb * nblk * kDkVals;
     double* d_part = nullptr;
-    if ((st = plan_solver_buf(pl, 2, 0, nval * sizeof(double) + nb * sizeof(unsigned), (void**)&d_part)) != BLOCH_OK)
+    if ((st = plan_solver_buf(pl, 2, 0, (nval + 1) * sizeof(double) + nb * sizeof(unsigned), (void**)&d_part)) != BLOCH_OK)
         return st;
-    unsigned* d_mx = (unsigned*)(d_part + nval);
+    unsigned* d_mx = (unsigned*)(d_part + nval + 1);
     if ((st = launch_absmax<T>(pl, nb, u, d_mx)) != BLOCH_OK) return st;
     ++pl->launches;
     k_dk_partial<T><<<dim3(nblk, nb), 256, 0, pl->stream>>>(u, w.E, MU, pl->uniform_rho ? pl->rho_uniform_scaled : 1.0,
                                                             w.qtab, geo_of<T>(pl), d_mx, d_part);
     BLOCH_CUDA_CHECK_RET(cudaGetLastError());
-    std::vector<double> h(nval);
-    BLOCH_CUDA_CHECK_RET(cudaMemcpyAsync(h.data(), d_part, nval * sizeof(double), cudaMemcpyDeviceToHost, pl->stream));
+    std::vector<double> h(nval + 1);
+    BLOCH_CUDA_CHECK_RET(
+        cudaMemcpyAsync(h.data(), d_part, h.size() * sizeof(double), cudaMemcpyDeviceToHost, pl->stream));
     BLOCH_CUDA_CHECK_RET(cudaStreamSynchronize(pl->stream));
+    if (h[nval] != 0.0 && (st = check_pass_err(pl)) != BLOCH_OK) return st;
     for (int b = 0; b < nb; ++b) {
         double s[kDkVals] = {0};
         for (int j = 0; j < nblk; ++j)
@@ -274,8 +278,7 @@ static bloch_status eigvec_real_impl(bloch_plan* pl, int nb, const cplx_t<T>* uh
         launch_strain_real<T>(pl, nb, uh, eps, T(1.0 / (pl->qscale * (double)pl->V)), d_ph + nb);
     }
     BLOCH_CUDA_CHECK_RET(cudaGetLastError());
-    BLOCH_CUDA_CHECK_RET(cudaStreamSynchronize(pl->stream));
-    return BLOCH_OK;
+    return check_pass_err(pl);   // synchronises
 }
 
 }  // namespace bloch

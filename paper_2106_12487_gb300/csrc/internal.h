@@ -119,7 +119,7 @@ struct bloch_plan {
     dfloat* d_rx = nullptr;
     int* d_nactive = nullptr;
     int* d_perr = nullptr;    // pass error word (a staging wait ran out), Geo::err
-    int* h_nactive = nullptr;     // pinned
+    int* h_nactive = nullptr;     // pinned: the active count, and the pass error word behind it
 
     bloch::Geo geo_f, geo_d, geo_x;     // FP32, FP64, float-float
     int pmax;                           // cap on pencils per CTA of the mixed-radix passes
