@@ -497,8 +497,17 @@ def alu_peaks_leg(p, opt, nb):
     return out
 
 
-# FP32, c = 8 B: K-apply 54c + 4 (its x pass also forms (p, Ap)), k_cg_update 9c, k_cg_pupdate 15c
+# FP32, c = 8 B, per voxel, system and iteration.  Plain-form baseline (fft_variant 2): K-apply
+# 54c + 4, k_cg_update 9c, k_cg_pupdate 15c.
 PCG_BYTES_PER_VOXEL = 628.0
+# The pass chain: passes 1-4 (9 + 12 + 12 + 12)c + 4, the divergence pass that updates r in place of
+# storing Ap 6c + 3c + 3c, k_cg_pupdate 15c.
+PCG_CHAIN_BYTES_PER_VOXEL = 580.0
+
+
+def pcg_bytes_per_voxel(fft_variant):
+    """Algorithmic bytes of one FP32 PCG iteration per voxel and system."""
+    return PCG_BYTES_PER_VOXEL if fft_variant == 2 else PCG_CHAIN_BYTES_PER_VOXEL
 
 
 def pcg_roofline(plan, p, nb, iters):
@@ -523,7 +532,7 @@ def pcg_roofline(plan, p, nb, iters):
     torch.cuda.synchronize()
     n_it = int(it.max())
     t_it = e0.elapsed_time(e1) / 1000.0 / max(n_it, 1)
-    alg = PCG_BYTES_PER_VOXEL * plan.V * nb
+    alg = pcg_bytes_per_voxel(plan.options.fft_variant) * plan.V * nb
     peak, peak_src = peaks()
     return {"bound": "hbm", "achieved": alg / t_it / 1e9, "peak": peak, "unit": "GB/s",
             "frac": alg / t_it / 1e9 / peak, "kernel": f"FP32 PCG iteration, {nb} systems at {tuple(p.grid)} "
