@@ -41,8 +41,6 @@ template <> const dfloat2* tw_of<dfloat>(const bloch_plan* pl, int axis) { retur
 template <typename T> static const T* ctab_of(const bloch_plan* pl);
 template <> const float* ctab_of<float>(const bloch_plan* pl) { return pl->d_Cf; }
 template <> const double* ctab_of<double>(const bloch_plan* pl) { return pl->d_Cd; }
-template <typename T> static const T* cpk_of(const bloch_plan* pl);
-template <> const float* cpk_of<float>(const bloch_plan* pl) { return pl->d_Cpf; }
 // ------------------------------------------------------------ host helpers
 static bool fast_axis(int N);
 static bool fast_x(int N);
@@ -59,7 +57,7 @@ static bool factor_ok(int n) {
 // strain pass holds two butterflies.
 static AxisPlan make_axis(int N, bool ff) {
     static const int ends[] = {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 14, 15, 16};
-    static const int mids[] = {1, 2, 3, 4, 5, 6, 7, 8};
+    static const int mids[] = {1, 3, 4, 5, 6, 7, 8};
     AxisPlan ap{};
     ap.N = N;
     int best = 1 << 30;
@@ -67,7 +65,7 @@ static AxisPlan make_axis(int N, bool ff) {
         for (int r2 : mids)
             for (int r3 : ends) {
                 if (r1 * r2 * r3 != N || (r1 > r3 && r3 > 1)) continue;
-                if (ff && (r1 == 12 || r1 == 14 || r3 == 12 || r3 == 14)) continue;
+                if (ff ? r1 == 12 || r1 == 14 || r3 == 12 || r3 == 14 : r2 == 4) continue;
                 const int cost = (r2 > 1 ? 1000 : 0) + r1 + r2 + r3;
                 if (cost < best) {
                     best = cost;

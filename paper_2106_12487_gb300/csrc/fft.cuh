@@ -35,8 +35,8 @@ __device__ __forceinline__ unsigned fdiv(unsigned n, const FastDiv& f) { return 
 
 // Radix schedule N = r1 * r2 * r3 of an axis (r2 = 1: two stages).  The first
 // and the last radix come from {1..10, 12, 14, 15, 16} (float-float: without
-// 12 and 14), the middle one from {1..8}; every length up to
-// 512 with prime factors in {2,3,5,7} has one.
+// 12 and 14), the middle one from {1, 3, 5, 6, 7, 8} (float-float: and 4); every
+// length up to 512 with prime factors in {2,3,5,7} has one.
 struct AxisPlan {
     int N;
     int r1, r2, r3;

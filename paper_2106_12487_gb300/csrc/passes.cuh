@@ -158,12 +158,20 @@ __device__ __forceinline__ void with_radix(int R, F&& f) {
         }
     }
 }
-template <typename F>
+// Middle radices that a schedule chooses: 4 occurs in float-float only (84 = 3 4 7,
+// 7 x 12 in the types that have a 12).
+template <typename T, typename F>
 __device__ __forceinline__ void with_mid_radix(int R, F&& f) {
     switch (R) {
-        BLOCH_RADIX(2) BLOCH_RADIX(3) BLOCH_RADIX(4) BLOCH_RADIX(5) BLOCH_RADIX(6) BLOCH_RADIX(7) BLOCH_RADIX(8)
-#undef BLOCH_RADIX
+        BLOCH_RADIX(3) BLOCH_RADIX(5) BLOCH_RADIX(6) BLOCH_RADIX(7) BLOCH_RADIX(8)
         default: break;
+    }
+    if constexpr (std::is_same<T, dfloat>::value) {
+        switch (R) {
+            BLOCH_RADIX(4)
+#undef BLOCH_RADIX
+            default: break;
+        }
     }
 }
 
@@ -197,7 +205,7 @@ __device__ __forceinline__ int slot_of(int k, const AxisPlan& a) {
 template <int DIR, typename C>
 __device__ __forceinline__ void pf_mid(C* buf, int nbuf, const AxisPlan& a, int lp, const C* tw, int tid, int nthr) {
     const int P1 = (1 << lp) - 1, NP = a.N << lp;
-    with_mid_radix(a.r2, [&](auto rc) {
+    with_mid_radix<real_t<C>>(a.r2, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         const int per = (a.N / R) << lp, r3 = a.r3;
         for (int t = tid; t < nbuf * per; t += nthr) {
@@ -552,7 +560,7 @@ __device__ __forceinline__ void lf_first(const C* Wb, long long V, C* buf, int n
 template <int DIR, bool FREQ, typename C>
 __device__ __forceinline__ void lf_mid(C* buf, int nrows, const AxisPlan& a, const C* tw, int tid, int nthr) {
     const int ld = xrow(a), gr = xgroup(a);
-    with_mid_radix(a.r2, [&](auto rc) {
+    with_mid_radix<real_t<C>>(a.r2, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         const int M = a.N / R;
         for (int t = tid; t < nrows * M; t += nthr) {
