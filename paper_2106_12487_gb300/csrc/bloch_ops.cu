@@ -54,7 +54,13 @@ static bool factor_ok(int n) {
 // Radix schedule of an axis: the fewest stages, then the smallest radices (the
 // sum of the radices is the work of the direct parts and the butterflies held
 // in registers), the first no larger than the last: the first stage of the
-// strain pass holds two butterflies.
+// strain pass holds two butterflies.  K-apply in us with this rule, with the larger
+// radix first, and with the least balanced schedule of two stages:
+//   120 x 100 x 84 FP32, 6 systems   662   687   726
+//   90^3 FP32, 4 systems             386   396   425
+//   60^3 FP32, 1 system               38    38    48
+//   60^3 FP64, 2 systems             688   699   680
+//   60^3 float-float, 2 systems      320   351   378
 static AxisPlan make_axis(int N, bool ff) {
     static const int ends[] = {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 14, 15, 16};
     static const int mids[] = {1, 3, 4, 5, 6, 7, 8};
@@ -86,10 +92,17 @@ static AxisPlan make_axis(int N, bool ff) {
 // Shared memory a CTA may take: two CTAs per SM for the z passes, whose rows
 // gain from width; four for the rows along x, whose do not.
 constexpr size_t kTileSmemZ = 104 * 1024, kTileSmemX = 55 * 1024;
-// CTAs wanted in a launch before a tile is worth its width: three per SM.
-// (48 x 40 x 36, FP32, 10 systems: 185 us per K-apply with tiles made for one
-// system, 95 us with tiles made for the launch.)
-constexpr long long kTileCtas = 456;
+// CTAs wanted in a launch before a tile is worth its width: three on each of the
+// 152 SMs, of every form.  K-apply in us with 1, 2, 3, 4 and 6 per SM:
+//   48 x 40 x 36 FP32, 2 systems          47   36   32   33   36
+//   60^3 FP32, 1 system                   52   46   38   38   42
+//   24 x 20 x 15 FP64, 4 systems          73   62   62   80   80
+//   36^3 FP64, 2 systems                 196  181  174  170  187
+//   60^3 float-float, 2 systems          340  341  320  320  360
+// The kernels' occupancy (kPassCtas: two to four CTAs) moves the line less than the
+// last wave does, so one figure serves all.  Launches of 90^3 and more, or ten
+// systems of 60^3, reach it with full tiles and do not change.
+constexpr long long kTileCtas = 3 * 152;
 
 // P pencils (rows) per CTA, a power of two of at most plan->pmax (half
 // of it along x): halved until the tile fits its shared memory, then while the
@@ -114,7 +127,8 @@ PassTile pass_tile(const bloch_plan* pl, PassKind kind, int nb) {
     while ((x_ ? P > 1 : P * el > 32) && npen * nb / P < kTileCtas) P >>= 1;
     while ((1 << t.lp) < P) ++t.lp;
     t.smem = row * P + tw;
-    // threads: the fewest idle butterfly slots over the first and last stage
+    // threads: the fewest idle butterfly slots over the first and last stage (120 x 100 x 84 FP32, 6
+    // systems: 662 us; 692 with 256 threads throughout, 757 with 128; 48 x 40 x 36, 2 systems: 32, 35, 37)
     long long best = -1;
     for (int n : {256, 224, 192, 160, 128}) {
         long long c = 0;
