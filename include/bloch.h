@@ -73,8 +73,9 @@ typedef struct {
     int32_t method;      /* BLOCH_LANCZOS (shift-invert Lanczos with thick restart, Section
                             3.3), BLOCH_SUBSPACE (Algorithm 1) or BLOCH_LOBPCG (locally
                             optimal block preconditioned CG on the pencil (A_k, M), block
-                            [X, W = T R, P] with T the Green preconditioner of Eq.
-                            (precond) and a rank-revealing Rayleigh-Ritz; no inner PCG;
+                            [X, W = T R less its part in X, P] with T the Green
+                            preconditioner of Eq. (precond) and a rank-revealing
+                            Rayleigh-Ritz that keeps X; no inner PCG;
                             block q = n + 2 unless set, 3q <= 44, 48 with a uniform
                             density).  Every method handles any density and k = 0.
                             Default BLOCH_SUBSPACE.                                     */

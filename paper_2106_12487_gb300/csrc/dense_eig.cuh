@@ -275,30 +275,97 @@ static __global__ void k_gen_herm_eig(int n, const double2* __restrict__ K, cons
     if (tid == 0) status[b] = conv ? 0 : 2;
 }
 
-// Rank-revealing Rayleigh-Ritz of a pencil (K, M) whose M may be singular
-// (SVQB, Stathopoulos & Wu 2002): the basis is first scaled to unit M-norm,
-// s_i = M_ii^-1/2 (0 for a zero column), M' = S M S, K' = S K S; then
-// M' = V D V^H (Jacobi), the directions with D > eps * max(D) are kept,
-// Z = V_keep D_keep^-1/2 (M'-orthonormal), C = Z^H K' Z = Y diag(lam) Y^H
-// (Jacobi) and the Ritz vectors in the original coordinates are Q = S Z Y.  One CTA per pencil (blockIdx.x); K, M, Q n x n
-// row-major (double2) at b * n * n; M scaled by mscale.  Out: lam[b][0..r)
-// ascending, Q[b] columns 0..r (the rest zero), rank[b] = r.  Shared memory:
-// gen_eig_smem(n, blockDim.x).
-static __global__ void k_svqb_eig(int n, const double2* __restrict__ K, const double2* __restrict__ M, double mscale,
-                                  double eps, double* __restrict__ lam, double2* __restrict__ Q,
-                                  int* __restrict__ rank) {
+constexpr int kLobQ = 16;   // most vectors of a LOBPCG block (one Gram pass over [X, W, P]: 3q <= 48)
+
+// Coefficients that take X out of W: from G = S^H (M S) on S = [X, W] (2q x 2q per
+// slot; the columns of X are read) the (2q x q) matrix [-(X^H M X)^-1 X^H M W; I].
+// X is nearly M-orthonormal but for a start block: Cholesky of the scaled X^H M X,
+// a vector dependent on those before it left out.  One CTA per slot.
+static __global__ void k_project_coef(int q, const double2* __restrict__ G, double2* __restrict__ Cf) {
+    __shared__ double2 L[kLobQ * kLobQ];
+    __shared__ double sc[kLobQ];
+    const int n = 2 * q, tid = threadIdx.x, nt = blockDim.x;
+    const double2* Gb = G + (size_t)blockIdx.x * n * n;
+    double2* Cb = Cf + (size_t)blockIdx.x * n * q;
+    for (int i = tid; i < q; i += nt) sc[i] = Gb[i * n + i].x > 0.0 ? 1.0 / sqrt(Gb[i * n + i].x) : 0.0;
+    __syncthreads();
+    for (int e = tid; e < q * q; e += nt) {
+        const int i = e / q, j = e % q;
+        const double f = 0.5 * sc[i] * sc[j];
+        L[e] = make_double2(f * (Gb[i * n + j].x + Gb[j * n + i].x), f * (Gb[i * n + j].y - Gb[j * n + i].y));
+    }
+    __syncthreads();
+    for (int c = 0; c < q; ++c) {
+        const double d2 = L[c * q + c].x, d = d2 > 1e-14 ? sqrt(d2) : 0.0;
+        __syncthreads();
+        for (int i = c + tid; i < q; i += nt) {
+            const double2 v = L[i * q + c];
+            L[i * q + c] = i == c ? make_double2(d, 0.0)
+                                  : (d > 0.0 ? make_double2(v.x / d, v.y / d) : make_double2(0.0, 0.0));
+        }
+        __syncthreads();
+        for (int e = tid; e < q * q; e += nt) {
+            const int i = e / q, j = e % q;
+            if (j > c && i >= j) L[e] = zsub(L[e], zmul(L[i * q + c], zconj(L[j * q + c])));
+        }
+        __syncthreads();
+    }
+    for (int c = tid; c < q; c += nt) {   // one column of W each: L y = X^H M w, L^H y = y
+        double2 y[kLobQ];
+        for (int i = 0; i < q; ++i) {
+            const double2 g = Gb[(q + c) * n + i];   // w^H M x_i
+            double2 v = make_double2(sc[i] * g.x, -sc[i] * g.y);
+            for (int k = 0; k < i; ++k) v = zsub(v, zmul(L[i * q + k], y[k]));
+            const double d = L[i * q + i].x;
+            y[i] = d > 0.0 ? make_double2(v.x / d, v.y / d) : make_double2(0.0, 0.0);
+        }
+        for (int i = q - 1; i >= 0; --i) {
+            double2 v = y[i];
+            for (int k = i + 1; k < q; ++k) v = zsub(v, zmul(zconj(L[k * q + i]), y[k]));
+            const double d = L[i * q + i].x;
+            y[i] = d > 0.0 ? make_double2(v.x / d, v.y / d) : make_double2(0.0, 0.0);
+        }
+        for (int i = 0; i < q; ++i) {
+            Cb[i * q + c] = make_double2(-sc[i] * y[i].x, -sc[i] * y[i].y);
+            Cb[(q + i) * q + c] = make_double2(i == c ? 1.0 : 0.0, 0.0);
+        }
+    }
+}
+
+// Rank-revealing Rayleigh-Ritz of a pencil (K, M) whose M may be singular, on a
+// basis whose first nx vectors are to be kept (LOBPCG's X).  The basis is first
+// scaled to unit M-norm, s_i = M_ii^-1/2 (0 for a zero column), M' = S M S,
+// K' = S K S; a Cholesky factorisation of M' with pivoting takes the first nx
+// vectors before the others.  Of these it takes the one whose part M'-orthogonal to
+// the vectors taken is largest against its part orthogonal to the first nx, and ends
+// when the ratio of the squared norms is at most eps; a part below noise (squared)
+// is rounding of the Gram sums and is dropped too.  Z = L^-H of the vectors taken
+// (M'-orthonormal), C = Z^H K' Z = Y diag(lam) Y^H (Jacobi) and the Ritz vectors in
+// the original coordinates are Q = S Z Y.
+// What is dropped is thus a direction of [W, P] that X and the others span: span(X)
+// stays inside the projection and no step loses what X has reached.  (Dropping small
+// eigenvectors of M' instead, as Stathopoulos & Wu 2002, takes combinations with X
+// out: at 12 x 10 x 8 in FP32 the residual went from 2e-4 back to 0.9 whenever
+// rounding put one below the line.)  One CTA per pencil (blockIdx.x); K, M, Q n x n
+// row-major (double2) at b * n * n, n <= 64; M scaled by mscale.  Out:
+// lam[b][0..r) ascending, Q[b] columns 0..r (the rest zero), rank[b] = r.  Shared
+// memory: gen_eig_smem(n, blockDim.x).
+static __global__ void k_rank_eig(int n, int nx, const double2* __restrict__ K, const double2* __restrict__ M,
+                                  double mscale, double eps, double noise, double* __restrict__ lam,
+                                  double2* __restrict__ Q, int* __restrict__ rank) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double2* A = reinterpret_cast<double2*>(smem_raw);   // M, then C
-    double2* Vm = A + n * n;                            // eigenvectors of M, then Z
+    double2* Vm = A + n * n;                            // L, then K Z
     double2* Kh = Vm + n * n;
-    double2* Y = Kh + n * n;
+    double2* Y = Kh + n * n;                            // Z
     double2* rot = Y + n * n;
-    double* w = reinterpret_cast<double*>(rot + jacobi_rot_slots(n));
+    double* w = reinterpret_cast<double*>(rot + jacobi_rot_slots(n));   // squared norms of the parts left
     double* red = w + n;
-    int* perm = reinterpret_cast<int*>(red + 2 * blockDim.x);
-    __shared__ int r_sh;
-    __shared__ double dmax_sh;
-    __shared__ double sc[64];   // s_i (n <= 64)
+    int* perm = reinterpret_cast<int*>(red + 2 * blockDim.x);           // vectors taken, in order
+    __shared__ int piv_sh;
+    __shared__ double d_sh;
+    __shared__ double sc[64];    // s_i
+    __shared__ double ref[64];   // squared norms of the parts orthogonal to the first nx
     const int tid = threadIdx.x, nt = blockDim.x;
     const int b = blockIdx.x;
     const double2* Kb = K + (size_t)b * n * n;
@@ -306,6 +373,7 @@ static __global__ void k_svqb_eig(int n, const double2* __restrict__ K, const do
     for (int i = tid; i < n; i += nt) {
         const double d = mscale * Mb[i * n + i].x;
         sc[i] = d > 0.0 ? 1.0 / sqrt(d) : 0.0;
+        w[i] = d > 0.0 ? 1.0 : 0.0;
     }
     __syncthreads();
     for (int e = tid; e < n * n; e += nt) {
@@ -315,27 +383,61 @@ static __global__ void k_svqb_eig(int n, const double2* __restrict__ K, const do
         A[e] = make_double2(0.5 * sij * mscale * (m1.x + m2.x), 0.5 * sij * mscale * (m1.y - m2.y));
         const double2 k1 = Kb[i * n + j], k2 = Kb[j * n + i];
         Kh[e] = make_double2(0.5 * sij * (k1.x + k2.x), 0.5 * sij * (k1.y - k2.y));
+        Y[e] = make_double2(0.0, 0.0);
     }
     __syncthreads();
-    jacobi_herm(n, A, Vm, w, red, rot);
-    if (tid == 0) {
-        double dm = 0.0;
-        for (int i = 0; i < n; ++i) dm = fmax(dm, w[i]);
-        dmax_sh = dm;
-        int r = 0;   // kept directions, compacted to the front in original order
-        for (int i = 0; i < n; ++i)
-            if (w[i] > eps * dm && dm > 0.0) perm[r++] = i;
-        r_sh = r;
+    int r = 0;
+    bool first = true;   // thread 0: among the first nx
+    for (; r < n; ++r) {
+        if (tid == 0) {
+            int p = -1;
+            double best = noise;
+            for (int i = 0; i < nx && first; ++i)
+                if (w[i] > best) {
+                    best = w[i];
+                    p = i;
+                }
+            if (p < 0) {
+                if (first)
+                    for (int i = nx; i < n; ++i) ref[i] = w[i];
+                first = false;
+                best = eps;
+                for (int i = nx; i < n; ++i)
+                    if (w[i] > noise && w[i] > best * ref[i]) {
+                        best = w[i] / ref[i];
+                        p = i;
+                    }
+            }
+            piv_sh = p;
+            d_sh = p < 0 ? 0.0 : sqrt(w[p]);
+            perm[r] = p;
+        }
+        __syncthreads();
+        const int p = piv_sh;
+        if (p < 0) break;
+        const double d = d_sh;
+        for (int i = tid; i < n; i += nt) {
+            if (i == p) {
+                Vm[i * n + r] = make_double2(d, 0.0);
+                w[i] = -1.0;   // taken
+            } else if (w[i] >= 0.0) {
+                double2 s = A[i * n + p];
+                for (int k = 0; k < r; ++k) s = zsub(s, zmul(Vm[i * n + k], zconj(Vm[p * n + k])));
+                const double2 l = make_double2(s.x / d, s.y / d);
+                Vm[i * n + r] = l;
+                w[i] = fmax(w[i] - (l.x * l.x + l.y * l.y), 0.0);
+            }
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    const int r = r_sh;
-    // Z[:, c] = Vm[:, perm[c]] / sqrt(w[perm[c]]) into Y (n x r, row-major n x n storage)
-    for (int e = tid; e < n * r; e += nt) {
-        const int i = e / r, c = e % r;
-        const double s = 1.0 / sqrt(w[perm[c]]);
-        const double2 v = Vm[i * n + perm[c]];
-        Y[i * n + c] = make_double2(v.x * s, v.y * s);
-    }
+    // Z[:, c] = rows perm[0..c] of L^-H, by back substitution
+    for (int c = tid; c < r; c += nt)
+        for (int k = c; k >= 0; --k) {
+            double2 s = make_double2(k == c ? 1.0 : 0.0, 0.0);
+            for (int j = k + 1; j <= c; ++j) s = zsub(s, zmul(zconj(Vm[perm[j] * n + k]), Y[perm[j] * n + c]));
+            const double d = Vm[perm[k] * n + k].x;
+            Y[perm[k] * n + c] = make_double2(s.x / d, s.y / d);
+        }
     __syncthreads();
     // T = Kh Z (n x r) into Vm
     for (int e = tid; e < n * r; e += nt) {
