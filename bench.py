@@ -78,7 +78,7 @@ def parse():
                     help="with --kapply-only: precision of the timed chain (form = the form's), with --fft-variant "
                          "taken as given")
     ap.add_argument("--fft-variant", type=int, default=0, choices=[0, 1, 2],
-                    help="0: two-stage register FFT passes, 1: shared-memory Stockham passes, 2: cuFFT baseline")
+                    help="0: two-stage register FFT passes, 1: mixed-radix passes everywhere, 2: cuFFT baseline")
     ap.add_argument("--precond", default="green", choices=["green", "learned"],
                     help="green: the Green operator P^-1 (the paper); learned: train the learned Fourier-space "
                          "preconditioner first (untimed, reported under 'precond') and solve with it")

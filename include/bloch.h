@@ -98,8 +98,8 @@ typedef struct {
                             0 = host-driven loop with one synchronisation per iteration.
                             Default 1.                                                  */
     int32_t fft_variant; /* 0 = two-stage register FFT passes where the axis length is a
-                            power of two in [16, 256], shared-memory Stockham passes
-                            elsewhere; 1 = shared-memory Stockham passes everywhere;
+                            power of two in [16, 256], mixed-radix passes elsewhere;
+                            1 = mixed-radix passes everywhere;
                             2 = plain-form baseline: cuFFT 3D transforms with unfused
                             pointwise kernels.  All compute the same operator.
                             Default 0.                                                  */

@@ -29,11 +29,11 @@ struct Workspace {
     C* r = nullptr;         // 3 x V x cg_cap
     C* p = nullptr;
     C* Ap = nullptr;
-    double* part3 = nullptr;  // cg_cap x part_blocks x 3
+    double* part3 = nullptr;  // cg_cap x (blocks of a vector kernel or CTAs of the divergence pass) x 3
     double2* part2 = nullptr; // cg_cap x nblk_max
     double2* dots = nullptr;  // cg_cap
     CGSys* sys = nullptr;     // cg_cap
-    double2* partz = nullptr; // cg_cap x zblk: (p, Ap) partials of the fused x-stress or z-divergence pass
+    double2* partz = nullptr; // cg_cap x zblk: (p, Ap) partials of the stress pass
     int zblk = 0;
 };
 

@@ -32,12 +32,12 @@
 // components of a tile are spread over the CTA, so small tiles still fill its
 // threads; registers stay below the launch bounds (kPassCtas).
 //
-// Against the Stockham form these passes had before (tiles copied in, between
-// two buffers per stage and out; odd radices with run-time sines), K-apply:
-//   120 x 100 x 84, FP32, 6 systems   14.30 -> 0.67 ms
-//   256^3, FP32, 2 systems            14.26 -> 3.78 ms
-//   64^3, FP64, 4 systems              1.73 -> 1.51 ms (bound by FP64 issue)
-//   128^3, float-float, 4 systems      7.92 -> 4.72 ms (bound by FP32 issue)
+// K-apply before and after this form replaced two-buffer Stockham tiles (copied in,
+// between the buffers per stage and out; odd radices with run-time sines):
+//   120 x 100 x 84, FP32, 6 systems   14.28 -> 0.67 ms
+//   256^3, FP32, 2 systems            14.17 -> 3.81 ms
+//   64^3, FP64, 4 systems              1.73 -> 1.50 ms (bound by FP64 issue)
+//   128^3, float-float, 4 systems      7.90 -> 4.70 ms (bound by FP32 issue)
 #pragma once
 
 #include "cg.cuh"
