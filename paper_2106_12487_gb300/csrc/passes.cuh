@@ -35,9 +35,9 @@
 // K-apply before and after this form replaced two-buffer Stockham tiles (copied in,
 // between the buffers per stage and out; odd radices with run-time sines):
 //   120 x 100 x 84, FP32, 6 systems   14.28 -> 0.67 ms
-//   256^3, FP32, 2 systems            14.17 -> 3.81 ms
+//   256^3, FP32, 2 systems            14.26 -> 3.75 ms
 //   64^3, FP64, 4 systems              1.73 -> 1.50 ms (bound by FP64 issue)
-//   128^3, float-float, 4 systems      7.90 -> 4.70 ms (bound by FP32 issue)
+//   128^3, float-float, 4 systems      7.92 -> 4.61 ms (bound by FP32 issue)
 #pragma once
 
 #include "cg.cuh"
@@ -296,7 +296,8 @@ __global__ void __launch_bounds__(256, kPassCtasZ<T, WIDE>)
             const C* src = Ub + (size_t)c * g.V + pi0 + (ok ? p : 0) + (size_t)j * plane;
             C* s = buf + 2 * c * NP + u;
             // the scaled transform reads its inputs again (from L1) where the
-            // registers cannot hold both
+            // registers cannot hold both; 32-bit indices into the q table (with
+            // 64-bit addresses the wide form spills: 256^3 3.84 against 3.75 ms)
             constexpr bool keep = sizeof(T) == 4 && R <= 8;
             C v[R];
             if constexpr (keep) {
@@ -304,7 +305,7 @@ __global__ void __launch_bounds__(256, kPassCtasZ<T, WIDE>)
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     v[r] = src[(unsigned)(r * M) * plane];
-                    w[r] = cscale(v[r], qs(qz[r * M + j]));
+                    w[r] = cscale(v[r], qs(qz[(unsigned)(r * M + j)]));
                 }
                 RegDFT<R, +1, C>::run(v);
                 RegDFT<R, +1, C>::run(w);
@@ -322,7 +323,7 @@ __global__ void __launch_bounds__(256, kPassCtasZ<T, WIDE>)
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
                         v[r] = src[(unsigned)(r * M) * plane];
-                        if (h) v[r] = cscale(v[r], qs(qz[r * M + j]));
+                        if (h) v[r] = cscale(v[r], qs(qz[(unsigned)(r * M + j)]));
                     }
                     RegDFT<R, +1, C>::run(v);
                     s[0] = v[0];
