@@ -37,12 +37,12 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FALLBACK_HBM = 6800.0
 KAPPLY_BYTES_PER_VOXEL = {1: 436.0, 0: 868.0, 2: 868.0}   # algorithmic bytes per voxel, 5-pass chain (FF: 16 B complex)
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum over the five passes) per system of the
-# FP32 fast-pass K-apply at 128^3, from one ncu capture of a 4-system launch (1845.6 MB read +
-# 1550.9 MB written); it scales with the systems per launch.  Valid only while the pass sources hash
+# FP32 fast-pass K-apply at 128^3, from one ncu capture of a 4-system launch (1832.1 MB read +
+# 1521.4 MB written); it scales with the systems per launch.  Valid only while the pass sources hash
 # to `sources_sha256` (fpasses.cuh, fft.cuh, common.cuh in that order); otherwise traffic is null.
 KAPPLY_TRAFFIC = {"grid": (128, 128, 128), "precision": 1, "fft_variant": 0,
-                  "bytes_per_system": 3353.61e6 / 4,
-                  "sources_sha256": "fea70b8d0f88a8855330d72ca564cdc8dde59c650a2944f323000a7696557de5"}
+                  "bytes_per_system": 3353.47e6 / 4,
+                  "sources_sha256": "f06f136dd1beb7cb1c707d9ef2f210dcea2edd7644760771e2ab5efd5df95a20"}
 
 
 def parse():
